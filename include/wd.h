@@ -234,8 +234,8 @@ WD_API wd_status wd_set_fusion(wd_ctx* ctx, int32_t mode);
  * recorded into a graph (a normal step with full active windows at once, any other step the second time its
  * configuration occurs) and replayed
  * from then on (at most 8 graphs per context, least recently used replaced); the planner kernel and the
- * copy of the result block stay ordinary launches on the caller's stream.  Graphs need the tensor-core
- * kernels (bf16, head_dim 128) and are used only while earlier steps are still queued: a caller that calls
+ * copy of the result block stay ordinary launches on the caller's stream.  bf16 models need the
+ * tensor-core kernels (head_dim 128) for it.  Graphs are used only while earlier steps are still queued: a caller that calls
  * wd_step_sync after every step gets direct launches, which are faster then.  Steps with debug taps, with
  * profiling on, with a fused-consumer mode, planned on the host, or issued on a stream that is itself being
  * captured or that cannot be captured (the legacy default stream) are launched directly.  Results are

@@ -1009,12 +1009,11 @@ static wd_status run_gemm(wd_ctx* c, const void* x, const WdTcX* x_map, const Wd
         *go = {n_split, (size_t)rows * ncol, 1, WD_GEMM_TCGEN05};
     } else {
         if ((size_t)rows * ncol > y_floats) return WD_ERR_CAPACITY;
-        int col = 0;
-        for (int i = 0; i < nseg; ++i) {
-            wd_launch_gemm_plain(c->d.dtype, x, segs[i].w, y + col, rows, segs[i].n, K, ncol, stream);
-            col += segs[i].n;
-        }
-        *go = {1, (size_t)rows * ncol, nseg, WD_GEMM_PLAIN};
+        const void* w[3];
+        int n[3];
+        for (int i = 0; i < nseg; ++i) { w[i] = segs[i].w; n[i] = segs[i].n; }
+        wd_launch_gemm_plain(c->d.dtype, x, w, n, nseg, y, rows, K, ncol, /*w_static=*/true, stream);
+        *go = {1, (size_t)rows * ncol, 1, WD_GEMM_PLAIN};
     }
     if (e1) WD_CUDA_TRY(cudaEventRecord(e1, stream));
     return WD_OK;
@@ -1480,10 +1479,11 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     // graph.  With an empty queue (a caller that syncs after every step) direct launches win, because the GPU
     // starts on the first kernels while the host is still launching the later ones (measured: 230 against 227
     // tokens/s end to end).
-    // The tensor-core attention only: the index-list kernel sizes its shared memory by the exact visible count,
-    // which a recorded launch would keep while the count grows.
-    const bool attn_by_tc = st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN;
-    if (c->graphs_on && dev_mode && !c->prof_on && !taps_on && !fused && !stream_capturing && use_tc(c) && attn_by_tc &&
+    // bf16 needs the tensor-core attention.  fp32 steps take the index-list kernel with room for whole key tiles (its
+    // scores in shared memory), so a recorded launch holds while the visible count grows within the last tile.
+    const bool attn_by_tc = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN;
+    const bool attn_by_tiles = d.dtype == WD_F32 && (wd_align_up((size_t)max_vis, 128) + dh) * 4 <= 200 * 1024;
+    if (c->graphs_on && dev_mode && !c->prof_on && !taps_on && !fused && !stream_capturing && (attn_by_tc || attn_by_tiles) &&
         !st->queue.empty()) {
         wd_ctx::StepKey key;
         key.state_uid = st->uid; key.batch = batch; key.rows = R_; key.n_act = NA; key.n_qtiles = (int)n_qtiles;
@@ -1819,7 +1819,7 @@ extern "C" wd_status wd_op_gemm(int32_t dtype, int32_t impl, const void* x, cons
     if (dtype != WD_F32 && dtype != WD_BF16) return WD_ERR_BAD_PARAM;
     if (impl == WD_GEMM_AUTO) impl = dtype == WD_BF16 ? WD_GEMM_TCGEN05 : WD_GEMM_PLAIN;
     if (impl == WD_GEMM_PLAIN) {
-        wd_launch_gemm_plain(dtype, x, w, y, rows, n_out, k_in, n_out, (cudaStream_t)stream);
+        wd_launch_gemm_plain(dtype, x, &w, &n_out, 1, y, rows, k_in, n_out, /*w_static=*/false, (cudaStream_t)stream);
         WD_CUDA_TRY(cudaGetLastError());
         return WD_OK;
     }

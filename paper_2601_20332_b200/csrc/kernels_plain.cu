@@ -2,9 +2,9 @@
 //
 // These are the bandwidth- and latency-bound pieces around the GEMMs (embedding
 // gather, RMSNorm, RoPE + K/V scatter, SwiGLU, residual add, unmask reduction)
-// plus CUDA-core versions of the GEMM and of attention that work for any dtype
-// and any index list; the fp32 configuration runs on them entirely and the
-// bf16 tensor-core kernels are cross-checked against them.
+// plus a CUDA-core version of attention that works for any dtype and any index
+// list; the fp32 configuration runs on it entirely and the bf16 tensor-core
+// kernel is cross-checked against it.
 #include <cstdlib>
 #include <cstring>
 #include <utility>
@@ -574,52 +574,6 @@ __global__ void __launch_bounds__(1024, 1) rmsnorm_fp4_kernel(float* __restrict_
     }
 }
 
-// ---------------------------------------------------------------- CUDA-core GEMM
-// y[rows, n] = x[rows, k] * w[n, k]^T.  32 x 64 output tile per block, 2 x 4 per thread.
-template <typename T>
-__global__ void gemm_plain_kernel(const T* __restrict__ x, const T* __restrict__ w, float* __restrict__ y,
-                                  int rows, int n, int k, int ldy) {
-    __shared__ float xs[32][33];
-    __shared__ float ws[64][33];
-    pdl_launch_dependents();
-    pdl_wait();
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;          // 16 x 16
-    const int r0 = blockIdx.y * 32, n0 = blockIdx.x * 64;
-    float acc[2][4] = {};
-    for (int k0 = 0; k0 < k; k0 += 32) {
-        for (int i = threadIdx.x; i < 32 * 32; i += 256) {
-            const int rr = i >> 5, kk = i & 31;
-            xs[rr][kk] = (r0 + rr < rows && k0 + kk < k) ? to_f(x[(size_t)(r0 + rr) * k + k0 + kk]) : 0.f;
-        }
-        for (int i = threadIdx.x; i < 64 * 32; i += 256) {
-            const int nn = i >> 5, kk = i & 31;
-            ws[nn][kk] = (n0 + nn < n && k0 + kk < k) ? to_f(w[(size_t)(n0 + nn) * k + k0 + kk]) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) {
-            const float a0 = xs[ty][kk], a1 = xs[ty + 16][kk];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float b = ws[tx + 16 * j][kk];
-                acc[0][j] += a0 * b;
-                acc[1][j] += a1 * b;
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int r = r0 + ty + 16 * i;
-        if (r >= rows) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = n0 + tx + 16 * j;
-            if (c < n) y[(size_t)r * ldy + c] = acc[i][j];
-        }
-    }
-}
-
 // ---------------------------------------------------------------- RoPE + K/V scatter
 // Adds the split-K slices of the fused q/k/v projection, rotates q and k heads by the row's
 // table, writes q and the K/V cache rows.  K cache [batch][Hkv][S][dh]; V cache transposed
@@ -744,14 +698,43 @@ __global__ void __launch_bounds__(256, 4) rope_scatter_kernel(const float* __res
 }
 
 // ---------------------------------------------------------------- CUDA-core attention
-// One block (128 threads) per (row, head).  Scores of all visible positions in shared
-// memory, then softmax, then the weighted sum of V rows.
-template <typename T>
-__global__ void attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
-                                       const T* __restrict__ vcache, const int32_t* __restrict__ row_seq,
-                                       const int32_t* __restrict__ vis_idx, const int32_t* __restrict__ vis_off,
-                                       T* __restrict__ out, float* __restrict__ tap, int nv_single, int Hq,
-                                       int Hkv, int dh, int S, int Sp, int batch, int32_t* __restrict__ status) {
+// One block (256 threads) per (row, head).  Scores of all visible positions in shared memory, then softmax, then the
+// weighted sum of V rows.  With few keys the block is as long as its chain of memory round trips, so both products keep
+// many loads in flight: a key takes eight lanes (16-byte loads of its row) and a warp sixteen keys at a time; V, stored
+// transposed ([dh][Sp]), takes eight head dims per warp at a time with the lanes over the positions, the eight sums
+// reduced together by halving.  kVec: head_dim is at most 4 * 8 * 16 bytes and a multiple of 16 bytes and the rows are
+// aligned; otherwise a key takes a whole warp, one element per lane.  Measured (fp32, 4 heads of 64, 56 to 96 keys, 9 to 60
+// rows): 4.6 to 5.7 us; with a key per warp and a head dim per warp at a time it took 25 to 31 us.
+template <typename T> struct Vec16;
+template <> struct Vec16<float> {
+    static constexpr int N = 4;
+    static __device__ __forceinline__ void load(const float* p, float (&v)[4]) {
+        const float4 u = *reinterpret_cast<const float4*>(p);
+        v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+    }
+};
+template <> struct Vec16<__nv_bfloat16> {
+    static constexpr int N = 8;
+    static __device__ __forceinline__ void load(const __nv_bfloat16* p, float (&v)[8]) {
+        const uint4 u = *reinterpret_cast<const uint4*>(p);
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v[2 * i] = __uint_as_float(w[i] << 16);
+            v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+        }
+    }
+};
+
+constexpr int kAttnThreads = 256;
+
+template <typename T, bool kVec>
+__global__ void __launch_bounds__(kAttnThreads)
+attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
+                       const T* __restrict__ vcache, const int32_t* __restrict__ row_seq,
+                       const int32_t* __restrict__ vis_idx, const int32_t* __restrict__ vis_off,
+                       T* __restrict__ out, float* __restrict__ tap, int nv_single, int Hq,
+                       int Hkv, int dh, int S, int Sp, int batch, int32_t* __restrict__ status) {
     extern __shared__ float sc[];                 // [n_vis] scores, then dh floats of q
     __shared__ float red[32];
     pdl_launch_dependents();
@@ -767,29 +750,80 @@ __global__ void attention_plain_kernel(const T* __restrict__ q, const T* __restr
     const int kvh = h / (Hq / Hkv);
     const T* kb = kcache + ((size_t)b * Hkv + kvh) * S * dh;
     const T* vb = vcache + ((size_t)b * Hkv + kvh) * dh * Sp;     // [dh][Sp]
-    float* qs = sc + nv;
-    for (int c = threadIdx.x; c < dh; c += blockDim.x) qs[c] = to_f(q[((size_t)r * Hq + h) * dh + c]);
-    __syncthreads();
+    const T* qr = q + ((size_t)r * Hq + h) * dh;
     const float scale = rsqrtf((float)dh);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int nw = kAttnThreads / 32;
     float mx = -INFINITY;
-    for (int j = wid; j < nv; j += nw) {
-        const int vi = vis_idx[v0 + j];
-        if ((unsigned)vi >= (unsigned)S) {             // index check: recorded, the position is left out (weight 0)
-            if (lane == 0) { atomicCAS(status, 0, WD_ERR_BOUNDS); sc[j] = -INFINITY; }
-            continue;
+    if (kVec) {
+        constexpr int N = Vec16<T>::N, kU = 4, kMaxVec = 4;    // keys in flight per lane group; 16-byte pieces of a row per lane
+        const int l8 = lane & 7, kg = lane >> 3, nvec = dh / N;
+        float qv[kMaxVec][N];
+#pragma unroll
+        for (int i = 0; i < kMaxVec; ++i)
+            if (l8 + 8 * i < nvec) Vec16<T>::load(qr + (l8 + 8 * i) * N, qv[i]);
+        for (int j0 = wid * 4 * kU; j0 < nv; j0 += nw * 4 * kU) {
+            int vi[kU];
+            bool ok[kU];
+            float a[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int j = j0 + 4 * u + kg;
+                vi[u] = j < nv ? vis_idx[v0 + j] : 0;
+                ok[u] = (unsigned)vi[u] < (unsigned)S;
+                a[u] = 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < kMaxVec; ++i) {
+                if (8 * i >= nvec) break;
+                float kv[kU][N];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (l8 + 8 * i < nvec) Vec16<T>::load(kb + (size_t)(ok[u] ? vi[u] : 0) * dh + (l8 + 8 * i) * N, kv[u]);
+                if (l8 + 8 * i < nvec) {
+#pragma unroll
+                    for (int u = 0; u < kU; ++u)
+#pragma unroll
+                        for (int e = 0; e < N; ++e) a[u] = fmaf(qv[i][e], kv[u][e], a[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int j = j0 + 4 * u + kg;
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) a[u] += __shfl_xor_sync(0xffffffffu, a[u], o);
+                if (j >= nv) continue;
+                // index check: a position outside the sequence is recorded and left out (weight 0)
+                const float s = ok[u] ? a[u] * scale : -INFINITY;
+                if (l8 == 0) {
+                    if (!ok[u]) atomicCAS(status, 0, WD_ERR_BOUNDS);
+                    sc[j] = s;
+                }
+                mx = fmaxf(mx, s);
+            }
         }
-        const T* kr = kb + (size_t)vi * dh;
-        float a = 0.f;
-        for (int c = lane; c < dh; c += 32) a += qs[c] * to_f(kr[c]);
-        a = warp_sum(a) * scale;
-        if (lane == 0) sc[j] = a;
-        mx = fmaxf(mx, a);
+    } else {
+        float* qs = sc + nv;
+        for (int c = threadIdx.x; c < dh; c += kAttnThreads) qs[c] = to_f(qr[c]);
+        __syncthreads();
+        for (int j = wid; j < nv; j += nw) {
+            const int vi = vis_idx[v0 + j];
+            if ((unsigned)vi >= (unsigned)S) {
+                if (lane == 0) { atomicCAS(status, 0, WD_ERR_BOUNDS); sc[j] = -INFINITY; }
+                continue;
+            }
+            const T* kr = kb + (size_t)vi * dh;
+            float a = 0.f;
+            for (int c = lane; c < dh; c += 32) a += qs[c] * to_f(kr[c]);
+            a = warp_sum(a) * scale;
+            if (lane == 0) sc[j] = a;
+            mx = fmaxf(mx, a);
+        }
     }
     mx = block_max(mx, red);
     __syncthreads();
     float sum = 0.f;
-    for (int j = threadIdx.x; j < nv; j += blockDim.x) {
+    for (int j = threadIdx.x; j < nv; j += kAttnThreads) {
         const float e = __expf(sc[j] - mx);
         sc[j] = e;
         sum += e;
@@ -797,20 +831,37 @@ __global__ void attention_plain_kernel(const T* __restrict__ q, const T* __restr
     sum = block_sum(sum, red);
     __syncthreads();
     const float inv = 1.f / sum;
-    // V is stored transposed ([dh][Sp]): each warp takes head dims c = wid, wid + nw, ... and its
-    // lanes stride over the visible positions, so consecutive lanes read consecutive positions
-    for (int c = wid; c < dh; c += nw) {
-        const T* vr = vb + (size_t)c * Sp;
-        float a = 0.f;
+    for (int c0 = 8 * wid; c0 < dh; c0 += 8 * nw) {
+        float a[8] = {};
+        const T* vr[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) vr[c] = vb + (size_t)min(c0 + c, dh - 1) * Sp;
+#pragma unroll 2
         for (int j = lane; j < nv; j += 32) {
             const int vi = vis_idx[v0 + j];
-            if ((unsigned)vi < (unsigned)S) a += sc[j] * to_f(vr[vi]);
+            if ((unsigned)vi < (unsigned)S) {
+                const float p = sc[j];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) a[c] = fmaf(p, to_f(vr[c][vi]), a[c]);
+            }
         }
-        a = warp_sum(a) * inv;
-        if (lane == 0) {
+        // eight sums over 32 lanes: after the steps over lane bits 4, 3, 2 a lane holds one of them
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            const bool up = (lane & (4 * o)) != 0;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+                const float send = up ? a[i] : a[i + o], keep = up ? a[i + o] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * o);
+            }
+        }
+        a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+        a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+        const int c = c0 + (lane >> 2);
+        if ((lane & 3) == 0 && c < dh) {
             const size_t o = ((size_t)r * Hq + h) * dh + c;
-            out[o] = from_f<T>(a);
-            if (tap) tap[o] = a;
+            out[o] = from_f<T>(a[0] * inv);
+            if (tap) tap[o] = a[0] * inv;
         }
     }
 }
@@ -1231,14 +1282,6 @@ void wd_launch_rmsnorm(int dtype, float* x, const float* part, int n_split, size
     }
 }
 
-void wd_launch_gemm_plain(int dtype, const void* x, const void* w, float* y, int rows, int n, int k,
-                          int ldy, cudaStream_t st) {
-    if (rows <= 0 || n <= 0) return;
-    dim3 grid(wd_ceil_div(n, 64), wd_ceil_div(rows, 32));
-    WD_DISPATCH(dtype, launch_pdl(gemm_plain_kernel<T>, grid, dim3(256), 0, st, (const T*)x, (const T*)w, y, rows, n,
-                                  k, ldy));
-}
-
 void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t split_stride,
                             const int32_t* row_seq, const int32_t* row_pos, const float2* rope_tab, void* q,
                             void* kcache, void* vcache, int n_rows, int Hq, int Hkv, int dh, int S, int Sp,
@@ -1254,25 +1297,37 @@ void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t sp
                                   Hkv, dh, S, Sp, n_qk, qk_groups, n_qk_blocks, batch, status));
 }
 
+template <typename T, bool kVec>
+static void launch_attention_plain(dim3 grid, size_t smem, cudaStream_t st, const void* q, const void* kcache, const void* vcache,
+                                   const int32_t* row_seq, const int32_t* vis_idx, const int32_t* vis_off, void* out, float* tap,
+                                   int max_vis, int Hq, int Hkv, int dh, int S, int Sp, int batch, int32_t* status) {
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(attention_plain_kernel<T, kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_pdl(attention_plain_kernel<T, kVec>, grid, dim3(kAttnThreads), smem, st, (const T*)q, (const T*)kcache, (const T*)vcache,
+               row_seq, vis_idx, vis_off, (T*)out, tap, max_vis, Hq, Hkv, dh, S, Sp, batch, status);
+}
+
 void wd_launch_attention_plain(int dtype, const void* q, const void* kcache, const void* vcache,
                                const int32_t* row_seq, const int32_t* vis_idx, const int32_t* vis_off,
                                void* out, float* tap, int n_rows, int max_vis, int Hq, int Hkv, int dh,
                                int S, int Sp, int batch, int32_t* status, cudaStream_t st) {
     if (n_rows <= 0) return;
-    const size_t smem = (size_t)(max_vis + dh) * sizeof(float);
-    dim3 grid(n_rows, Hq);
+    // room for a multiple of 128 scores, so that the launch does not depend on the exact visible count: a recorded step
+    // keeps it while the count grows within a key tile (up to the 200 KB that a single call may ask for)
+    const size_t room = (size_t)wd_align_up((size_t)max_vis, 128) + dh;
+    const size_t smem = (room * 4 <= 200 * 1024 ? room : (size_t)max_vis + dh) * sizeof(float);
+    const dim3 grid(n_rows, Hq);
+    const bool vec = (dh * (int)wd_elt_size(dtype)) % 16 == 0 && dh * (int)wd_elt_size(dtype) <= 512 &&
+                     ((uintptr_t)q | (uintptr_t)kcache) % 16 == 0;
+#define WD_ATTN_ARGS grid, smem, st, q, kcache, vcache, row_seq, vis_idx, vis_off, out, tap, max_vis, Hq, Hkv, dh, S, Sp, batch, status
     if (dtype == WD_F32) {
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(attention_plain_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(attention_plain_kernel<float>, grid, dim3(128), smem, st, (const float*)q, (const float*)kcache,
-                   (const float*)vcache, row_seq, vis_idx, vis_off, (float*)out, tap, max_vis, Hq, Hkv, dh, S, Sp, batch, status);
+        if (vec) launch_attention_plain<float, true>(WD_ATTN_ARGS);
+        else launch_attention_plain<float, false>(WD_ATTN_ARGS);
     } else {
-        using T = __nv_bfloat16;
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(attention_plain_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(attention_plain_kernel<T>, grid, dim3(128), smem, st, (const T*)q, (const T*)kcache,
-                   (const T*)vcache, row_seq, vis_idx, vis_off, (T*)out, tap, max_vis, Hq, Hkv, dh, S, Sp, batch, status);
+        if (vec) launch_attention_plain<__nv_bfloat16, true>(WD_ATTN_ARGS);
+        else launch_attention_plain<__nv_bfloat16, false>(WD_ATTN_ARGS);
     }
+#undef WD_ATTN_ARGS
 }
 
 void wd_launch_swiglu(int dtype, const float* part, int n_split, size_t split_stride, void* h,

@@ -112,9 +112,10 @@ void wd_launch_rmsnorm(int dtype, float* x, const float* part, int n_split, size
 // (xq != null: FP8 output instead of xn: e4m3 codes [n_rows][d] and one scale per row;
 //  x4 != null: NVFP4 output instead of xn, quantised from the bfloat16 rounding of the normalised row; d % 16 == 0)
 
-// plain GEMM: y[rows, n] (float) = x[rows,k] * w[n,k]^T
-void wd_launch_gemm_plain(int dtype, const void* x, const void* w, float* y, int rows, int n, int k,
-                          int ldy, cudaStream_t st);
+// plain GEMM (gemm_plain.cu): y[rows, n_0 + n_1 + ...] (float, leading dimension ldy) = x[rows,k] * [w_0; w_1; ...]^T for up
+// to three matrices.  w_static: the weights were complete before the previous kernel of the stream started.
+void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const int* n, int n_mat, float* y, int rows, int k,
+                          int ldy, bool w_static, cudaStream_t st);
 
 // qkv partials -> RoPE -> q (dtype) and K/V cache rows.
 //   part: [n_split][n_rows][(Hq+2Hkv)*dh] float, columns = [q | k | v]
