@@ -18,10 +18,15 @@
 //   warp 1      MMA issuer
 //   warps 2-5   epilogue: tcgen05.ld, row scales, coalesced fp32 stores of this K slice's partial sums
 //   warps 6-9   block scales: shared memory -> tensor memory
-// Work units are (weight tile, token tile, K slice), dealt round-robin to one CTA per SM; K slices are
-// written side by side ([slice][tok][n]) and added by the consumer, as in the bf16 kernel.
+// Persistent, one CTA per SM: the K blocks of all (weight tile, token tile) units form one line that is cut into
+// equal shares (stream-K), or whole units per CTA when that is cheaper.  The partial sums of a unit that several
+// CTAs share are written side by side ([slice][tok][n]) and added by the consumer, as in the bf16 kernel.
+// Measured at 34 rows, quantised input to summed result, 12288 x 4096 / 24576 x 4096 / 4096 x 12288: 16.9 / 22.1 / 17.9 us
+// against 4.7 / 9.3 / 4.6 us for the bytes alone; what remains is start-up (2-3 us to the first complete stage, 2 us from the
+// last MMA to the stores) around 0.44 us a stage.  (Bringing the weights into the L2 ahead of the dependency wait made it
+// slower: 24.4 instead of 23.8 us for the middle shape, 107 instead of 90 us at 600 rows.)
 // Every wait is bounded; on expiry the CTA records WD_ERR_DEVICE_TIMEOUT and leaves.
-#include <cstdlib>
+#include <algorithm>
 #include <cstring>
 
 #include <cuda_fp8.h>
@@ -40,7 +45,8 @@ constexpr int kSfW = kBM * 16;        // 2 KB of weight block scales
 constexpr int kThreads = 320;
 
 struct Fp4Params {
-    int rows, n_out, bn, kb_total, tok_tiles, n_tiles, n_slices, n_units, n_stages, buf_cols;
+    int rows, n_out, bn, kb_total, tok_tiles, n_slices, n_units, n_stages, buf_cols;
+    int aligned;                      // whole units per CTA (one slice) instead of equal pieces of the K-block line
     int w_static;                     // the weights were written before the previous kernel started
     float* y;
     size_t split_stride;
@@ -76,26 +82,24 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     uint64_t* sf_free = sf_full + 2;
     uint32_t* tmem_slot = (uint32_t*)(sf_free + 2);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    float* gx_s = (float*)(tmem_slot + 4);           // [128] row scales of the epilogue's token tile
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int G = gridDim.x, c = blockIdx.x;
-    const int n_my = c < p.n_units ? (p.n_units - c + G - 1) / G : 0;
-    // unit -> (tile, token tile, K slice); slices innermost, so neighbouring CTAs share a weight tile's rows
-    auto decode = [&](int u, int& n0, int& tok0, int& sl, int& kb0, int& kbn) {
-        const int unit = c + u * G;
-        sl = unit % p.n_slices;
-        const int rest = unit / p.n_slices;
-        tok0 = (rest % p.tok_tiles) * p.bn;
-        n0 = (rest / p.tok_tiles) * kBM;
-        kb0 = sl * p.kb_total / p.n_slices;
-        kbn = (sl + 1) * p.kb_total / p.n_slices - kb0;
+    // This CTA's share [g_begin, g_end) of the line of K blocks of all units, unit = weight tile * tok_tiles + token tile
+    // (neighbouring units share a weight tile): equal shares, so every SM streams the same bytes, or whole units.
+    const int G = gridDim.x, c = blockIdx.x, KB = p.kb_total, W = p.n_units * KB;
+    const int g_begin = p.aligned ? (int)((long long)c * p.n_units / G) * KB : (int)((long long)c * W / G);
+    const int g_end = p.aligned ? (int)((long long)(c + 1) * p.n_units / G) * KB : (int)((long long)(c + 1) * W / G);
+    const int n_total = g_end - g_begin;
+    // the piece that starts at K block g of the line: its unit's rows and tokens, first K block and length
+    auto piece_at = [&](int g, int& unit, int& n0, int& tok0, int& kb0, int& len) {
+        unit = g / KB;
+        kb0 = g - unit * KB;
+        len = min(KB - kb0, g_end - g);
+        const int tile = unit / p.tok_tiles;
+        n0 = tile * kBM;
+        tok0 = (unit - tile * p.tok_tiles) * p.bn;
     };
-    int n_total = 0;
-    for (int u = 0; u < n_my; ++u) {
-        int n0, tok0, sl, kb0, kbn;
-        decode(u, n0, tok0, sl, kb0, kbn);
-        n_total += kbn;
-    }
     const uint32_t tmem_cols = 2u * (uint32_t)p.buf_cols + 64u <= 128u ? 128u : (2u * (uint32_t)p.buf_cols + 64u <= 256u ? 256u : 512u);
 
     pdl_launch_dependents();
@@ -112,6 +116,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (const CUtensorMap* m : {&map_w, &map_sw, &map_x, &map_sx}) asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(tmem_slot), tmem_cols);
     tc_fence_before();
@@ -125,16 +130,15 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             // ------------------------------------------------ TMA producer
             uint64_t pol_stream;
             asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
-            struct Walk { int u, left, kb, n0, tok0; };
+            struct Walk { int g, left, kb, n0, tok0; };
             auto enter = [&](Walk& w) {
-                int sl, kb0, kbn;
-                decode(w.u, w.n0, w.tok0, sl, kb0, kbn);
-                w.kb = kb0;
-                w.left = kbn;
+                int unit;
+                piece_at(w.g, unit, w.n0, w.tok0, w.kb, w.left);
             };
             auto advance = [&](Walk& w) {
                 ++w.kb;
-                if (--w.left == 0 && ++w.u < n_my) enter(w);
+                ++w.g;
+                if (--w.left == 0 && w.g < g_end) enter(w);
             };
             auto load_w = [&](const Walk& w, int s) {
                 const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes), full = smem_u32(&bars[s]);
@@ -148,14 +152,18 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 tma_load_2d(sa + kStageW + x_bytes + kSfW, &map_sx, full, w.kb * 16, w.tok0);
             };
             Walk w, wx;
-            w.u = 0;
+            w.g = g_begin;
             enter(w);
             wx = w;
             const int n_pre = n_total < NS ? n_total : NS;
-            if (!p.w_static) pdl_wait();
-            for (int i = 0; i < n_pre; ++i, advance(w)) load_w(w, i);        // weights first when they depend on nothing
-            if (p.w_static) pdl_wait();
-            for (int i = 0; i < n_pre; ++i, advance(wx)) load_x(wx, i);
+            if (p.w_static) {        // weights first: they depend on nothing
+                for (int i = 0; i < n_pre; ++i, advance(w)) load_w(w, i);
+                pdl_wait();
+                for (int i = 0; i < n_pre; ++i, advance(wx)) load_x(wx, i);
+            } else {                 // stage by stage, so that the first is complete as early as possible
+                pdl_wait();
+                for (int i = 0; i < n_pre; ++i, advance(w)) { load_w(w, i); load_x(w, i); }
+            }
             int s = n_pre % NS;
             uint32_t ph = (uint32_t)(n_pre / NS) & 1u;
             for (int i = n_pre; i < n_total; ++i, advance(w)) {
@@ -176,9 +184,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             bool ok = true;
             int s = 0, i = 0;
             uint32_t ph = 0;
-            for (int u = 0; u < n_my && ok; ++u) {
-                int n0, tok0, sl, kb0, kbn;
-                decode(u, n0, tok0, sl, kb0, kbn);
+            for (int g = g_begin, u = 0; g < g_end && ok; ++u) {
+                int unit, n0, tok0, kb0, kbn;
+                piece_at(g, unit, n0, tok0, kb0, kbn);
+                g += kbn;
                 const int buf = u & 1;
                 const uint32_t par = (uint32_t)(u >> 1) & 1u;
                 if (!(ok = mbar_wait(smem_u32(&acc_empty[buf]), par ^ 1u, abort_flag))) break;
@@ -214,18 +223,29 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         const int n_local = quarter * 32 + lane;
         pdl_wait();
         bool ok = true;
-        for (int u = 0; u < n_my; ++u) {
-            int n0, tok0, sl, kb0, kbn;
-            decode(u, n0, tok0, sl, kb0, kbn);
+        for (int g = g_begin, u = 0; g < g_end; ++u) {
+            int unit, n0, tok0, kb0, kbn;
+            piece_at(g, unit, n0, tok0, kb0, kbn);
+            g += kbn;
+            // slice: this CTA's place among those that share the unit
+            const int sl = p.aligned ? 0 : c - (int)((((long long)unit * KB + 1) * G - 1) / W);
             const int buf = u & 1;
             const uint32_t par = (uint32_t)(u >> 1) & 1u;
             const int n = n0 + n_local;
             const bool n_ok = n < p.n_out;
+            // the row scales while the MMAs still run: the tokens' through shared memory, the weight row's in a register
+            asm volatile("bar.sync 1, 128;" ::: "memory");          // the previous piece's readers are done
+            const int e = (int)threadIdx.x - 64;
+            if (e < p.bn) gx_s[e] = tok0 + e < p.rows ? __ldg(p.gx + tok0 + e) : 0.f;
+            const float gwn = n_ok ? p.gw[n] : 0.f;
+            asm volatile("bar.sync 1, 128;" ::: "memory");
             ok = ok && mbar_wait(smem_u32(&acc_full[buf]), par, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
+            if (!ok) {               // (stays in the loop: every warp reaches the same barriers)
+                *abort_flag = 1;
+                continue;
+            }
             tc_fence_after();
-            const float gwn = n_ok ? p.gw[n] : 0.f;
             float* ys = p.y + (size_t)sl * p.split_stride + n;
             const uint32_t t_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.buf_cols);
             for (int cc = 0; cc < p.bn; cc += 16) {
@@ -236,12 +256,19 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 #pragma unroll
                     for (int t = 0; t < 16; ++t) {
                         const int tok = tok0 + cc + t;
-                        if (tok < p.rows) ys[(size_t)tok * p.n_out] = __uint_as_float(v[t]) * gwn * __ldg(p.gx + tok);
+                        if (tok < p.rows) ys[(size_t)tok * p.n_out] = __uint_as_float(v[t]) * gwn * gx_s[cc + t];
                     }
                 }
             }
             tc_fence_before();
             mbar_arrive(smem_u32(&acc_empty[buf]));
+            if (kb0 + kbn == KB && n_ok) {
+                // this CTA finished the unit: slices that nobody wrote must read as zero
+                for (int z = sl + 1; z < p.n_slices; ++z) {
+                    float* yz = p.y + (size_t)z * p.split_stride + n;
+                    for (int tok = tok0; tok < tok0 + p.bn && tok < p.rows; ++tok) yz[(size_t)tok * p.n_out] = 0.f;
+                }
+            }
         }
         if (!ok && lane == 0) {
             *abort_flag = 1;
@@ -293,47 +320,86 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 }
 
 // ---------------------------------------------------------------- quantisation
-template <typename T> __device__ __forceinline__ float ldf(const T* p);
-template <> __device__ __forceinline__ float ldf<float>(const float* p) { return __bfloat162float(__float2bfloat16_rn(*p)); }
-template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+// sixteen elements as bfloat16 pairs in eight words (a float input is rounded to bfloat16 first)
+__device__ __forceinline__ void ld_block16(const float* p, bool vec, uint32_t (&w)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float2 v = vec ? reinterpret_cast<const float2*>(p)[i] : make_float2(p[2 * i], p[2 * i + 1]);
+        const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+        w[i] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+}
+__device__ __forceinline__ void ld_block16(const __nv_bfloat16* p, bool vec, uint32_t (&w)[8]) {
+    if (vec) {
+        const uint4 a = reinterpret_cast<const uint4*>(p)[0], b = reinterpret_cast<const uint4*>(p)[1];
+        w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+    } else {
+        const uint16_t* q = reinterpret_cast<const uint16_t*>(p);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = (uint32_t)q[2 * i] | ((uint32_t)q[2 * i + 1] << 16);
+    }
+}
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+__device__ __forceinline__ float block_amax(const uint32_t (&w)[8]) {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = fmaxf(m, fmaxf(fabsf(bf_lo(w[i])), fabsf(bf_hi(w[i]))));
+    return m;
+}
 
 // One block per row: row scale g = max|row| / (6 * 448) (1 for a zero row); per 16-element block the scale
-// s = e4m3((max|block| / 6) / g) and the codes e2m1(x / (s * g)).  The input is taken as bfloat16 (a float
-// input is rounded first).  K is a multiple of 16.
+// s = e4m3((max|block| / 6) / g) and the codes e2m1(x / (s * g)).  The input is taken as bfloat16.  K is a multiple of 16.
+// A thread owns one 16-element block, loaded once in two 16-byte pieces and kept in registers between the two passes (the
+// blocks beyond kQuantThreads of a long row are read again from the L1): with few rows the kernel is one memory round trip,
+// one reduction and the arithmetic.  Measured with 34 rows: K 4096 2.9 us, K 12288 4.3 us (6.2 and 15.1 us with single
+// elements read in either pass).
+constexpr int kQuantThreads = 1024;
 template <typename T>
-__global__ void quantize_nvfp4_kernel(const T* __restrict__ x, int K, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
-                                      float* __restrict__ g_out) {
+__global__ void __launch_bounds__(kQuantThreads)
+quantize_nvfp4_kernel(const T* __restrict__ x, int K, int vec, uint8_t* __restrict__ codes, uint8_t* __restrict__ sf,
+                      float* __restrict__ g_out) {
     __shared__ float red[32];
     pdl_launch_dependents();
     pdl_wait();
     const size_t row = blockIdx.x;
     const T* xr = x + row * (size_t)K;
-    float amax = 0.f;
-    for (int i = threadIdx.x; i < K; i += blockDim.x) amax = fmaxf(amax, fabsf(ldf<T>(xr + i)));
+    const int nb = K >> 4;
+    uint32_t w[8];
+    float bmax = 0.f, amax = 0.f;
+    if ((int)threadIdx.x < nb) {
+        ld_block16(xr + 16 * threadIdx.x, vec != 0, w);
+        amax = bmax = block_amax(w);
+    }
+    for (int b = threadIdx.x + blockDim.x; b < nb; b += blockDim.x) {
+        uint32_t t[8];
+        ld_block16(xr + 16 * b, vec != 0, t);
+        amax = fmaxf(amax, block_amax(t));
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
     __syncthreads();
-    amax = 0.f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) amax = fmaxf(amax, red[i]);
+    amax = (threadIdx.x & 31) < (blockDim.x >> 5) ? red[threadIdx.x & 31] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     const float g = amax > 0.f ? __fdiv_rn(amax, 6.0f * 448.0f) : 1.f;
     if (threadIdx.x == 0) g_out[row] = g;
-    for (int b = threadIdx.x; b < K / 16; b += blockDim.x) {
-        float v[16];
-        float bmax = 0.f;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            v[i] = ldf<T>(xr + 16 * b + i);
-            bmax = fmaxf(bmax, fabsf(v[i]));
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        if (b != (int)threadIdx.x) {
+            ld_block16(xr + 16 * b, vec != 0, w);
+            bmax = block_amax(w);
         }
         const uint32_t sc = (uint32_t)__nv_cvt_float_to_fp8(__fdiv_rn(__fdiv_rn(bmax, 6.0f), g), __NV_SATFINITE, __NV_E4M3);
         const float d = __fmul_rn(e4m3_value(sc), g);
-        sf[row * (size_t)(K / 16) + b] = (uint8_t)sc;
+        sf[row * (size_t)nb + b] = (uint8_t)sc;
         uint32_t lo = 0, hi = 0;
+        if (d > 0.f) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            lo |= (d > 0.f ? e2m1_code(__fdiv_rn(v[i], d)) : 0u) << (4 * i);
-            hi |= (d > 0.f ? e2m1_code(__fdiv_rn(v[8 + i], d)) : 0u) << (4 * i);
+            for (int i = 0; i < 4; ++i) {
+                lo |= (e2m1_code(__fdiv_rn(bf_lo(w[i]), d)) | (e2m1_code(__fdiv_rn(bf_hi(w[i]), d)) << 4)) << (8 * i);
+                hi |= (e2m1_code(__fdiv_rn(bf_lo(w[4 + i]), d)) | (e2m1_code(__fdiv_rn(bf_hi(w[4 + i]), d)) << 4)) << (8 * i);
+            }
         }
         *reinterpret_cast<uint2*>(codes + row * (size_t)(K / 2) + 8 * b) = make_uint2(lo, hi);
     }
@@ -391,7 +457,7 @@ void wd_launch_quantize_nvfp4(int dtype, const void* x, int n_rows, int K, const
     if (n_rows <= 0) return;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n_rows);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3((unsigned)std::min(kQuantThreads, wd_ceil_div(K / 16, 32) * 32));
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -399,8 +465,10 @@ void wd_launch_quantize_nvfp4(int dtype, const void* x, int n_rows, int K, const
     cfg.attrs = attr;
     cfg.numAttrs = wd_pdl_enabled ? 1 : 0;
     ++wd_launch_counter;
-    if (dtype == WD_F32) cudaLaunchKernelEx(&cfg, quantize_nvfp4_kernel<float>, (const float*)x, K, op->codes, op->sf, op->g);
-    else cudaLaunchKernelEx(&cfg, quantize_nvfp4_kernel<__nv_bfloat16>, (const __nv_bfloat16*)x, K, op->codes, op->sf, op->g);
+    for (const void* f : {(const void*)quantize_nvfp4_kernel<float>, (const void*)quantize_nvfp4_kernel<__nv_bfloat16>}) wd_prefer_max_shared(f);
+    const int vec = (uintptr_t)x % 16 == 0 ? 1 : 0;
+    if (dtype == WD_F32) cudaLaunchKernelEx(&cfg, quantize_nvfp4_kernel<float>, (const float*)x, K, vec, op->codes, op->sf, op->g);
+    else cudaLaunchKernelEx(&cfg, quantize_nvfp4_kernel<__nv_bfloat16>, (const __nv_bfloat16*)x, K, vec, op->codes, op->sf, op->g);
 }
 
 wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, size_t y_floats, int sm_count, int32_t* status,
@@ -415,33 +483,36 @@ wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, si
     p.tok_tiles = (rows + 127) / 128;
     p.bn = ((rows + p.tok_tiles - 1) / p.tok_tiles + 15) / 16 * 16;        // balanced token tiles, <= 128
     p.kb_total = K / kKB;
-    p.n_tiles = (n_out + kBM - 1) / kBM;
+    const int n_tiles = (n_out + kBM - 1) / kBM;
+    p.n_units = n_tiles * p.tok_tiles;
     const size_t slice = (size_t)rows * n_out;
     if (slice > y_floats) return WD_ERR_CAPACITY;
-    // K slices while (weight tile, token tile) pairs alone would leave SMs idle and the partial sums fit
-    // K slices: the split count that minimises (waves of units over the SMs) x (stages per unit) x (time one SM
-    // needs to take in a stage, about 63 GB/s whatever the source) + the write and re-read of one more partial
-    // result per slice at HBM speed
-    int ns = 1;
-    if (!force_single_split) {
-        const double t_stage = (double)(kStageW + p.bn * 128 + kSfW + p.bn * 16) / 63e9;
-        const double t_slice = (double)slice * 8.0 / 6.5e12;
-        double best = 1e30;
-        for (int c = 1; c <= WD_TC_MAX_SPLIT && c <= p.kb_total && (size_t)c * slice <= y_floats; ++c) {
-            const int units = p.n_tiles * p.tok_tiles * c;
-            const double t = (double)((units + sm_count - 1) / sm_count) * ((p.kb_total + c - 1) / c) * t_stage + c * t_slice;
-            if (t < best * 0.999) { best = t; ns = c; }
-        }
+    // Equal shares of the K-block line over all SMs, or whole units per CTA (one slice): whichever takes less, with the time
+    // one SM needs to take in a stage (about 63 GB/s whatever the source) and the write and re-read of a further slice at
+    // HBM speed.  (Units of a fixed K slice dealt round-robin had rounds that were not full: 12 and 24 stages per SM for the
+    // q/k/v and gate/up shapes at 34 rows where the line gives 10.4 and 20.8, and 3 slices of gate/up instead of 2.)
+    const long long W = (long long)p.n_units * p.kb_total;
+    const int G_line = (int)std::min<long long>(sm_count, W);
+    const bool many = p.n_units >= 4 * sm_count;        // rounds of whole units are full enough
+    int n_slices = 1;
+    for (long long u = 0; u < p.n_units && !many; ++u) {
+        const long long first = ((u * p.kb_total + 1) * G_line - 1) / W, last = (((u + 1) * p.kb_total) * G_line - 1) / W;
+        n_slices = std::max(n_slices, (int)(last - first) + 1);
     }
-    p.n_slices = ns;
-    p.n_units = p.n_tiles * p.tok_tiles * ns;
+    const int G_unit = std::min(sm_count, p.n_units);
+    const double t_stage = (double)(kStageW + p.bn * 128 + kSfW + p.bn * 16) / 63e9;
+    const double t_line = (double)((W + G_line - 1) / G_line) * t_stage + (n_slices - 1) * (double)slice * 8.0 / 6.5e12;
+    const double t_unit = (double)((p.n_units + G_unit - 1) / G_unit) * p.kb_total * t_stage;
+    p.aligned = force_single_split || many || t_unit <= t_line || n_slices > WD_TC_MAX_SPLIT || (size_t)n_slices * slice > y_floats;
+    p.n_slices = p.aligned ? 1 : n_slices;
+    const int grid = p.aligned ? G_unit : G_line;
     int cols = 32;
     while (cols < p.bn) cols <<= 1;
     p.buf_cols = cols;
     const int stage = (kStageW + p.bn * 128 + kSfW + p.bn * 16 + 1023) & ~1023;
     p.n_stages = (200 * 1024) / stage;
     if (p.n_stages > 10) p.n_stages = 10;
-    const size_t smem = (size_t)p.n_stages * stage + (2 * p.n_stages + 8) * 8 + 64 + 1024;
+    const size_t smem = (size_t)p.n_stages * stage + (2 * p.n_stages + 8) * 8 + 64 + 512 + 1024;
     p.y = y;
     p.split_stride = slice;
     p.gw = w->g;
@@ -467,7 +538,7 @@ wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, si
         attr_done[dev] = true;
     }
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)(p.n_units < sm_count ? p.n_units : sm_count));
+    lc.gridDim = dim3((unsigned)grid);
     lc.blockDim = dim3(kThreads);
     lc.dynamicSmemBytes = smem;
     lc.stream = stream;
@@ -478,6 +549,6 @@ wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, si
     lc.numAttrs = wd_pdl_enabled ? 1 : 0;
     ++wd_launch_counter;
     WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_fp4_kernel, mx, mw, msx, msw, p));
-    if (n_split_out) *n_split_out = ns;
+    if (n_split_out) *n_split_out = p.n_slices;
     return WD_OK;
 }

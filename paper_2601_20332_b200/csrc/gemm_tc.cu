@@ -1369,13 +1369,30 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
 }
 
-// y = sum of split-K slices
-__global__ void reduce_slices_kernel(const float* __restrict__ part, int n_split, size_t stride, float* __restrict__ y,
-                                     size_t total) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        float v = 0.f;
-        for (int s = 0; s < n_split; ++s) v += part[s * stride + i];
-        y[i] = v;
+// y = sum of split-K slices, in slice order; four outputs per thread (the slices start on 16 bytes when kVec)
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+reduce_slices_kernel(const float* __restrict__ part, int n_split, size_t stride, float* __restrict__ y, size_t total) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i >= total) return;
+    if (kVec) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s0 = 0; s0 < n_split; s0 += 4) {
+            float4 t[4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) t[s] = s0 + s < n_split ? ldcg4(part + (size_t)(s0 + s) * stride + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) add4(v, t[s]);
+        }
+        *reinterpret_cast<float4*>(y + i) = v;
+    } else {
+        for (size_t j = i; j < total && j < i + 4; ++j) {
+            float v = 0.f;
+            for (int s = 0; s < n_split; ++s) v += part[s * stride + j];
+            y[j] = v;
+        }
     }
 }
 
@@ -1930,9 +1947,19 @@ wd_status wd_tc_chain(const WdTcChainItem* items, int n, int rows, float* y, siz
 }
 
 void wd_launch_reduce_slices(const float* part, int n_split, size_t stride, float* y, size_t total, cudaStream_t st) {
-    const int blocks = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)((total + 1023) / 1024));
+    lc.blockDim = dim3(256);
+    lc.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = wd_pdl_enabled ? 1 : 0;
     ++wd_launch_counter;
-    reduce_slices_kernel<<<blocks, 256, 0, st>>>(part, n_split, stride, y, total);
+    wd_prefer_max_shared((const void*)reduce_slices_kernel<true>);
+    const bool vec = total % 4 == 0 && stride % 4 == 0 && ((uintptr_t)part | (uintptr_t)y) % 16 == 0;
+    cudaLaunchKernelEx(&lc, vec ? reduce_slices_kernel<true> : reduce_slices_kernel<false>, part, n_split, stride, y, total);
 }
 
 wd_status wd_tc_encode_fp8(CUtensorMap* m, const void* ptr, int n_rows, int K, int box_rows) {
@@ -1972,9 +1999,7 @@ wd_status wd_tc_gemm_standalone(const void* x, const void* w, float* y, int rows
     int ns = 1;
     s = wd_tc_gemm(&xm, &seg, 1, rows, k_in, (float*)scratch, scratch_bytes / 4, sm, status, stream, &ns, false);
     if (s != WD_OK) return s;
-    const int blocks = (int)((slice + 255) / 256 < 1184 ? (slice + 255) / 256 : 1184);
-    ++wd_launch_counter;
-    reduce_slices_kernel<<<blocks, 256, 0, stream>>>((const float*)scratch, ns, slice, y, slice);
+    wd_launch_reduce_slices((const float*)scratch, ns, slice, y, slice, stream);
     WD_CUDA_TRY(cudaGetLastError());
     return WD_OK;
 }
@@ -2001,9 +2026,7 @@ wd_status wd_tc_gemm_standalone_fp8(const uint8_t* xq, const float* sx, const ui
     int ns = 1;
     s = wd_tc_gemm(&xm, &seg, 1, rows, k_in, slices, slice_floats, sm, status, stream, &ns, false, nullptr, &f8);
     if (s != WD_OK) return s;
-    const int blocks = (int)((slice + 255) / 256 < 1184 ? (slice + 255) / 256 : 1184);
-    ++wd_launch_counter;
-    reduce_slices_kernel<<<blocks, 256, 0, stream>>>(slices, ns, slice, y, slice);
+    wd_launch_reduce_slices(slices, ns, slice, y, slice, stream);
     WD_CUDA_TRY(cudaGetLastError());
     return WD_OK;
 }
@@ -2067,9 +2090,7 @@ extern "C" wd_status wd_op_gemm_noalloc(const void* x, const void* w, float* y, 
     int ns = 1;
     s = wd_tc_gemm(&xm, &seg, 1, rows, k_in, scratch, (size_t)WD_NOALLOC_SCRATCH_FLOATS, sm, status, stream, &ns, false);
     if (s != WD_OK) return s;
-    const int blocks = (int)((slice + 255) / 256 < 1184 ? (slice + 255) / 256 : 1184);
-    ++wd_launch_counter;
-    reduce_slices_kernel<<<blocks, 256, 0, stream>>>(scratch, ns, slice, y, slice);
+    wd_launch_reduce_slices(scratch, ns, slice, y, slice, stream);
     WD_CUDA_TRY(cudaGetLastError());
     return WD_OK;
 }

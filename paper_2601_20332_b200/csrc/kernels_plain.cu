@@ -17,6 +17,22 @@
 
 bool wd_pdl_enabled = true;
 
+// Every small kernel asks for the largest shared-memory carve-out although it uses next to none: an SM keeps its
+// carve-out while blocks are resident, and the next GEMM's blocks (some 200 KB each, launched early under
+// programmatic dependent launch so that they can fetch weights ahead of their dependency) become resident
+// beside a small kernel's blocks only if the SM is already configured for that much shared memory.
+void wd_prefer_max_shared(const void* kernel) {
+    thread_local std::vector<std::pair<const void*, int>> done;      // (kernel, device) pairs already configured
+    int dev = 0;
+    static const bool off = getenv("WD_NO_CARVEOUT") && atoi(getenv("WD_NO_CARVEOUT"));
+    if (off) return;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return; }
+    for (const auto& e : done) if (e.first == kernel && e.second == dev) return;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+        cudaGetLastError();
+    done.emplace_back(kernel, dev);
+}
+
 namespace {
 
 using wdk::pdl_launch_dependents;
@@ -55,24 +71,9 @@ extern "C" __attribute__((visibility("default"))) int wd_debug_small_trace(unsig
 
 // Launch with programmatic stream serialization: the kernel may start while its predecessor
 // is still draining; it calls pdl_wait() before touching anything the predecessor wrote.
-// Every small kernel asks for the largest shared-memory carve-out although it uses next to none: an SM keeps its
-// carve-out while blocks are resident, and the next GEMM's blocks (some 200 KB each, launched early under
-// programmatic dependent launch so that they can fetch weights ahead of their dependency) become resident
-// beside a small kernel's blocks only if the SM is already configured for that much shared memory.
-static void prefer_max_shared(const void* kernel) {
-    static std::vector<std::pair<const void*, int>> done;      // (kernel, device) pairs already configured
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return; }
-    for (const auto& e : done) if (e.first == kernel && e.second == dev) return;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-        cudaGetLastError();
-    done.emplace_back(kernel, dev);
-}
-
 template <typename... KArgs, typename... Args>
 void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-    static const bool carve = !(getenv("WD_NO_CARVEOUT") && atoi(getenv("WD_NO_CARVEOUT")));
-    if (carve) prefer_max_shared((const void*)kernel);
+    wd_prefer_max_shared((const void*)kernel);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -1369,14 +1370,9 @@ static wd_status launch_swiglu_quant(const float* part, int n_split, size_t spli
     lc.numAttrs = wd_pdl_enabled ? 2 : 1;
     const int per_thread = ((f4 + 3) / 4 + 255) / 256;          // float4 per thread
     cudaError_t e;
-    {
-        static const bool carve = !(getenv("WD_NO_CARVEOUT") && atoi(getenv("WD_NO_CARVEOUT")));
-        if (carve) {
-            prefer_max_shared((const void*)swiglu_fp4_kernel<3>); prefer_max_shared((const void*)swiglu_fp4_kernel<5>);
-            prefer_max_shared((const void*)swiglu_fp4_kernel<8>); prefer_max_shared((const void*)swiglu_fp8_kernel<3>);
-            prefer_max_shared((const void*)swiglu_fp8_kernel<5>); prefer_max_shared((const void*)swiglu_fp8_kernel<8>);
-        }
-    }
+    for (const void* f : {(const void*)swiglu_fp4_kernel<3>, (const void*)swiglu_fp4_kernel<5>, (const void*)swiglu_fp4_kernel<8>,
+                          (const void*)swiglu_fp8_kernel<3>, (const void*)swiglu_fp8_kernel<5>, (const void*)swiglu_fp8_kernel<8>})
+        wd_prefer_max_shared(f);
     if (h4p) {
         if (per_thread <= 3) e = cudaLaunchKernelEx(&lc, swiglu_fp4_kernel<3>, part, n_split, split_stride, F, h4);
         else if (per_thread <= 5) e = cudaLaunchKernelEx(&lc, swiglu_fp4_kernel<5>, part, n_split, split_stride, F, h4);

@@ -193,4 +193,5 @@ void wd_launch_fill_qtiles(int32_t* lists, int n_rows, int n_vis, cudaStream_t s
 
 wd_status wd_launch_wait_expire(cudaStream_t st);
 int32_t* wd_op_status_ptr();   // device address of the single-operation status word
+void wd_prefer_max_shared(const void* kernel);   // ask for the largest shared-memory carve-out (see the definition)
 extern bool wd_pdl_enabled;    // programmatic dependent launch on every kernel (default on)
