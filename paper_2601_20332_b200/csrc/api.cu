@@ -976,7 +976,7 @@ static bool use_tc(const wd_ctx* c) {
 static wd_status run_gemm(wd_ctx* c, const void* x, const WdTcX* x_map, const WdTcSeg* segs, int nseg,
                           int rows, int K, float* y, size_t y_floats, int32_t* status, cudaStream_t stream,
                           GemmOut* go, bool single_split = false, const WdTcFuse* fuse = nullptr,
-                          const WdTcFp8* fp8 = nullptr, const WdTcSwiglu* sg = nullptr) {
+                          const WdTcFp8* fp8 = nullptr, const WdTcEpi* epi = nullptr) {
     int ncol = 0;
     for (int i = 0; i < nseg; ++i) ncol += segs[i].n;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1002,10 +1002,10 @@ static wd_status run_gemm(wd_ctx* c, const void* x, const WdTcX* x_map, const Wd
     } else if (use_tc(c)) {
         int n_split = 1;
         wd_status s = wd_tc_gemm(x_map, segs, nseg, rows, K, y, y_floats, c->sm_count, status, stream, &n_split,
-                                 single_split, fuse, fp8, sg);
+                                 single_split, fuse, fp8, epi);
         if (s != WD_OK) return s;
         // SwiGLU done by the GEMM: bf16 h instead of the fp32 gate/up sums
-        if (sg && sg->done && c->prof_on) c->prof_step_bytes -= (double)rows * ncol * 4 - (double)rows * (ncol / 2) * 2;
+        if (epi && epi->sg && epi->sg->done && c->prof_on) c->prof_step_bytes -= (double)rows * ncol * 4 - (double)rows * (ncol / 2) * 2;
         *go = {n_split, (size_t)rows * ncol, 1, WD_GEMM_TCGEN05};
     } else {
         if ((size_t)rows * ncol > y_floats) return WD_ERR_CAPACITY;
@@ -1260,6 +1260,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     // before the copy of the result block); launched directly, or recorded into a CUDA graph and replayed
     auto run_kernels = [&]() -> wd_status {
     c->tc.x_map_attn.smem_cap = 0;          // set per block below, and only beside the single-key-tile attention
+    bool down_pending = false;          // x still lacks the previous block's FFN output (partial sums in part)
+    GemmOut down_go = {1, 0, 0, 0};
     if (fused) {
         // Five kernels per block.  The GEMM input is bf16(x * gain) without the 1/rms factor; the CTA
         // that completes an output tile applies it (from per-block sums of squares written by the
@@ -1342,8 +1344,6 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     } else {
     wd_launch_embed(d.dtype, c->tok_embed, st->ids_dev, row_seq, row_pos, c->x, c->rope_tab, R_, D, S, d.vocab, dh,
                     d.rope_theta, status, stream);
-    bool down_pending = false;          // x still lacks the previous block's FFN output
-    GemmOut down_go = {1, 0, 0, 0};
     for (int l = 0; l < d.n_layers; ++l) {
         char* kc = st->kcache + (size_t)l * st->kv_layer_bytes;
         char* vc = st->vcache + (size_t)l * st->v_layer_bytes;
@@ -1377,10 +1377,16 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         // (measured: 215 KB for the two CTAs together still fits an SM, 222 KB does not)
         c->tc.x_map_attn.smem_cap = (attn_smem > 0 && attn_smem <= 110 * 1024 && R_ <= 128) ? (int)(223232 - attn_smem) : 0;
         WdTcSeg wo[1] = {{c->wo[l], D, c->tc.get(WD_TC_WO, l)}};
-        if ((s = run_gemm(c, c->attn, &c->tc.x_map_attn, wo, 1, R_, hq, c->part, c->part_floats, status, stream, &go)) != WD_OK)
+        WdTcResid resid_o, resid_d;
+        resid_o.x = resid_d.x = c->x;
+        WdTcEpi epi_o, epi_d;
+        epi_o.resid = &resid_o;
+        epi_d.resid = &resid_d;
+        if ((s = run_gemm(c, c->attn, &c->tc.x_map_attn, wo, 1, R_, hq, c->part, c->part_floats, status, stream, &go, false, nullptr,
+                          nullptr, &epi_o)) != WD_OK)
             return s;
         // feed-forward half
-        wd_launch_rmsnorm(d.dtype, c->x, c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, c->xn,
+        wd_launch_rmsnorm(d.dtype, c->x, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, c->xn,
                           nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_d : nullptr);
         if (fp4) {
             if ((s = run_gemm_fp4(c, &c->f4gu[l], R_, D, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
@@ -1404,19 +1410,24 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         WdTcSeg gu[2] = {{c->wg[l], F, c->tc.get(WD_TC_WG, l)}, {c->wu[l], F, c->tc.get(WD_TC_WU, l)}};
         WdTcSwiglu sg;
         sg.h = use_tc(c) ? (__nv_bfloat16*)c->h : nullptr;
+        WdTcEpi epi_sg;
+        epi_sg.sg = &sg;
         if ((s = run_gemm(c, c->xn, &c->tc.x_map_d, gu, 2, R_, D, c->part, c->part_floats, status, stream, &go, false,
-                          nullptr, nullptr, &sg)) != WD_OK)
+                          nullptr, nullptr, &epi_sg)) != WD_OK)
             return s;
         if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, R_, F, stream);
         WdTcSeg wdn[1] = {{c->wd[l], D, c->tc.get(WD_TC_WD, l)}};
-        if ((s = run_gemm(c, c->h, &c->tc.x_map_h, wdn, 1, R_, F, c->part, c->part_floats, status, stream, &go)) != WD_OK)
+        if ((s = run_gemm(c, c->h, &c->tc.x_map_h, wdn, 1, R_, F, c->part, c->part_floats, status, stream, &go, false, nullptr,
+                          nullptr, &epi_d)) != WD_OK)
             return s;
         }
-        if (st->taps.layer_out || l == d.n_layers - 1) {
-            float* tap = st->taps.layer_out ? st->taps.layer_out + (size_t)l * R_ * D : nullptr;
-            wd_launch_residual_add(c->x, c->part, go.n_split, go.split_stride, tap, R_, D, stream);
+        if (resid_d.done) {             // x is complete
+            if (st->taps.layer_out)
+                WD_CUDA_TRY(cudaMemcpyAsync(st->taps.layer_out + (size_t)l * R_ * D, c->x, (size_t)R_ * D * 4, cudaMemcpyDeviceToDevice, stream));
+        } else if (st->taps.layer_out) {
+            wd_launch_residual_add(c->x, c->part, go.n_split, go.split_stride, st->taps.layer_out + (size_t)l * R_ * D, R_, D, stream);
         } else {
-            down_pending = true;     // folded into the next block's RMSNorm
+            down_pending = true;     // folded into the next block's RMSNorm, or the final one (which needs the active rows only)
             down_go = go;
         }
     }
@@ -1425,8 +1436,9 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     bool lm_fused = false;
     int lm_chunks = wd_unmask_chunks(d.vocab);
     if (NA > 0) {
-        wd_launch_rmsnorm(d.dtype, c->x, nullptr, 0, 0, c->final_norm, d.rms_eps, c->xn, act_row, NA, D, stream,
+        wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride, c->final_norm, d.rms_eps, c->xn, act_row, NA, D, stream,
                           fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_lm : nullptr);
+        float* logits = st->taps.logits ? st->taps.logits : c->logits;      // a tap takes them directly
         WdTcSeg lm[1] = {{c->lm_head, d.vocab, c->tc.get(WD_TC_LM, 0)}};
         WdTcFp8 f8lm;
         if (fp8) {
@@ -1441,18 +1453,15 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         fl.write_logits = st->taps.logits ? 1 : 0;
         lm_fused = use_tc(c) && NA <= 1024 && c->sm_count % 4 == 0 && !fp4;     // one CTA group per tile of <= 256 active rows
         if (fp4) {
-            if ((s = run_gemm_fp4(c, &c->f4lm, NA, D, c->logits, (size_t)d.max_active * d.vocab, status, stream, &go,
+            if ((s = run_gemm_fp4(c, &c->f4lm, NA, D, logits, (size_t)d.max_active * d.vocab, status, stream, &go,
                                   /*single_split=*/true)) != WD_OK)
                 return s;
-        } else if ((s = run_gemm(c, fp8 ? (const void*)c->xn8 : c->xn, fp8 ? &c->x8_d : &c->tc.x_map_d, lm, 1, NA, D, c->logits,
+        } else if ((s = run_gemm(c, fp8 ? (const void*)c->xn8 : c->xn, fp8 ? &c->x8_d : &c->tc.x_map_d, lm, 1, NA, D, logits,
                           (size_t)d.max_active * d.vocab, status, stream, &go, /*single_split=*/true,
                           lm_fused ? &fl : nullptr, fp8 ? &f8lm : nullptr)) != WD_OK)
             return s;
         if (lm_fused) lm_chunks = fl.n_chunks;
-        else wd_launch_rowstats(c->logits, NA, d.vocab, c->ch_max, c->ch_idx, c->ch_sum, stream);
-        if (st->taps.logits)
-            WD_CUDA_TRY(cudaMemcpyAsync(st->taps.logits, c->logits, (size_t)NA * d.vocab * 4, cudaMemcpyDeviceToDevice,
-                                        stream));
+        else wd_launch_rowstats(logits, NA, d.vocab, c->ch_max, c->ch_idx, c->ch_sum, stream);
     }
     int32_t* n_sel = c->result + 1;
     int32_t* sel_pos = n_sel + batch;

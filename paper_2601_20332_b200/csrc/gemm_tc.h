@@ -107,12 +107,25 @@ struct WdTcSwiglu {
     mutable bool done = false;
 };
 
+// Output and down projections with many rows: where the GEMM works on whole tiles, its epilogue adds the result to the
+// residual stream x[rows, n] (float) and nothing goes to y.  `done`: whether that happened; if not, y holds the sums as usual.
+struct WdTcResid {
+    float* x = nullptr;
+    mutable bool done = false;
+};
+
+// What a launch may do in its epilogue instead of writing y, if its schedule allows it
+struct WdTcEpi {
+    const WdTcSwiglu* sg = nullptr;
+    const WdTcResid* resid = nullptr;
+};
+
 // y[split][rows][sum n_i] = x * [w_0; w_1; ...]^T, split-K partial sums side by side
 // (split_stride = rows * sum n_i floats).  The consumer adds the slices.
 wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, int K, float* y, size_t y_floats,
                      int sm_count, int32_t* status, cudaStream_t stream, int* n_split_out,
                      bool force_single_split = false, const WdTcFuse* fuse = nullptr, const WdTcFp8* fp8 = nullptr,
-                     const WdTcSwiglu* sg = nullptr);
+                     const WdTcEpi* epi = nullptr);
 // Chain kernel (few rows): up to four consecutive fused GEMMs (modes QKV / RESID / SWIGLU) in one persistent
 // launch whose weight stream never stops; each GEMM's input is the previous one's finished tiles.
 struct WdTcChainItem {
