@@ -65,10 +65,10 @@ struct wd_ctx {
     // configuration (StepKey) has been seen before is captured once and replayed afterwards
     struct StepKey {
         uint64_t state_uid = 0;
-        int batch = 0, rows = 0, n_act = 0, n_qtiles = 0, key_tiles = 0, max_tile_rows = 0, k_eff = 0, mode = 0, impl = 0, attn_impl = 0;
+        int batch = 0, rows = 0, n_act = 0, n_qtiles = 0, key_tiles = 0, max_tile_rows = 0, max_seq_tiles = 0, k_eff = 0, mode = 0, impl = 0, attn_impl = 0;
         bool operator==(const StepKey& o) const {
             return state_uid == o.state_uid && batch == o.batch && rows == o.rows && n_act == o.n_act && n_qtiles == o.n_qtiles &&
-                   key_tiles == o.key_tiles && max_tile_rows == o.max_tile_rows && k_eff == o.k_eff && mode == o.mode &&
+                   key_tiles == o.key_tiles && max_tile_rows == o.max_tile_rows && max_seq_tiles == o.max_seq_tiles && k_eff == o.k_eff && mode == o.mode &&
                    impl == o.impl && attn_impl == o.attn_impl;
         }
     };
@@ -188,7 +188,7 @@ static void carve_ctx(const wd_model_dims* d, Carve& c, size_t off[24]) {
     off[7] = c.take(MA * 4);                                    // row_token
     off[8] = c.take(MA * 8);                                    // row_sumexp
     off[9] = c.take(MA * 4);                                    // row_conf
-    const size_t plan_ints = 2 * MR + 2 * MA + 2 * ((size_t)d->max_batch + 1) + (size_t)d->max_batch * d->max_seq +
+    const size_t plan_ints = 2 * MR + 2 * MA + 3 * ((size_t)d->max_batch + 1) + (size_t)d->max_batch * d->max_seq +
                              3 * (MR / 128 + (size_t)d->max_batch + 1) + 2 * (size_t)d->max_batch +
                              (size_t)d->max_batch * d->max_seq;      // + staging of the external windows
     off[10] = c.take(plan_ints * 4);                            // plan
@@ -1070,7 +1070,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     pend.cp.assign(batch, WdCountPlan());
     bool all_done = true, any_refresh = false, all_contig = true;
     size_t n_rows = 0, n_act = 0, n_vis = 0, n_qtiles = 0;
-    int max_vis = 0, max_tile_rows = 0;
+    int max_vis = 0, max_tile_rows = 0, max_seq_tiles = 0;
     if (!dev_mode) {
         st->plans.assign(batch, WdSeqPlan());
         for (int b = 0; b < batch; ++b) {
@@ -1112,6 +1112,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         n_qtiles += (cp.n_rows + 127) / 128;
         max_vis = std::max(max_vis, (int)cp.n_vis);
         max_tile_rows = std::max(max_tile_rows, std::min(128, (int)cp.n_rows));
+        max_seq_tiles = std::max(max_seq_tiles, ((int)cp.n_rows + 127) / 128);
     }
     if (all_done) return WD_DONE;
     if (n_rows > (size_t)d.max_rows || n_act > (size_t)d.max_active ||
@@ -1131,6 +1132,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     const size_t o_qt_row0 = o; o += n_qtiles;
     const size_t o_qt_n = o; o += n_qtiles;
     const size_t o_nvis = o; o += batch;
+    const size_t o_qt_off = o; o += batch + 1;
     const size_t o_tseq = o; o += batch;          // step index of each sequence (for the decode-step stamps)
     const size_t o_vis_idx = o; o += n_vis;       // last: every other offset depends on rows, active rows and tiles only
     if (o > c->plan_ints) return WD_ERR_CAPACITY;
@@ -1156,6 +1158,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         pl.act_off_dev = c->plan + o_act_off; pl.vis_off_dev = c->plan + o_vis_off; pl.vis_idx = c->plan + o_vis_idx;
         pl.qt_seq = c->plan + o_qt_seq; pl.qt_row0 = c->plan + o_qt_row0; pl.qt_n = c->plan + o_qt_n;
         pl.nvis_dev = c->plan + o_nvis; pl.tseq_dev = c->plan + o_tseq;
+        pl.qt_off_dev = c->plan + o_qt_off;
         pl.status = c->result;
         wd_launch_plan(pl, stream);
     } else {
@@ -1166,6 +1169,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             ph[o_vis_off + b] = (int32_t)v;
             ph[o_nvis + b] = p.done ? 0 : (int32_t)p.vis.size();
             ph[o_tseq + b] = st->seqs[b].t;
+            ph[o_qt_off + b] = (int32_t)qt;
             if (p.done) continue;
             for (size_t t0 = 0; t0 < p.rows.size(); t0 += 128, ++qt) {
                 ph[o_qt_seq + qt] = b;
@@ -1187,6 +1191,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             v += p.vis.size();
         }
         ph[o_act_off + batch] = (int32_t)a;
+        ph[o_qt_off + batch] = (int32_t)qt;
         ph[o_vis_off + batch] = (int32_t)v;
         WD_CUDA_TRY(cudaMemcpyAsync(c->plan, ph, o * 4, cudaMemcpyHostToDevice, stream));
         // keep the device copy of the planner state complete (the unmask kernel maintains the flags
@@ -1251,7 +1256,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         if (st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN)
             return wd_attn_tc_launch(c->q, R_, (int)n_qtiles, c->plan + o_qt_seq, c->plan + o_qt_row0, c->plan + o_qt_n,
                                      c->plan + o_nvis, &st->map_k, &st->map_vt, c->attn, attn_tap, Hq, Hkv, dh, l, max_vis,
-                                     c->sm_count, status, stream, max_tile_rows, &attn_smem);
+                                     c->sm_count, status, stream, max_tile_rows, &attn_smem, c->plan + o_qt_off, batch, max_seq_tiles);
         wd_launch_attention_plain(d.dtype, c->q, kc, vc, row_seq, vis_idx, vis_off, c->attn, attn_tap, R_, max_vis, Hq,
                                   Hkv, dh, S, Sp, batch, status, stream);
         return WD_OK;
@@ -1496,7 +1501,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         !st->queue.empty()) {
         wd_ctx::StepKey key;
         key.state_uid = st->uid; key.batch = batch; key.rows = R_; key.n_act = NA; key.n_qtiles = (int)n_qtiles;
-        key.key_tiles = (max_vis + 127) / 128; key.max_tile_rows = max_tile_rows; key.k_eff = k_eff;
+        key.key_tiles = (max_vis + 127) / 128; key.max_tile_rows = max_tile_rows; key.max_seq_tiles = max_seq_tiles; key.k_eff = k_eff;
         key.mode = (c->fp8_on ? 1 : 0) | (c->fp4_on ? 2 : 0) | (st->attn_tc ? 4 : 0);
         key.impl = c->gemm_impl; key.attn_impl = c->attn_impl;
         wd_ctx::StepGraph* hit = nullptr;
@@ -1857,7 +1862,7 @@ extern "C" wd_status wd_op_attention(int32_t dtype, const void* q, const void* k
 
 extern "C" size_t wd_op_attention_tc_scratch_bytes(int32_t n_rows) {
     if (n_rows < 1) return 0;
-    return wd_align_up((size_t)(3 * ((n_rows + 127) / 128) + 1) * 4, 256);
+    return wd_align_up((size_t)(3 * ((n_rows + 127) / 128) + 3) * 4, 256);
 }
 
 extern "C" wd_status wd_op_attention_tc(const void* q, const void* kcache, const void* vcache_t, void* out,
@@ -1886,7 +1891,7 @@ extern "C" wd_status wd_op_attention_tc(const void* q, const void* kcache, const
     WD_CUDA_TRY(cudaGetLastError());
     return wd_attn_tc_launch(q, n_rows, n_tiles, lists, lists + n_tiles, lists + 2 * n_tiles, lists + 3 * n_tiles, &map_k,
                              &map_vt, out, nullptr, n_q_heads, n_kv_heads, 128, 0, max_vis, sm, status, stream,
-                             std::min(n_rows, 128));
+                             std::min(n_rows, 128), nullptr, lists + 3 * n_tiles + 1, 1, n_tiles);
 }
 
 extern "C" size_t wd_op_lm_unmask_scratch_bytes(int32_t n, int32_t vocab) {

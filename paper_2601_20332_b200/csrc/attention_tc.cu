@@ -50,6 +50,7 @@ struct AttnParams {
     const int32_t* qtile_row0;   // [n_tiles] first row (index into the step's row list)
     const int32_t* qtile_n;      // [n_tiles] valid rows
     const int32_t* seq_nvis;     // [batch] visible positions [0, n_vis)
+    const int32_t* seq_qt_off;   // [batch + 1] first tile of each sequence (two-tile kernel)
     __nv_bfloat16* out;          // [rows][Hq*dh]
     float* tap;                  // optional fp32 copy
     int Hq, Hkv, layer;
@@ -548,6 +549,309 @@ attention_tc_single_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
     attention_tc_body<true>(map_q, map_k, map_vt, p);
 }
 
+// ------------------------------------------------------------------------------------------
+// Two query tiles per CTA: launches of more than one wave of single-tile CTAs
+// ------------------------------------------------------------------------------------------
+// A single-tile CTA is bound by its softmax warps: 2800 cycles per key tile, one phase after another (scores, maxima, a barrier
+// between the two halves of a row, exponentials, P, the rescale of O in registers), against 1024 of the tensor core.  Here a CTA
+// works on two query tiles over the same keys: consecutive (row tile, query head) items of one sequence and KV head.
+//   warps 0, 1         TMA, MMA (2 and 3 are there to make a warpgroup, which hands its registers to the others)
+//   warps 4-7 / 8-11   softmax of tile 0 / tile 1, one thread per query row: no exchange between threads, a row's 128 scores in
+//                      registers, and while one tile's scores are exponentiated the tensor core works on the other's
+//   O                  stays in tensor memory: P V accumulates over the key tiles, and a warp rescales its rows only when a row's
+//                      maximum has grown by more than 2^8 since the reference value in use (any reference cancels in O / l)
+// Tensor memory: S (and P over it) 2 x 128 columns, O 2 x 128.  Shared memory: two Q tiles, two K and two V stages, 192 KB.
+// The tensor core runs Q K^T and P V in issue order, so S(i + 1) complete means P V(i) has read P(i) and has been added to O;
+// one barrier each for S and P of a tile suffices (P(i + 1) needs S(i + 1), which is issued only after P(i) has been seen).
+// Measured per launch against the single-tile kernel: see wd_attn_tc_launch.
+constexpr int kDThreads = 384;
+// Registers per thread after the hand-over: 56 for the first warpgroup, 224 for the other two.  The launch has 168 for each of
+// the 384 threads (the most that fit the register file), and 128 * 56 + 256 * 224 = 384 * 168.
+constexpr int kDBars = 14;
+constexpr int kDQ = 0, kDKFull = 1, kDKEmpty = 3, kDVFull = 5, kDVEmpty = 7, kDSFull = 9, kDPFull = 11, kDODone = 13;
+constexpr size_t kDualSmem = 6 * (size_t)kOperand + (kDBars + 2) * 8 + 1024;
+
+__device__ __forceinline__ uint64_t f32x2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void f32x2_get(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__global__ void __launch_bounds__(kDThreads, 1)
+attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                         const __grid_constant__ CUtensorMap map_vt, const AttnParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* sQ = smem;                              // two tiles
+    uint8_t* sK = smem + 2 * kOperand;               // two stages
+    uint8_t* sV = sK + 2 * kOperand;                 // two stages (transposed V tiles)
+    uint64_t* bars = (uint64_t*)(sV + 2 * kOperand);
+    uint32_t* tmem_slot = (uint32_t*)(bars + kDBars);
+    volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    pdl_launch_dependents();
+    // (the index lists are complete before this kernel can start: see attention_tc_body)
+    const int b = blockIdx.z, kvh = blockIdx.y, item0 = 2 * (int)blockIdx.x;
+    const int tile0 = p.seq_qt_off[b], n_items = (p.seq_qt_off[b + 1] - tile0) * p.tiles_per_kv;
+    if (item0 >= n_items) return;                    // a shorter sequence of the batch
+    const int n_q = min(2, n_items - item0);         // query tiles of this CTA
+    const int n_vis = p.seq_nvis[b], n_kt = (n_vis + kTile - 1) / kTile;
+    const int group = p.Hq / p.Hkv;
+    struct Item { int row0, n_valid, h, n_slots; };
+    auto item = [&](int t) {
+        const int e = item0 + t, hg = e % p.tiles_per_kv;
+        const int tile = tile0 + e / p.tiles_per_kv;
+        Item r;
+        r.row0 = p.qtile_row0[tile];
+        r.n_valid = p.qtile_n[tile];
+        r.h = kvh * group + hg * p.pack;             // query head of slot 0
+        r.n_slots = min(p.pack, group - hg * p.pack);
+        return r;
+    };
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kDBars; ++i) mbar_init(smem_u32(&bars[i]), (i == kDPFull || i == kDPFull + 1) ? 128u : 1u);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (const CUtensorMap* m : {&map_q, &map_k, &map_vt}) asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+    }
+    if (warp == 1) tmem_alloc(smem_u32(tmem_slot), (uint32_t)kTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();                                      // q and the cache rows come from the previous kernel
+    // (the hand-over stands inside the branches: the compiler gives each the registers it has after it)
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (warp == 0) {
+            if (lane == 0) {
+                // ---------------------------------------------------- TMA producer
+                const uint32_t qf = smem_u32(&bars[kDQ]);
+                const Item q0 = item(0), q1 = item(n_q - 1);
+                const int bh = b * p.Hkv + kvh;
+                mbar_expect_tx(qf, (uint32_t)((q0.n_slots + (n_q == 2 ? q1.n_slots : 0)) * p.slot * 256));
+                for (int t = 0; t < n_q; ++t) {
+                    const Item q = t ? q1 : q0;
+                    for (int j = 0; j < q.n_slots; ++j) {
+                        const uint32_t dst = smem_u32(sQ) + (uint32_t)(t * kOperand + j * p.slot * 128);
+                        tma_load_2d(dst, &map_q, qf, (q.h + j) * kTile, q.row0);
+                        tma_load_2d(dst + kAtom, &map_q, qf, (q.h + j) * kTile + 64, q.row0);
+                    }
+                }
+                bool ok = true;
+                for (int i = 0; i < n_kt && ok; ++i) {
+                    const int s = i & 1, kv0 = i * kTile;
+                    const uint32_t ph = ((uint32_t)(i >> 1) & 1u) ^ 1u;
+                    const uint32_t kf = smem_u32(&bars[kDKFull + s]), vf = smem_u32(&bars[kDVFull + s]);
+                    const uint32_t sk = smem_u32(sK + (size_t)s * kOperand), sv = smem_u32(sV + (size_t)s * kOperand);
+                    if (!(ok = mbar_wait(smem_u32(&bars[kDKEmpty + s]), ph, abort_flag))) break;
+                    mbar_expect_tx(kf, kOperand);
+                    tma_load_4d(sk, &map_k, kf, 0, kv0, bh, p.layer);             // keys kv0.., dims 0..63
+                    tma_load_4d(sk + kAtom, &map_k, kf, 64, kv0, bh, p.layer);    // dims 64..127
+                    if (!(ok = mbar_wait(smem_u32(&bars[kDVEmpty + s]), ph, abort_flag))) break;
+                    mbar_expect_tx(vf, kOperand);
+                    tma_load_4d(sv, &map_vt, vf, kv0, 0, bh, p.layer);            // all dims, keys kv0..kv0+63
+                    tma_load_4d(sv + kAtom, &map_vt, vf, kv0 + 64, 0, bh, p.layer);
+                }
+                if (!ok) {
+                    *abort_flag = 1;
+                    atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
+                }
+            }
+            __syncwarp();
+        } else if (warp == 1) {
+            if (lane == 0) {
+                // ---------------------------------------------------- MMA issuer
+                bool ok = mbar_wait(smem_u32(&bars[kDQ]), 0, abort_flag);
+                auto issue_qk = [&](int t, int i) {                   // S_t = Q_t K(i)^T
+                    const uint64_t qd = make_sdesc(smem_u32(sQ + (size_t)t * kOperand));
+                    const uint64_t kd = make_sdesc(smem_u32(sK + (size_t)(i & 1) * kOperand));
+                    const uint32_t acc = tmem_base + (uint32_t)(t * kTile);
+    #pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {
+                        const uint64_t o = (uint64_t)((kk >> 2) * (kAtom >> 4) + 2 * (kk & 3));
+                        umma_bf16(acc, qd + o, kd + o, p.idesc, kk > 0);
+                    }
+                    umma_commit(smem_u32(&bars[kDSFull + t]));
+                    if (t == n_q - 1) umma_commit(smem_u32(&bars[kDKEmpty + (i & 1)]));     // K stage free
+                };
+                ok = ok && mbar_wait(smem_u32(&bars[kDKFull]), 0, abort_flag);
+                if (ok) {
+                    tc_fence_after();
+                    for (int t = 0; t < n_q; ++t) issue_qk(t, 0);
+                }
+                for (int i = 0; i < n_kt && ok; ++i) {
+                    const uint32_t ph = (uint32_t)(i >> 1) & 1u;
+                    if (!(ok = mbar_wait(smem_u32(&bars[kDVFull + (i & 1)]), ph, abort_flag))) break;          // V(i) landed
+                    for (int t = 0; t < n_q; ++t) {
+                        if (!(ok = mbar_wait(smem_u32(&bars[kDPFull + t]), (uint32_t)i & 1u, abort_flag))) break;   // P_t(i) written, O_t rescaled
+                        tc_fence_after();
+                        const uint64_t vd = make_sdesc(smem_u32(sV + (size_t)(i & 1) * kOperand));
+                        const uint32_t acc = tmem_base + (uint32_t)(2 * kTile + t * kTile), pa = tmem_base + (uint32_t)(t * kTile);
+    #pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)                // 16 keys = 8 columns of P per MMA
+                            umma_bf16_ta(acc, pa + 8 * kk, vd + (uint64_t)((kk >> 2) * (kAtom >> 4) + 2 * (kk & 3)), p.idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                        if (t == n_q - 1) umma_commit(smem_u32(&bars[kDVEmpty + (i & 1)]));     // V stage free
+                        if (i + 1 < n_kt) {
+                            if (t == 0 && !(ok = mbar_wait(smem_u32(&bars[kDKFull + ((i + 1) & 1)]), (uint32_t)((i + 1) >> 1) & 1u, abort_flag))) break;
+                            tc_fence_after();
+                            issue_qk(t, i + 1);
+                        }
+                    }
+                }
+                if (ok) umma_commit(smem_u32(&bars[kDODone]));
+                if (!ok) {
+                    *abort_flag = 1;
+                    atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
+                }
+            }
+            __syncwarp();
+        }
+        __syncwarp();
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        // -------------------------------------------------------- softmax, one thread per query row
+        const int t = (warp - 4) >> 2, quarter = warp & 3;        // query tile; TMEM lanes 32*quarter .. +31
+        const int r = quarter * 32 + lane;
+        bool ok = true;
+        if (t < n_q) {
+            const Item q = item(t);
+            // warps whose rows are all beyond the valid ones only keep the barrier counts right (the test is per warp:
+            // tcgen05.ld and .st are warp-collective)
+            const int sj = r >> p.slot_shift, rr = r & (p.slot - 1);          // slot (head q.h + sj) and row within it
+            const bool live = ((quarter * 32) >> p.slot_shift) < q.n_slots && ((quarter * 32) & (p.slot - 1)) < q.n_valid;
+            const uint32_t t_s = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * kTile);
+            const uint32_t t_o = t_s + (uint32_t)(2 * kTile);
+            const uint64_t c2 = f32x2(p.scale_log2e, p.scale_log2e);
+            float m = 0.f, l = 0.f;
+            for (int i = 0; i < n_kt; ++i) {
+                if (!(ok = mbar_wait(smem_u32(&bars[kDSFull + t]), (uint32_t)i & 1u, abort_flag))) break;
+                tc_fence_after();
+                const int n_keys = min(kTile, n_vis - i * kTile);             // valid keys of this tile
+                // keys past n_vis may hold anything: zero their V columns so that 0 * garbage stays 0 (tile 0's threads, row r
+                // of the transposed V tile = head dim r; P V of either tile is issued after tile 0's P has been seen)
+                if (n_keys < kTile && t == 0) {
+                    if (!(ok = mbar_wait(smem_u32(&bars[kDVFull + (i & 1)]), (uint32_t)(i >> 1) & 1u, abort_flag))) break;
+                    uint8_t* vt = sV + (size_t)(i & 1) * kOperand + r * 128;
+                    for (int kv = n_keys; kv < kTile; ++kv)
+                        *reinterpret_cast<uint16_t*>(vt + (kv >> 6) * kAtom + ((((kv & 63) >> 3) ^ (r & 7)) << 4) + (kv & 7) * 2) = 0;
+                    fence_proxy_async_smem();
+                }
+                if (live) {
+                    uint32_t sc[4][32];
+                    float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        tmem_ld32(t_s + (uint32_t)(32 * c), sc[c]);
+                        if (n_keys < kTile) {
+#pragma unroll
+                            for (int k = 0; k < 32; ++k)
+                                if (32 * c + k >= n_keys) sc[c][k] = __float_as_uint(-INFINITY);
+                        }
+#pragma unroll
+                        for (int k = 0; k < 32; k += 2) {
+                            mx0 = fmaxf(mx0, __uint_as_float(sc[c][k]));
+                            mx1 = fmaxf(mx1, __uint_as_float(sc[c][k + 1]));
+                        }
+                    }
+                    const float mx = fmaxf(mx0, mx1) * p.scale_log2e;          // the scale is positive
+                    if (i == 0) {
+                        m = mx;
+                    } else if (__any_sync(0xffffffffu, mx > m + 8.f)) {
+                        // (P V(i - 1) is complete: S(i) was issued behind it)
+                        const float mn = fmaxf(m, mx), alpha = ex2_approx(m - mn);
+                        m = mn;
+                        l *= alpha;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t v[32];
+                            tmem_ld32(t_o + (uint32_t)(32 * c), v);
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) v[k] = __float_as_uint(__uint_as_float(v[k]) * alpha);
+                            tmem_st32(t_o + (uint32_t)(32 * c), v);
+                        }
+                    }
+                    const uint64_t nm2 = f32x2(-m, -m);
+                    uint64_t l2[2] = {0ull, 0ull};
+#pragma unroll
+                    for (int hc = 0; hc < 2; ++hc) {
+                        uint32_t pw[32];
+#pragma unroll
+                        for (int g = 0; g < 32; ++g) {
+                            // masked keys: fma(-inf, c, -m) = -inf, exp2(-inf) = 0
+                            const uint32_t* q2 = &sc[2 * hc + (g >> 4)][2 * (g & 15)];
+                            float a, c;
+                            f32x2_get(f32x2_fma(f32x2(__uint_as_float(q2[0]), __uint_as_float(q2[1])), c2, nm2), a, c);
+                            a = ex2_approx(a);
+                            c = ex2_approx(c);
+                            l2[g & 1] = f32x2_add(l2[g & 1], f32x2(a, c));
+                            pw[g] = pack_bf16(a, c);
+                        }
+                        tmem_st32(t_s + (uint32_t)(32 * hc), pw);             // P over the S columns: all scores are in registers
+                    }
+                    float a, c;
+                    f32x2_get(f32x2_add(l2[0], l2[1]), a, c);
+                    l += a + c;
+                }
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bars[kDPFull + t]));
+            }
+            ok = ok && mbar_wait(smem_u32(&bars[kDODone]), 0, abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            tc_fence_after();
+            if (ok && live) {
+                const bool valid = sj < q.n_slots && rr < q.n_valid;
+                const float inv = 1.f / l;
+                const size_t base = ((size_t)(q.row0 + rr) * p.Hq + q.h + sj) * kTile;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t v[32];
+                    tmem_ld32(t_o + (uint32_t)(32 * c), v);
+                    if (valid) {
+                        uint4* dst = reinterpret_cast<uint4*>(p.out + base + 32 * c);
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            uint4 u;
+                            u.x = pack_bf16(__uint_as_float(v[8 * g]) * inv, __uint_as_float(v[8 * g + 1]) * inv);
+                            u.y = pack_bf16(__uint_as_float(v[8 * g + 2]) * inv, __uint_as_float(v[8 * g + 3]) * inv);
+                            u.z = pack_bf16(__uint_as_float(v[8 * g + 4]) * inv, __uint_as_float(v[8 * g + 5]) * inv);
+                            u.w = pack_bf16(__uint_as_float(v[8 * g + 6]) * inv, __uint_as_float(v[8 * g + 7]) * inv);
+                            dst[g] = u;
+                        }
+                        if (p.tap) {
+#pragma unroll
+                            for (int k = 0; k < 32; ++k) p.tap[base + 32 * c + k] = __uint_as_float(v[k]) * inv;
+                        }
+                    }
+                }
+            }
+            if (!ok) {
+                *abort_flag = 1;
+                if (lane == 0) atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
+            }
+        }
+        tc_fence_before();
+    }
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)kTmemCols);
+    }
+}
+
 #ifdef WD_GEMM_TRACE
 extern "C" __attribute__((visibility("default"))) int wd_debug_attn_stamps(unsigned long long* host /*[160][8]*/) {
     cudaDeviceSynchronize();
@@ -611,7 +915,7 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
                             const int32_t* qtile_n, const int32_t* seq_nvis, const CUtensorMap* map_k,
                             const CUtensorMap* map_vt, void* out, float* tap, int Hq, int Hkv, int dh, int layer,
                             int max_vis, int sm_count, int32_t* status, cudaStream_t stream, int max_tile_rows,
-                            size_t* smem_used) {
+                            size_t* smem_used, const int32_t* seq_qt_off, int batch, int max_seq_tiles) {
     if (dh != kTile) return WD_ERR_BAD_PARAM;
     if (n_tiles <= 0) return WD_OK;
     EncodeTiledFn enc = get_encode();
@@ -660,6 +964,34 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
     p.slot_shift = pack == 1 ? 7 : (pack == 2 ? 6 : 5);
     p.tiles_per_kv = (group + pack - 1) / pack;
     const int grid_y = Hkv * p.tiles_per_kv;
+    static bool attr_done[64] = {};     // the attribute is per device
+    // More single-tile CTAs than SMs: two tiles per CTA (the rule is the wave: up to one of them the single-tile kernel, with its
+    // keys split over a cluster when SMs are left over, has the shorter chain).  Measured, single / two tiles, in us: 583 rows,
+    // 32 heads 32.8 / 24.8; 1536 rows, 32 heads 78.8 / 70.3 (192 CTAs for 148 SMs); eight sequences of 672 rows, 28 query and 4
+    // KV heads 158 / 113, of 66 rows over 830 keys 38.9 / 28.8; 1792 rows, 128 heads 360 / 257.
+    static const int dual_on = getenv("WD_ATTN_DUAL") ? atoi(getenv("WD_ATTN_DUAL")) : 1;
+    if (dual_on && seq_qt_off && n_tiles * grid_y > sm_count) {
+        static bool dual_done[64] = {};
+        if (!dual_done[dev]) {
+            WD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_dual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDualSmem));
+            dual_done[dev] = true;
+        }
+        p.seq_qt_off = seq_qt_off;
+        if (smem_used) *smem_used = kDualSmem;
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3((unsigned)((max_seq_tiles * p.tiles_per_kv + 1) / 2), (unsigned)Hkv, (unsigned)batch);
+        lc.blockDim = dim3(kDThreads);
+        lc.dynamicSmemBytes = kDualSmem;
+        lc.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        lc.attrs = attr;
+        lc.numAttrs = wd_pdl_enabled ? 1 : 0;
+        ++wd_launch_counter;
+        WD_CUDA_TRY(cudaLaunchKernelEx(&lc, attention_tc_dual_kernel, mq, *map_k, *map_vt, p));
+        return WD_OK;
+    }
     int want = sm_count / (n_tiles * grid_y);
     if (want < 1) want = 1;
     if (want > kMaxCluster) want = kMaxCluster;
@@ -672,7 +1004,6 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
                                (1 + 2) * (size_t)kOperand + (kBars + 1) * 8 + 16 + 2 * kTile * 4 + 1024};
     const size_t smem = smem_of[single ? 1 : 0];
     if (smem_used) *smem_used = smem;
-    static bool attr_done[64] = {};     // the attribute is per device
     if (!attr_done[dev]) {
         WD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of[0]));
         WD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_single_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of[1]));

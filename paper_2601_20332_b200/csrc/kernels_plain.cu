@@ -199,7 +199,7 @@ struct PlanArgs {
     const int32_t* dec_step;
     int32_t* wex;                 // [batch][S]
     int32_t *row_seq, *row_pos, *act_row, *act_pos, *act_off_dev, *vis_off_dev, *vis_idx, *qt_seq, *qt_row0, *qt_n, *nvis_dev,
-        *tseq_dev;
+        *tseq_dev, *qt_off_dev;
     int32_t* status;
 };
 
@@ -231,7 +231,9 @@ __global__ void plan_kernel(const PlanArgs a) {
         a.vis_off_dev[b] = a.vis_off[b];
         a.nvis_dev[b] = a.done[b] ? 0 : a.n_vis[b];
         a.tseq_dev[b] = a.t[b];
-        if (b == a.batch - 1) { a.act_off_dev[a.batch] = a.act_off[a.batch]; a.vis_off_dev[a.batch] = a.vis_off[a.batch]; }
+        a.qt_off_dev[b] = a.qt_off[b];
+        if (b == a.batch - 1) {
+            a.qt_off_dev[a.batch] = a.qt_off[a.batch]; a.act_off_dev[a.batch] = a.act_off[a.batch]; a.vis_off_dev[a.batch] = a.vis_off[a.batch]; }
     }
     if (a.done[b]) return;
     const int S = a.S, row0 = a.row_off[b], act0 = a.act_off[b];
@@ -1453,7 +1455,7 @@ void wd_launch_plan(const WdPlanLaunch& h, cudaStream_t st) {
     a.decoded = h.decoded; a.dec_step = h.dec_step; a.wex = h.wex;
     a.row_seq = h.row_seq; a.row_pos = h.row_pos; a.act_row = h.act_row; a.act_pos = h.act_pos;
     a.act_off_dev = h.act_off_dev; a.vis_off_dev = h.vis_off_dev; a.vis_idx = h.vis_idx;
-    a.qt_seq = h.qt_seq; a.qt_row0 = h.qt_row0; a.qt_n = h.qt_n; a.nvis_dev = h.nvis_dev; a.tseq_dev = h.tseq_dev;
+    a.qt_seq = h.qt_seq; a.qt_row0 = h.qt_row0; a.qt_n = h.qt_n; a.nvis_dev = h.nvis_dev; a.tseq_dev = h.tseq_dev; a.qt_off_dev = h.qt_off_dev;
     a.status = h.status;
     launch_pdl(plan_kernel, dim3(h.batch), dim3(256), 0, st, a);
 }
@@ -1493,7 +1495,8 @@ int32_t* wd_op_status_ptr() {
 }
 
 // Query-tile lists of ONE sequence whose n_rows rows all see positions [0, n_vis): tile t covers
-// rows [128 t, 128 t + n).  Layout of `lists`: seq[n_tiles] | row0[n_tiles] | n[n_tiles] | n_vis[1].
+// rows [128 t, 128 t + n).  Layout of `lists`: seq[n_tiles] | row0[n_tiles] | n[n_tiles] | n_vis[1] | first tile of
+// the sequence and of the one after it [2].
 __global__ void fill_qtiles_kernel(int32_t* lists, int n_rows, int n_vis) {
     const int n_tiles = (n_rows + 127) / 128;
     for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
@@ -1501,7 +1504,11 @@ __global__ void fill_qtiles_kernel(int32_t* lists, int n_rows, int n_vis) {
         lists[n_tiles + t] = 128 * t;
         lists[2 * n_tiles + t] = min(128, n_rows - 128 * t);
     }
-    if (threadIdx.x == 0) lists[3 * n_tiles] = n_vis;
+    if (threadIdx.x == 0) {
+        lists[3 * n_tiles] = n_vis;
+        lists[3 * n_tiles + 1] = 0;
+        lists[3 * n_tiles + 2] = n_tiles;
+    }
 }
 
 void wd_launch_fill_qtiles(int32_t* lists, int n_rows, int n_vis, cudaStream_t st) {

@@ -183,7 +183,7 @@ struct WdPlanLaunch {
     const int32_t* dec_step;      // [batch][S] device
     int32_t* wex;                 // [batch][S] device: external window of the phase
     int32_t *row_seq, *row_pos, *act_row, *act_pos, *act_off_dev, *vis_off_dev, *vis_idx, *qt_seq, *qt_row0, *qt_n, *nvis_dev,
-        *tseq_dev;
+        *tseq_dev, *qt_off_dev;
     int32_t* status;
 };
 void wd_launch_plan(const WdPlanLaunch& h, cudaStream_t st);

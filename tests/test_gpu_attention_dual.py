@@ -1,0 +1,35 @@
+"""The attention kernel with two query tiles per CTA (launches of more single-tile CTAs than SMs), against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import wd_oracle as wo
+from paper_2601_20332_b200 import binding as wd
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+# more than 148 (row tile, query head) items: an odd number of tiles (a CTA with one), a last tile of one row, one key tile,
+# one key in the last tile, one below and one above a tile; grouped-query heads whose items pair across row tiles (7 per
+# tile); packed heads (two and four per tile) with empty slots; scores whose row maxima grow by tens of units from tile to
+# tile, so that the accumulated output is rescaled, and mild ones, where it is not
+@pytest.mark.parametrize("rows,nv,Hq,Hkv,S,qs", [(257, 128, 64, 64, 136, 1.5), (300, 127, 64, 64, 128, 8.0),
+                                                 (260, 129, 56, 8, 136, 8.0), (130, 1025, 84, 12, 1032, 8.0),
+                                                 (640, 400, 32, 32, 400, 1.5), (33, 300, 320, 64, 304, 8.0),
+                                                 (20, 700, 693, 99, 704, 1.5), (128, 1, 160, 160, 8, 1.5)])
+def test_two_tiles_per_cta_vs_oracle(rows, nv, Hq, Hkv, S, qs):
+    g = torch.Generator(device=DEV).manual_seed(rows + nv)
+    q = (torch.randn(rows, Hq, 128, device=DEV, generator=g) * qs).to(torch.bfloat16)
+    kc = torch.randn(Hkv, S, 128, device=DEV, generator=g).to(torch.bfloat16)
+    kc *= torch.linspace(0.5, 2.0, S, device=DEV).to(torch.bfloat16)[None, :, None]        # later keys score higher
+    vc = torch.randn(Hkv, S, 128, device=DEV, generator=g).to(torch.bfloat16)
+    K = kc.double().cpu().numpy().transpose(1, 0, 2)[:nv]
+    V = vc.double().cpu().numpy().transpose(1, 0, 2)[:nv]
+    kc[:, nv:] = float("nan")                       # what must not be read as a value
+    vc[:, nv:] = float("nan")
+    out = wd.op_attention_tc(q, kc, vc.transpose(1, 2).contiguous(), nv).float().cpu().numpy().astype(np.float64)
+    assert wd.op_status() == 0 and np.isfinite(out).all()
+    ref, _ = wo.attention_rows(q.double().cpu().numpy(), K, V, Hq // Hkv)
+    # P and the result rounded to bf16: as in test_attention_tc_kernel_vs_oracle
+    assert np.abs(out - ref).max() / np.abs(ref).max() < 2e-2
