@@ -65,10 +65,11 @@ struct wd_ctx {
     // configuration (StepKey) has been seen before is captured once and replayed afterwards
     struct StepKey {
         uint64_t state_uid = 0;
-        int batch = 0, rows = 0, n_act = 0, n_qtiles = 0, key_tiles = 0, max_tile_rows = 0, max_seq_tiles = 0, k_eff = 0, mode = 0, impl = 0, attn_impl = 0;
+        int batch = 0, rows = 0, n_act = 0, n_qtiles = 0, key_tiles = 0, max_tile_rows = 0, max_seq_tiles = 0, n_aqt = 0, max_seq_act_tiles = 0, max_act_tile_rows = 0, k_eff = 0, mode = 0, impl = 0, attn_impl = 0;
         bool operator==(const StepKey& o) const {
             return state_uid == o.state_uid && batch == o.batch && rows == o.rows && n_act == o.n_act && n_qtiles == o.n_qtiles &&
-                   key_tiles == o.key_tiles && max_tile_rows == o.max_tile_rows && max_seq_tiles == o.max_seq_tiles && k_eff == o.k_eff && mode == o.mode &&
+                   key_tiles == o.key_tiles && max_tile_rows == o.max_tile_rows && max_seq_tiles == o.max_seq_tiles && n_aqt == o.n_aqt &&
+                   max_seq_act_tiles == o.max_seq_act_tiles && max_act_tile_rows == o.max_act_tile_rows && k_eff == o.k_eff && mode == o.mode &&
                    impl == o.impl && attn_impl == o.attn_impl;
         }
     };
@@ -94,6 +95,11 @@ struct wd_ctx {
     float* ch_max = nullptr;     // [max_active][chunks] unmask stage-1 statistics
     int32_t* ch_idx = nullptr;
     double* ch_sum = nullptr;
+    // the last block's rows of a refresh step: the active ones, one after the other
+    float* x_act = nullptr;      // [max_active, d]
+    void* xn_act = nullptr;      // [max_active, d] (model dtype)
+    float2* rope_act = nullptr;  // [max_active][dh/2]
+    int32_t* seq_act = nullptr;  // [max_active]
     float2* rope_tab = nullptr;  // [max_rows][dh/2] (cos, sin) of this step's rows
     float* sumsq = nullptr;      // [d/128][max_rows] partial sums of squares of the residual rows
     int32_t* tile_counters = nullptr;  // arrival counters of the fused GEMM epilogues (kept zero)
@@ -175,7 +181,7 @@ static size_t part_floats_for(const wd_model_dims* d) {
     return std::max((size_t)d->max_rows * cols, (size_t)WD_TC_MAX_SPLIT * small_rows * cols);
 }
 
-static void carve_ctx(const wd_model_dims* d, Carve& c, size_t off[24]) {
+static void carve_ctx(const wd_model_dims* d, Carve& c, size_t off[28]) {
     const size_t e = wd_elt_size(d->dtype);
     const size_t MR = d->max_rows, MA = d->max_active, hq = (size_t)d->n_q_heads * d->head_dim;
     off[0] = c.take(MR * d->d_model * 4);                       // x
@@ -188,8 +194,8 @@ static void carve_ctx(const wd_model_dims* d, Carve& c, size_t off[24]) {
     off[7] = c.take(MA * 4);                                    // row_token
     off[8] = c.take(MA * 8);                                    // row_sumexp
     off[9] = c.take(MA * 4);                                    // row_conf
-    const size_t plan_ints = 2 * MR + 2 * MA + 3 * ((size_t)d->max_batch + 1) + (size_t)d->max_batch * d->max_seq +
-                             3 * (MR / 128 + (size_t)d->max_batch + 1) + 2 * (size_t)d->max_batch +
+    const size_t plan_ints = 2 * MR + 2 * MA + 4 * ((size_t)d->max_batch + 1) + (size_t)d->max_batch * d->max_seq +
+                             3 * (MR / 128 + (size_t)d->max_batch + 1) + 3 * (MA / 128 + (size_t)d->max_batch + 1) + 2 * (size_t)d->max_batch +
                              (size_t)d->max_batch * d->max_seq;      // + staging of the external windows
     off[10] = c.take(plan_ints * 4);                            // plan
     off[11] = c.take((1 + (size_t)d->max_batch + 3 * MA) * 4);  // result
@@ -204,13 +210,17 @@ static void carve_ctx(const wd_model_dims* d, Carve& c, size_t off[24]) {
     off[18] = c.take(((max_gemm_cols(d) + 127) / 128) * (MR / 256 + 2) * 4);   // tile counters
     off[19] = ((max_gemm_cols(d) + 127) / 128) * (MR / 256 + 2);
     off[20] = c.take(256);                                       // chain kernel counters
-    off[21] = c.off;
+    off[21] = c.take(MA * d->d_model * 4);                      // x_act
+    off[22] = c.take(MA * d->d_model * e);                      // xn_act
+    off[23] = c.take(MA * (size_t)(d->head_dim / 2) * 8);       // rope_act
+    off[24] = c.take(MA * 4);                                   // seq_act
+    off[25] = c.off;
 }
 
 extern "C" size_t wd_workspace_bytes(const wd_model_dims* dims) {
     if (!dims_valid(dims)) return 0;
     Carve c;
-    size_t off[24];
+    size_t off[28];
     carve_ctx(dims, c, off);
     return c.off;
 }
@@ -272,12 +282,13 @@ extern "C" wd_status wd_create(const wd_model_dims* dims, const wd_weights* w, v
         c->attn_norm.push_back(w->attn_norm[l]); c->ffn_norm.push_back(w->ffn_norm[l]);
     }
     Carve cv;
-    size_t off[24];
+    size_t off[28];
     carve_ctx(dims, cv, off);
     char* base = (char*)workspace;
     c->x = (float*)(base + off[0]);
     c->xn = base + off[1];
     c->q = base + off[2];
+    c->x_act = (float*)(base + off[21]); c->xn_act = base + off[22]; c->rope_act = (float2*)(base + off[23]); c->seq_act = (int32_t*)(base + off[24]);
     c->attn = base + off[3];
     c->h = base + off[4];
     c->part = (float*)(base + off[5]);
@@ -304,7 +315,7 @@ extern "C" wd_status wd_create(const wd_model_dims* dims, const wd_weights* w, v
 
     if (dims->dtype == WD_BF16) {
         wd_status s = wd_tc_weights_init(&c->tc, dims, c->tok_embed, c->lm_head, c->wq, c->wk, c->wv, c->wo,
-                                         c->wg, c->wu, c->wd, c->xn, c->attn, c->h);
+                                         c->wg, c->wu, c->wd, c->xn, c->attn, c->h, c->xn_act);
         if (s != WD_OK) { delete c; return s; }
     }
     *out = c;
@@ -1071,6 +1082,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     bool all_done = true, any_refresh = false, all_contig = true;
     size_t n_rows = 0, n_act = 0, n_vis = 0, n_qtiles = 0;
     int max_vis = 0, max_tile_rows = 0, max_seq_tiles = 0;
+    int n_aqt = 0, max_act_tile_rows = 0, max_seq_act_tiles = 0;        // query tiles over the active rows alone
     if (!dev_mode) {
         st->plans.assign(batch, WdSeqPlan());
         for (int b = 0; b < batch; ++b) {
@@ -1113,6 +1125,9 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         max_vis = std::max(max_vis, (int)cp.n_vis);
         max_tile_rows = std::max(max_tile_rows, std::min(128, (int)cp.n_rows));
         max_seq_tiles = std::max(max_seq_tiles, ((int)cp.n_rows + 127) / 128);
+        n_aqt += ((int)cp.n_active + 127) / 128;
+        max_act_tile_rows = std::max(max_act_tile_rows, std::min(128, (int)cp.n_active));
+        max_seq_act_tiles = std::max(max_seq_act_tiles, ((int)cp.n_active + 127) / 128);
     }
     if (all_done) return WD_DONE;
     if (n_rows > (size_t)d.max_rows || n_act > (size_t)d.max_active ||
@@ -1133,6 +1148,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     const size_t o_qt_n = o; o += n_qtiles;
     const size_t o_nvis = o; o += batch;
     const size_t o_qt_off = o; o += batch + 1;
+    const size_t o_aqt_seq = o; o += n_aqt;
+    const size_t o_aqt_row0 = o; o += n_aqt;
+    const size_t o_aqt_n = o; o += n_aqt;
+    const size_t o_aqt_off = o; o += batch + 1;
     const size_t o_tseq = o; o += batch;          // step index of each sequence (for the decode-step stamps)
     const size_t o_vis_idx = o; o += n_vis;       // last: every other offset depends on rows, active rows and tiles only
     if (o > c->plan_ints) return WD_ERR_CAPACITY;
@@ -1141,16 +1160,20 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         WdPlanLaunch pl;
         memset(&pl, 0, sizeof(pl));
         pl.batch = batch; pl.S = S; pl.A = A; pl.T = T;
-        int32_t r = 0, a = 0, v = 0, qt = 0;
+        int32_t r = 0, a = 0, v = 0, qt = 0, aqt = 0;
         for (int b = 0; b < batch; ++b) {
             const WdCountPlan& cp = pend.cp[b];
-            pl.row_off[b] = r; pl.act_off[b] = a; pl.vis_off[b] = v; pl.qt_off[b] = qt;
+            pl.row_off[b] = r; pl.act_off[b] = a; pl.vis_off[b] = v; pl.qt_off[b] = qt; pl.aqt_off[b] = aqt;
             pl.done[b] = cp.done; pl.refresh[b] = cp.refresh; pl.n_wex[b] = cp.n_wex; pl.n_vis[b] = cp.n_vis;
             pl.t[b] = st->counts[b].t;
             pl.window_refresh[b] = cp.window_refresh ? 1 : 0; pl.prev_phase_start[b] = cp.prev_phase_start;
             if (cp.done) continue;
             r += cp.n_rows; a += cp.n_active; v += cp.n_vis; qt += (cp.n_rows + 127) / 128;
+            aqt += (cp.n_active + 127) / 128;
         }
+        pl.aqt_off[batch] = aqt;
+        pl.aqt_seq = c->plan + o_aqt_seq; pl.aqt_row0 = c->plan + o_aqt_row0; pl.aqt_n = c->plan + o_aqt_n;
+        pl.aqt_off_dev = c->plan + o_aqt_off;
         pl.row_off[batch] = r; pl.act_off[batch] = a; pl.vis_off[batch] = v; pl.qt_off[batch] = qt;
         pl.decoded = st->decoded_dev; pl.dec_step = st->dec_step_dev; pl.wex = st->wex_dev;
         pl.row_seq = c->plan + o_row_seq; pl.row_pos = c->plan + o_row_pos;
@@ -1162,7 +1185,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         pl.status = c->result;
         wd_launch_plan(pl, stream);
     } else {
-        size_t r = 0, a = 0, v = 0, qt = 0;
+        size_t r = 0, a = 0, v = 0, qt = 0, aqt = 0;
         for (int b = 0; b < batch; ++b) {
             const WdSeqPlan& p = st->plans[b];
             ph[o_act_off + b] = (int32_t)a;
@@ -1170,11 +1193,17 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             ph[o_nvis + b] = p.done ? 0 : (int32_t)p.vis.size();
             ph[o_tseq + b] = st->seqs[b].t;
             ph[o_qt_off + b] = (int32_t)qt;
+            ph[o_aqt_off + b] = (int32_t)aqt;
             if (p.done) continue;
             for (size_t t0 = 0; t0 < p.rows.size(); t0 += 128, ++qt) {
                 ph[o_qt_seq + qt] = b;
                 ph[o_qt_row0 + qt] = (int32_t)(r + t0);
                 ph[o_qt_n + qt] = (int32_t)std::min<size_t>(128, p.rows.size() - t0);
+            }
+            for (size_t t0 = 0; t0 < p.active.size(); t0 += 128, ++aqt) {
+                ph[o_aqt_seq + aqt] = b;
+                ph[o_aqt_row0 + aqt] = (int32_t)(a + t0);
+                ph[o_aqt_n + aqt] = (int32_t)std::min<size_t>(128, p.active.size() - t0);
             }
             size_t ai = 0;
             for (size_t i = 0; i < p.rows.size(); ++i) {
@@ -1192,6 +1221,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         }
         ph[o_act_off + batch] = (int32_t)a;
         ph[o_qt_off + batch] = (int32_t)qt;
+        ph[o_aqt_off + batch] = (int32_t)aqt;
         ph[o_vis_off + batch] = (int32_t)v;
         WD_CUDA_TRY(cudaMemcpyAsync(c->plan, ph, o * 4, cudaMemcpyHostToDevice, stream));
         // keep the device copy of the planner state complete (the unmask kernel maintains the flags
@@ -1251,8 +1281,12 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         wd_fp4_operand_split(c->fp4_x, NA, D, &x4_lm);
     }
     size_t attn_smem = 0;               // shared memory of an attention CTA (tensor-core form), for the projection after it
-    auto attention = [&](int l, char* kc, char* vc) -> wd_status {
+    auto attention = [&](int l, char* kc, char* vc, bool act_only = false) -> wd_status {
         float* attn_tap = st->taps.attn_out ? st->taps.attn_out + (size_t)l * R_ * hq : nullptr;
+        if (act_only)       // q holds the active rows, one after the other
+            return wd_attn_tc_launch(c->q, NA, n_aqt, c->plan + o_aqt_seq, c->plan + o_aqt_row0, c->plan + o_aqt_n, c->plan + o_nvis,
+                                     &st->map_k, &st->map_vt, c->attn, nullptr, Hq, Hkv, dh, l, max_vis, c->sm_count, status, stream,
+                                     max_act_tile_rows, &attn_smem, c->plan + o_aqt_off, batch, max_seq_act_tiles);
         if (st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN)
             return wd_attn_tc_launch(c->q, R_, (int)n_qtiles, c->plan + o_qt_seq, c->plan + o_qt_row0, c->plan + o_qt_n,
                                      c->plan + o_nvis, &st->map_k, &st->map_vt, c->attn, attn_tap, Hq, Hkv, dh, l, max_vis,
@@ -1261,6 +1295,13 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                                   Hkv, dh, S, Sp, batch, status, stream);
         return WD_OK;
     };
+    // Nothing reads the last block's output but the final norm, and that only at the active rows: a refresh step's last block
+    // computes keys and values of every row (the cache wants them) and the rest for the active rows, which a gather puts one
+    // after the other.  From 257 rows on, where the GEMMs' time depends on their rows, and when it at least halves them (352 rows,
+    // 32 active: 225 us of a block -> 120; 28672 rows, 2048 active: 11.2 ms -> 2.3 ms; a step of 104 rows streams weights either
+    // way and would pay three more launches).  Not for a model of one block, and not when a tap wants every row of every block.
+    const bool act_last = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN && !fp8 && !fp4 && !fused &&
+                          d.n_layers > 1 && NA > 0 && R_ > 256 && 2 * NA <= R_ && !st->taps.layer_out && !st->taps.attn_out;
     // ---- the kernels of the step, from the embedding to the selection (everything after the planner and
     // before the copy of the result block); launched directly, or recorded into a CUDA graph and replayed
     auto run_kernels = [&]() -> wd_status {
@@ -1352,6 +1393,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     for (int l = 0; l < d.n_layers; ++l) {
         char* kc = st->kcache + (size_t)l * st->kv_layer_bytes;
         char* vc = st->vcache + (size_t)l * st->v_layer_bytes;
+        const bool act = act_last && l == d.n_layers - 1;
         // attention half (FP8 mode: the normalised rows leave the RMSNorm as e4m3 codes + row scales)
         wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
                           c->attn_norm[l], d.rms_eps, c->xn, nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn,
@@ -1367,6 +1409,16 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             if ((s = run_gemm(c, c->xn8, &c->x8_d, qkv, 3, R_, D, c->part, c->part_floats, status, stream, &go, false,
                               nullptr, &f8)) != WD_OK)
                 return s;
+        } else if (act) {
+            // keys and values of every row
+            WdTcSeg kv[2] = {{c->wk[l], hkv, c->tc.get(WD_TC_WK, l)}, {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
+            if ((s = run_gemm(c, c->xn, &c->tc.x_map_d, kv, 2, R_, D, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
+            wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, row_seq, row_pos, c->rope_tab, c->q, kc, vc, R_, 0, Hkv,
+                                   dh, S, Sp, batch, status, stream);
+            // queries of the active rows
+            wd_launch_gather_active(c->x, c->xn, c->rope_tab, row_seq, act_row, c->x_act, c->xn_act, c->rope_act, c->seq_act, NA, D, dh / 2, stream);
+            WdTcSeg wq[1] = {{c->wq[l], hq, c->tc.get(WD_TC_WQ, l)}};
+            if ((s = run_gemm(c, c->xn_act, &c->tc.x_map_act, wq, 1, NA, D, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
         } else {
         WdTcSeg qkv[3] = {{c->wq[l], hq, c->tc.get(WD_TC_WQ, l)}, {c->wk[l], hkv, c->tc.get(WD_TC_WK, l)},
                           {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
@@ -1374,25 +1426,34 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             return s;
         }
         impl_used = go.impl;
-        wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, row_seq, row_pos, c->rope_tab, c->q, kc,
-                               vc, R_, Hq, Hkv, dh, S, Sp, batch, status, stream);
-        if ((s = attention(l, kc, vc)) != WD_OK) return s;
+        if (act)
+            wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, c->seq_act, act_pos, c->rope_act, c->q, kc, vc, NA, Hq, 0,
+                                   dh, S, Sp, batch, status, stream);
+        else
+            wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, row_seq, row_pos, c->rope_tab, c->q, kc,
+                                   vc, R_, Hq, Hkv, dh, S, Sp, batch, status, stream);
+        if ((s = attention(l, kc, vc, act)) != WD_OK) return s;
+        // from here on the block works on these rows
+        const int Rb = act ? NA : R_;
+        float* xb = act ? c->x_act : c->x;
+        void* xnb = act ? c->xn_act : c->xn;
+        const WdTcX* xmb = act ? &c->tc.x_map_act : &c->tc.x_map_d;
         // the output projection's CTAs beside the attention's (when those take less than half an SM's shared
         // memory): a shorter ring, but its weights are on their way while the attention still runs
         // (measured: 215 KB for the two CTAs together still fits an SM, 222 KB does not)
-        c->tc.x_map_attn.smem_cap = (attn_smem > 0 && attn_smem <= 110 * 1024 && R_ <= 128) ? (int)(223232 - attn_smem) : 0;
+        c->tc.x_map_attn.smem_cap = (attn_smem > 0 && attn_smem <= 110 * 1024 && Rb <= 128) ? (int)(223232 - attn_smem) : 0;
         WdTcSeg wo[1] = {{c->wo[l], D, c->tc.get(WD_TC_WO, l)}};
         WdTcResid resid_o, resid_d;
-        resid_o.x = resid_d.x = c->x;
+        resid_o.x = resid_d.x = xb;
         WdTcEpi epi_o, epi_d;
         epi_o.resid = &resid_o;
         epi_d.resid = &resid_d;
-        if ((s = run_gemm(c, c->attn, &c->tc.x_map_attn, wo, 1, R_, hq, c->part, c->part_floats, status, stream, &go, false, nullptr,
+        if ((s = run_gemm(c, c->attn, &c->tc.x_map_attn, wo, 1, Rb, hq, c->part, c->part_floats, status, stream, &go, false, nullptr,
                           nullptr, &epi_o)) != WD_OK)
             return s;
         // feed-forward half
-        wd_launch_rmsnorm(d.dtype, c->x, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, c->xn,
-                          nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_d : nullptr);
+        wd_launch_rmsnorm(d.dtype, xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, xnb,
+                          nullptr, Rb, D, stream, fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_d : nullptr);
         if (fp4) {
             if ((s = run_gemm_fp4(c, &c->f4gu[l], R_, D, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
             if ((s = wd_launch_swiglu_fp4(c->part, go.n_split, go.split_stride, &x4_f, R_, F, stream)) != WD_OK) return s;
@@ -1417,12 +1478,12 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         sg.h = use_tc(c) ? (__nv_bfloat16*)c->h : nullptr;
         WdTcEpi epi_sg;
         epi_sg.sg = &sg;
-        if ((s = run_gemm(c, c->xn, &c->tc.x_map_d, gu, 2, R_, D, c->part, c->part_floats, status, stream, &go, false,
+        if ((s = run_gemm(c, xnb, xmb, gu, 2, Rb, D, c->part, c->part_floats, status, stream, &go, false,
                           nullptr, nullptr, &epi_sg)) != WD_OK)
             return s;
-        if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, R_, F, stream);
+        if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream);
         WdTcSeg wdn[1] = {{c->wd[l], D, c->tc.get(WD_TC_WD, l)}};
-        if ((s = run_gemm(c, c->h, &c->tc.x_map_h, wdn, 1, R_, F, c->part, c->part_floats, status, stream, &go, false, nullptr,
+        if ((s = run_gemm(c, c->h, &c->tc.x_map_h, wdn, 1, Rb, F, c->part, c->part_floats, status, stream, &go, false, nullptr,
                           nullptr, &epi_d)) != WD_OK)
             return s;
         }
@@ -1441,7 +1502,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     bool lm_fused = false;
     int lm_chunks = wd_unmask_chunks(d.vocab);
     if (NA > 0) {
-        wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride, c->final_norm, d.rms_eps, c->xn, act_row, NA, D, stream,
+        wd_launch_rmsnorm(d.dtype, act_last ? c->x_act : c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
+                          c->final_norm, d.rms_eps, c->xn, act_last ? nullptr : act_row, NA, D, stream,
                           fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_lm : nullptr);
         float* logits = st->taps.logits ? st->taps.logits : c->logits;      // a tap takes them directly
         WdTcSeg lm[1] = {{c->lm_head, d.vocab, c->tc.get(WD_TC_LM, 0)}};
@@ -1501,7 +1563,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         !st->queue.empty()) {
         wd_ctx::StepKey key;
         key.state_uid = st->uid; key.batch = batch; key.rows = R_; key.n_act = NA; key.n_qtiles = (int)n_qtiles;
-        key.key_tiles = (max_vis + 127) / 128; key.max_tile_rows = max_tile_rows; key.max_seq_tiles = max_seq_tiles; key.k_eff = k_eff;
+        key.key_tiles = (max_vis + 127) / 128; key.max_tile_rows = max_tile_rows; key.max_seq_tiles = max_seq_tiles; key.n_aqt = n_aqt;
+        key.max_seq_act_tiles = max_seq_act_tiles; key.max_act_tile_rows = max_act_tile_rows; key.k_eff = k_eff;
         key.mode = (c->fp8_on ? 1 : 0) | (c->fp4_on ? 2 : 0) | (st->attn_tc ? 4 : 0);
         key.impl = c->gemm_impl; key.attn_impl = c->attn_impl;
         wd_ctx::StepGraph* hit = nullptr;

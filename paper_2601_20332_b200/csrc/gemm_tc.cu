@@ -55,7 +55,6 @@ struct TcParams {
     // time share a few weight tiles and one group of token tiles (working set well inside the L2)
     int tok_grp;
     __nv_bfloat16* swiglu_h;        // dual == 2: [rows, ncol] with ncol = FFN width
-    float* resid_x;                 // pair kernel, kEpi == kEpiResid: [rows, ncol]
     // FP8 operands: K blocks of 128 elements, outputs scaled by sw[segment][n] * sx[token]
     int fp8;
     const float* sw[3];
@@ -65,7 +64,7 @@ struct TcParams {
     int seg_n[3];
     int seg_col[3];
     long long W;                    // total K blocks of the launch = n_units * kb_total
-    float* y;
+    float* y;                       // (kEpiResid: the residual stream)
     size_t split_stride;
     int32_t* status;
     uint32_t idesc;
@@ -598,7 +597,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     if (n_ok && p.f.write_logits) {
 #pragma unroll
                         for (int t = 0; t < 32; ++t)
-                            if (u.tok0 + cc + t < p.rows) yb[(size_t)(u.tok0 + cc + t) * p.ncol] = __uint_as_float(v[t]);
+                            if (cc + t < p.bn && u.tok0 + cc + t < p.rows)      // (the last chunk may reach beyond the token tile)
+                                yb[(size_t)(u.tok0 + cc + t) * p.ncol] = __uint_as_float(v[t]);
                     }
 #pragma unroll
                     for (int t = 0; t < 32; ++t) tr[t * 129 + n_local] = n_ok ? __uint_as_float(v[t]) : -INFINITY;
@@ -1312,7 +1312,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 for (int cc = 16 * hf; cc < p.bn && u.tok0 + cc < p.rows; cc += col_step) {
                     uint32_t v[16];
                     float xv[16];
-                    float* xs = p.resid_x + (size_t)(u.tok0 + cc) * p.ncol + n;
+                    float* xs = p.y + (size_t)(u.tok0 + cc) * p.ncol + n;
 #pragma unroll
                     for (int t = 0; t < 16; ++t) xv[t] = n_ok && u.tok0 + cc + t < p.rows ? xs[(size_t)t * p.ncol] : 0.f;
                     tmem_ld16(t_acc + (uint32_t)cc, v);
@@ -1679,7 +1679,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     const CUtensorMap& m2 = *segs[nseg > 2 ? 2 : 0].map;
     if (sg) sg->done = p.dual == 2;
     if (resid) resid->done = epi == kEpiResid;
-    if (epi == kEpiResid) p.resid_x = resid->x;
+    if (epi == kEpiResid) p.y = resid->x;
     ++wd_launch_counter;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)(2 * G * ts));
@@ -1708,7 +1708,8 @@ wd_status wd_tc_weights_init(WdTcWeights* tc, const wd_model_dims* d, const void
                              const std::vector<const void*>& wq, const std::vector<const void*>& wk,
                              const std::vector<const void*>& wv, const std::vector<const void*>& wo,
                              const std::vector<const void*>& wg, const std::vector<const void*>& wu,
-                             const std::vector<const void*>& wd, const void* xn, const void* attn, const void* h) {
+                             const std::vector<const void*>& wd, const void* xn, const void* attn, const void* h,
+                             const void* xn_act) {
     (void)tok_embed;
     const int L = d->n_layers, hq = d->n_q_heads * d->head_dim, hkv = d->n_kv_heads * d->head_dim;
     tc->n_layers = L;
@@ -1727,6 +1728,7 @@ wd_status wd_tc_weights_init(WdTcWeights* tc, const wd_model_dims* d, const void
     tc->x_map_d = {xn, d->d_model};
     tc->x_map_attn = {attn, hq};
     tc->x_map_h = {h, d->d_ffn};
+    tc->x_map_act = {xn_act, d->d_model};
     return WD_OK;
 }
 

@@ -35,7 +35,7 @@ struct WdTcX {
 struct WdTcWeights {
     std::vector<CUtensorMap> maps;      // [kind][layer]
     int n_layers = 0;
-    WdTcX x_map_d, x_map_attn, x_map_h;
+    WdTcX x_map_d, x_map_attn, x_map_h, x_map_act;
     const CUtensorMap* get(int kind, int l) const {
         return maps.empty() ? nullptr : &maps[(size_t)kind * n_layers + l];
     }
@@ -45,7 +45,8 @@ wd_status wd_tc_weights_init(WdTcWeights* tc, const wd_model_dims* d, const void
                              const std::vector<const void*>& wq, const std::vector<const void*>& wk,
                              const std::vector<const void*>& wv, const std::vector<const void*>& wo,
                              const std::vector<const void*>& wg, const std::vector<const void*>& wu,
-                             const std::vector<const void*>& wd, const void* xn, const void* attn, const void* h);
+                             const std::vector<const void*>& wd, const void* xn, const void* attn, const void* h,
+                             const void* xn_act);
 
 // What the CTA that completes an output tile does with the summed tile ("fused epilogue").
 // The tile sums still pass through the partial-sum slices in y; these modes only add the

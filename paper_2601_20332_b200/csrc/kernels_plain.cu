@@ -200,6 +200,8 @@ struct PlanArgs {
     int32_t* wex;                 // [batch][S]
     int32_t *row_seq, *row_pos, *act_row, *act_pos, *act_off_dev, *vis_off_dev, *vis_idx, *qt_seq, *qt_row0, *qt_n, *nvis_dev,
         *tseq_dev, *qt_off_dev;
+    int32_t aqt_off[WD_PLAN_MAX_BATCH + 1];
+    int32_t *aqt_seq, *aqt_row0, *aqt_n, *aqt_off_dev;
     int32_t* status;
 };
 
@@ -232,7 +234,9 @@ __global__ void plan_kernel(const PlanArgs a) {
         a.nvis_dev[b] = a.done[b] ? 0 : a.n_vis[b];
         a.tseq_dev[b] = a.t[b];
         a.qt_off_dev[b] = a.qt_off[b];
+        a.aqt_off_dev[b] = a.aqt_off[b];
         if (b == a.batch - 1) {
+            a.aqt_off_dev[a.batch] = a.aqt_off[a.batch];
             a.qt_off_dev[a.batch] = a.qt_off[a.batch]; a.act_off_dev[a.batch] = a.act_off[a.batch]; a.vis_off_dev[a.batch] = a.vis_off[a.batch]; }
     }
     if (a.done[b]) return;
@@ -248,6 +252,11 @@ __global__ void plan_kernel(const PlanArgs a) {
         a.qt_seq[a.qt_off[b] + j] = b;
         a.qt_row0[a.qt_off[b] + j] = row0 + 128 * j;
         a.qt_n[a.qt_off[b] + j] = min(128, n_rows - 128 * j);
+    }
+    for (int j = threadIdx.x; j < a.aqt_off[b + 1] - a.aqt_off[b]; j += blockDim.x) {
+        a.aqt_seq[a.aqt_off[b] + j] = b;
+        a.aqt_row0[a.aqt_off[b] + j] = act0 + 128 * j;
+        a.aqt_n[a.aqt_off[b] + j] = min(128, n_act - 128 * j);
     }
     if (a.refresh[b]) {
         // ordered compaction of the undecoded positions: the first n_wex form the window
@@ -575,6 +584,23 @@ __global__ void __launch_bounds__(1024, 1) rmsnorm_fp4_kernel(float* __restrict_
         const int c4 = threadIdx.x + u * blockDim.x;
         wdk::nvfp4_emit4(v[u], gr, c4 < nv, x4.codes + (size_t)i * (d >> 1), x4.sf + (size_t)i * (d >> 4), c4);
     }
+}
+
+// ---------------------------------------------------------------- gather of the active rows
+__global__ void __launch_bounds__(256) gather_active_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ xn,
+                                                            const float2* __restrict__ rope_tab, const int32_t* __restrict__ row_seq,
+                                                            const int32_t* __restrict__ act_row, float* __restrict__ x_act,
+                                                            __nv_bfloat16* __restrict__ xn_act, float2* __restrict__ rope_act,
+                                                            int32_t* __restrict__ seq_act, int d, int half) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int i = blockIdx.x, r = act_row[i];
+    const float4* xs = reinterpret_cast<const float4*>(x + (size_t)r * d);
+    const uint4* ns = reinterpret_cast<const uint4*>(xn + (size_t)r * d);
+    for (int c = threadIdx.x; c < d / 4; c += blockDim.x) reinterpret_cast<float4*>(x_act + (size_t)i * d)[c] = xs[c];
+    for (int c = threadIdx.x; c < d / 8; c += blockDim.x) reinterpret_cast<uint4*>(xn_act + (size_t)i * d)[c] = ns[c];
+    for (int c = threadIdx.x; c < half; c += blockDim.x) rope_act[(size_t)i * half + c] = rope_tab[(size_t)r * half + c];
+    if (threadIdx.x == 0) seq_act[i] = row_seq[r];
 }
 
 // ---------------------------------------------------------------- RoPE + K/V scatter
@@ -1285,6 +1311,13 @@ void wd_launch_rmsnorm(int dtype, float* x, const float* part, int n_split, size
     }
 }
 
+void wd_launch_gather_active(const float* x, const void* xn, const float2* rope_tab, const int32_t* row_seq, const int32_t* act_row,
+                             float* x_act, void* xn_act, float2* rope_act, int32_t* seq_act, int n_act, int d, int half, cudaStream_t st) {
+    if (n_act <= 0) return;
+    launch_pdl(gather_active_kernel, dim3(n_act), dim3(256), 0, st, x, (const __nv_bfloat16*)xn, rope_tab, row_seq, act_row, x_act,
+               (__nv_bfloat16*)xn_act, rope_act, seq_act, d, half);
+}
+
 void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t split_stride,
                             const int32_t* row_seq, const int32_t* row_pos, const float2* rope_tab, void* q,
                             void* kcache, void* vcache, int n_rows, int Hq, int Hkv, int dh, int S, int Sp,
@@ -1450,12 +1483,14 @@ void wd_launch_plan(const WdPlanLaunch& h, cudaStream_t st) {
     }
     for (int b = 0; b <= h.batch; ++b) {
         a.row_off[b] = h.row_off[b]; a.act_off[b] = h.act_off[b]; a.vis_off[b] = h.vis_off[b]; a.qt_off[b] = h.qt_off[b];
+        a.aqt_off[b] = h.aqt_off[b];
     }
     a.S = h.S; a.A = h.A; a.T = h.T; a.batch = h.batch;
     a.decoded = h.decoded; a.dec_step = h.dec_step; a.wex = h.wex;
     a.row_seq = h.row_seq; a.row_pos = h.row_pos; a.act_row = h.act_row; a.act_pos = h.act_pos;
     a.act_off_dev = h.act_off_dev; a.vis_off_dev = h.vis_off_dev; a.vis_idx = h.vis_idx;
     a.qt_seq = h.qt_seq; a.qt_row0 = h.qt_row0; a.qt_n = h.qt_n; a.nvis_dev = h.nvis_dev; a.tseq_dev = h.tseq_dev; a.qt_off_dev = h.qt_off_dev;
+    a.aqt_seq = h.aqt_seq; a.aqt_row0 = h.aqt_row0; a.aqt_n = h.aqt_n; a.aqt_off_dev = h.aqt_off_dev;
     a.status = h.status;
     launch_pdl(plan_kernel, dim3(h.batch), dim3(256), 0, st, a);
 }

@@ -126,6 +126,11 @@ void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t sp
                             int batch, int32_t* status, cudaStream_t st);
 // (a row whose position or sequence index is outside the state records WD_ERR_BOUNDS and writes no cache row)
 
+// The active rows of a step, one after the other: x_act[i] = x[act_row[i]], xn_act (bf16), rope_act and seq_act likewise.
+// d % 8 == 0, half = head_dim / 2 even.
+void wd_launch_gather_active(const float* x, const void* xn, const float2* rope_tab, const int32_t* row_seq, const int32_t* act_row,
+                             float* x_act, void* xn_act, float2* rope_act, int32_t* seq_act, int n_act, int d, int half, cudaStream_t st);
+
 // general (index-list) attention, CUDA cores.
 //   row_seq[r]: sequence of row r (null: one sequence)
 //   vis_idx: concatenated visible positions, sequence b at [vis_off[b], vis_off[b+1])
@@ -184,6 +189,8 @@ struct WdPlanLaunch {
     int32_t* wex;                 // [batch][S] device: external window of the phase
     int32_t *row_seq, *row_pos, *act_row, *act_pos, *act_off_dev, *vis_off_dev, *vis_idx, *qt_seq, *qt_row0, *qt_n, *nvis_dev,
         *tseq_dev, *qt_off_dev;
+    int32_t aqt_off[WD_PLAN_MAX_BATCH + 1];                      // query tiles over the active rows alone
+    int32_t *aqt_seq, *aqt_row0, *aqt_n, *aqt_off_dev;
     int32_t* status;
 };
 void wd_launch_plan(const WdPlanLaunch& h, cudaStream_t st);
