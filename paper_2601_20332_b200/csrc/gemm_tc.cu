@@ -18,6 +18,7 @@
 // Split-K partial sums are written side by side ([slice][tok][n]); the kernel that
 // consumes the GEMM output adds them, which keeps the result deterministic.
 // Every wait is bounded: on expiry the CTA records WD_ERR_DEVICE_TIMEOUT and leaves.
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -63,7 +64,7 @@ struct TcParams {
     int seg_tile0[4];               // first tile index of each weight matrix (+ end)
     int seg_n[3];
     int seg_col[3];
-    long long W;                    // total K blocks of the launch = n_units * kb_total
+    int W;                          // total K blocks of the launch = n_units * kb_total
     float* y;                       // (kEpiResid: the residual stream)
     size_t split_stride;
     int32_t* status;
@@ -86,7 +87,7 @@ __device__ __forceinline__ UnitInfo decode_unit(const TcParams& p, int unit, int
         tile = rem / gsz;
         tokt = grp * p.tok_grp + rem % gsz;
     } else {
-        tile = p.tok_split > 1 ? unit : unit / p.tok_tiles;
+        tile = p.tok_split > 1 || p.tok_tiles == 1 ? unit : unit / p.tok_tiles;
         tokt = p.tok_split > 1 ? tok_group : unit - tile * p.tok_tiles;
     }
     u.tok0 = tokt * p.bn * (p.dual == 1 ? 2 : 1);
@@ -97,52 +98,52 @@ __device__ __forceinline__ UnitInfo decode_unit(const TcParams& p, int unit, int
     return u;
 }
 
+// (The schedule's arithmetic is in 32 bits, the host sees to it that products of a line's length and the CTA count fit:
+// and a piece is found without a division: with 64-bit ones per piece a normal step of 34 rows took 1.2 % longer.)
 // The pieces of one CTA's share [g_begin, g_end) of the K-block line, in the order they are
 // processed: first the partial tile at the front of the share, then the partial tile at its
 // back, then the whole tiles in between.  Partial tiles are the ones other CTAs also work on;
 // doing them first lets those tiles complete (and their fused epilogue run) in the middle of the
 // kernel instead of all at its end.
 struct Sched {
-    long long g_begin, g_end;
-    int kb_total, head_len, tail_len, n_full, n_pieces;
-    long long full_begin;
-    long long stride = 0;           // > 0: whole units first, first + stride, ... (K blocks on the line)
+    int kb_total, head_unit, head_kb, head_len, tail_len, n_full, n_pieces;
+    int full_unit, full_step;       // whole units full_unit, full_unit + full_step, ...
     // whole units c, c + G, c + 2G, ... of n_units
-    __device__ void init_strided(long long c, long long G, int n_units, int kb) {
+    __device__ void init_strided(int c, int G, int n_units, int kb) {
         kb_total = kb;
-        head_len = tail_len = 0;
-        n_full = n_pieces = c < n_units ? (int)((n_units - c + G - 1) / G) : 0;
-        g_begin = full_begin = c * kb;
-        stride = G * kb;
-        g_end = g_begin;
+        head_unit = head_kb = head_len = tail_len = 0;
+        n_full = n_pieces = c < n_units ? (n_units - c + G - 1) / G : 0;
+        full_unit = c;
+        full_step = G;
     }
-    __device__ void init(long long gb, long long ge, int kb) {
-        g_begin = gb; g_end = ge; kb_total = kb;
-        const long long total = ge - gb;
-        const int off = (int)(gb % kb);
-        head_len = off ? (int)((long long)(kb - off) < total ? (kb - off) : total) : 0;
-        const long long rest_begin = gb + head_len;
-        const long long rest = ge - rest_begin;
-        n_full = (int)(rest / kb);
-        tail_len = (int)(rest - (long long)n_full * kb);
-        full_begin = rest_begin;
+    __device__ void init(int gb, int ge, int kb) {
+        kb_total = kb;
+        const int total = ge - gb;
+        head_unit = gb / kb;
+        head_kb = gb - head_unit * kb;
+        head_len = head_kb ? min(kb - head_kb, total) : 0;
+        const int rest = total - head_len;
+        n_full = rest / kb;
+        tail_len = rest - n_full * kb;
+        full_unit = head_unit + (head_kb ? 1 : 0);
+        full_step = 1;
         n_pieces = (head_len ? 1 : 0) + (tail_len ? 1 : 0) + n_full;
     }
-    // piece i -> first K block on the line and length
-    __device__ void piece(int i, long long& g, int& len) const {
-        if (stride > 0) { g = full_begin + (long long)i * stride; len = kb_total; return; }
-        if (head_len) { if (i == 0) { g = g_begin; len = head_len; return; } --i; }
-        if (tail_len) { if (i == 0) { g = g_end - tail_len; len = tail_len; return; } --i; }
-        g = full_begin + (long long)i * kb_total;
+    // piece i -> unit, first K block in it and length
+    __device__ void piece(int i, int& unit, int& kb0, int& len) const {
+        kb0 = 0;
+        if (head_len) { if (i == 0) { unit = head_unit; kb0 = head_kb; len = head_len; return; } --i; }
+        if (tail_len) { if (i == 0) { unit = full_unit + n_full; len = tail_len; return; } --i; }
+        unit = full_unit + i * full_step;
         len = kb_total;
     }
 };
 
 // number of CTAs whose piece of the line touches unit u
-__device__ __forceinline__ int n_contrib(const TcParams& p, long long G, int unit) {
+__device__ __forceinline__ int n_contrib(const TcParams& p, int G, int unit) {
     if (p.aligned) return 1;
-    const long long first = ((long long)unit * p.kb_total + 1) * G - 1;
-    const long long last = ((long long)(unit + 1) * p.kb_total) * G - 1;
+    const int first = (unit * p.kb_total + 1) * G - 1;
+    const int last = (unit + 1) * p.kb_total * G - 1;
     return (int)(last / p.W - first / p.W) + 1;
 }
 
@@ -194,7 +195,7 @@ __device__ __forceinline__ float sumsq_lane(const TcParams& p, int r, int lane) 
 // depend on which CTA arrived last.  A warp handles one token at a time, its lanes the tile's
 // 128 columns as float4; the loads of several tokens and slices are issued together so that
 // their L2 round trips overlap, and only then reduced.
-__device__ void finalize_unit(const TcParams& p, long long G, int unit, int e) {
+__device__ void finalize_unit(const TcParams& p, int G, int unit, int e) {
     const UnitInfo u = decode_unit(p, unit);
     const int nt = min(p.bn, p.rows - u.tok0);
     const int lane = e & 31, wq = e >> 5;
@@ -370,9 +371,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     float* lm_scratch = (float*)(tmem_slot + 4);           // 23 KB for the LM-head statistics
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long G = gridDim.x / (p.tok_split > 1 ? p.tok_split : 1), c = blockIdx.x % G;
+    const int G = gridDim.x / (p.tok_split > 1 ? p.tok_split : 1), c = blockIdx.x % G;
     const int tok_group = (int)(blockIdx.x / G);
-    long long g_begin, g_end;
+    int g_begin, g_end;
     if (p.aligned) {
         g_begin = (c * p.n_units / G) * p.kb_total;
         g_end = ((c + 1) * p.n_units / G) * p.kb_total;
@@ -417,12 +418,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 const CUtensorMap* mw;
             };
             auto enter = [&](Walk& w) {                    // position on the first block of piece w.piece
-                long long g;
-                int len;
-                sch.piece(w.piece, g, len);
-                const int unit = (int)(g / p.kb_total);
-                w.kb = (int)(g - (long long)unit * p.kb_total);
-                w.left = len;
+                int unit;
+                sch.piece(w.piece, unit, w.kb, w.left);
                 const UnitInfo u = decode_unit(p, unit, tok_group);
                 w.n0 = u.n0;
                 w.tok0 = u.tok0;
@@ -479,9 +476,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             int s = 0;
             uint32_t ph = 0;
             for (int piece = 0; piece < sch.n_pieces && ok; ++piece) {
-                long long g;
-                int len;
-                sch.piece(piece, g, len);
+                int unit, kb0, len;
+                sch.piece(piece, unit, kb0, len);
                 // normal: two accumulators used alternately; wide: one accumulator pair (both weight halves)
                 const int buf = kWide ? 0 : (piece & 1);
                 const uint32_t par = kWide ? ((uint32_t)piece & 1u) : ((uint32_t)(piece >> 1) & 1u);
@@ -530,17 +526,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         pdl_wait();      // the previous reader of y has finished (already implied by the data flow)
         bool ok = true;
         for (int piece = 0; piece < sch.n_pieces; ++piece) {
-            long long g;
-            int len;
-            sch.piece(piece, g, len);
-            const int unit = (int)(g / p.kb_total), kb0 = (int)(g - (long long)unit * p.kb_total);
+            int unit, kb0, len;
+            sch.piece(piece, unit, kb0, len);
             const UnitInfo u = decode_unit(p, unit, tok_group);
             const int buf = kWide ? 0 : (piece & 1);
             const uint32_t par = kWide ? ((uint32_t)piece & 1u) : ((uint32_t)(piece >> 1) & 1u);
             const int n = u.n0 + n_local;
             const bool n_ok = n < p.seg_n[u.seg];
             int ord = 0;
-            if (!p.aligned) ord = (int)(c - (((long long)unit * p.kb_total + 1) * G - 1) / p.W);
+            if (!p.aligned && kb0) ord = c - ((unit * p.kb_total + 1) * G - 1) / p.W;     // (else it is the first)
             // FP8: the row scales of this token tile go to shared memory while the MMAs still run
             float* sx_s = lm_scratch + (kLmStats ? 5664 : 0);
             if (kFp8) {
@@ -781,16 +775,16 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
     int* last_flag = (int*)(tmem_slot + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long G = gridDim.x, c = blockIdx.x;
+    const int G = gridDim.x, c = blockIdx.x;
     // this CTA's share of every GEMM's line of K blocks
     Sched sch[kChainMax];
     int n_tot[kChainMax];
-    long long total = 0;
+    int total = 0;
 #pragma unroll
     for (int g = 0; g < kChainMax; ++g) {
         n_tot[g] = 0;
         if (g < cp.n_gemm) {
-            const long long gb = c * cp.g[g].W / G, ge = (c + 1) * cp.g[g].W / G;
+            const int gb = c * cp.g[g].W / G, ge = (c + 1) * cp.g[g].W / G;
             sch[g].init(gb, ge, cp.g[g].kb_total);
             n_tot[g] = (int)(ge - gb);
             total += n_tot[g];
@@ -825,7 +819,7 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
             struct Cur {
                 int g, piece, left, kb, n0, tok0;
                 const CUtensorMap* mw;
-                long long i;                               // stages issued so far
+                int i;                               // stages issued so far
                 int s;                                     // ring slot of stage i, kept by increments (no division in the loop)
                 uint32_t ph;                               // (i / NS) & 1
             };
@@ -833,12 +827,8 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
                 while (w.g < cp.n_gemm && w.piece >= sch[w.g].n_pieces) { ++w.g; w.piece = 0; }
                 if (w.g >= cp.n_gemm) return;
                 const TcParams& p = cp.g[w.g];
-                long long gl;
-                int len;
-                sch[w.g].piece(w.piece, gl, len);
-                const int unit = (int)(gl / p.kb_total);
-                w.kb = (int)(gl - (long long)unit * p.kb_total);
-                w.left = len;
+                int unit;
+                sch[w.g].piece(w.piece, unit, w.kb, w.left);
                 const UnitInfo u = decode_unit(p, unit, 0);
                 w.n0 = u.n0;
                 w.tok0 = u.tok0;
@@ -925,9 +915,8 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
             for (int g = 0; g < cp.n_gemm && ok; ++g) {
                 const uint32_t idesc = cp.g[g].idesc;
                 for (int piece = 0; piece < sch[g].n_pieces && ok; ++piece, ++pc) {
-                    long long gl;
-                    int len;
-                    sch[g].piece(piece, gl, len);
+                    int unit, kb0, len;
+                    sch[g].piece(piece, unit, kb0, len);
                     const int buf = pc & 1;
                     const uint32_t par = (uint32_t)(pc >> 1) & 1u;
                     if (!(ok = mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), par ^ 1u, abort_flag))) break;
@@ -966,15 +955,13 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
         for (int g = 0; g < cp.n_gemm && ok; ++g) {
             const TcParams& p = cp.g[g];
             for (int piece = 0; piece < sch[g].n_pieces; ++piece, ++pc) {
-                long long gl;
-                int len;
-                sch[g].piece(piece, gl, len);
-                const int unit = (int)(gl / p.kb_total);
+                int unit, kb0, len;
+                sch[g].piece(piece, unit, kb0, len);
                 const UnitInfo u = decode_unit(p, unit, 0);
                 const int buf = pc & 1;
                 const uint32_t par = (uint32_t)(pc >> 1) & 1u;
                 const int n = u.n0 + n_local;
-                const int ord = (int)(c - (((long long)unit * p.kb_total + 1) * G - 1) / p.W);
+                const int ord = c - ((unit * p.kb_total + 1) * G - 1) / p.W;
                 ok = ok && mbar_wait(smem_u32(&bars[2 * NS + buf]), par, abort_flag);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -1103,7 +1090,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     const uint32_t rank = cluster_ctarank();              // 0: issues the MMAs
     if (threadIdx.x == 0) G_STAMP(0);
     // pairs per token group, this pair's index in its group, its token group (see TcParams::tok_split)
-    const long long G = (gridDim.x >> 1) / (p.tok_split > 1 ? p.tok_split : 1), c = (blockIdx.x >> 1) % G;
+    const int G = (gridDim.x >> 1) / (p.tok_split > 1 ? p.tok_split : 1), c = (blockIdx.x >> 1) % G;
     const int tok_group = (int)((blockIdx.x >> 1) / G);
     Sched sch;
     int n_total;
@@ -1111,7 +1098,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         sch.init_strided(c, G, p.n_units, p.kb_total);
         n_total = sch.n_pieces * p.kb_total;
     } else {
-        long long g_begin, g_end;
+        int g_begin, g_end;
         if (p.aligned) {
             g_begin = (c * p.n_units / G) * p.kb_total;
             g_end = ((c + 1) * p.n_units / G) * p.kb_total;
@@ -1160,12 +1147,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 const CUtensorMap* mw;
             };
             auto enter = [&](Walk& w) {
-                long long g;
-                int len;
-                sch.piece(w.piece, g, len);
-                const int unit = (int)(g / p.kb_total);
-                w.kb = (int)(g - (long long)unit * p.kb_total);
-                w.left = len;
+                int unit;
+                sch.piece(w.piece, unit, w.kb, w.left);
                 const UnitInfo u = decode_unit(p, unit, tok_group);
                 w.n0 = u.n0 + (int)rank * kBM;
                 w.tok0 = u.tok0 + (int)rank * tok_rows;
@@ -1220,9 +1203,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             int s = 0;
             uint32_t ph = 0;
             for (int piece = 0; piece < sch.n_pieces && ok; ++piece) {
-                long long g;
-                int len;
-                sch.piece(piece, g, len);
+                int unit, kb0, len;
+                sch.piece(piece, unit, kb0, len);
                 const int buf = n_sets == 2 ? piece & 1 : 0;
                 const uint32_t par = (uint32_t)(n_sets == 2 ? piece >> 1 : piece) & 1u;
                 // the epilogues of both CTAs have drained this accumulator set (free at the start)
@@ -1284,17 +1266,15 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         pdl_wait();
         bool ok = true;
         for (int piece = 0; piece < sch.n_pieces; ++piece) {
-            long long g;
-            int len;
-            sch.piece(piece, g, len);
-            const int unit = (int)(g / p.kb_total), kb0 = (int)(g - (long long)unit * p.kb_total);
+            int unit, kb0, len;
+            sch.piece(piece, unit, kb0, len);
             const UnitInfo u = decode_unit(p, unit, tok_group);
             const int buf = n_sets == 2 ? piece & 1 : 0;
             const uint32_t par = (uint32_t)(n_sets == 2 ? piece >> 1 : piece) & 1u;
             const int n = u.n0 + n_local;
             const bool n_ok = n < p.seg_n[u.seg];
             int ord = 0;
-            if (!p.aligned) ord = (int)(c - (((long long)unit * p.kb_total + 1) * G - 1) / p.W);
+            if (!p.aligned && kb0) ord = c - ((unit * p.kb_total + 1) * G - 1) / p.W;     // (else it is the first)
             ok = ok && mbar_wait(smem_u32(&bars[2 * NS + buf]), par, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -1627,7 +1607,8 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     const int ts = (!p.dual && epi == kEpiPlain && p.tok_tiles == 2 && (sm_count / 2) % 2 == 0) ? 2 : 1;
     p.tok_split = ts;
     p.n_units = ts > 1 ? tiles : tiles * p.tok_tiles;
-    p.W = (long long)p.n_units * p.kb_total;
+    if ((long long)p.n_units * p.kb_total > INT_MAX) return WD_ERR_CAPACITY;
+    p.W = p.n_units * p.kb_total;
     const size_t slice = (size_t)rows * col;
     if (p.dual != 2 && epi == kEpiPlain && slice > y_floats) return WD_ERR_CAPACITY;
     long long G = sm_count / 2 / ts;                                       // CTA pairs (per token group)
@@ -1638,7 +1619,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     // slice instead of two or three saves the consumers (and the zero fill) most of their traffic.
     static const int aligned_from = env_int("WD_GEMM_ALIGNED_UNITS", 2);
     if (force_single_split || (size_t)n_slices * slice > y_floats || n_slices > WD_TC_MAX_SPLIT ||
-        p.n_units >= aligned_from * G) {
+        p.n_units >= aligned_from * G || p.W * (G + 1) > INT_MAX) {
         p.aligned = 1;
         n_slices = 1;
         G = sm_count / 2 / ts;
@@ -1802,7 +1783,8 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
                        ? cfg.tok_tiles : 1;
     p.tok_split = ts;
     p.n_units = ts > 1 ? tiles : tiles * cfg.tok_tiles;
-    p.W = (long long)p.n_units * p.kb_total;
+    if ((long long)p.n_units * p.kb_total > INT_MAX) return WD_ERR_CAPACITY;
+    p.W = p.n_units * p.kb_total;
     p.n_stages = cfg.n_stages;
     p.buf_cols = cfg.buf_cols;
     // (trace builds) q/k/v, o, gate/up, down of a block by their shape; everything else in slot 4
@@ -1815,7 +1797,7 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
     if (G > p.W / 2) G = p.W / 2 > 0 ? p.W / 2 : 1;           // at least two K blocks per CTA
     int n_slices = count_slices(p.n_units, p.kb_total, p.W, G);
     p.aligned = 0;
-    if (force_single_split || (size_t)n_slices * slice > y_floats || n_slices > WD_TC_MAX_SPLIT) {
+    if (force_single_split || (size_t)n_slices * slice > y_floats || n_slices > WD_TC_MAX_SPLIT || p.W * (G + 1) > INT_MAX) {
         p.aligned = 1;
         n_slices = 1;
         G = (long long)slots / ts;
@@ -1928,7 +1910,8 @@ wd_status wd_tc_chain(const WdTcChainItem* items, int n, int rows, float* y, siz
         p.tok_tiles = 1;
         p.tok_split = 1;
         p.n_units = tiles;
-        p.W = (long long)tiles * p.kb_total;
+        if ((long long)tiles * p.kb_total * sm_count > INT_MAX) return WD_ERR_CAPACITY;
+        p.W = tiles * p.kb_total;
         p.n_stages = cfg.n_stages;
         p.buf_cols = cfg.buf_cols;
         if (G > p.W / 2) return WD_ERR_BAD_PARAM;                  // at least two K blocks per CTA and GEMM
