@@ -1016,6 +1016,7 @@ static wd_status run_gemm(wd_ctx* c, const void* x, const WdTcX* x_map, const Wd
                                  single_split, fuse, fp8, epi);
         if (s != WD_OK) return s;
         // SwiGLU done by the GEMM: bf16 h instead of the fp32 gate/up sums
+        if (epi && epi->rope && epi->rope->done && c->prof_on) c->prof_step_bytes -= (double)rows * ncol * 2;    // (bf16 q, k, v)
         if (epi && epi->sg && epi->sg->done && c->prof_on) c->prof_step_bytes -= (double)rows * ncol * 4 - (double)rows * (ncol / 2) * 2;
         *go = {n_split, (size_t)rows * ncol, 1, WD_GEMM_TCGEN05};
     } else {
@@ -1394,6 +1395,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         char* kc = st->kcache + (size_t)l * st->kv_layer_bytes;
         char* vc = st->vcache + (size_t)l * st->v_layer_bytes;
         const bool act = act_last && l == d.n_layers - 1;
+        WdTcRope rope;
+        WdTcEpi epi_rope;
         // attention half (FP8 mode: the normalised rows leave the RMSNorm as e4m3 codes + row scales)
         wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
                           c->attn_norm[l], d.rms_eps, c->xn, nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn,
@@ -1422,11 +1425,22 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         } else {
         WdTcSeg qkv[3] = {{c->wq[l], hq, c->tc.get(WD_TC_WQ, l)}, {c->wk[l], hkv, c->tc.get(WD_TC_WK, l)},
                           {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
-        if ((s = run_gemm(c, c->xn, &c->tc.x_map_d, qkv, 3, R_, D, c->part, c->part_floats, status, stream, &go)) != WD_OK)
+        // (Not for grouped-query heads: their narrow q/k/v has 85 % full rounds at 5376 rows, the rotation's kernel is 50 us of a
+        // 2.1 ms block, and the epilogue would save about half of it.)
+        if (use_tc(c) && dh == 128 && Hq == Hkv) {
+            rope.map_q = c->tc.get(WD_TC_WQ_ROT, l); rope.map_k = c->tc.get(WD_TC_WK_ROT, l);
+            rope.row_seq = row_seq; rope.row_pos = row_pos; rope.rope_tab = c->rope_tab;
+            rope.q = (__nv_bfloat16*)c->q; rope.kcache = (__nv_bfloat16*)kc; rope.vcache = (__nv_bfloat16*)vc;
+            rope.Hq = Hq; rope.Hkv = Hkv; rope.S = S; rope.Sp = Sp; rope.batch = batch;
+            epi_rope.rope = &rope;
+        }
+        if ((s = run_gemm(c, c->xn, &c->tc.x_map_d, qkv, 3, R_, D, c->part, c->part_floats, status, stream, &go, false, nullptr, nullptr,
+                          &epi_rope)) != WD_OK)
             return s;
         }
         impl_used = go.impl;
-        if (act)
+        if (rope.done) {
+        } else if (act)
             wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, c->seq_act, act_pos, c->rope_act, c->q, kc, vc, NA, Hq, 0,
                                    dh, S, Sp, batch, status, stream);
         else

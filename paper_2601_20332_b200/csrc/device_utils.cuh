@@ -165,6 +165,14 @@ __device__ __forceinline__ void tma2_load_2d_hint(uint32_t dst, const CUtensorMa
         ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "l"(policy)
         : "memory");
 }
+// the same for a 5-D box that starts at 0 in the three dimensions between the first and the last
+__device__ __forceinline__ void tma2_load_5d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c4,
+                                                  uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %4, %4, %5}], [%2], %6;"
+        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(0), "r"(c4), "l"(policy)
+        : "memory");
+}
 __device__ __forceinline__ void tmem2_alloc(uint32_t slot_smem_addr, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_smem_addr), "r"(cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");

@@ -1055,18 +1055,101 @@ extern "C" __attribute__((visibility("default"))) int wd_debug_chain_trace(unsig
 // accumulator set and the epilogue of a unit does not overlap the next unit's MMAs.
 // Whole-tile schedule: units are dealt round-robin in (token group, weight tile, token tile) order so
 // that the pairs running at one time share a few weight tiles and one token group in the L2.
-// kEpi: what the epilogue does with a finished tile.  Partial sums or fp32 results to y (or h, dual == 2); the residual add
-// (WdTcResid), which takes whole tiles and single accumulators.  The add reads and writes the residual stream once, beside the
+// kEpi: what the epilogue does with a finished tile.  Partial sums or fp32 results to y (or h, dual == 2); RoPE and the cache write
+// (WdTcRope); the residual add (WdTcResid).  The last two take whole tiles and single accumulators.  The add reads and writes the residual stream once, beside the
 // next unit's MMAs; as fp32 sums followed by the RMSNorm's own add it was written, read, and the stream read and written.
 // Measured (28672 rows of 4096 / 5376 of 3584): output projection 676 -> 721 us / 104 -> 110 us, the RMSNorm that follows
 // 330 -> 161 us / 65 -> 30 us; down projection and its RMSNorm alike.
-enum { kEpiPlain = 0, kEpiResid = 2 };
+enum { kEpiPlain = 0, kEpiRope = 1, kEpiResid = 2 };
+
+// RoPE epilogue, a warp's 32 accumulator rows (weight rows of one head) x 16 tokens at a time.  What bounds it are round trips
+// and small stores (with the table loaded per chunk and results stored two bytes a lane, 583 rows took 73 to 81 us instead of 60): the next
+// chunk's table rows and positions are on their way while a chunk is worked on, and results are collected in shared memory and
+// written 16 bytes a lane.
+// A rotated head (q, k): lane l < 16 holds dimension 16 quarter + l, lane l + 16 its partner 64 dimensions on; a token's
+// dimensions of this warp are two runs of 16.  v: the lane is one head dimension of the transposed cache; its 16 tokens, when
+// they are consecutive positions from a multiple of eight on, are two 16-byte stores.
+// Measured, 32 heads, with a rotation kernel / with this epilogue, in us: 583 rows 61.6 + 19.6 / 60.4; 1551 rows of four
+// sequences 127 + 47 / 132; 28672 rows 2020 + 877 / 2023.
+constexpr int kRopeSmem = 2048 + 32 * 48;       // per warp: [16 tokens][16] (cos, sin), results
+template <int kEpi> struct EpiArgs {};
+template <> struct EpiArgs<kEpiRope> { WdTcRope rope; };
+struct RopeNext {
+    float4 cs[4];
+    int pos, seq;
+};
+__device__ __forceinline__ void rope_fetch(const WdTcRope& rp, RopeNext& nx, bool rotated, int quarter, int lane, int tok0, int rows) {
+    if (tok0 >= rows) return;
+    if (rotated) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int f = 32 * k + lane;            // float4 f of the chunk: token f / 8, two (cos, sin) pairs
+            nx.cs[k] = __ldg(reinterpret_cast<const float4*>(rp.rope_tab + (size_t)min(tok0 + (f >> 3), rows - 1) * 64 + 16 * quarter) + (f & 7));
+        }
+    }
+    const int t = min(tok0 + (lane & 15), rows - 1);
+    nx.pos = __ldg(rp.row_pos + t);
+    nx.seq = __ldg(rp.row_seq + t);
+}
+// head: of its segment.  The caller has put the chunk's table rows into buf (__syncwarp() behind it).
+__device__ __forceinline__ void rope_chunk(const WdTcRope& rp, const uint32_t (&v)[16], int pos, int seq, int seg, int head, int quarter,
+                                           int lane, int tok0, int rows, uint8_t* buf, int32_t* status) {
+    const int n_tok = min(16, rows - tok0);
+    const bool in_range = (unsigned)pos < (unsigned)rp.S && (unsigned)seq < (unsigned)rp.batch;     // this lane's token (lane & 15)
+    if (!in_range && lane < n_tok) atomicCAS(status, 0, WD_ERR_BOUNDS);                              // recorded; its cache row is not written
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(buf + 2048);
+    if (seg < 2) {
+        const int half = lane >> 4, jj = lane & 15;
+        const float2* cs = reinterpret_cast<const float2*>(buf) + jj;
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            const float own = __uint_as_float(v[t]), other = __shfl_xor_sync(0xffffffffu, own, 16);
+            const float2 c = cs[16 * t];
+            out[32 * t + lane] = __float2bfloat16_rn(own * c.x + (half ? other : -other) * c.y);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int t = 8 * i + (lane >> 2), run = (lane >> 1) & 1, part = lane & 1;      // 16 bytes: eight dimensions of token t
+            const uint4 w = *reinterpret_cast<const uint4*>(out + 32 * t + 16 * run + 8 * part);
+            const int tp = __shfl_sync(0xffffffffu, pos, t), ts = __shfl_sync(0xffffffffu, seq, t);
+            const bool ok = __shfl_sync(0xffffffffu, in_range ? 1 : 0, t) != 0;
+            __nv_bfloat16* dst = seg == 0 ? rp.q + ((size_t)(tok0 + t) * rp.Hq + head) * 128
+                                          : rp.kcache + (((size_t)ts * rp.Hkv + head) * rp.S + tp) * 128;
+            if (t < n_tok && (seg == 0 || ok)) *reinterpret_cast<uint4*>(dst + 64 * run + 16 * quarter + 8 * part) = w;
+        }
+        return;
+    }
+    uint32_t w[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const __nv_bfloat162 p2 = __floats2bfloat162_rn(__uint_as_float(v[2 * t]), __uint_as_float(v[2 * t + 1]));
+        w[t] = *reinterpret_cast<const uint32_t*>(&p2);
+    }
+    const int pos0 = __shfl_sync(0xffffffffu, pos, 0), seq0 = __shfl_sync(0xffffffffu, seq, 0);
+    if (n_tok == 16 && (pos0 & 7) == 0 && __all_sync(0xffffffffu, in_range && seq == seq0 && pos == pos0 + (lane & 15))) {
+        uint4* dst = reinterpret_cast<uint4*>(rp.vcache + (((size_t)seq0 * rp.Hkv + head) * 128 + 32 * quarter + lane) * rp.Sp + pos0);
+        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        return;
+    }
+    uint4* row = reinterpret_cast<uint4*>(buf + 2048 + 48 * lane);
+    row[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    row[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    __syncwarp();
+    const int t = lane & 15;
+    if (t < n_tok && in_range) {                    // half a warp a dimension, its lanes over the tokens
+        __nv_bfloat16* dst = rp.vcache + (((size_t)seq * rp.Hkv + head) * 128 + 32 * quarter) * rp.Sp + pos;
+#pragma unroll
+        for (int dd = lane >> 4; dd < 32; dd += 2) dst[(size_t)dd * rp.Sp] = *reinterpret_cast<const __nv_bfloat16*>(buf + 2048 + 48 * dd + 2 * t);
+    }
+}
 
 template <bool kFp8, int kEpi = kEpiPlain>
 __global__ void __launch_bounds__(kThreadsPair)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w0,
                     const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w2,
-                    const TcParams p) {
+                    const TcParams p, const __grid_constant__ EpiArgs<kEpi> ep) {
     constexpr int kKE = kFp8 ? 128 : kBK;                 // K elements per block
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -1085,6 +1168,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     // [2NS+2, 2NS+3] accumulator empty (used in the even CTA; every epilogue warp of both CTAs arrives once)
     uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NS + 4);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    uint8_t* rope_buf = (uint8_t*)(((uintptr_t)(tmem_slot + 2) + 15) & ~(uintptr_t)15);     // kEpiRope: kRopeSmem per epilogue warp
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();              // 0: issues the MMAs
@@ -1145,6 +1229,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             struct Walk {
                 int piece, left, kb, n0, tok0;
                 const CUtensorMap* mw;
+                bool rot;               // kEpiRope: a q or k head, rows in rotation order
             };
             auto enter = [&](Walk& w) {
                 int unit;
@@ -1153,6 +1238,11 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 w.n0 = u.n0 + (int)rank * kBM;
                 w.tok0 = u.tok0 + (int)rank * tok_rows;
                 w.mw = u.seg == 0 ? &map_w0 : (u.seg == 1 ? &map_w1 : &map_w2);
+                w.rot = kEpi == kEpiRope && u.seg < 2;
+            };
+            auto load_w = [&](const Walk& w, uint32_t dst, uint32_t full) {
+                if (kEpi == kEpiRope && w.rot) tma2_load_5d_hint(dst, w.mw, full, w.kb * kKE, w.n0 >> 7, pol_stream);
+                else tma2_load_2d_hint(dst, w.mw, full, w.kb * kKE, w.n0, pol_stream);
             };
             auto advance = [&](Walk& w) {
                 ++w.kb;
@@ -1165,8 +1255,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             Walk w = w0;
             for (int i = 0; i < n_pre; ++i, advance(w)) {
                 if (rank == 0) mbar_expect_tx(smem_u32(&bars[i]), 2u * (uint32_t)stage_bytes);
-                tma2_load_2d_hint(smem_u32(smem + (size_t)i * stage_bytes), w.mw, cluster_map(smem_u32(&bars[i]), 0),
-                                  w.kb * kKE, w.n0, pol_stream);
+                load_w(w, smem_u32(smem + (size_t)i * stage_bytes), cluster_map(smem_u32(&bars[i]), 0));
                 if (gate_up)
                     tma2_load_2d_hint(smem_u32(smem + (size_t)i * stage_bytes) + kStageA, &map_w1,
                                       cluster_map(smem_u32(&bars[i]), 0), w.kb * kKE, w.n0, pol_stream);
@@ -1189,7 +1278,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 const uint32_t full = cluster_map(smem_u32(&bars[s]), 0);
                 const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
                 if (rank == 0) mbar_expect_tx(smem_u32(&bars[s]), 2u * (uint32_t)stage_bytes);
-                tma2_load_2d_hint(sa, w.mw, full, w.kb * kKE, w.n0, pol_stream);
+                load_w(w, sa, full);
                 if (gate_up) tma2_load_2d_hint(sa + kStageA, &map_w1, full, w.kb * kKE, w.n0, pol_stream);
                 tma2_load_2d(sa + stage_a, &map_x, full, w.kb * kKE, w.tok0);
                 if (++s == NS) { s = 0; ph ^= 1u; }
@@ -1275,6 +1364,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             const bool n_ok = n < p.seg_n[u.seg];
             int ord = 0;
             if (!p.aligned && kb0) ord = c - ((unit * p.kb_total + 1) * G - 1) / p.W;     // (else it is the first)
+            RopeNext nx = {};
+            if constexpr (kEpi == kEpiRope) rope_fetch(ep.rope, nx, u.seg < 2, quarter, lane, u.tok0 + 16 * hf, min(p.rows, u.tok0 + p.bn));
             ok = ok && mbar_wait(smem_u32(&bars[2 * NS + buf]), par, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -1299,6 +1390,22 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
 #pragma unroll
                     for (int t = 0; t < 16; ++t)
                         if (n_ok && u.tok0 + cc + t < p.rows) xs[(size_t)t * p.ncol] = xv[t] + __uint_as_float(v[t]);
+                }
+            } else if constexpr (kEpi == kEpiRope) {
+                for (int cc = 16 * hf; cc < p.bn && u.tok0 + cc < p.rows; cc += col_step) {
+                    uint32_t v[16];
+                    // (a head is 128 weight rows: this CTA's rows exist or not as a whole)
+                    uint8_t* wb = rope_buf + (size_t)(warp - 2) * kRopeSmem;
+                    const int pos = nx.pos, seq = nx.seq;
+                    __syncwarp();               // the previous chunk's readers of wb are done
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) reinterpret_cast<float4*>(wb)[32 * k + lane] = nx.cs[k];
+                    rope_fetch(ep.rope, nx, u.seg < 2, quarter, lane, u.tok0 + cc + col_step, min(p.rows, u.tok0 + p.bn));
+                    tmem_ld16(t_acc + (uint32_t)cc, v);
+                    __syncwarp();
+                    if (n_ok)
+                        rope_chunk(ep.rope, v, pos, seq, u.seg, (u.n0 >> 7) + (int)rank, quarter, lane, u.tok0 + cc, min(p.rows, u.tok0 + p.bn),
+                                   wb, p.status);
                 }
             } else if (gate_up) {
                 // h = silu(gate) * up
@@ -1432,6 +1539,22 @@ wd_status encode_2d(CUtensorMap* m, const void* ptr, int n_rows, int K, int box_
     return r == CUDA_SUCCESS ? WD_OK : WD_ERR_CUDA;
 }
 
+// [heads * 128, K] bf16 row-major as (K, 16, 2, 4, heads): a box is 64 (K) of one head whose rows arrive in the order 0-15,
+// 64-79, 16-31, 80-95, ...; 128-byte swizzle
+wd_status encode_rot(CUtensorMap* m, const void* ptr, int heads, int K) {
+    EncodeTiledFn enc = get_encode();
+    if (!enc) return WD_ERR_CUDA;
+    if ((uintptr_t)ptr % 16 || ((size_t)K * 2) % 16) return WD_ERR_MISALIGNED;
+    cuuint64_t dims[5] = {(cuuint64_t)K, 16, 2, 4, (cuuint64_t)heads};
+    cuuint64_t strides[4] = {(cuuint64_t)K * 2, (cuuint64_t)K * 2 * 64, (cuuint64_t)K * 2 * 16, (cuuint64_t)K * 2 * 128};
+    cuuint32_t box[5] = {(cuuint32_t)kBK, 16, 2, 4, 1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? WD_OK : WD_ERR_CUDA;
+}
+
 // [n_rows, K] bytes (e4m3 codes) row-major, box = 128 (K) x box_rows, 128-byte swizzle
 wd_status encode_2d8(CUtensorMap* m, const void* ptr, int n_rows, int K, int box_rows) {
     EncodeTiledFn enc = get_encode();
@@ -1517,6 +1640,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     memset(&p, 0, sizeof(p));
     const WdTcSwiglu* sg = epi_opt ? epi_opt->sg : nullptr;
     const WdTcResid* resid = epi_opt ? epi_opt->resid : nullptr;
+    const WdTcRope* rope = epi_opt ? epi_opt->rope : nullptr;
     int epi = kEpiPlain;
     if (fp8) {
         p.fp8 = 1;
@@ -1550,12 +1674,14 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
             const long long gu_units = (long long)((segs[0].n + p.tile_rows - 1) / p.tile_rows) * ((rows + 255) / 256);
             if (full_rounds(gu_units)) p.dual = 2;
         }
-        // the residual add in the epilogue: the same condition on whole units of one accumulator (with shares of the K-block
+        // RoPE or the residual add in the epilogue: the same condition on whole units of one accumulator (with shares of the K-block
         // line a tile's sum is in several pieces)
         static const int epi_on = env_int("WD_GEMM_EPI", 3);
-        if (!fp8 && p.dual != 2 && resid && resid->x && nseg == 1 && (epi_on & 2) &&
-            full_rounds((long long)tiles_all * ((rows + 255) / 256))) {
-            epi = kEpiResid;
+        if (!fp8 && p.dual != 2 && full_rounds((long long)tiles_all * ((rows + 255) / 256))) {
+            if (rope && nseg == 3 && (epi_on & 1)) epi = kEpiRope;
+            else if (resid && resid->x && nseg == 1 && (epi_on & 2)) epi = kEpiResid;
+        }
+        if (epi != kEpiPlain) {
             p.dual = 0;
             force_single_split = true;
         }
@@ -1575,7 +1701,8 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     const int stage = (p.dual == 2 ? 2 : 1) * kStageA + tok_rows * kBK * 2;
     p.n_stages = (192 * 1024) / stage;
     if (p.n_stages > 10) p.n_stages = 10;
-    const size_t smem = (size_t)p.n_stages * stage + (2 * p.n_stages + 4) * 8 + 16 + 256 + 1024;
+    const size_t smem = (size_t)p.n_stages * stage + (2 * p.n_stages + 4) * 8 + 16 + 256 + 1024 +
+                        (epi == kEpiRope ? 8 * kRopeSmem : 0);
     int tiles = 0, col = 0;
     for (int i = 0; i < nseg; ++i)
         if (!segs[i].map) return WD_ERR_NULL;
@@ -1652,13 +1779,15 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     if (!attr_done[dev]) {
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_pair_kernel<false, kEpiRope>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_pair_kernel<false, kEpiResid>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         attr_done[dev] = true;
     }
-    const CUtensorMap& m0 = *segs[0].map;
-    const CUtensorMap& m1 = *segs[(nseg > 1 || p.dual == 2) ? 1 : 0].map;
+    const CUtensorMap& m0 = epi == kEpiRope ? *rope->map_q : *segs[0].map;
+    const CUtensorMap& m1 = epi == kEpiRope ? *rope->map_k : *segs[(nseg > 1 || p.dual == 2) ? 1 : 0].map;
     const CUtensorMap& m2 = *segs[nseg > 2 ? 2 : 0].map;
     if (sg) sg->done = p.dual == 2;
+    if (rope) rope->done = epi == kEpiRope;
     if (resid) resid->done = epi == kEpiResid;
     if (epi == kEpiResid) p.y = resid->x;
     ++wd_launch_counter;
@@ -1676,9 +1805,12 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = wd_pdl_enabled ? 2 : 1;
-    if (fp8) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<true>, mx, m0, m1, m2, p));
-    else if (epi == kEpiResid) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<false, kEpiResid>, mx, m0, m1, m2, p));
-    else WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<false>, mx, m0, m1, m2, p));
+    EpiArgs<kEpiRope> er;
+    if (rope) er.rope = *rope;
+    if (fp8) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<true>, mx, m0, m1, m2, p, EpiArgs<kEpiPlain>()));
+    else if (epi == kEpiRope) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<false, kEpiRope>, mx, m0, m1, m2, p, er));
+    else if (epi == kEpiResid) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<false, kEpiResid>, mx, m0, m1, m2, p, EpiArgs<kEpiResid>()));
+    else WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_pair_kernel<false>, mx, m0, m1, m2, p, EpiArgs<kEpiPlain>()));
     if (n_split_out) *n_split_out = p.n_slices;
     return WD_OK;
 }
@@ -1700,6 +1832,10 @@ wd_status wd_tc_weights_init(WdTcWeights* tc, const wd_model_dims* d, const void
         if ((s = encode_2d(&tc->maps[(size_t)WD_TC_WQ * L + l], wq[l], hq, d->d_model, kBM)) != WD_OK) return s;
         if ((s = encode_2d(&tc->maps[(size_t)WD_TC_WK * L + l], wk[l], hkv, d->d_model, kBM)) != WD_OK) return s;
         if ((s = encode_2d(&tc->maps[(size_t)WD_TC_WV * L + l], wv[l], hkv, d->d_model, kBM)) != WD_OK) return s;
+        if (d->head_dim == 128) {
+            if ((s = encode_rot(&tc->maps[(size_t)WD_TC_WQ_ROT * L + l], wq[l], d->n_q_heads, d->d_model)) != WD_OK) return s;
+            if ((s = encode_rot(&tc->maps[(size_t)WD_TC_WK_ROT * L + l], wk[l], d->n_kv_heads, d->d_model)) != WD_OK) return s;
+        }
         if ((s = encode_2d(&tc->maps[(size_t)WD_TC_WO * L + l], wo[l], d->d_model, hq, kBM)) != WD_OK) return s;
         if ((s = encode_2d(&tc->maps[(size_t)WD_TC_WG * L + l], wg[l], d->d_ffn, d->d_model, kBM)) != WD_OK) return s;
         if ((s = encode_2d(&tc->maps[(size_t)WD_TC_WU * L + l], wu[l], d->d_ffn, d->d_model, kBM)) != WD_OK) return s;
@@ -1718,6 +1854,7 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
                      const WdTcFuse* fuse, const WdTcFp8* fp8, const WdTcEpi* epi) {
     if (!x || !segs || !y || !status || nseg < 1 || nseg > 3) return WD_ERR_BAD_PARAM;
     if (epi && epi->sg) epi->sg->done = false;
+    if (epi && epi->rope) epi->rope->done = false;
     if (epi && epi->resid) epi->resid->done = false;
     if (rows < 1 || K < 8 || K % 8) return WD_ERR_BAD_PARAM;
     TcParams p;

@@ -7,7 +7,9 @@
 #define WD_TC_MAX_SPLIT 16          // most split-K slices
 #define WD_TC_SPLITK_MAX_ROWS 256   // split-K only while the token tile count is 1
 
-enum { WD_TC_WQ = 0, WD_TC_WK, WD_TC_WV, WD_TC_WO, WD_TC_WG, WD_TC_WU, WD_TC_WD, WD_TC_LM, WD_TC_KINDS };
+enum { WD_TC_WQ = 0, WD_TC_WK, WD_TC_WV, WD_TC_WO, WD_TC_WG, WD_TC_WU, WD_TC_WD, WD_TC_LM,
+       WD_TC_WQ_ROT, WD_TC_WK_ROT,        // q and k with the rows of a head in rotation order (WdTcRope)
+       WD_TC_KINDS };
 
 // One weight matrix [n, K] taking part in a GEMM (its rows become output columns).
 struct WdTcSeg {
@@ -115,9 +117,23 @@ struct WdTcResid {
     mutable bool done = false;
 };
 
+// q/k/v launches with head_dim 128 and many rows: where the GEMM works on whole tiles, its epilogue rotates the q and k
+// heads by the rows' table and writes q and the K / transposed-V cache rows; nothing goes to y.  map_q, map_k: the weights
+// with the 128 rows of a head in the order 0-15, 64-79, 16-31, 80-95, ... (a rotation pair is then 16 accumulator rows apart,
+// so two lanes of one warp hold it).  `done` as above.
+struct WdTcRope {
+    const CUtensorMap *map_q = nullptr, *map_k = nullptr;
+    const int32_t *row_seq = nullptr, *row_pos = nullptr;
+    const float2* rope_tab = nullptr;      // [rows][64] (cos, sin)
+    __nv_bfloat16 *q = nullptr, *kcache = nullptr, *vcache = nullptr;
+    int Hq = 0, Hkv = 0, S = 0, Sp = 0, batch = 1;
+    mutable bool done = false;
+};
+
 // What a launch may do in its epilogue instead of writing y, if its schedule allows it
 struct WdTcEpi {
     const WdTcSwiglu* sg = nullptr;
+    const WdTcRope* rope = nullptr;
     const WdTcResid* resid = nullptr;
 };
 
