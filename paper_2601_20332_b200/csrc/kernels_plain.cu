@@ -1371,8 +1371,9 @@ void wd_launch_swiglu(int dtype, const float* part, int n_split, size_t split_st
     if (n_rows <= 0) return;
     const size_t total = (size_t)n_rows * (F >> 2);
     static const int sw_rows = getenv("WD_SWIGLU_ROWS") ? atoi(getenv("WD_SWIGLU_ROWS")) : 1;
-    // up to about a hundred rows (measured: -1.4 % on a 68-row step, +1 % at 352 rows, where two positions per thread pay)
-    static const int sw_rows_max = getenv("WD_SWIGLU_ROWS_MAX") ? atoi(getenv("WD_SWIGLU_ROWS_MAX")) : 148 * 8 * 256;
+    // up to 600 thousand positions, 195 rows of 12288 (measured per launch, one / two positions per thread: 5.2 / 11.9 us at 136
+    // rows, 10.4 / 7.7 us at 352 rows, where two pay)
+    static const int sw_rows_max = getenv("WD_SWIGLU_ROWS_MAX") ? atoi(getenv("WD_SWIGLU_ROWS_MAX")) : 600000;
     if (sw_rows && total <= (size_t)sw_rows_max) {
         WD_DISPATCH(dtype, launch_pdl(swiglu_rows_kernel<T>, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, part, n_split,
                                       split_stride, (T*)h, n_rows, F));
