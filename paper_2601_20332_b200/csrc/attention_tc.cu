@@ -563,12 +563,19 @@ attention_tc_single_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
 // Tensor memory: S (and P over it) 2 x 128 columns, O 2 x 128.  Shared memory: two Q tiles, two K and two V stages, 192 KB.
 // The tensor core runs Q K^T and P V in issue order, so S(i + 1) complete means P V(i) has read P(i) and has been added to O;
 // one barrier each for S and P of a tile suffices (P(i + 1) needs S(i + 1), which is issued only after P(i) has been seen).
+// What bounds it: 3900 cycles per key tile and pair of query tiles.  The MMAs alone, issued without waiting for any softmax, take
+// 3280 (M = N = 128 runs at 62 % of the peak rate: both operands' slices of a Q K^T use up the shared-memory bandwidth), the
+// softmax without the MMAs 3100, and the K/V loads hide completely.  Beside the loop a CTA spends 3 us until its first scores, 1.1
+// us after the last exponentials and the write of O, so a few key tiles are dominated by both ends: one row of O per thread took
+// 2.1-4.6 us (a warp's store touched 32 lines), staged through shared memory 0.5-1; loading tile 0 and its keys before tile 1, and
+// zeroing V columns by 16 bytes while the scores are still being computed, the rest of 113 -> 98 us for eight sequences of
+// 672 rows, 28 query and 4 KV heads, and 257 -> 249 us for 1792 rows, 128 heads.
 // Measured per launch against the single-tile kernel: see wd_attn_tc_launch.
 constexpr int kDThreads = 384;
 // Registers per thread after the hand-over: 56 for the first warpgroup, 224 for the other two.  The launch has 168 for each of
 // the 384 threads (the most that fit the register file), and 128 * 56 + 256 * 224 = 384 * 168.
-constexpr int kDBars = 14;
-constexpr int kDQ = 0, kDKFull = 1, kDKEmpty = 3, kDVFull = 5, kDVEmpty = 7, kDSFull = 9, kDPFull = 11, kDODone = 13;
+constexpr int kDBars = 16;
+constexpr int kDQ = 0, kDKFull = 2, kDKEmpty = 4, kDVFull = 6, kDVEmpty = 8, kDSFull = 10, kDPFull = 12, kDODone = 14;
 constexpr size_t kDualSmem = 6 * (size_t)kOperand + (kDBars + 2) * 8 + 1024;
 
 __device__ __forceinline__ uint64_t f32x2(float a, float b) {
@@ -639,18 +646,18 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         if (warp == 0) {
             if (lane == 0) {
                 // ---------------------------------------------------- TMA producer
-                const uint32_t qf = smem_u32(&bars[kDQ]);
-                const Item q0 = item(0), q1 = item(n_q - 1);
                 const int bh = b * p.Hkv + kvh;
-                mbar_expect_tx(qf, (uint32_t)((q0.n_slots + (n_q == 2 ? q1.n_slots : 0)) * p.slot * 256));
-                for (int t = 0; t < n_q; ++t) {
-                    const Item q = t ? q1 : q0;
+                auto load_q = [&](int t) {
+                    const Item q = item(t);
+                    const uint32_t qf = smem_u32(&bars[kDQ + t]);
+                    mbar_expect_tx(qf, (uint32_t)(q.n_slots * p.slot * 256));
                     for (int j = 0; j < q.n_slots; ++j) {
                         const uint32_t dst = smem_u32(sQ) + (uint32_t)(t * kOperand + j * p.slot * 128);
                         tma_load_2d(dst, &map_q, qf, (q.h + j) * kTile, q.row0);
                         tma_load_2d(dst + kAtom, &map_q, qf, (q.h + j) * kTile + 64, q.row0);
                     }
-                }
+                };
+                load_q(0);                                             // the first tile and its keys come first: S(0) of tile 0 starts on them
                 bool ok = true;
                 for (int i = 0; i < n_kt && ok; ++i) {
                     const int s = i & 1, kv0 = i * kTile;
@@ -661,6 +668,7 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     mbar_expect_tx(kf, kOperand);
                     tma_load_4d(sk, &map_k, kf, 0, kv0, bh, p.layer);             // keys kv0.., dims 0..63
                     tma_load_4d(sk + kAtom, &map_k, kf, 64, kv0, bh, p.layer);    // dims 64..127
+                    if (i == 0 && n_q == 2) load_q(1);
                     if (!(ok = mbar_wait(smem_u32(&bars[kDVEmpty + s]), ph, abort_flag))) break;
                     mbar_expect_tx(vf, kOperand);
                     tma_load_4d(sv, &map_vt, vf, kv0, 0, bh, p.layer);            // all dims, keys kv0..kv0+63
@@ -675,7 +683,6 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
         } else if (warp == 1) {
             if (lane == 0) {
                 // ---------------------------------------------------- MMA issuer
-                bool ok = mbar_wait(smem_u32(&bars[kDQ]), 0, abort_flag);
                 auto issue_qk = [&](int t, int i) {                   // S_t = Q_t K(i)^T
                     const uint64_t qd = make_sdesc(smem_u32(sQ + (size_t)t * kOperand));
                     const uint64_t kd = make_sdesc(smem_u32(sK + (size_t)(i & 1) * kOperand));
@@ -688,10 +695,11 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     umma_commit(smem_u32(&bars[kDSFull + t]));
                     if (t == n_q - 1) umma_commit(smem_u32(&bars[kDKEmpty + (i & 1)]));     // K stage free
                 };
-                ok = ok && mbar_wait(smem_u32(&bars[kDKFull]), 0, abort_flag);
-                if (ok) {
+                bool ok = mbar_wait(smem_u32(&bars[kDKFull]), 0, abort_flag);
+                for (int t = 0; t < n_q && ok; ++t) {
+                    if (!(ok = mbar_wait(smem_u32(&bars[kDQ + t]), 0, abort_flag))) break;
                     tc_fence_after();
-                    for (int t = 0; t < n_q; ++t) issue_qk(t, 0);
+                    issue_qk(t, 0);
                 }
                 for (int i = 0; i < n_kt && ok; ++i) {
                     const uint32_t ph = (uint32_t)(i >> 1) & 1u;
@@ -705,6 +713,7 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                         for (int kk = 0; kk < 8; ++kk)                // 16 keys = 8 columns of P per MMA
                             umma_bf16_ta(acc, pa + 8 * kk, vd + (uint64_t)((kk >> 2) * (kAtom >> 4) + 2 * (kk & 3)), p.idesc, (i > 0 || kk > 0) ? 1u : 0u);
                         if (t == n_q - 1) umma_commit(smem_u32(&bars[kDVEmpty + (i & 1)]));     // V stage free
+                        if (i == n_kt - 1) umma_commit(smem_u32(&bars[kDODone + t]));
                         if (i + 1 < n_kt) {
                             if (t == 0 && !(ok = mbar_wait(smem_u32(&bars[kDKFull + ((i + 1) & 1)]), (uint32_t)((i + 1) >> 1) & 1u, abort_flag))) break;
                             tc_fence_after();
@@ -712,7 +721,6 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                         }
                     }
                 }
-                if (ok) umma_commit(smem_u32(&bars[kDODone]));
                 if (!ok) {
                     *abort_flag = 1;
                     atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
@@ -738,18 +746,20 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             const uint64_t c2 = f32x2(p.scale_log2e, p.scale_log2e);
             float m = 0.f, l = 0.f;
             for (int i = 0; i < n_kt; ++i) {
-                if (!(ok = mbar_wait(smem_u32(&bars[kDSFull + t]), (uint32_t)i & 1u, abort_flag))) break;
-                tc_fence_after();
                 const int n_keys = min(kTile, n_vis - i * kTile);             // valid keys of this tile
                 // keys past n_vis may hold anything: zero their V columns so that 0 * garbage stays 0 (tile 0's threads, row r
                 // of the transposed V tile = head dim r; P V of either tile is issued after tile 0's P has been seen)
                 if (n_keys < kTile && t == 0) {
                     if (!(ok = mbar_wait(smem_u32(&bars[kDVFull + (i & 1)]), (uint32_t)(i >> 1) & 1u, abort_flag))) break;
                     uint8_t* vt = sV + (size_t)(i & 1) * kOperand + r * 128;
-                    for (int kv = n_keys; kv < kTile; ++kv)
-                        *reinterpret_cast<uint16_t*>(vt + (kv >> 6) * kAtom + ((((kv & 63) >> 3) ^ (r & 7)) << 4) + (kv & 7) * 2) = 0;
+                    auto at = [&](int kv) { return vt + (kv >> 6) * kAtom + ((((kv & 63) >> 3) ^ (r & 7)) << 4) + (kv & 7) * 2; };
+                    int kv = n_keys;
+                    for (; kv & 7; ++kv) *reinterpret_cast<uint16_t*>(at(kv)) = 0;
+                    for (; kv < kTile; kv += 8) *reinterpret_cast<uint4*>(at(kv)) = make_uint4(0, 0, 0, 0);
                     fence_proxy_async_smem();
                 }
+                if (!(ok = mbar_wait(smem_u32(&bars[kDSFull + t]), (uint32_t)i & 1u, abort_flag))) break;
+                tc_fence_after();
                 if (live) {
                     uint32_t sc[4][32];
                     float mx0 = -INFINITY, mx1 = -INFINITY;
@@ -809,33 +819,45 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 tc_fence_before();
                 mbar_arrive(smem_u32(&bars[kDPFull + t]));
             }
-            ok = ok && mbar_wait(smem_u32(&bars[kDODone]), 0, abort_flag);
+            ok = ok && mbar_wait(smem_u32(&bars[kDODone + t]), 0, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
             if (ok && live) {
-                const bool valid = sj < q.n_slots && rr < q.n_valid;
+                // through shared memory (the warp's rows of the Q tile, which no MMA reads any more), so that a store instruction
+                // writes two whole rows of 256 bytes: with a thread to a row it touched 32 lines
                 const float inv = 1.f / l;
-                const size_t base = ((size_t)(q.row0 + rr) * p.Hq + q.h + sj) * kTile;
+                const int rr0 = (quarter * 32) & (p.slot - 1), n_out = min(32, q.n_valid - rr0);     // the warp's valid rows
+                uint8_t* st = sQ + (size_t)t * kOperand + quarter * 8192;
+                __nv_bfloat16* out = p.out + ((size_t)(q.row0 + rr0) * p.Hq + q.h + sj) * kTile;
+                const size_t pitch = (size_t)p.Hq * kTile;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint32_t v[32];
                     tmem_ld32(t_o + (uint32_t)(32 * c), v);
-                    if (valid) {
-                        uint4* dst = reinterpret_cast<uint4*>(p.out + base + 32 * c);
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            uint4 u;
-                            u.x = pack_bf16(__uint_as_float(v[8 * g]) * inv, __uint_as_float(v[8 * g + 1]) * inv);
-                            u.y = pack_bf16(__uint_as_float(v[8 * g + 2]) * inv, __uint_as_float(v[8 * g + 3]) * inv);
-                            u.z = pack_bf16(__uint_as_float(v[8 * g + 4]) * inv, __uint_as_float(v[8 * g + 5]) * inv);
-                            u.w = pack_bf16(__uint_as_float(v[8 * g + 6]) * inv, __uint_as_float(v[8 * g + 7]) * inv);
-                            dst[g] = u;
-                        }
-                        if (p.tap) {
-#pragma unroll
-                            for (int k = 0; k < 32; ++k) p.tap[base + 32 * c + k] = __uint_as_float(v[k]) * inv;
-                        }
+                    for (int g = 0; g < 4; ++g) {
+                        uint4 u;
+                        u.x = pack_bf16(__uint_as_float(v[8 * g]) * inv, __uint_as_float(v[8 * g + 1]) * inv);
+                        u.y = pack_bf16(__uint_as_float(v[8 * g + 2]) * inv, __uint_as_float(v[8 * g + 3]) * inv);
+                        u.z = pack_bf16(__uint_as_float(v[8 * g + 4]) * inv, __uint_as_float(v[8 * g + 5]) * inv);
+                        u.w = pack_bf16(__uint_as_float(v[8 * g + 6]) * inv, __uint_as_float(v[8 * g + 7]) * inv);
+                        *reinterpret_cast<uint4*>(st + lane * 256 + (((4 * c + g) ^ (lane & 7)) << 4)) = u;
                     }
+                    if (p.tap && lane < n_out) {
+#pragma unroll
+                        for (int k = 0; k < 32; ++k)
+                            p.tap[((size_t)(q.row0 + rr) * p.Hq + q.h + sj) * kTile + 32 * c + k] = __uint_as_float(v[k]) * inv;
+                    }
+                }
+                __syncwarp();
+                for (int r0 = lane >> 4; r0 < n_out; r0 += 8) {
+                    uint4 u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        u[k] = *reinterpret_cast<const uint4*>(st + (r0 + 2 * k) * 256 + (((lane & 15) ^ ((r0 + 2 * k) & 7)) << 4));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (r0 + 2 * k < n_out) *reinterpret_cast<uint4*>(out + (r0 + 2 * k) * pitch + 8 * (lane & 15)) = u[k];
                 }
             }
             if (!ok) {
@@ -967,8 +989,8 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
     static bool attr_done[64] = {};     // the attribute is per device
     // More single-tile CTAs than SMs: two tiles per CTA (the rule is the wave: up to one of them the single-tile kernel, with its
     // keys split over a cluster when SMs are left over, has the shorter chain).  Measured, single / two tiles, in us: 583 rows,
-    // 32 heads 32.8 / 24.8; 1536 rows, 32 heads 78.8 / 70.3 (192 CTAs for 148 SMs); eight sequences of 672 rows, 28 query and 4
-    // KV heads 158 / 113, of 66 rows over 830 keys 38.9 / 28.8; 1792 rows, 128 heads 360 / 257.
+    // 32 heads 32.8 / 23.4; 1536 rows, 32 heads 78.8 / 67.7 (192 CTAs for 148 SMs); eight sequences of 672 rows, 28 query and 4
+    // KV heads 158 / 98, of 66 rows over 830 keys 38.9 / 27.1; 1792 rows, 128 heads 360 / 249.
     static const int dual_on = getenv("WD_ATTN_DUAL") ? atoi(getenv("WD_ATTN_DUAL")) : 1;
     if (dual_on && seq_qt_off && n_tiles * grid_y > sm_count) {
         static bool dual_done[64] = {};
