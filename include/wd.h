@@ -591,9 +591,9 @@ WD_API size_t wd_op_lm_unmask_scratch_bytes(int32_t n, int32_t vocab);
  * call.  Synchronises the device. */
 WD_API wd_status wd_op_status(void);
 
-/* Exercises the library's error path for device-side waits without any fault: one
- * thread waits, with the same bounded wait every kernel of the library uses, on a
- * shared-memory barrier that nothing ever signals.  The wait gives up after its
+/* Exercises the library's error path for device-side waits without any fault: a
+ * warp waits, with the same bounded wait every kernel of the library uses, half of its
+ * lanes on a shared-memory barrier that nothing ever signals.  The wait gives up after its
  * time limit (two seconds), the kernel records
  * WD_ERR_DEVICE_TIMEOUT in the operations' status word and returns normally; the
  * context stays usable.  wd_op_status() then reports and clears the code.

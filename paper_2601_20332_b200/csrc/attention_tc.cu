@@ -301,7 +301,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
         // time to finish while this thread was busy with the next tile's softmax
         auto fold = [&](int j, float alpha) {
             const int s = j & 1;
-            if (!mbar_wait(smem_u32(&bars[kOFull + s]), (uint32_t)(j >> 1) & 1u, abort_flag)) { *abort_flag = 1; ok = false; }
+            mbar_wait_stay(smem_u32(&bars[kOFull + s]), (uint32_t)(j >> 1) & 1u, abort_flag, ok);
             tc_fence_after();
             if (live) {
 #pragma unroll
@@ -317,17 +317,16 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
         };
         for (int i = 0; i < n_kt; ++i) {
             const int s = i & 1;
-            // A failed wait must not leave the loop before the named barrier below (the other
-            // warps would wait there for ever): it raises the CTA's abort flag, every thread still
-            // reaches the barrier, and all of them leave together right after it.
-            if (!mbar_wait(smem_u32(&bars[kSFull + s]), (uint32_t)(i >> 1) & 1u, abort_flag)) *abort_flag = 1;
+            // A failed wait must not leave the loop: the other warps would wait at the named barrier below for ever.  It
+            // raises the CTA's abort flag, and every thread goes through the remaining tiles, whose waits give up at once.
+            mbar_wait_stay(smem_u32(&bars[kSFull + s]), (uint32_t)(i >> 1) & 1u, abort_flag, ok);
             tc_fence_after();
             if (threadIdx.x == 64 && i == 0) A_STAMP(2);
             const int n_keys = min(kTile, n_vis - (kt_begin + i) * kTile);   // valid keys in this tile
             // keys past n_vis may hold anything: zero their V columns so that 0 * garbage stays 0.
             // Thread (r, hf) owns row r (a head dim) of atom hf (keys 64*hf..) of the transposed V tile.
             if (n_keys < c_off + 64) {
-                if (!mbar_wait(smem_u32(&bars[kVFull + i % NS]), (uint32_t)(i / NS) & 1u, abort_flag)) *abort_flag = 1;   // V landed
+                mbar_wait_stay(smem_u32(&bars[kVFull + i % NS]), (uint32_t)(i / NS) & 1u, abort_flag, ok);   // V landed
                 uint8_t* vt = sV + (size_t)(i % NS) * kOperand + hf * kAtom + r * 128;
                 for (int kv = max(n_keys - c_off, 0); kv < 64; ++kv)
                     *reinterpret_cast<uint16_t*>(vt + (((kv >> 3) ^ (r & 7)) << 4) + (kv & 7) * 2) = 0;
@@ -370,7 +369,6 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
                 xm[((i & 1) * 2 + hf) * kTile + r] = (uint16_t)(mb >> 16);
             }
             asm volatile("bar.sync 1, 256;" ::: "memory");
-            if (*abort_flag) { ok = false; break; }
             float alpha = 0.f;
             if (live) {
                 mx = fmaxf(fmaxf(mx, __uint_as_float((uint32_t)xm[((i & 1) * 2 + (hf ^ 1)) * kTile + r] << 16)), m);
@@ -403,7 +401,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
             if (!kSingle && i > 0) fold(i - 1, alpha_prev);
             alpha_prev = alpha;
         }
-        if (ok && n_kt > 0) fold(n_kt - 1, alpha_prev);
+        if (n_kt > 0) fold(n_kt - 1, alpha_prev);
         if (threadIdx.x == 64) A_STAMP(4);
         // row sum = sum of the two halves (same running maximum on both sides)
         asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -750,7 +748,7 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 // keys past n_vis may hold anything: zero their V columns so that 0 * garbage stays 0 (tile 0's threads, row r
                 // of the transposed V tile = head dim r; P V of either tile is issued after tile 0's P has been seen)
                 if (n_keys < kTile && t == 0) {
-                    if (!(ok = mbar_wait(smem_u32(&bars[kDVFull + (i & 1)]), (uint32_t)(i >> 1) & 1u, abort_flag))) break;
+                    mbar_wait_stay(smem_u32(&bars[kDVFull + (i & 1)]), (uint32_t)(i >> 1) & 1u, abort_flag, ok);
                     uint8_t* vt = sV + (size_t)(i & 1) * kOperand + r * 128;
                     auto at = [&](int kv) { return vt + (kv >> 6) * kAtom + ((((kv & 63) >> 3) ^ (r & 7)) << 4) + (kv & 7) * 2; };
                     int kv = n_keys;
@@ -758,7 +756,7 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     for (; kv < kTile; kv += 8) *reinterpret_cast<uint4*>(at(kv)) = make_uint4(0, 0, 0, 0);
                     fence_proxy_async_smem();
                 }
-                if (!(ok = mbar_wait(smem_u32(&bars[kDSFull + t]), (uint32_t)i & 1u, abort_flag))) break;
+                mbar_wait_stay(smem_u32(&bars[kDSFull + t]), (uint32_t)i & 1u, abort_flag, ok);      // (a failed wait goes on: its output is not written)
                 tc_fence_after();
                 if (live) {
                     uint32_t sc[4][32];
@@ -819,7 +817,7 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                 tc_fence_before();
                 mbar_arrive(smem_u32(&bars[kDPFull + t]));
             }
-            ok = ok && mbar_wait(smem_u32(&bars[kDODone + t]), 0, abort_flag);
+            mbar_wait_stay(smem_u32(&bars[kDODone + t]), 0, abort_flag, ok);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
             if (ok && live) {

@@ -64,6 +64,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
     return false;
 }
+// The same wait by a whole warp that goes on either way.  Every lane polls with its own clock, so lanes may give up at different
+// times, and what follows (tcgen05.ld / .st, votes over the full mask) takes the whole warp: a lane that gave up raises the flag,
+// which ends every later wait of the block early, clears ok, and stays with the others.  Nothing that another thread waits for
+// may be left out on that path.
+__device__ __forceinline__ void mbar_wait_stay(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool& ok) {
+    if (!mbar_wait(bar, parity, abort_flag)) {
+        *abort_flag = 1;
+        ok = false;
+    }
+    __syncwarp();
+}
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
     asm volatile(

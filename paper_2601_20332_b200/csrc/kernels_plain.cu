@@ -1496,16 +1496,26 @@ void wd_launch_plan(const WdPlanLaunch& h, cudaStream_t st) {
     launch_pdl(plan_kernel, dim3(h.batch), dim3(256), 0, st, a);
 }
 
-// A bounded wait that is never satisfied: the barrier expects one arrival and nobody arrives.
+// A bounded wait of a warp that half of its lanes never see satisfied: odd lanes poll a barrier that expects one arrival and gets
+// none, even lanes one whose phase is complete.  The warp is whole afterwards and the flag is up: the next wait on the first
+// barrier, by all lanes, gives up too, without waiting for its time to run out.
 __global__ void wait_expire_kernel(int32_t* status) {
-    __shared__ uint64_t bar;
+    __shared__ uint64_t bar[2];
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        wdk::mbar_init(wdk::smem_u32(&bar), 1);
+        for (int i = 0; i < 2; ++i) wdk::mbar_init(wdk::smem_u32(&bar[i]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (!wdk::mbar_wait(wdk::smem_u32(&bar), 0, &abort_flag)) atomicCAS(status, 0, WD_ERR_DEVICE_TIMEOUT);
+        wdk::mbar_arrive(wdk::smem_u32(&bar[0]));
     }
+    __syncwarp();
+    bool ok = true, again = true;
+    wdk::mbar_wait_stay(wdk::smem_u32(&bar[threadIdx.x & 1]), 0, &abort_flag, ok);
+    const unsigned met = __ballot_sync(0xffffffffu, ok);
+    const unsigned long long t0 = wdk::global_ns();
+    wdk::mbar_wait_stay(wdk::smem_u32(&bar[1]), 0, &abort_flag, again);
+    const unsigned met_again = __ballot_sync(0xffffffffu, again || wdk::global_ns() - t0 > wdk::kWaitNs / 2);
+    if (threadIdx.x == 0) atomicCAS(status, 0, met == 0x55555555u && met_again == 0 ? WD_ERR_DEVICE_TIMEOUT : WD_ERR_CUDA);
 }
 
 wd_status wd_launch_wait_expire(cudaStream_t st) {
