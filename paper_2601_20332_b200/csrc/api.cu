@@ -1,6 +1,7 @@
 // C ABI of libwd.so: context, sequence state, the step driver and the single
 // operations.  Host code; every step of the path runs in the kernels it launches.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cstdio>
 #include <cstdlib>
@@ -111,6 +112,7 @@ struct wd_ctx {
     size_t result_ints = 0;
 
     WdTcWeights tc;              // tensor maps of the weights (bf16 only)
+    WdAttnQ attn_q;
     WdTcChainState chain;        // counters of the chain kernel (WD_FUSION_CHAIN)
     bool chain_dirty = false;    // a device-side error may have left them out of step: zero them before the next launch
 
@@ -545,7 +547,7 @@ extern "C" wd_status wd_profile_read(const wd_ctx* ctx, double* gemm_ms, double*
 // ---------------------------------------------------------------------------
 static const int kQueueCap = 32;        // most steps enqueued without wd_step_sync
 
-static uint64_t g_state_uid = 0;
+static std::atomic<uint64_t> g_state_uid{0};
 
 struct wd_state {
     wd_ctx* ctx = nullptr;
@@ -1287,11 +1289,11 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         if (act_only)       // q holds the active rows, one after the other
             return wd_attn_tc_launch(c->q, NA, n_aqt, c->plan + o_aqt_seq, c->plan + o_aqt_row0, c->plan + o_aqt_n, c->plan + o_nvis,
                                      &st->map_k, &st->map_vt, c->attn, nullptr, Hq, Hkv, dh, l, max_vis, c->sm_count, status, stream,
-                                     max_act_tile_rows, &attn_smem, c->plan + o_aqt_off, batch, max_seq_act_tiles);
+                                     max_act_tile_rows, &attn_smem, c->plan + o_aqt_off, batch, max_seq_act_tiles, &c->attn_q);
         if (st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN)
             return wd_attn_tc_launch(c->q, R_, (int)n_qtiles, c->plan + o_qt_seq, c->plan + o_qt_row0, c->plan + o_qt_n,
                                      c->plan + o_nvis, &st->map_k, &st->map_vt, c->attn, attn_tap, Hq, Hkv, dh, l, max_vis,
-                                     c->sm_count, status, stream, max_tile_rows, &attn_smem, c->plan + o_qt_off, batch, max_seq_tiles);
+                                     c->sm_count, status, stream, max_tile_rows, &attn_smem, c->plan + o_qt_off, batch, max_seq_tiles, &c->attn_q);
         wd_launch_attention_plain(d.dtype, c->q, kc, vc, row_seq, vis_idx, vis_off, c->attn, attn_tap, R_, max_vis, Hq,
                                   Hkv, dh, S, Sp, batch, status, stream);
         return WD_OK;

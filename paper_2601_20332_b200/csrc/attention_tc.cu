@@ -888,16 +888,12 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn get_encode() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {      // looked up once, by whichever thread comes first
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
+        return cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess ? (EncodeTiledFn)p : nullptr;
+    }();
     return fn;
 }
 
@@ -935,15 +931,11 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
                             const int32_t* qtile_n, const int32_t* seq_nvis, const CUtensorMap* map_k,
                             const CUtensorMap* map_vt, void* out, float* tap, int Hq, int Hkv, int dh, int layer,
                             int max_vis, int sm_count, int32_t* status, cudaStream_t stream, int max_tile_rows,
-                            size_t* smem_used, const int32_t* seq_qt_off, int batch, int max_seq_tiles) {
+                            size_t* smem_used, const int32_t* seq_qt_off, int batch, int max_seq_tiles, WdAttnQ* q_maps) {
     if (dh != kTile) return WD_ERR_BAD_PARAM;
     if (n_tiles <= 0) return WD_OK;
     EncodeTiledFn enc = get_encode();
     if (!enc) return WD_ERR_CUDA;
-    // the query descriptor depends only on (buffer, rows, heads): the same for every layer of a step
-    static CUtensorMap mq;
-    static const void* mq_ptr = nullptr;
-    static int mq_rows = -1, mq_hq = -1, mq_dev = -1, mq_slot = -1;
     int dev = 0;
     WD_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return WD_ERR_CUDA;
@@ -959,7 +951,15 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
         if (pack == 2 && max_tile_rows > 64) pack = 1;
     }
     const int slot = kTile / pack;
-    if (mq_ptr != q || mq_rows != n_rows || mq_hq != Hq || mq_dev != dev || mq_slot != slot) {
+    CUtensorMap mq;
+    const WdAttnQ::Entry* known = nullptr;
+    for (int i = 0; q_maps && i < 2; ++i) {
+        const WdAttnQ::Entry& e = q_maps->entries[i];
+        if (e.q == q && e.rows == n_rows && e.heads == Hq && e.slot == slot) known = &e;
+    }
+    if (known) {
+        mq = known->map;
+    } else {
         cuuint64_t dims[2] = {(cuuint64_t)Hq * dh, (cuuint64_t)n_rows};
         cuuint64_t strides[1] = {(cuuint64_t)Hq * dh * 2};
         cuuint32_t box[2] = {64, (cuuint32_t)slot}, estr[2] = {1, 1};
@@ -967,7 +967,10 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return WD_ERR_CUDA;
-        mq_ptr = q; mq_rows = n_rows; mq_hq = Hq; mq_dev = dev; mq_slot = slot;
+        if (q_maps) {
+            q_maps->entries[q_maps->next] = {q, n_rows, Hq, slot, mq};
+            q_maps->next ^= 1;
+        }
     }
     AttnParams p;
     memset(&p, 0, sizeof(p));

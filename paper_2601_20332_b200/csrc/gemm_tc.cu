@@ -1511,16 +1511,12 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn get_encode() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {      // looked up once, by whichever thread comes first
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
+        return cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess ? (EncodeTiledFn)p : nullptr;
+    }();
     return fn;
 }
 
@@ -2011,8 +2007,8 @@ wd_status wd_tc_chain(const WdTcChainItem* items, int n, int rows, float* y, siz
     if (n < 1 || n > kChainMax || !wd_tc_chain_rows_ok(rows)) return WD_ERR_BAD_PARAM;
     const TcConfig cfg = pick_config(rows, false, false);
     if (cfg.tok_tiles != 1 || cfg.ctas_per_sm != 1) return WD_ERR_BAD_PARAM;
-    static ChainParams cp;              // large: kept off the stack (host threads do not step one context concurrently)
-    static ChainMaps maps;
+    thread_local ChainParams cp;        // large: kept off the stack
+    thread_local ChainMaps maps;
     memset(&cp, 0, sizeof(cp));
     cp.n_gemm = n;
     cp.ready = cs->ready_dev;
