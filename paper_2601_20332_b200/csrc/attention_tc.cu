@@ -548,7 +548,7 @@ attention_tc_single_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
 }
 
 // ------------------------------------------------------------------------------------------
-// Two query tiles per CTA: launches of more than one wave of single-tile CTAs
+// Two query tiles per CTA (the rule stands in wd_attn_tc_launch)
 // ------------------------------------------------------------------------------------------
 // A single-tile CTA is bound by its softmax warps: 2800 cycles per key tile, one phase after another (scores, maxima, a barrier
 // between the two halves of a row, exponentials, P, the rescale of O in registers), against 1024 of the tensor core.  Here a CTA
@@ -988,12 +988,21 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
     p.tiles_per_kv = (group + pack - 1) / pack;
     const int grid_y = Hkv * p.tiles_per_kv;
     static bool attr_done[64] = {};     // the attribute is per device
-    // More single-tile CTAs than SMs: two tiles per CTA (the rule is the wave: up to one of them the single-tile kernel, with its
-    // keys split over a cluster when SMs are left over, has the shorter chain).  Measured, single / two tiles, in us: 583 rows,
-    // 32 heads 32.8 / 23.4; 1536 rows, 32 heads 78.8 / 67.7 (192 CTAs for 148 SMs); eight sequences of 672 rows, 28 query and 4
-    // KV heads 158 / 98, of 66 rows over 830 keys 38.9 / 27.1; 1792 rows, 128 heads 360 / 249.
+    // Two tiles per CTA when that takes fewer rounds over the SMs: a CTA with two tiles takes 1.05-1.4 times a CTA with one, so
+    // halving the rounds pays and the same number of rounds does not (pairs are formed inside one sequence and KV head: with one
+    // tile for each there are none).  Measured, single / two tiles, in us; rounds 2 and 1: 583 rows, 32 heads 33 / 23.4; 128 keys
+    // 700 rows, 28 query and 4 KV heads 14.8 / 10.0; 2048 keys, 640 rows, 40 heads 63 / 42.5.  3 and 2: 290 rows, 100 heads, 512
+    // keys 32.5 / 28.2.  2 and 2: 34 rows, 160 heads, 512 keys 21.7 / 24.2; 290 rows, 80 heads, 2048 keys 65 / 75; 640 rows, 50
+    // heads, 1024 keys 37.6 / 42.7.  With the same rounds it still wins where a CTA is mostly start and end, one key tile and
+    // more than 64 rows in a tile (128 rows, 160 heads 14.3 / 13.2; 64 rows 12.7 / 13.1) or two and more than 96 (256 keys: 97
+    // rows 17.5 / 17.1, 128 rows 17.8 / 17.0, 80 rows 16.6 / 16.9; at 512 keys 128 rows 23.8 / 24.2).
     static const int dual_on = getenv("WD_ATTN_DUAL") ? atoi(getenv("WD_ATTN_DUAL")) : 1;
-    if (dual_on && seq_qt_off && n_tiles * grid_y > sm_count) {
+    const int ctas_one = n_tiles * grid_y;
+    const int ctas_two = Hkv * ((n_tiles * p.tiles_per_kv + (p.tiles_per_kv & 1 ? batch : 0)) / 2);   // (each sequence may end in half a pair)
+    const int rounds_one = (ctas_one + sm_count - 1) / sm_count, rounds_two = (ctas_two + sm_count - 1) / sm_count;
+    const int tile_rows = max_tile_rows > 0 ? max_tile_rows : kTile;
+    const bool short_ctas = rounds_one > 1 && ((max_kt == 1 && tile_rows > 64) || (max_kt == 2 && tile_rows > 96));
+    if (dual_on && seq_qt_off && (rounds_two < rounds_one || (rounds_two == rounds_one && short_ctas))) {
         static bool dual_done[64] = {};
         if (!dual_done[dev]) {
             WD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_dual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDualSmem));

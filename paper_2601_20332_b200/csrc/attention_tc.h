@@ -35,5 +35,5 @@ wd_status wd_attn_tc_launch(const void* q, int n_rows, int n_tiles, const int32_
 // smem_used (optional): the dynamic shared memory of one CTA of the launch (the single-key-tile form takes less than
 // half an SM's, so that the next kernel's CTAs can be resident beside it).
 // seq_qt_off (optional): device [batch + 1], first query tile of each sequence (tiles in sequence order); max_seq_tiles = most
-// tiles of any sequence.  With them a launch of more CTAs than SMs takes two query tiles per CTA.
+// tiles of any sequence.  With them a launch may take two query tiles per CTA (see the rule in wd_attn_tc_launch).
 // q_maps (optional): where the query descriptor is kept; without it, it is made for this launch.

@@ -1,4 +1,4 @@
-"""The attention kernel with two query tiles per CTA (launches of more single-tile CTAs than SMs), against the oracle."""
+"""The attention kernel with two query tiles per CTA (where that takes fewer rounds over the SMs), against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -13,11 +13,14 @@ DEV = "cuda"
 # more than 148 (row tile, query head) items: an odd number of tiles (a CTA with one), a last tile of one row, one key tile,
 # one key in the last tile, one below and one above a tile; grouped-query heads whose items pair across row tiles (7 per
 # tile); packed heads (two and four per tile) with empty slots; scores whose row maxima grow by tens of units from tile to
-# tile, so that the accumulated output is rescaled, and mild ones, where it is not
+# tile, so that the accumulated output is rescaled, and mild ones, where it is not; then both sides of the rule at an equal
+# number of rounds (one tile per KV head: 64 and 65 rows over one key tile, 96 and 97 over two, three key tiles)
 @pytest.mark.parametrize("rows,nv,Hq,Hkv,S,qs", [(257, 128, 64, 64, 136, 1.5), (300, 127, 64, 64, 128, 8.0),
                                                  (260, 129, 56, 8, 136, 8.0), (130, 1025, 84, 12, 1032, 8.0),
                                                  (640, 400, 32, 32, 400, 1.5), (33, 300, 320, 64, 304, 8.0),
-                                                 (20, 700, 693, 99, 704, 1.5), (128, 1, 160, 160, 8, 1.5)])
+                                                 (20, 700, 693, 99, 704, 1.5), (128, 1, 160, 160, 8, 1.5),
+                                                 (64, 128, 160, 160, 128, 1.5), (65, 128, 160, 160, 128, 8.0), (96, 256, 160, 160, 256, 8.0),
+                                                 (97, 256, 160, 160, 256, 1.5), (128, 257, 160, 160, 264, 8.0)])
 def test_two_tiles_per_cta_vs_oracle(rows, nv, Hq, Hkv, S, qs):
     g = torch.Generator(device=DEV).manual_seed(rows + nv)
     q = (torch.randn(rows, Hq, 128, device=DEV, generator=g) * qs).to(torch.bfloat16)
