@@ -19,9 +19,9 @@
 //   warps 2-5   epilogue: tcgen05.ld, row scales, coalesced fp32 stores of this K slice's partial sums
 //   warps 6-9   block scales: shared memory -> tensor memory
 // Persistent, one CTA per SM: the K blocks of all (weight tile, token tile) units form one line that is cut into
-// equal shares (stream-K), or whole units per CTA when that is cheaper.  The partial sums of a unit that several
+// equal shares (stream-K, see choose_split), or whole units per CTA when that is cheaper.  The partial sums of a unit that several
 // CTAs share are written side by side ([slice][tok][n]) and added by the consumer, as in the bf16 kernel.
-// Measured at 34 rows, quantised input to summed result, 12288 x 4096 / 24576 x 4096 / 4096 x 12288: 16.9 / 22.1 / 17.9 us
+// Measured at 34 rows, quantised input to summed result, 12288 x 4096 / 24576 x 4096 / 4096 x 12288: 15.4 / 22.8 / 16.0 us
 // against 4.7 / 9.3 / 4.6 us for the bytes alone; what remains is start-up (2-3 us to the first complete stage, 2 us from the
 // last MMA to the stores) around 0.44 us a stage.  (Bringing the weights into the L2 ahead of the dependency wait made it
 // slower: 24.4 instead of 23.8 us for the middle shape, 107 instead of 90 us at 600 rows.)
@@ -434,6 +434,54 @@ wd_status encode_bytes(CUtensorMap* m, const void* ptr, int n_rows, int row_byte
     return r == CUDA_SUCCESS ? WD_OK : WD_ERR_CUDA;
 }
 
+// How the K blocks of all units are dealt out: whole units per CTA (one slice), or the line of all K blocks cut into `grid` equal
+// shares, a unit's sums then being spread over up to n_slices slices.
+struct Split { int grid, n_slices, aligned; };
+
+// Most CTAs that share a unit when the line of n units is cut into G equal shares: with G / n = a + r / q in lowest terms a unit
+// covers at most ceil((q - 1) / q + G / n) of them.
+int sharers(int n, int G) {
+    const int a = G / n;
+    int r = G % n, q = n, x = r;
+    if (r == 0) return a;
+    while (x) { const int t = q % x; q = x; x = t; }       // q = gcd(r, n)
+    return a + (r / q == 1 ? 1 : 2);
+}
+
+// Time of a split: the stages of the longest share, t_stage each, and for every further slice its write and re-read at HBM speed
+// (t_slice) and 0.3 us, for the zero fill where nobody wrote it and for its place in the chain of the kernel that adds the slices
+// (between 0.15 and 1 us the choice is the same).  Beside all SMs the grids tried give G / n_units a denominator of at most eight:
+// shares then start with a unit every few units, which costs hardly a stage and saves slices.  With fewer slices allowed than all
+// SMs would make (a long K with few units, little scratch) it is a smaller grid, not whole units.
+// Measured at 34 rows, step of eight blocks 4096 / 12288 wide: 740 us; with all SMs whenever the line is cut 766, its down
+// projections leaving six slices after 11 stages instead of four after 12, its q/k/v three instead of two after the same 11;
+// fixed K splits dealt round-robin 739, but 850 at 68 rows against 830.  5 rows of 300, K 16384, quantiser and sum with it:
+// 12.3 us (48 CTAs), with whole units 34.8 (3 CTAs).
+Split choose_split(int n_units, int kb, int sm_count, int max_slices, double t_stage, double t_slice) {
+    const long long W = (long long)n_units * kb;
+    const int g_unit = std::min(sm_count, n_units);
+    Split best = {g_unit, 1, 1};
+    if (n_units >= 4 * sm_count) return best;               // rounds of whole units are full enough
+    double t_best = (double)((n_units + g_unit - 1) / g_unit) * kb * t_stage;
+    auto consider = [&](long long G) {
+        if (G < 1 || G > sm_count || G > W) return;
+        const int ns = sharers(n_units, (int)G);
+        if (ns > max_slices) return;
+        const double t = (double)((W + G - 1) / G) * t_stage + (ns - 1) * (t_slice + 0.3e-6);
+        if (t < t_best * 0.999) {
+            t_best = t;
+            best = {(int)G, ns, 0};
+        }
+    };
+    for (int q = 1; q <= 8; ++q) {
+        long long j = (long long)sm_count * q / n_units;
+        if (q == 1) j = std::min<long long>(j, max_slices);
+        if (n_units * j % q == 0) consider(n_units * j / q);
+    }
+    consider(sm_count);
+    return best;
+}
+
 }  // namespace
 
 size_t wd_fp4_operand_bytes(int n_rows, int K) {
@@ -483,25 +531,12 @@ wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, si
     p.n_units = n_tiles * p.tok_tiles;
     const size_t slice = (size_t)rows * n_out;
     if (slice > y_floats) return WD_ERR_CAPACITY;
-    // Equal shares of the K-block line over all SMs, or whole units per CTA (one slice): whichever takes less, with the time
-    // one SM needs to take in a stage (about 63 GB/s whatever the source) and the write and re-read of a further slice at
-    // HBM speed.  (Units of a fixed K slice dealt round-robin had rounds that were not full: 12 and 24 stages per SM for the
-    // q/k/v and gate/up shapes at 34 rows where the line gives 10.4 and 20.8, and 3 slices of gate/up instead of 2.)
-    const long long W = (long long)p.n_units * p.kb_total;
-    const int G_line = (int)std::min<long long>(sm_count, W);
-    const bool many = p.n_units >= 4 * sm_count;        // rounds of whole units are full enough
-    int n_slices = 1;
-    for (long long u = 0; u < p.n_units && !many; ++u) {
-        const long long first = ((u * p.kb_total + 1) * G_line - 1) / W, last = (((u + 1) * p.kb_total) * G_line - 1) / W;
-        n_slices = std::max(n_slices, (int)(last - first) + 1);
-    }
-    const int G_unit = std::min(sm_count, p.n_units);
-    const double t_stage = (double)(kStageW + p.bn * 128 + kSfW + p.bn * 16) / 63e9;
-    const double t_line = (double)((W + G_line - 1) / G_line) * t_stage + (n_slices - 1) * (double)slice * 8.0 / 6.5e12;
-    const double t_unit = (double)((p.n_units + G_unit - 1) / G_unit) * p.kb_total * t_stage;
-    p.aligned = force_single_split || many || t_unit <= t_line || n_slices > WD_TC_MAX_SPLIT || (size_t)n_slices * slice > y_floats;
-    p.n_slices = p.aligned ? 1 : n_slices;
-    const int grid = p.aligned ? G_unit : G_line;
+    const int max_slices = (int)std::min<size_t>(WD_TC_MAX_SPLIT, y_floats / slice);
+    const double t_stage = (double)(kStageW + p.bn * 128 + kSfW + p.bn * 16) / 63e9;      // what one SM takes in, whatever the source
+    const Split sp = choose_split(p.n_units, p.kb_total, sm_count, force_single_split ? 1 : max_slices, t_stage, (double)slice * 8.0 / 6.5e12);
+    p.aligned = sp.aligned;
+    p.n_slices = sp.n_slices;
+    const int grid = sp.grid;
     int cols = 32;
     while (cols < p.bn) cols <<= 1;
     p.buf_cols = cols;

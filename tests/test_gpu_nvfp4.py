@@ -33,9 +33,11 @@ def test_quantise_edges_are_the_oracles_bytes(rows, k, shift):
     np.testing.assert_array_equal(gr, rg)
 
 
-# a unit shared by many SMs, units that start and end inside a share, whole units per SM because the shares would need too
-# many slices, and because there are many units
-@pytest.mark.parametrize("rows,n,k", [(34, 1000, 4096), (129, 2000, 1024), (5, 300, 16384), (600, 16000, 256)])
+# a unit shared by many SMs, units that start and end inside a share, a grid cut down to the most slices (three units, one unit),
+# whole units per SM because there are many; two units in three equal shares, every share a fixed part of a unit, more sharers
+# than units
+@pytest.mark.parametrize("rows,n,k", [(34, 1000, 4096), (129, 2000, 1024), (5, 300, 16384), (600, 16000, 256), (5, 128, 16384),
+                                      (34, 12288, 4096), (16, 4096, 1024), (64, 600, 8192)])
 def test_gemm_edges(rows, n, k):
     g = torch.Generator(device=DEV).manual_seed(rows + n)
     x = torch.randn(rows, k, device=DEV, generator=g).to(torch.bfloat16)
