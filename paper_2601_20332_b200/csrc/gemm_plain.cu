@@ -1,6 +1,8 @@
 // CUDA-core GEMM: y[rows, n] = x[rows, k] * w[n, k]^T for any dtype, fp32 multiply and accumulate.  The fp32 models run
 // on it entirely; for bf16 it is the cross-check of the tensor-core kernels.  Up to three weight matrices that share
 // the input (q/k/v; gate/up) go in one launch, their outputs side by side.
+#include <algorithm>
+
 #include "wd_internal.h"
 #include "device_utils.cuh"
 
@@ -205,6 +207,15 @@ void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const 
         vec = vec && (uintptr_t)segs.w[i] % 16 == 0;
     }
     if (end <= 0) return;
+    constexpr int kMostRows = 65535 * 8;        // of one launch (a grid holds 65535 blocks in y)
+    if (rows > kMostRows) {
+        const size_t size = dtype == WD_F32 ? 4 : 2;
+        for (int r0 = 0; r0 < rows; r0 += kMostRows) {
+            const int m = std::min(rows - r0, kMostRows);
+            wd_launch_gemm_plain(dtype, (const char*)x + (size_t)r0 * k * size, w, n, n_mat, y + (size_t)r0 * ldy, m, k, ldy, w_static, st);
+            if (rows - r0 <= kMostRows) return;
+        }
+    }
     // Tiles when the rows kernel (17 TFLOP/s from a few hundred rows on) would take longer than the tiles' rounds over the
     // machine, two tiles per SM: 30 us each at k = 256 (768 columns: 24 us against 29 at 1024 rows, 47 against 30 at 2048,
     // 108 against 59 at 4800).

@@ -11,10 +11,11 @@ DEV = "cuda"
 
 
 # rows kernel: one piece, ragged pieces, k not a multiple of 4 (no vector loads), of 128, above 256, above one block of
-# three 128-element loads; tile kernel: from 1 M results up, ragged in rows, columns and k
+# three 128-element loads; tile kernel: from 1 M results up, ragged in rows, columns and k; more rows than
+# one grid holds
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("rows,n,k", [(1, 1, 5), (8, 16, 256), (9, 17, 64), (130, 101, 257), (33, 70, 388), (17, 36, 900),
-                                      (1100, 1030, 36), (1031, 1024, 260)])
+                                      (1100, 1030, 36), (1031, 1024, 260), (524289, 3, 5)])
 def test_gemm_plain_edges(dtype, rows, n, k):
     g = torch.Generator(device=DEV).manual_seed(rows * 7 + n)
     x = torch.randn(rows, k, device=DEV, generator=g).to(dtype)
