@@ -11,8 +11,7 @@ DEV = "cuda"
 
 
 # rows kernel: one piece, ragged pieces, k not a multiple of 4 (no vector loads), of 128, above 256, above one block of
-# three 128-element loads; tile kernel: from 1 M results up, ragged in rows, columns and k; more rows than
-# one grid holds
+# three 128-element loads; tile kernel, ragged in rows, columns and k; more rows than one grid holds
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("rows,n,k", [(1, 1, 5), (8, 16, 256), (9, 17, 64), (130, 101, 257), (33, 70, 388), (17, 36, 900),
                                       (1100, 1030, 36), (1031, 1024, 260), (524289, 3, 5)])
@@ -26,6 +25,20 @@ def test_gemm_plain_edges(dtype, rows, n, k):
     # values sum to |x| |w|^T
     bound = (k + 1) * 2.0 ** -24 * (x.double().abs() @ w.double().abs().T)
     assert ((y.double() - ref).abs() <= bound + 1e-30).all()
+
+
+# tiles filled through registers: k odd, rows that start off a 16-byte boundary, ragged rows,
+# columns and k, a last row tile with one row, a first one with 33
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("rows,n,k,shift", [(1100, 1030, 35, 0), (257, 2100, 255, 0), (640, 1030, 256, 1),
+                                            (33, 8200, 687, 0), (129, 4097, 18, 3)])
+def test_gemm_plain_unaligned(dtype, rows, n, k, shift):
+    g = torch.Generator(device=DEV).manual_seed(rows * 7 + n)
+    x = torch.randn(rows * k + shift, device=DEV, generator=g).to(dtype)[shift:].view(rows, k)
+    w = torch.randn(n * k + shift, device=DEV, generator=g).to(dtype)[shift:].view(n, k)
+    y = wd.op_gemm(x, w, wd.WD_GEMM_PLAIN)
+    bound = (k + 1) * 2.0 ** -24 * (x.double().abs() @ w.double().abs().T)         # as above
+    assert ((y.double() - x.double() @ w.double().T).abs() <= bound + 1e-30).all()
 
 
 # eight lanes per key with one to four 16-byte pieces per lane, fewer pieces than lanes, rows not a multiple of 16 bytes
