@@ -158,7 +158,12 @@ typedef struct wd_step_out {
  *   attn_out  [n_layers][n_rows][n_q_heads*head_dim]   attention outputs before
  *             the output projection
  *   logits    [n_act][vocab]   logits of the active rows
- * all float.  Capacities are for max_rows / max_active. */
+ * all float.  Capacities are for max_rows / max_active.
+ * layer_out and attn_out change what is computed: without them a step of more than 256 rows, at most
+ * half of them active, computes the last block for the active rows only (nothing else reads its output), and its
+ * products there are split otherwise, so that the logits of a step with and without these two taps may
+ * differ in their last bits.  logits alone changes nothing: the LM head writes there instead of to its own
+ * buffer. */
 typedef struct wd_debug_taps {
     float* layer_out;
     float* attn_out;

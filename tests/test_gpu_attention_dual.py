@@ -5,6 +5,8 @@ import torch
 
 from oracle import wd_oracle as wo
 from paper_2601_20332_b200 import binding as wd
+from paper_2601_20332_b200 import synth
+from wd_harness import Parity
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -36,3 +38,19 @@ def test_two_tiles_per_cta_vs_oracle(rows, nv, Hq, Hkv, S, qs):
     ref, _ = wo.attention_rows(q.double().cpu().numpy(), K, V, Hq // Hkv)
     # P and the result rounded to bf16: as in test_attention_tc_kernel_vs_oracle
     assert np.abs(out - ref).max() / np.abs(ref).max() < 2e-2
+
+
+# six, three and one query tiles of 16 heads: 160 single tiles, 96 pairs, CTAs beyond a shorter sequence's last pair leave at once
+# and odd sequences end in half a pair; with grouped heads (five to a KV head) pairs cross row tiles
+@pytest.mark.parametrize("Hq,Hkv", [(16, 16), (20, 4)])
+def test_sequences_of_different_lengths(Hq, Hkv):
+    cfg = synth.get_config("llada8b", L=1, d=256, Hq=Hq, Hkv=Hkv, dh=128, F=512, V=1000, P=650, G=80)
+    w = synth.make_weights(cfg, DEV, gain_jitter=0.1)
+    ids = synth.make_prompts(cfg, batch=3)
+    ids[1, 300:] = cfg["mask_id"]
+    ids[2, 50:] = cfg["mask_id"]
+    par = Parity(cfg, w, ids)
+    for _ in range(2):
+        info = par.step(16, 40, 4, 2, 1)["info"]
+    assert par.log[0]["info"]["n_rows"] == 706 + 356 + 106
+    par.close()

@@ -4,6 +4,7 @@ import torch
 
 from paper_2601_20332_b200 import binding as wd
 from paper_2601_20332_b200 import synth
+from wd_harness import Parity
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -44,3 +45,22 @@ def test_active_rows_of_the_last_block(Hq, Hkv, batch, P, G, A, B):
     for full, act in zip(*runs):
         # the same bf16 pipeline with other splits of the sums: bounded by the tolerance of a block's output
         assert float((full - act).norm() / full.norm()) < 1e-2
+
+
+# grouped-query heads and three sequences, one of them shorter; full heads, more active rows than a query tile and fewer than half
+@pytest.mark.parametrize("Hq,Hkv,batch,P,G,A,B", [(4, 1, 3, 150, 90, 16, 20), (2, 2, 2, 300, 300, 140, 60)])
+def test_untapped_blocks_against_the_oracle(Hq, Hkv, batch, P, G, A, B):
+    """The path that steps take in use: only the logits are tapped.  Index sets, logits, chosen tokens of a refresh step, of the
+    two normal steps that read the cache it wrote, and of the next refresh."""
+    cfg = synth.get_config("llada8b", L=2, d=256, Hq=Hq, Hkv=Hkv, dh=128, F=512, V=1000, P=P, G=G)
+    w = synth.make_weights(cfg, DEV, gain_jitter=0.1)
+    ids = synth.make_prompts(cfg, batch=batch)
+    ids[1, P - 40:] = cfg["mask_id"]
+    par = Parity(cfg, w, ids, block_taps=False)
+    for i in range(4):
+        info = par.step(A, B, 3, 2, 1)["info"]
+        assert info["is_refresh"] == (i % 3 == 0)
+        if info["is_refresh"]:
+            assert info["n_rows"] > 256 and 2 * info["n_active"] <= info["n_rows"]
+    par.check_state_mirror()
+    par.close()

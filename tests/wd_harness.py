@@ -34,8 +34,10 @@ def max_rel(a, b):
 class Parity:
     def __init__(self, cfg, weights, ids, decoded=None, gemm_impl=wd.WD_GEMM_AUTO, oracle_seqs=None,
                  max_rows=None, max_active=None, fusion=wd.WD_FUSION_AUTO, eos_id=None, refresh_mode=0, fp8=False,
-                 follow_rounded=False, stagger=False, fp4=False):
-        """follow_rounded: a second oracle follower per sequence runs in the bfloat16 storage-points mode
+                 follow_rounded=False, stagger=False, fp4=False, block_taps=True):
+        """block_taps=False: no taps of the blocks, only of the logits (with them a step computes the last block for
+        every row); the layers are then not compared.
+        follow_rounded: a second oracle follower per sequence runs in the bfloat16 storage-points mode
         (the same teacher-forced trajectory); `step` then also records, per block, the GPU's distance to it
         and its own distance to the plain float64 follower: what the storage format alone costs at that
         depth, the yardstick for the GPU's error in a deep model."""
@@ -62,7 +64,11 @@ class Parity:
         self.t_layer = torch.zeros(L * max_rows * d, dtype=torch.float32, device=dev)
         self.t_attn = torch.zeros(L * max_rows * hq, dtype=torch.float32, device=dev)
         self.t_logits = torch.zeros(max_active * V, dtype=torch.float32, device=dev)
-        self.st.set_taps(self.t_layer, self.t_attn, self.t_logits)
+        self.block_taps = block_taps
+        if block_taps:
+            self.st.set_taps(self.t_layer, self.t_attn, self.t_logits)
+        else:
+            self.st.set_taps(logits=self.t_logits)
         self.model = synth.OracleModelView(weights)
         if fp8:
             self.model.dims = dict(self.model.dims, fp8=True)
@@ -124,7 +130,7 @@ class Parity:
                 assert p[name] == op[oname], (name, b)
             r0, r1 = row_off[b], row_off[b + 1]
             a0, a1 = act_off[b], act_off[b + 1]
-            for l in range(L):
+            for l in range(L if self.block_taps else 0):
                 e_l = rel_rms(lay[l, r0:r1], o["layer_out"][l])
                 e_a = max_rel(att[l, r0:r1], o["attn_out"][l])
                 worst["layer"] = max(worst["layer"], e_l)
