@@ -1302,7 +1302,9 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     // computes keys and values of every row (the cache wants them) and the rest for the active rows, which a gather puts one
     // after the other.  From 257 rows on, where the GEMMs' time depends on their rows, and when it at least halves them (352 rows,
     // 32 active: 225 us of a block -> 120; 28672 rows, 2048 active: 11.2 ms -> 2.3 ms; a step of 104 rows streams weights either
-    // way and would pay three more launches).  Not for a model of one block, and not when a tap wants every row of every block.
+    // way and would pay three more launches).  At the edges, step of two blocks in us without / with it: 32 of 260 rows active 472
+    // / 412, 128 of 260 483 / 439, 256 of 512 585 / 552, 300 of 620 655 / 646, 1024 of 2100 1840 / 1602.  Not for a model of one
+    // block, and not when a tap wants every row of every block.
     const bool act_last = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN && !fp8 && !fp4 && !fused &&
                           d.n_layers > 1 && NA > 0 && R_ > 256 && 2 * NA <= R_ && !st->taps.layer_out && !st->taps.attn_out;
     // ---- the kernels of the step, from the embedding to the selection (everything after the planner and
@@ -1427,8 +1429,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         } else {
         WdTcSeg qkv[3] = {{c->wq[l], hq, c->tc.get(WD_TC_WQ, l)}, {c->wk[l], hkv, c->tc.get(WD_TC_WK, l)},
                           {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
-        // (Not for grouped-query heads: their narrow q/k/v has 85 % full rounds at 5376 rows, the rotation's kernel is 50 us of a
-        // 2.1 ms block, and the epilogue would save about half of it.)
+        // (Heads without grouping only, so far.  With 28 query over 4 KV heads a refresh of four blocks would also be 1-2 % faster
+        // for it where the rounds are full: 5376 rows 7370 / 7270 us, 6080 rows 8000 / 7830, 6880 rows 9150 / 8990.)
         if (use_tc(c) && dh == 128 && Hq == Hkv) {
             rope.map_q = c->tc.get(WD_TC_WQ_ROT, l); rope.map_k = c->tc.get(WD_TC_WK_ROT, l);
             rope.row_seq = row_seq; rope.row_pos = row_pos; rope.rope_tab = c->rope_tab;

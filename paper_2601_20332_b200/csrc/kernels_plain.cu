@@ -1372,7 +1372,8 @@ void wd_launch_swiglu(int dtype, const float* part, int n_split, size_t split_st
     const size_t total = (size_t)n_rows * (F >> 2);
     static const int sw_rows = getenv("WD_SWIGLU_ROWS") ? atoi(getenv("WD_SWIGLU_ROWS")) : 1;
     // up to 600 thousand positions, 195 rows of 12288 (measured per launch, one / two positions per thread: 5.2 / 11.9 us at 136
-    // rows, 10.4 / 7.7 us at 352 rows, where two pay)
+    // rows, 10.4 / 7.7 us at 352 rows, where two pay).  Normal step of four blocks, one / two, in us: 12288 wide 170 rows 665 / 687,
+    // 204 rows 730 / 753, 238 rows 777 / 798, 272 rows 958 / 958; 18944 wide 140 rows 589 / 585, 210 rows 686 / 678.
     static const int sw_rows_max = getenv("WD_SWIGLU_ROWS_MAX") ? atoi(getenv("WD_SWIGLU_ROWS_MAX")) : 600000;
     if (sw_rows && total <= (size_t)sw_rows_max) {
         WD_DISPATCH(dtype, launch_pdl(swiglu_rows_kernel<T>, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, part, n_split,
