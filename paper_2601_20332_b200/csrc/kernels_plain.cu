@@ -755,10 +755,12 @@ template <> struct Vec16<__nv_bfloat16> {
     }
 };
 
-constexpr int kAttnThreads = 256;
+// kFew: 128 threads, a key per warp and one head dim per warp at a time, for many blocks with little in each (at most 32 head dims:
+// with eight dims to a warp most of its warps would have none).
+constexpr int kAttnThreads = 256, kAttnThreadsFew = 128;
 
-template <typename T, bool kVec>
-__global__ void __launch_bounds__(kAttnThreads)
+template <typename T, bool kVec, bool kFew>
+__global__ void __launch_bounds__(kFew ? kAttnThreadsFew : kAttnThreads)
 attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
                        const T* __restrict__ vcache, const int32_t* __restrict__ row_seq,
                        const int32_t* __restrict__ vis_idx, const int32_t* __restrict__ vis_off,
@@ -782,7 +784,7 @@ attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
     const T* qr = q + ((size_t)r * Hq + h) * dh;
     const float scale = rsqrtf((float)dh);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int nw = kAttnThreads / 32;
+    constexpr int kThreads = kFew ? kAttnThreadsFew : kAttnThreads, nw = kThreads / 32;
     float mx = -INFINITY;
     if (kVec) {
         constexpr int N = Vec16<T>::N, kU = 4, kMaxVec = 4;    // keys in flight per lane group; 16-byte pieces of a row per lane
@@ -833,7 +835,7 @@ attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
         }
     } else {
         float* qs = sc + nv;
-        for (int c = threadIdx.x; c < dh; c += kAttnThreads) qs[c] = to_f(qr[c]);
+        for (int c = threadIdx.x; c < dh; c += kThreads) qs[c] = to_f(qr[c]);
         __syncthreads();
         for (int j = wid; j < nv; j += nw) {
             const int vi = vis_idx[v0 + j];
@@ -852,7 +854,7 @@ attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
     mx = block_max(mx, red);
     __syncthreads();
     float sum = 0.f;
-    for (int j = threadIdx.x; j < nv; j += kAttnThreads) {
+    for (int j = threadIdx.x; j < nv; j += kThreads) {
         const float e = __expf(sc[j] - mx);
         sc[j] = e;
         sum += e;
@@ -860,6 +862,23 @@ attention_plain_kernel(const T* __restrict__ q, const T* __restrict__ kcache,
     sum = block_sum(sum, red);
     __syncthreads();
     const float inv = 1.f / sum;
+    if (kFew) {
+        for (int c = wid; c < dh; c += nw) {
+            const T* vr = vb + (size_t)c * Sp;
+            float a = 0.f;
+            for (int j = lane; j < nv; j += 32) {
+                const int vi = vis_idx[v0 + j];
+                if ((unsigned)vi < (unsigned)S) a = fmaf(sc[j], to_f(vr[vi]), a);
+            }
+            a = warp_sum(a) * inv;
+            if (lane == 0) {
+                const size_t o = ((size_t)r * Hq + h) * dh + c;
+                out[o] = from_f<T>(a);
+                if (tap) tap[o] = a;
+            }
+        }
+        return;
+    }
     for (int c0 = 8 * wid; c0 < dh; c0 += 8 * nw) {
         float a[8] = {};
         const T* vr[8];
@@ -1333,13 +1352,13 @@ void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t sp
                                   Hkv, dh, S, Sp, n_qk, qk_groups, n_qk_blocks, batch, status));
 }
 
-template <typename T, bool kVec>
+template <typename T, bool kVec, bool kFew>
 static void launch_attention_plain(dim3 grid, size_t smem, cudaStream_t st, const void* q, const void* kcache, const void* vcache,
                                    const int32_t* row_seq, const int32_t* vis_idx, const int32_t* vis_off, void* out, float* tap,
                                    int max_vis, int Hq, int Hkv, int dh, int S, int Sp, int batch, int32_t* status) {
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(attention_plain_kernel<T, kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(attention_plain_kernel<T, kVec>, grid, dim3(kAttnThreads), smem, st, (const T*)q, (const T*)kcache, (const T*)vcache,
+        cudaFuncSetAttribute(attention_plain_kernel<T, kVec, kFew>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_pdl(attention_plain_kernel<T, kVec, kFew>, grid, dim3(kFew ? kAttnThreadsFew : kAttnThreads), smem, st, (const T*)q, (const T*)kcache, (const T*)vcache,
                row_seq, vis_idx, vis_off, (T*)out, tap, max_vis, Hq, Hkv, dh, S, Sp, batch, status);
 }
 
@@ -1356,12 +1375,21 @@ void wd_launch_attention_plain(int dtype, const void* q, const void* kcache, con
     const bool vec = (dh * (int)wd_elt_size(dtype)) % 16 == 0 && dh * (int)wd_elt_size(dtype) <= 512 &&
                      ((uintptr_t)q | (uintptr_t)kcache) % 16 == 0;
 #define WD_ATTN_ARGS grid, smem, st, q, kcache, vcache, row_seq, vis_idx, vis_off, out, tap, max_vis, Hq, Hkv, dh, S, Sp, batch, status
+    // kFew for many blocks of at most 32 head dims: where rows cannot be loaded 16 bytes at a time, up to the visible counts whose
+    // scores leave room for only a few blocks on an SM, or with next to no keys.  Measured, 256 threads / 128, in us: fp32, 4 heads
+    // of 6, 1500 rows, 1 key 24.5 / 13.0, 1000 keys 919 / 630, 20000 keys 34.9 / 56.7 ms, 200 rows of 1000 keys 177 / 187; bf16, 4
+    // heads of 20, 1500 rows, 6000 keys 5.67 / 4.92 ms; fp32, 4 heads of 16, 1500 rows, 1 key 32 / 18, 40 keys 39 / 46.
+    // (Eight dims to a warp want lists that ascend, as a step's do: 1500 rows, 4 heads of 128, 1000 keys in order 627, in random
+    // order 3250 us, one dim at a time 1320 / 2450.  Looking at the order inside the kernel cost the ordered lists up to half.)
+    const bool few = dh <= 32 && (long long)n_rows * Hq >= 16 * 148 && (vec ? max_vis <= 8 : max_vis <= 8192);
     if (dtype == WD_F32) {
-        if (vec) launch_attention_plain<float, true>(WD_ATTN_ARGS);
-        else launch_attention_plain<float, false>(WD_ATTN_ARGS);
+        if (few) launch_attention_plain<float, false, true>(WD_ATTN_ARGS);
+        else if (vec) launch_attention_plain<float, true, false>(WD_ATTN_ARGS);
+        else launch_attention_plain<float, false, false>(WD_ATTN_ARGS);
     } else {
-        if (vec) launch_attention_plain<__nv_bfloat16, true>(WD_ATTN_ARGS);
-        else launch_attention_plain<__nv_bfloat16, false>(WD_ATTN_ARGS);
+        if (few) launch_attention_plain<__nv_bfloat16, false, true>(WD_ATTN_ARGS);
+        else if (vec) launch_attention_plain<__nv_bfloat16, true, false>(WD_ATTN_ARGS);
+        else launch_attention_plain<__nv_bfloat16, false, false>(WD_ATTN_ARGS);
     }
 #undef WD_ATTN_ARGS
 }

@@ -64,6 +64,26 @@ def test_attention_plain_edges(dtype, dh, n_vis):
     assert ((out - ref).abs() <= tol).all()
 
 
+# many blocks of few head dims (128 threads, a dim per warp): rows that are not 16-byte pieces, next to no keys, and both sides of
+# the line between the two forms (2368 blocks, 8 keys for aligned rows)
+@pytest.mark.parametrize("dtype,dh,rows,n_vis", [(torch.float32, 6, 592, 33), (torch.float32, 6, 591, 33), (torch.float32, 16, 700, 1),
+                                                 (torch.float32, 32, 700, 8), (torch.float32, 32, 700, 9), (torch.bfloat16, 20, 600, 130),
+                                                 (torch.bfloat16, 2, 1200, 5)])
+def test_attention_plain_many_small_blocks(dtype, dh, rows, n_vis):
+    Hq, Hkv, S = 4, 2, 136
+    g = torch.Generator(device=DEV).manual_seed(dh + n_vis)
+    q = torch.randn(rows, Hq, dh, device=DEV, generator=g).to(dtype)
+    k = torch.randn(Hkv, S, dh, device=DEV, generator=g).to(dtype)
+    v = torch.randn(Hkv, dh, S, device=DEV, generator=g).to(dtype)
+    vis = torch.randperm(S, device=DEV, generator=g)[:n_vis].sort().values.to(torch.int32)
+    out = wd.op_attention(q, k, v, vis).double()
+    kk = k.double()[:, vis.long()].repeat_interleave(Hq // Hkv, 0)
+    vv = v.double()[:, :, vis.long()].repeat_interleave(Hq // Hkv, 0)
+    ref = torch.einsum("rhj,hdj->rhd", (torch.einsum("rhd,hjd->rhj", q.double(), kk) / dh ** 0.5).softmax(-1), vv)
+    tol = 1e-5 * float(v.abs().max()) + (2.0 ** -8 * ref.abs() if dtype == torch.bfloat16 else 0.0)        # as above
+    assert ((out - ref).abs() <= tol).all()
+
+
 def test_fp32_steps_replayed_from_graphs():
     """Queued fp32 steps are recorded and replayed; the generation is the one that direct launches give."""
     cfg = synth.get_config("tiny", P=100, G=60)            # the visible range grows across a key tile (128) on the way
