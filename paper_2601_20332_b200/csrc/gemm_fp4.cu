@@ -27,6 +27,7 @@
 // slower: 24.4 instead of 23.8 us for the middle shape, 107 instead of 90 us at 600 rows.)
 // Every wait is bounded; on expiry the CTA records WD_ERR_DEVICE_TIMEOUT and leaves.
 #include <algorithm>
+#include <climits>
 #include <cstring>
 
 #include <cuda_fp8.h>
@@ -88,8 +89,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     // This CTA's share [g_begin, g_end) of the line of K blocks of all units, unit = weight tile * tok_tiles + token tile
     // (neighbouring units share a weight tile): equal shares, so every SM streams the same bytes, or whole units.
     const int G = gridDim.x, c = blockIdx.x, KB = p.kb_total, W = p.n_units * KB;
-    const int g_begin = p.aligned ? (int)((long long)c * p.n_units / G) * KB : (int)((long long)c * W / G);
-    const int g_end = p.aligned ? (int)((long long)(c + 1) * p.n_units / G) * KB : (int)((long long)(c + 1) * W / G);
+    // (32-bit: the host sees to it that the products fit)
+    const int g_begin = p.aligned ? c * p.n_units / G * KB : c * W / G;
+    const int g_end = p.aligned ? (c + 1) * p.n_units / G * KB : (c + 1) * W / G;
     const int n_total = g_end - g_begin;
     // the piece that starts at K block g of the line: its unit's rows and tokens, first K block and length
     auto piece_at = [&](int g, int& unit, int& n0, int& tok0, int& kb0, int& len) {
@@ -228,7 +230,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             piece_at(g, unit, n0, tok0, kb0, kbn);
             g += kbn;
             // slice: this CTA's place among those that share the unit
-            const int sl = p.aligned ? 0 : c - (int)((((long long)unit * KB + 1) * G - 1) / W);
+            const int sl = p.aligned || kb0 == 0 ? 0 : c - ((unit * KB + 1) * G - 1) / W;
             const int buf = u & 1;
             const uint32_t par = (uint32_t)(u >> 1) & 1u;
             const int n = n0 + n_local;
@@ -464,7 +466,7 @@ Split choose_split(int n_units, int kb, int sm_count, int max_slices, double t_s
     if (n_units >= 4 * sm_count) return best;               // rounds of whole units are full enough
     double t_best = (double)((n_units + g_unit - 1) / g_unit) * kb * t_stage;
     auto consider = [&](long long G) {
-        if (G < 1 || G > sm_count || G > W) return;
+        if (G < 1 || G > sm_count || G > W || W * (G + 1) > INT_MAX) return;
         const int ns = sharers(n_units, (int)G);
         if (ns > max_slices) return;
         const double t = (double)((W + G - 1) / G) * t_stage + (ns - 1) * (t_slice + 0.3e-6);
@@ -528,6 +530,7 @@ wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, si
     p.bn = ((rows + p.tok_tiles - 1) / p.tok_tiles + 15) / 16 * 16;        // balanced token tiles, <= 128
     p.kb_total = K / kKB;
     const int n_tiles = (n_out + kBM - 1) / kBM;
+    if ((long long)n_tiles * p.tok_tiles * std::max(p.kb_total, sm_count + 1) > INT_MAX) return WD_ERR_CAPACITY;
     p.n_units = n_tiles * p.tok_tiles;
     const size_t slice = (size_t)rows * n_out;
     if (slice > y_floats) return WD_ERR_CAPACITY;
