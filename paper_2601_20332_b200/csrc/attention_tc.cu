@@ -558,6 +558,8 @@ attention_tc_single_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
 //                      registers, and while one tile's scores are exponentiated the tensor core works on the other's
 //   O                  stays in tensor memory: P V accumulates over the key tiles, and a warp rescales its rows only when a row's
 //                      maximum has grown by more than 2^8 since the reference value in use (any reference cancels in O / l)
+// (Two tiles in turn and the rescale left out while the maximum grows little are the steps that FlashAttention-4 made known;
+// written here from their description.)
 // Tensor memory: S (and P over it) 2 x 128 columns, O 2 x 128.  Shared memory: two Q tiles, two K and two V stages, 192 KB.
 // The tensor core runs Q K^T and P V in issue order, so S(i + 1) complete means P V(i) has read P(i) and has been added to O;
 // one barrier each for S and P of a tile suffices (P(i + 1) needs S(i + 1), which is issued only after P(i) has been seen).
