@@ -341,8 +341,11 @@ __device__ void finalize_unit(const TcParams& p, int G, int unit, int e) {
 // by piece boundaries gets one partial sum per CTA that touched it, written to slice
 // (CTA - first CTA of the tile); the CTA that finishes the tile zero-fills the unused slices.
 // kWide: two weight halves per CTA (many tokens).  kLmStats: the LM-head epilogue that reduces
-// the logits to per-row statistics.  Separate instantiations keep the plain weight-streaming
-// kernel free of the other variants' code (its issue loops are sensitive to it).
+// the logits to per-row statistics.  kFused: the CTA that completes a tile finishes it (finalize_unit).
+// Separate instantiations keep the plain weight-streaming kernel free of the other variants' code
+// (its issue loops are sensitive to it), and give finalize_unit the registers that its loads in flight
+// want: inside the plain kernel, at 79 registers, it had made the WD_FUSION_TILE step 2-5 % slower
+// (normal step of eight blocks, 34 rows: 1373 us, with 148 registers 1305).
 #ifdef WD_GEMM_TRACE
 // clock stamps of the last launch per slot (q/k/v, o, gate/up, down, other): [slot][CTA][event]
 __device__ unsigned long long g_gemm_trace[8][160][8];
@@ -351,8 +354,8 @@ __device__ unsigned long long g_gemm_trace[8][160][8];
 #define G_STAMP(k) do { } while (0)
 #endif
 
-template <bool kWide, bool kLmStats, bool kFp8 = false>
-__global__ void __launch_bounds__(kWide ? kThreadsWide : kThreads)
+template <bool kWide, bool kLmStats, bool kFp8 = false, bool kFused = false>
+__global__ void __launch_bounds__(kWide ? kThreadsWide : kThreads, kFused ? 1 : 0)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w0,
                const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w2,
                const TcParams p) {
@@ -641,7 +644,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             }
             tc_fence_before();
             mbar_arrive(smem_u32(&bars[2 * NS + 2 + buf]));       // accumulator may be overwritten
-            if (p.f.mode != WD_FUSE_NONE && p.f.mode != WD_FUSE_LMSTATS) {
+            if constexpr (kFused) {
                 // count this piece's arrival at its tile; the CTA that arrives last finishes the tile
                 const int e = (int)threadIdx.x - 64;
                 __threadfence();
@@ -666,7 +669,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 epi_sync();
                 if (*last_flag) finalize_unit(p, G, unit, e);
                 epi_sync();
-            } else if (kb0 + len == p.kb_total && n_ok && p.f.mode == WD_FUSE_NONE) {
+            } else if (kb0 + len == p.kb_total && n_ok && !kLmStats) {
                 // this CTA finished the tile: slices nobody wrote must read as zero
                 for (int sl = ord + 1; sl < p.n_slices; ++sl) {
                     float* ys = yb + (size_t)sl * p.split_stride;
@@ -1971,6 +1974,7 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, false, false, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, false, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, true, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         attr_done[dev] = true;
@@ -1993,6 +1997,7 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
     else if (fp8) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, (gemm_tc_kernel<false, false, true>), mx, m0, m1, m2, p));
     else if (cfg.wide) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_kernel<true, false>, mx, m0, m1, m2, p));
     else if (p.f.mode == WD_FUSE_LMSTATS) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_kernel<false, true>, mx, m0, m1, m2, p));
+    else if (fused) WD_CUDA_TRY(cudaLaunchKernelEx(&lc, (gemm_tc_kernel<false, false, false, true>), mx, m0, m1, m2, p));
     else WD_CUDA_TRY(cudaLaunchKernelEx(&lc, gemm_tc_kernel<false, false>, mx, m0, m1, m2, p));
     if (n_split_out) *n_split_out = p.n_slices;
     return WD_OK;
