@@ -989,10 +989,12 @@ static bool use_tc(const wd_ctx* c) {
 static wd_status run_gemm(wd_ctx* c, const void* x, const WdTcX* x_map, const WdTcSeg* segs, int nseg,
                           int rows, int K, float* y, size_t y_floats, int32_t* status, cudaStream_t stream,
                           GemmOut* go, bool single_split = false, const WdTcFuse* fuse = nullptr,
-                          const WdTcFp8* fp8 = nullptr, const WdTcEpi* epi = nullptr) {
+                          const WdTcFp8* fp8 = nullptr, const WdTcEpi* epi = nullptr, WdPlainFuse* plain = nullptr) {
     int ncol = 0;
     for (int i = 0; i < nseg; ++i) ncol += segs[i].n;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    const size_t prof_used0 = c->prof_used;
+    const double prof_bytes0 = c->prof_step_bytes;
     if (c->prof_on) {
         while (c->prof_events.size() < c->prof_used + 2) {
             cudaEvent_t e;
@@ -1026,7 +1028,13 @@ static wd_status run_gemm(wd_ctx* c, const void* x, const WdTcX* x_map, const Wd
         const void* w[3];
         int n[3];
         for (int i = 0; i < nseg; ++i) { w[i] = segs[i].w; n[i] = segs[i].n; }
-        wd_launch_gemm_plain(c->d.dtype, x, w, n, nseg, y, rows, K, ncol, /*w_static=*/true, stream);
+        if (plain && !wd_launch_gemm_plain_fused(*plain, w, n, nseg, rows, K, stream)) {
+            c->prof_used = prof_used0;
+            c->prof_step_bytes = prof_bytes0;
+            return WD_OK;                   // plain->done stays false
+        }
+        if (plain) plain->done = true;
+        else wd_launch_gemm_plain(c->d.dtype, x, w, n, nseg, y, rows, K, ncol, /*w_static=*/true, stream);
         *go = {1, (size_t)rows * ncol, 1, WD_GEMM_PLAIN};
     }
     if (e1) WD_CUDA_TRY(cudaEventRecord(e1, stream));
@@ -1275,6 +1283,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         for (int i = 0; i < 4; ++i) c->chain.ready_host[i] = 0;
         c->chain_dirty = false;
     }
+    const bool f32 = d.dtype == WD_F32;
     const bool fp8 = c->fp8_on && use_tc(c) && !fused;      // FP8 projections (q/k/v, gate/up, down, LM head)
     const bool fp4 = c->fp4_on && use_tc(c) && !fused;      // NVFP4 projections (the same ones)
     WdFp4Operand x4_d, x4_f, x4_lm;                         // the step's quantised activations, by use
@@ -1401,12 +1410,27 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         const bool act = act_last && l == d.n_layers - 1;
         WdTcRope rope;
         WdTcEpi epi_rope;
+        // fp32, few rows: the element-wise kernels inside the projections where x is complete (see wd_launch_gemm_plain_fused)
+        WdPlainFuse pq, po, pg, pd;
+        if (f32 && !down_pending) {
+            pq.epi = WD_PLAIN_QKV;
+            pq.x = c->x; pq.gain = c->attn_norm[l]; pq.eps = d.rms_eps;
+            pq.row_seq = row_seq; pq.row_pos = row_pos; pq.rope_tab = c->rope_tab;
+            pq.q = (float*)c->q; pq.kcache = (float*)kc; pq.vcache = (float*)vc;
+            pq.Hq = Hq; pq.Hkv = Hkv; pq.dh = dh; pq.S = S; pq.Sp = Sp; pq.batch = batch; pq.status = status;
+            WdTcSeg qkv[3] = {{c->wq[l], hq, nullptr}, {c->wk[l], hkv, nullptr}, {c->wv[l], hkv, nullptr}};
+            if ((s = run_gemm(c, c->x, nullptr, qkv, 3, R_, D, c->part, c->part_floats, status, stream, &go, false, nullptr, nullptr,
+                              nullptr, &pq)) != WD_OK)
+                return s;
+        }
         // attention half (FP8 mode: the normalised rows leave the RMSNorm as e4m3 codes + row scales)
-        wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
+        if (!pq.done)
+            wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
                           c->attn_norm[l], d.rms_eps, c->xn, nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn,
                           fp4 ? &x4_d : nullptr);
         down_pending = false;
-        if (fp4) {
+        if (pq.done) {
+        } else if (fp4) {
             if ((s = run_gemm_fp4(c, &c->f4qkv[l], R_, D, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
         } else if (fp8) {
             WdTcSeg qkv[3] = {{c->f8q[l].q, hq, &c->f8q[l].map}, {c->f8k[l].q, hkv, &c->f8k[l].map},
@@ -1443,7 +1467,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             return s;
         }
         impl_used = go.impl;
-        if (rope.done) {
+        if (rope.done || pq.done) {
         } else if (act)
             wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, c->seq_act, act_pos, c->rope_act, c->q, kc, vc, NA, Hq, 0,
                                    dh, S, Sp, batch, status, stream);
@@ -1466,21 +1490,39 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         WdTcEpi epi_o, epi_d;
         epi_o.resid = &resid_o;
         epi_d.resid = &resid_d;
-        if ((s = run_gemm(c, c->attn, &c->tc.x_map_attn, wo, 1, Rb, hq, c->part, c->part_floats, status, stream, &go, false, nullptr,
-                          nullptr, &epi_o)) != WD_OK)
+        WdTcSeg gu[2] = {{c->wg[l], F, c->tc.get(WD_TC_WG, l)}, {c->wu[l], F, c->tc.get(WD_TC_WU, l)}};
+        if (f32) {
+            po.epi = WD_PLAIN_ADD;
+            po.x = (const float*)c->attn; po.y = c->x; po.ldy = D;
+            if ((s = run_gemm(c, c->attn, nullptr, wo, 1, R_, hq, c->part, c->part_floats, status, stream, &go, false, nullptr, nullptr,
+                              nullptr, &po)) != WD_OK)
+                return s;
+        }
+        if (po.done) {
+            resid_o.done = true;
+            pg.epi = WD_PLAIN_SWIGLU;
+            pg.x = c->x; pg.gain = c->ffn_norm[l]; pg.eps = d.rms_eps;
+            pg.y = (float*)c->h; pg.ldy = pg.F = F;
+            if ((s = run_gemm(c, c->x, nullptr, gu, 2, R_, D, c->part, c->part_floats, status, stream, &go, false, nullptr, nullptr,
+                              nullptr, &pg)) != WD_OK)
+                return s;
+        } else if ((s = run_gemm(c, c->attn, &c->tc.x_map_attn, wo, 1, Rb, hq, c->part, c->part_floats, status, stream, &go, false, nullptr,
+                                 nullptr, &epi_o)) != WD_OK) {
             return s;
+        }
         // feed-forward half
-        wd_launch_rmsnorm(d.dtype, xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, xnb,
+        if (!pg.done)
+            wd_launch_rmsnorm(d.dtype, xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, xnb,
                           nullptr, Rb, D, stream, fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_d : nullptr);
         if (fp4) {
             if ((s = run_gemm_fp4(c, &c->f4gu[l], R_, D, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
             if ((s = wd_launch_swiglu_fp4(c->part, go.n_split, go.split_stride, &x4_f, R_, F, stream)) != WD_OK) return s;
             if ((s = run_gemm_fp4(c, &c->f4d[l], R_, F, c->part, c->part_floats, status, stream, &go)) != WD_OK) return s;
         } else if (fp8) {
-            WdTcSeg gu[2] = {{c->f8g[l].q, F, &c->f8g[l].map}, {c->f8u[l].q, F, &c->f8u[l].map}};
+            WdTcSeg gu8[2] = {{c->f8g[l].q, F, &c->f8g[l].map}, {c->f8u[l].q, F, &c->f8u[l].map}};
             WdTcFp8 f8;
             f8.sw[0] = c->f8g[l].s; f8.sw[1] = c->f8u[l].s; f8.sx = c->sxn;
-            if ((s = run_gemm(c, c->xn8, &c->x8_d, gu, 2, R_, D, c->part, c->part_floats, status, stream, &go, false, nullptr,
+            if ((s = run_gemm(c, c->xn8, &c->x8_d, gu8, 2, R_, D, c->part, c->part_floats, status, stream, &go, false, nullptr,
                               &f8)) != WD_OK)
                 return s;
             if ((s = wd_launch_swiglu_fp8(c->part, go.n_split, go.split_stride, c->h8, c->sh, R_, F, stream)) != WD_OK) return s;
@@ -1491,17 +1533,26 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                               &f8d)) != WD_OK)
                 return s;
         } else {
-        WdTcSeg gu[2] = {{c->wg[l], F, c->tc.get(WD_TC_WG, l)}, {c->wu[l], F, c->tc.get(WD_TC_WU, l)}};
         WdTcSwiglu sg;
         sg.h = use_tc(c) ? (__nv_bfloat16*)c->h : nullptr;
         WdTcEpi epi_sg;
         epi_sg.sg = &sg;
-        if ((s = run_gemm(c, xnb, xmb, gu, 2, Rb, D, c->part, c->part_floats, status, stream, &go, false,
-                          nullptr, nullptr, &epi_sg)) != WD_OK)
-            return s;
-        if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream);
+        if (!pg.done) {
+            if ((s = run_gemm(c, xnb, xmb, gu, 2, Rb, D, c->part, c->part_floats, status, stream, &go, false,
+                              nullptr, nullptr, &epi_sg)) != WD_OK)
+                return s;
+            if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream);
+        }
         WdTcSeg wdn[1] = {{c->wd[l], D, c->tc.get(WD_TC_WD, l)}};
-        if ((s = run_gemm(c, c->h, &c->tc.x_map_h, wdn, 1, Rb, F, c->part, c->part_floats, status, stream, &go, false, nullptr,
+        if (f32) {                      // (x is complete: the output projection or the RMSNorm after it has added its sums)
+            pd.epi = WD_PLAIN_ADD;
+            pd.x = (const float*)c->h; pd.y = c->x; pd.ldy = D;
+            if ((s = run_gemm(c, c->h, nullptr, wdn, 1, R_, F, c->part, c->part_floats, status, stream, &go, false, nullptr, nullptr,
+                              nullptr, &pd)) != WD_OK)
+                return s;
+        }
+        resid_d.done = pd.done;
+        if (!pd.done && (s = run_gemm(c, c->h, &c->tc.x_map_h, wdn, 1, Rb, F, c->part, c->part_floats, status, stream, &go, false, nullptr,
                           nullptr, &epi_d)) != WD_OK)
             return s;
         }
@@ -1520,11 +1571,20 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     bool lm_fused = false;
     int lm_chunks = wd_unmask_chunks(d.vocab);
     if (NA > 0) {
-        wd_launch_rmsnorm(d.dtype, act_last ? c->x_act : c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
-                          c->final_norm, d.rms_eps, c->xn, act_last ? nullptr : act_row, NA, D, stream,
-                          fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_lm : nullptr);
         float* logits = st->taps.logits ? st->taps.logits : c->logits;      // a tap takes them directly
         WdTcSeg lm[1] = {{c->lm_head, d.vocab, c->tc.get(WD_TC_LM, 0)}};
+        WdPlainFuse pl;
+        if (f32 && !down_pending) {
+            pl.x = c->x; pl.row_idx = act_row; pl.gain = c->final_norm; pl.eps = d.rms_eps;
+            pl.y = logits; pl.ldy = d.vocab;
+            if ((s = run_gemm(c, c->x, nullptr, lm, 1, NA, D, logits, (size_t)d.max_active * d.vocab, status, stream, &go, false, nullptr,
+                              nullptr, nullptr, &pl)) != WD_OK)
+                return s;
+        }
+        if (!pl.done)
+            wd_launch_rmsnorm(d.dtype, act_last ? c->x_act : c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
+                          c->final_norm, d.rms_eps, c->xn, act_last ? nullptr : act_row, NA, D, stream,
+                          fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_lm : nullptr);
         WdTcFp8 f8lm;
         if (fp8) {
             lm[0] = {c->f8lm.q, d.vocab, &c->f8lm.map};
@@ -1537,7 +1597,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         fl.st_max = c->ch_max; fl.st_idx = c->ch_idx; fl.st_sum = c->ch_sum;
         fl.write_logits = st->taps.logits ? 1 : 0;
         lm_fused = use_tc(c) && NA <= 1024 && c->sm_count % 4 == 0 && !fp4;     // one CTA group per tile of <= 256 active rows
-        if (fp4) {
+        if (pl.done) {
+        } else if (fp4) {
             if ((s = run_gemm_fp4(c, &c->f4lm, NA, D, logits, (size_t)d.max_active * d.vocab, status, stream, &go,
                                   /*single_split=*/true)) != WD_OK)
                 return s;

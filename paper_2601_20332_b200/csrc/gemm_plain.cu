@@ -71,29 +71,90 @@ __device__ __forceinline__ float4 ld_row4(const T* p, int kk, int k) {
 // first NC * 128 elements are in registers before the dependency wait.  Bound by latency up to about a hundred rows, then by
 // the loads from L1 (17 TFLOP/s).  Measured, 768 columns, k = 256: 2.3 us at 9 rows, 2.9 at 64; a [32 x 64]-tile kernel with
 // K tiles of 32 through shared memory, a barrier on either side of each, took 19 us at 9 rows.
-template <typename T, int NC, bool kVec>
+//
+// kEpi and kNorm (WdPlainFuse) take the kernels on either side of a projection in, each of which is another link of 2-3 us in the
+// step's chain however little it does:
+//   kNorm    RMSNorm of the rows: their gains are multiplied into the weights before the dependency wait, the sum of squares of a
+//            row is reduced like the products (the lane that ends up with a row's result has that row's sum too), and 1 / rms is
+//            applied to the finished sums
+//   kEpiQkv  a warp's four columns are two rotation pairs of a q or k head (or four dims of a v head): rotated and written to q and
+//            the cache.  kEpiSwiglu: two gate and the two up columns that belong to them.  kEpiAdd: added to y.
+// Measured, normal step of the fp32 model (two blocks of 256 / 688, 9 rows): 24 launches and 75 us with separate kernels, 15 and 52 us
+// with these; a projection with its neighbours in it takes 2.1-2.9 us where the three kernels took 5.5 together.
+enum { kEpiNone = 0, kEpiQkv = 1, kEpiSwiglu = 2, kEpiAdd = 3 };
+template <int kEpi, bool kNorm> struct RowsArgs { WdPlainFuse f; };
+template <> struct RowsArgs<kEpiNone, false> {};
+
+// output column (of the concatenated matrices) that a warp of column group g computes as its c-th
+template <int kEpi>
+__device__ __forceinline__ int group_col(const WdPlainFuse& f, int g, int c) {
+    if (kEpi == kEpiSwiglu) return 2 * g + (c & 1) + (c >> 1) * f.F;
+    if (kEpi == kEpiQkv) {
+        const int half = f.dh >> 1, rotated = (f.Hq + f.Hkv) * (half >> 1);     // groups of rotation pairs
+        if (g < rotated) {
+            const int h = g / (half >> 1);
+            return h * f.dh + 2 * (g - h * (half >> 1)) + (c & 1) + (c >> 1) * half;
+        }
+        return (f.Hq + f.Hkv) * f.dh + 4 * (g - rotated) + c;
+    }
+    return 4 * g + c;
+}
+
+template <typename T, int kR, int NC, bool kVec, int kEpi = kEpiNone, bool kNorm = false>
 __global__ void __launch_bounds__(128)
-gemm_rows_kernel(const T* __restrict__ x, const Segs segs, float* __restrict__ y, int rows, int n, int k, int ldy, int w_static) {
-    constexpr int kC = 4, kR = 8;
+gemm_rows_kernel(const T* __restrict__ x, const Segs segs, float* __restrict__ y, int rows, int n, int k, int ldy, int w_static,
+                 const RowsArgs<kEpi, kNorm> ra) {
+    constexpr int kC = 4, kV = kR * kC, kDup = 32 / kV;      // sums of a warp, lanes that end up with the same one
+    constexpr bool kFused = kEpi != kEpiNone || kNorm;
+    WdPlainFuse f;
+    if constexpr (kFused) f = ra.f;
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31, col0 = (int)(blockIdx.x * 4 + (threadIdx.x >> 5)) * kC, row0 = (int)blockIdx.y * kR;
-    if (col0 >= n) return;
+    const int lane = threadIdx.x & 31, group = (int)(blockIdx.x * 4 + (threadIdx.x >> 5)), row0 = (int)blockIdx.y * kR;
+    if (group * kC >= n) return;
     const T* wp[kC];
 #pragma unroll
-    for (int c = 0; c < kC; ++c) wp[c] = weight_row<T>(segs, min(col0 + c, n - 1), k);
+    for (int c = 0; c < kC; ++c) wp[c] = weight_row<T>(segs, min(group_col<kEpi>(f, group, c), n - 1), k);
     float4 w[NC][kC];
     auto load_w = [&](int kb) {
 #pragma unroll
         for (int i = 0; i < NC; ++i)
 #pragma unroll
             for (int c = 0; c < kC; ++c) w[i][c] = ld_row4<T, kVec>(wp[c], kb + 128 * i + 4 * lane, k);
+        if (kNorm) {
+#pragma unroll
+            for (int i = 0; i < NC; ++i) {
+                const float4 g = ld_row4<float, true>(f.gain, kb + 128 * i + 4 * lane, k);
+#pragma unroll
+                for (int c = 0; c < kC; ++c) w[i][c] = make_float4(w[i][c].x * g.x, w[i][c].y * g.y, w[i][c].z * g.z, w[i][c].w * g.w);
+            }
+        }
     };
     if (!w_static) pdl_wait();
     load_w(0);
     if (w_static) pdl_wait();
-    float acc[kR * kC];
+    // this lane's result, and what its epilogue needs beside the product
+    const int own = lane / kDup, r = row0 + (own >> 2), c = group_col<kEpi>(f, group, own & 3);
+    const bool mine = r < rows && c < n && lane % kDup == 0;
+    float2 cs = make_float2(1.f, 0.f);
+    float old = 0.f;
+    int pos = 0, seq = 0;
+    if (kEpi == kEpiQkv && mine) {
+        pos = f.row_pos[r];
+        seq = f.row_seq[r];
+        if (c < (f.Hq + f.Hkv) * f.dh) cs = f.rope_tab[(size_t)r * (f.dh >> 1) + c % (f.dh >> 1)];
+    }
+    if (kEpi == kEpiAdd) old = Raw<float>::value(Raw<float>::load(y + (size_t)r * ldy + c, mine));
+    const T* xp[kR];
+#pragma unroll
+    for (int i = 0; i < kR; ++i) {
+        const int row = min(row0 + i, rows - 1);
+        xp[i] = x + (size_t)(kNorm && f.row_idx ? f.row_idx[row] : row) * k;
+    }
+    float acc[kR * kC], ss[kR];
 #pragma unroll
     for (int i = 0; i < kR * kC; ++i) acc[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < kR; ++i) ss[i] = 0.f;
     for (int kb = 0; kb < k; kb += 128 * NC) {
         if (kb > 0) load_w(kb);
 #pragma unroll
@@ -101,31 +162,68 @@ gemm_rows_kernel(const T* __restrict__ x, const Segs segs, float* __restrict__ y
             const int kk = kb + 128 * i + 4 * lane;
             float4 xv[kR];
 #pragma unroll
-            for (int r = 0; r < kR; ++r) xv[r] = ld_row4<T, kVec>(x + (size_t)min(row0 + r, rows - 1) * k, kk, k);
+            for (int rr = 0; rr < kR; ++rr) xv[rr] = ld_row4<T, kVec>(xp[rr], kk, k);
 #pragma unroll
-            for (int r = 0; r < kR; ++r)
+            for (int rr = 0; rr < kR; ++rr) {
+                if (kNorm) ss[rr] = fmaf(xv[rr].x, xv[rr].x, fmaf(xv[rr].y, xv[rr].y, fmaf(xv[rr].z, xv[rr].z, fmaf(xv[rr].w, xv[rr].w, ss[rr]))));
 #pragma unroll
-                for (int c = 0; c < kC; ++c) {
-                    float& a = acc[r * kC + c];
-                    a = fmaf(xv[r].x, w[i][c].x, a);
-                    a = fmaf(xv[r].y, w[i][c].y, a);
-                    a = fmaf(xv[r].z, w[i][c].z, a);
-                    a = fmaf(xv[r].w, w[i][c].w, a);
+                for (int cc = 0; cc < kC; ++cc) {
+                    float& a = acc[rr * kC + cc];
+                    a = fmaf(xv[rr].x, w[i][cc].x, a);
+                    a = fmaf(xv[rr].y, w[i][cc].y, a);
+                    a = fmaf(xv[rr].z, w[i][cc].z, a);
+                    a = fmaf(xv[rr].w, w[i][cc].w, a);
                 }
+            }
         }
     }
-    // after the step over lane bit b a lane keeps the values whose index has bit b equal to its own
+    // after the step over lane bit b a lane keeps the values whose index has that bit equal to its own, while there is more than one
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int step = 0; step < 5; ++step) {
+        const int o = 16 >> step, nv = kV >> (step + 1), ns = kR >> (step + 1);
         const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int i = 0; i < o; ++i) {
-            const float send = up ? acc[i] : acc[i + o], keep = up ? acc[i + o] : acc[i];
+        for (int i = 0; i < kV / 2; ++i) {
+            if (i >= nv) break;
+            const float send = up ? acc[i] : acc[i + nv], keep = up ? acc[i + nv] : acc[i];
             acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
+        if (nv == 0) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+        if (kNorm) {
+#pragma unroll
+            for (int i = 0; i < kR / 2; ++i) {
+                if (i >= ns) break;
+                const float send = up ? ss[i] : ss[i + ns], keep = up ? ss[i + ns] : ss[i];
+                ss[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+            if (ns == 0) ss[0] += __shfl_xor_sync(0xffffffffu, ss[0], o);
+        }
     }
-    const int r = row0 + (lane >> 2), c = col0 + (lane & 3);
-    if (r < rows && c < n) y[(size_t)r * ldy + c] = acc[0];
+    float v = acc[0];
+    if (kNorm) v *= rsqrtf(ss[0] / (float)k + f.eps);
+    if constexpr (kEpi == kEpiQkv) {
+        const float other = __shfl_xor_sync(0xffffffffu, v, 2 * kDup);         // the partner of a rotation pair
+        if (!mine) return;
+        const int h = c / f.dh, j = c - h * f.dh;
+        if (h < f.Hq + f.Hkv) v = v * cs.x + ((own & 2) ? other : -other) * cs.y;
+        if (h < f.Hq) {
+            f.q[(size_t)r * f.Hq * f.dh + c] = v;
+            return;
+        }
+        // index check: a cache row outside the state is recorded and not written
+        if ((unsigned)pos >= (unsigned)f.S || (unsigned)seq >= (unsigned)f.batch) {
+            atomicCAS(f.status, 0, WD_ERR_BOUNDS);
+            return;
+        }
+        const int kh = h < f.Hq + f.Hkv ? h - f.Hq : h - f.Hq - f.Hkv;
+        if (h < f.Hq + f.Hkv) f.kcache[(((size_t)seq * f.Hkv + kh) * f.S + pos) * f.dh + j] = v;
+        else f.vcache[(((size_t)seq * f.Hkv + kh) * f.dh + j) * f.Sp + pos] = v;
+    } else if constexpr (kEpi == kEpiSwiglu) {
+        const float up = __shfl_xor_sync(0xffffffffu, v, 2 * kDup);
+        if (mine && !(own & 2)) y[(size_t)r * ldy + c] = v / (1.f + __expf(-v)) * up;
+    } else {
+        if (mine) y[(size_t)r * ldy + c] = kEpi == kEpiAdd ? old + v : v;
+    }
 }
 
 // Many rows: [128 x 64] tiles, 256 threads with 8 x 4 results each (bound by the multiply-adds then: 12 shared-memory loads of
@@ -253,10 +351,26 @@ void launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaS
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-template <typename T, bool kVec>
-void launch_rows(const void* x, const Segs& segs, float* y, int rows, int n, int k, int ldy, bool w_static, cudaStream_t st) {
-    launch(k <= 256 ? gemm_rows_kernel<T, 2, kVec> : gemm_rows_kernel<T, 3, kVec>,
-           dim3((unsigned)wd_ceil_div(n, 16), (unsigned)wd_ceil_div(rows, 8)), 128, 0, st, (const T*)x, segs, y, rows, n, k, ldy, w_static ? 1 : 0);
+constexpr int kFusedBlocks = 9 * 148;       // see wd_launch_gemm_plain_fused
+
+template <typename T, bool kVec, int kEpi = kEpiNone, bool kNorm = false>
+void launch_rows(const void* x, const Segs& segs, float* y, int rows, int n, int k, int ldy, bool w_static, cudaStream_t st,
+                 const RowsArgs<kEpi, kNorm>& ra = {}) {
+    auto kernel = k <= 256 ? gemm_rows_kernel<T, 8, 2, kVec, kEpi, kNorm> : gemm_rows_kernel<T, 8, 3, kVec, kEpi, kNorm>;
+    int r = 8;
+    if constexpr (kEpi != kEpiNone || kNorm) {
+        // Four rows to a warp while the grid stays small (nine rows waste less, and each warp has half the loads and sums in its
+        // chain); then also the whole of k up to 768 in one go, one round trip instead of two.  Step of the fp32 model, two blocks of
+        // 256 / 688: 9 rows 63 -> 52 us, 40 81 -> 72, 72 98 -> 89; with 13 blocks to an SM instead of nine 96.  (The add after a
+        // short k is the exception: eight rows 2.3 us, four 3.7, always; not understood.)
+        if (!(kEpi == kEpiAdd && k <= 256) && (long long)wd_ceil_div(n, 16) * wd_ceil_div(rows, 4) <= kFusedBlocks) {
+            r = 4;
+            kernel = k <= 256 ? gemm_rows_kernel<T, 4, 2, kVec, kEpi, kNorm>
+                              : k <= 768 ? gemm_rows_kernel<T, 4, 6, kVec, kEpi, kNorm> : gemm_rows_kernel<T, 4, 3, kVec, kEpi, kNorm>;
+        }
+    }
+    launch(kernel, dim3((unsigned)wd_ceil_div(n, 16), (unsigned)wd_ceil_div(rows, r)), 128, 0, st, (const T*)x, segs, y, rows, n, k, ldy,
+           w_static ? 1 : 0, ra);
 }
 
 template <typename T, bool kAsync>
@@ -272,6 +386,35 @@ void launch_tiles(const void* x, const Segs& segs, float* y, int rows, int n, in
            (const T*)x, segs, y, rows, n, k, ldy);
 }
 
+// Tiles when the rows kernel would take longer: it works at 16 TFLOP/s in fp32 (8 where rows are not aligned) and at 15 (10)
+// in bf16, 20 (14.5) from k = 257 on, three loads in flight instead of two; a tile takes 0.85 us (1.05 through registers) of
+// its SM per 16 of K, and a lone one 0.4 more.  Measured, rows / tiles / the [32 x 64]-tile kernel before either, in us: fp32
+// 130 x 8000 k = 688 84 / 77 / 138; 520 x 2048, k = 256 33 / 29 / 51; k = 255 1024 x 2048 131 / 38 / 65, 130 x 8000 68 / 36 / 53,
+// 34 x 8000 18 / 22 / 28; bf16 2048 x 2048, k = 256 130 / 72 / 120, k = 255 201 / 72 / 120, 300 x 2048, k = 687 60 / 69 / 100.
+// In a step the rows kernel also has its weights before the previous kernel ends, about 5 us of a launch (528 rows, gate/up
+// of 2 x 688, k = 256, alike alone: normal step of the fp32 model 319 us, with tiles 332).
+bool tiles_pay(bool f32, bool vec, int rows, int n, int k, bool w_static) {
+    const double rate = f32 ? (vec ? 16.0 : 8.0) : k <= 256 ? (vec ? 15.0 : 10.0) : (vec ? 20.0 : 14.5);
+    const long long n_tiles = (long long)wd_ceil_div(n, kTileC) * wd_ceil_div(rows, kTileR);
+    const double us_rows = 2e-6 * rows * n * k / rate;
+    const double us_tiles = wd_ceil_div(k, kTileK) * (0.4 + (f32 && vec ? 0.85 : 1.05) * (double)((n_tiles + 147) / 148));
+    return us_tiles + (w_static ? 5.0 : 0.0) < us_rows;
+}
+
+// the matrices side by side; false unless rows of k elements can be read four at a time
+bool make_segs(const void* x, const void* const* w, const int* n, int n_mat, int k, Segs* segs, int* n_all) {
+    int end = 0;
+    bool vec = k % 4 == 0 && (uintptr_t)x % 16 == 0;
+    for (int i = 0; i < 3; ++i) {
+        segs->w[i] = w[i < n_mat ? i : n_mat - 1];
+        if (i < n_mat) end += n[i];
+        segs->end[i] = end;
+        vec = vec && (uintptr_t)segs->w[i] % 16 == 0;
+    }
+    *n_all = end;
+    return vec;
+}
+
 }  // namespace
 
 void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const int* n, int n_mat, float* y, int rows, int k,
@@ -279,13 +422,7 @@ void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const 
     if (rows <= 0 || n_mat < 1 || n_mat > 3) return;
     Segs segs;
     int end = 0;
-    bool vec = k % 4 == 0 && (uintptr_t)x % 16 == 0;
-    for (int i = 0; i < 3; ++i) {
-        segs.w[i] = w[i < n_mat ? i : n_mat - 1];
-        if (i < n_mat) end += n[i];
-        segs.end[i] = end;
-        vec = vec && (uintptr_t)segs.w[i] % 16 == 0;
-    }
+    const bool vec = make_segs(x, w, n, n_mat, k, &segs, &end);
     if (end <= 0) return;
     constexpr int kMostRows = 65535 * 8;        // of one launch (a grid holds 65535 blocks in y)
     if (rows > kMostRows) {
@@ -296,19 +433,7 @@ void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const 
             if (rows - r0 <= kMostRows) return;
         }
     }
-    // Tiles when the rows kernel would take longer: it works at 16 TFLOP/s in fp32 (8 where rows are not aligned) and at 15 (10)
-    // in bf16, 20 (14.5) from k = 257 on, three loads in flight instead of two; a tile takes 0.85 us (1.05 through registers) of
-    // its SM per 16 of K, and a lone one 0.4 more.  Measured, rows / tiles / the [32 x 64]-tile kernel before either, in us: fp32
-    // 130 x 8000 k = 688 84 / 77 / 138; 520 x 2048, k = 256 33 / 29 / 51; k = 255 1024 x 2048 131 / 38 / 65, 130 x 8000 68 / 36 / 53,
-    // 34 x 8000 18 / 22 / 28; bf16 2048 x 2048, k = 256 130 / 72 / 120, k = 255 201 / 72 / 120, 300 x 2048, k = 687 60 / 69 / 100.
-    // In a step the rows kernel also has its weights before the previous kernel ends, about 5 us of a launch (528 rows, gate/up
-    // of 2 x 688, k = 256, alike alone: normal step of the fp32 model 319 us, with tiles 332).
-    const bool f32 = dtype == WD_F32;
-    const double rate = f32 ? (vec ? 16.0 : 8.0) : k <= 256 ? (vec ? 15.0 : 10.0) : (vec ? 20.0 : 14.5);
-    const long long n_tiles = (long long)wd_ceil_div(end, kTileC) * wd_ceil_div(rows, kTileR);
-    const double us_rows = 2e-6 * rows * end * k / rate;
-    const double us_tiles = wd_ceil_div(k, kTileK) * (0.4 + (f32 && vec ? 0.85 : 1.05) * (double)((n_tiles + 147) / 148));
-    const bool tiles = us_tiles + (w_static ? 5.0 : 0.0) < us_rows;
+    const bool f32 = dtype == WD_F32, tiles = tiles_pay(f32, vec, rows, end, k, w_static);
     if (dtype == WD_F32) {
         if (tiles && vec) launch_tiles<float, true>(x, segs, y, rows, end, k, ldy, st);
         else if (tiles) launch_tiles<float, false>(x, segs, y, rows, end, k, ldy, st);
@@ -319,4 +444,35 @@ void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const 
         else if (vec) launch_rows<__nv_bfloat16, true>(x, segs, y, rows, end, k, ldy, w_static, st);
         else launch_rows<__nv_bfloat16, false>(x, segs, y, rows, end, k, ldy, w_static, st);
     }
+}
+
+bool wd_launch_gemm_plain_fused(const WdPlainFuse& f, const void* const* w, const int* n, int n_mat, int rows, int k, cudaStream_t st) {
+    if (!f.x || rows < 1 || n_mat < 1 || n_mat > 3) return false;
+    Segs segs;
+    int end = 0;
+    const bool vec = make_segs(f.x, w, n, n_mat, k, &segs, &end) && (uintptr_t)f.gain % 16 == 0;
+    // While the step is a chain of latencies: up to nine blocks of the eight-row form to an SM.  Beyond, the sums of squares taken
+    // again by every group of columns cost more than the launches saved (step of the fp32 model: 300 rows 187 us with separate
+    // kernels, 201 without this limit; 120 rows 101 and 99; 56 rows 75 and 64; 9 rows 74 and 52).
+    if (!vec || end < 4 || end % 4 || (long long)wd_ceil_div(end, 16) * wd_ceil_div(rows, 8) > kFusedBlocks ||
+        tiles_pay(true, true, rows, end, k, true))
+        return false;
+    switch (f.epi) {
+        case WD_PLAIN_STORE:
+            if (f.gain) launch_rows<float, true, kEpiNone, true>(f.x, segs, f.y, rows, end, k, f.ldy, true, st, {f});
+            return f.gain != nullptr;
+        case WD_PLAIN_QKV:
+            if (!f.gain || f.dh % 4) return false;
+            launch_rows<float, true, kEpiQkv, true>(f.x, segs, nullptr, rows, end, k, 0, true, st, {f});
+            return true;
+        case WD_PLAIN_SWIGLU:
+            if (!f.gain || f.F % 2 || end != 2 * f.F) return false;
+            launch_rows<float, true, kEpiSwiglu, true>(f.x, segs, f.y, rows, end, k, f.ldy, true, st, {f});
+            return true;
+        case WD_PLAIN_ADD:
+            if (f.gain) return false;
+            launch_rows<float, true, kEpiAdd, false>(f.x, segs, f.y, rows, end, k, f.ldy, true, st, {f});
+            return true;
+    }
+    return false;
 }

@@ -117,6 +117,30 @@ void wd_launch_rmsnorm(int dtype, float* x, const float* part, int n_split, size
 void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const int* n, int n_mat, float* y, int rows, int k,
                           int ldy, bool w_static, cudaStream_t st);
 
+// The same for few fp32 rows with the kernels on either side of the projection in it: RMSNorm of the rows (gain != null; with
+// row_idx the rows x[row_idx[i]]), and one of the epilogues below.  Returns false, with nothing launched, where the rows kernel
+// does not apply (alignment, many rows).  The weights are complete before the previous kernel of the stream started.
+enum { WD_PLAIN_STORE = 0,      // y = product
+       WD_PLAIN_QKV = 1,        // RoPE -> q and the K/V cache rows (as wd_launch_rope_scatter); y is not written
+       WD_PLAIN_SWIGLU = 2,     // w = [gate; up]: y[rows, F] = silu(gate) * up
+       WD_PLAIN_ADD = 3 };      // y += product
+struct WdPlainFuse {
+    int epi = WD_PLAIN_STORE;
+    bool done = false;              // (the callers' note that it was launched)
+    const float* x = nullptr;
+    float* y = nullptr;
+    int ldy = 0;
+    const float* gain = nullptr;
+    float eps = 0.f;
+    const int32_t* row_idx = nullptr;
+    const int32_t *row_seq = nullptr, *row_pos = nullptr;
+    const float2* rope_tab = nullptr;
+    float *q = nullptr, *kcache = nullptr, *vcache = nullptr;
+    int Hq = 0, Hkv = 0, dh = 0, S = 0, Sp = 0, batch = 0, F = 0;
+    int32_t* status = nullptr;
+};
+bool wd_launch_gemm_plain_fused(const WdPlainFuse& f, const void* const* w, const int* n, int n_mat, int rows, int k, cudaStream_t st);
+
 // qkv partials -> RoPE -> q (dtype) and K/V cache rows.
 //   part: [n_split][n_rows][(Hq+2Hkv)*dh] float, columns = [q | k | v]
 //   kcache: [batch][Hkv][S][dh]; vcache: [batch][Hkv][dh][Sp] (this layer's slices)

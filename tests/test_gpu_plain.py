@@ -102,3 +102,23 @@ def test_fp32_steps_replayed_from_graphs():
         ctx.close()
     assert np.array_equal(runs[0][0], runs[1][0])
     assert runs[0][1] == (0, 0) and runs[1][1][1] > 15
+
+
+# fp32 steps with the element-wise kernels inside the projections (few rows) and beside them, against the float64 oracle: refresh
+# and normal steps of one row to a few hundred, on either side of the four-row form's, the eight-row form's and the tiles' limits;
+# grouped heads, rotation pairs that do not fill a group of columns' block, head_dim not a multiple of 4 (separate kernels),
+# reduction lengths below one load, of one and of several blocks.  1e-5: rounding of fp32 sums over up to 900 terms, two blocks deep.
+@pytest.mark.parametrize("over,batch,P,A,B", [
+    (dict(), 1, 1, 1, 2), (dict(Hkv=2), 2, 33, 5, 7), (dict(), 1, 60, 24, 1), (dict(d=100, Hq=5, Hkv=1, dh=12, F=36, V=257), 3, 19, 4, 3),
+    (dict(d=64, Hq=3, Hkv=3, dh=6, F=900, V=130), 1, 40, 9, 4), (dict(d=900, Hq=2, Hkv=1, dh=36, F=772, V=300), 1, 9, 3, 2),
+    (dict(), 2, 120, 16, 40)])
+def test_fused_rows_steps(over, batch, P, A, B):
+    from wd_harness import Parity
+    cfg = synth.get_config("tiny", **over)
+    ids = synth.make_prompts(cfg, batch=batch, P=P, G=A + B + 6)
+    p = Parity(cfg, synth.make_weights(cfg, DEV, gain_jitter=0.1), ids)
+    for _ in range(4):
+        r = p.step(A, B, 3, 2, 1, tol_layer=1e-5, tol_attn=1e-5)
+        assert r["worst"]["logits"] <= 1e-5
+    p.check_state_mirror()
+    p.close()
