@@ -108,8 +108,8 @@ struct wd_ctx {
     int fuse = WD_FUSION_AUTO;   // where the consumers of the GEMMs run (wd_set_fusion)
     int32_t* plan = nullptr;     // packed index lists of the step
     size_t plan_ints = 0;
-    int32_t* result = nullptr;   // [status | n_sel[batch] | pos | tok | conf]
-    size_t result_ints = 0;
+    int32_t* status = nullptr;   // status word of the steps
+    size_t result_ints = 0;      // of a step's block in a state's ring: [status | n_sel[batch] | pos | tok | conf]
 
     WdTcWeights tc;              // tensor maps of the weights (bf16 only)
     WdAttnQ attn_q;
@@ -197,10 +197,10 @@ static void carve_ctx(const wd_model_dims* d, Carve& c, size_t off[28]) {
     off[8] = c.take(MA * 8);                                    // row_sumexp
     off[9] = c.take(MA * 4);                                    // row_conf
     const size_t plan_ints = 2 * MR + 2 * MA + 4 * ((size_t)d->max_batch + 1) + (size_t)d->max_batch * d->max_seq +
-                             3 * (MR / 128 + (size_t)d->max_batch + 1) + 3 * (MA / 128 + (size_t)d->max_batch + 1) + 2 * (size_t)d->max_batch +
+                             3 * (MR / 128 + (size_t)d->max_batch + 1) + 3 * (MA / 128 + (size_t)d->max_batch + 1) + 2 * (size_t)d->max_batch + 1 +
                              (size_t)d->max_batch * d->max_seq;      // + staging of the external windows
     off[10] = c.take(plan_ints * 4);                            // plan
-    off[11] = c.take((1 + (size_t)d->max_batch + 3 * MA) * 4);  // result
+    off[11] = c.take(4);                                        // status
     off[12] = plan_ints;
     // unmask statistics: per vocabulary chunk (CUDA-core path) or per 128-logit GEMM tile (LM-head epilogue)
     const size_t nch = std::max<size_t>((size_t)wd_unmask_chunks(d->vocab), 256);   // or one per CTA of the LM head
@@ -301,7 +301,7 @@ extern "C" wd_status wd_create(const wd_model_dims* dims, const wd_weights* w, v
     c->row_conf = (float*)(base + off[9]);
     c->plan = (int32_t*)(base + off[10]);
     c->plan_ints = off[12];
-    c->result = (int32_t*)(base + off[11]);
+    c->status = (int32_t*)(base + off[11]);
     c->result_ints = 1 + (size_t)dims->max_batch + 3 * (size_t)dims->max_active;
     c->ch_max = (float*)(base + off[13]);
     c->ch_idx = (int32_t*)(base + off[14]);
@@ -313,7 +313,7 @@ extern "C" wd_status wd_create(const wd_model_dims* dims, const wd_weights* w, v
     WD_CUDA_TRY(cudaMemset(c->tile_counters, 0, c->n_tile_counters * 4));
     c->chain.ready_dev = (int32_t*)(base + off[20]);
     WD_CUDA_TRY(cudaMemset(c->chain.ready_dev, 0, 256));
-    WD_CUDA_TRY(cudaMemset(c->result, 0, 4));
+    WD_CUDA_TRY(cudaMemset(c->status, 0, 4));
 
     if (dims->dtype == WD_BF16) {
         wd_status s = wd_tc_weights_init(&c->tc, dims, c->tok_embed, c->lm_head, c->wq, c->wk, c->wv, c->wo,
@@ -703,6 +703,10 @@ extern "C" wd_status wd_state_reset(wd_state* st, const int32_t* token_ids, cons
         if (token_ids[i] < 0 || token_ids[i] >= st->ctx->d.vocab) return WD_ERR_BAD_PARAM;
     // the pinned staging buffers may still be the source of an earlier reset's copies
     if (st->staged_recorded) WD_CUDA_TRY(cudaEventSynchronize(st->staged));
+    // Launch configurations met once are counted within a generation.  Counted across resets, every refresh step of a second request
+    // of the same lengths was recorded, replayed once and pushed out again: 17 of 230 us each in 64 steps of the small fp32 model.
+    std::vector<wd_ctx::StepKey>& seen = st->ctx->seen;
+    seen.erase(std::remove_if(seen.begin(), seen.end(), [&](const wd_ctx::StepKey& k) { return k.state_uid == st->uid; }), seen.end());
     load_host_mirror(st, token_ids, decoded);
     st->poisoned = false;
     WD_CUDA_TRY(upload_plan_state(st, (cudaStream_t)stream));
@@ -1164,8 +1168,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     const size_t o_aqt_n = o; o += n_aqt;
     const size_t o_aqt_off = o; o += batch + 1;
     const size_t o_tseq = o; o += batch;          // step index of each sequence (for the decode-step stamps)
+    const size_t o_slot = o; o += 1;              // the result ring's block of this step
     const size_t o_vis_idx = o; o += n_vis;       // last: every other offset depends on rows, active rows and tiles only
     if (o > c->plan_ints) return WD_ERR_CAPACITY;
+    const int slot = (int)st->queue.size();
     if (dev_mode) {
         // the device builds the lists; the host passes counts and offsets as kernel arguments
         WdPlanLaunch pl;
@@ -1193,7 +1199,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         pl.qt_seq = c->plan + o_qt_seq; pl.qt_row0 = c->plan + o_qt_row0; pl.qt_n = c->plan + o_qt_n;
         pl.nvis_dev = c->plan + o_nvis; pl.tseq_dev = c->plan + o_tseq;
         pl.qt_off_dev = c->plan + o_qt_off;
-        pl.status = c->result;
+        pl.slot = slot; pl.slot_dev = c->plan + o_slot;
+        pl.status = c->status;
         wd_launch_plan(pl, stream);
     } else {
         size_t r = 0, a = 0, v = 0, qt = 0, aqt = 0;
@@ -1231,6 +1238,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             v += p.vis.size();
         }
         ph[o_act_off + batch] = (int32_t)a;
+        ph[o_slot] = slot;
         ph[o_qt_off + batch] = (int32_t)qt;
         ph[o_aqt_off + batch] = (int32_t)aqt;
         ph[o_vis_off + batch] = (int32_t)v;
@@ -1255,7 +1263,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     const int32_t* act_off = c->plan + o_act_off;
     const int32_t* vis_off = c->plan + o_vis_off;
     const int32_t* vis_idx = c->plan + o_vis_idx;
-    int32_t* status = c->result;
+    int32_t* status = c->status;
 
     const int R_ = (int)n_rows, NA = (int)n_act;
     const int Hq = d.n_q_heads, Hkv = d.n_kv_heads, dh = d.head_dim, D = d.d_model, F = d.d_ffn;
@@ -1317,7 +1325,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     const bool act_last = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN && !fp8 && !fp4 && !fused &&
                           d.n_layers > 1 && NA > 0 && R_ > 256 && 2 * NA <= R_ && !st->taps.layer_out && !st->taps.attn_out;
     // ---- the kernels of the step, from the embedding to the selection (everything after the planner and
-    // before the copy of the result block); launched directly, or recorded into a CUDA graph and replayed
+    // before the event that a sync waits for); launched directly, or recorded into a CUDA graph and replayed
     auto run_kernels = [&]() -> wd_status {
     c->tc.x_map_attn.smem_cap = 0;          // set per block below, and only beside the single-key-tile attention
     bool down_pending = false;          // x still lacks the previous block's FFN output (partial sums in part)
@@ -1609,13 +1617,11 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         if (lm_fused) lm_chunks = fl.n_chunks;
         else wd_launch_rowstats(logits, NA, d.vocab, c->ch_max, c->ch_idx, c->ch_sum, stream);
     }
-    int32_t* n_sel = c->result + 1;
-    int32_t* sel_pos = n_sel + batch;
-    int32_t* sel_tok = sel_pos + (size_t)batch * std::max(k_eff, 1);
-    float* sel_conf = (float*)(sel_tok + (size_t)batch * std::max(k_eff, 1));
+    // the results go straight to the step's block of the host's ring
     wd_launch_select(c->ch_max, c->ch_idx, c->ch_sum, lm_chunks, c->row_token, c->row_sumexp, act_pos,
-                     act_off, 0, batch, k_eff, st->ids_dev, S, n_sel, sel_pos, sel_tok, sel_conf, c->row_conf,
-                     st->decoded_dev, st->dec_step_dev, c->plan + o_tseq, stream);
+                     act_off, 0, batch, k_eff, st->ids_dev, S, nullptr, nullptr, nullptr, nullptr, c->row_conf,
+                     st->decoded_dev, st->dec_step_dev, c->plan + o_tseq, stream, st->result_host, (int)st->result_slot_ints,
+                     c->plan + o_slot, status);
     return WD_OK;
     };
     // A device-planned step whose launch configuration has occurred before is replayed from a graph: the
@@ -1714,10 +1720,6 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         }
     }
     if (!graphed && (s = run_kernels()) != WD_OK) return s;
-    // this step's result block goes to its own slot of the pinned ring
-    const size_t res_ints = 1 + (size_t)batch + 3 * (size_t)batch * std::max(k_eff, 1);
-    int32_t* slot = st->result_host + st->queue.size() * st->result_slot_ints;
-    WD_CUDA_TRY(cudaMemcpyAsync(slot, c->result, res_ints * 4, cudaMemcpyDeviceToHost, stream));
     WD_CUDA_TRY(cudaEventRecord(st->done, stream));
     WD_CUDA_TRY(cudaGetLastError());
     if (!dev_mode) pend.plans = st->plans;
@@ -1757,7 +1759,7 @@ static wd_status drain_queue(wd_state* st, wd_step_out* outs, bool every_step, i
         const int32_t* tok = pos + (size_t)batch * kk;
         const float* conf = (const float*)(tok + (size_t)batch * kk);
         if (res[0] != 0) {
-            cudaMemset(st->ctx->result, 0, 4);
+            cudaMemset(st->ctx->status, 0, 4);
             result = res[0] == WD_ERR_DEVICE_TIMEOUT ? WD_ERR_DEVICE_TIMEOUT : WD_ERR_BOUNDS;
             break;
         }

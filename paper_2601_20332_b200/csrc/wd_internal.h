@@ -196,7 +196,10 @@ void wd_launch_select(const float* ch_max, const int32_t* ch_idx, const double* 
                       int32_t* row_token, double* row_sumexp, const int32_t* act_pos, const int32_t* act_off,
                       int n_single, int batch, int k, int32_t* ids, int S, int32_t* n_sel, int32_t* sel_pos,
                       int32_t* sel_token, float* sel_conf, float* row_conf, uint8_t* decoded, int32_t* dec_step,
-                      const int32_t* step_of_seq, cudaStream_t st);
+                      const int32_t* step_of_seq, cudaStream_t st, int32_t* slots = nullptr, int slot_ints = 0,
+                      const int32_t* slot = nullptr, const int32_t* status = nullptr);
+// (slots != null: n_sel, positions, tokens and confidences go to block *slot of the ring at slots, slot_ints ints a block, behind the
+//  status word read from *status; n_sel, sel_* are then not used)
 
 // Device-side planner (one block per sequence): builds the step's index lists from the device
 // copy of the state; the host supplies counts and offsets only.  Up to WD_PLAN_MAX_BATCH sequences.
@@ -215,6 +218,8 @@ struct WdPlanLaunch {
         *tseq_dev, *qt_off_dev;
     int32_t aqt_off[WD_PLAN_MAX_BATCH + 1];                      // query tiles over the active rows alone
     int32_t *aqt_seq, *aqt_row0, *aqt_n, *aqt_off_dev;
+    int32_t slot;                 // block of the result ring that this step's results go to
+    int32_t* slot_dev;
     int32_t* status;
 };
 void wd_launch_plan(const WdPlanLaunch& h, cudaStream_t st);
