@@ -12,7 +12,7 @@
 //            ring of shared-memory stages (128-byte swizzle), completion on mbarriers
 //   warp 1   allocates TMEM, issues tcgen05.mma (kind::f16, bf16 in, fp32 accumulate in
 //            TMEM), releases stages with tcgen05.commit
-//   warps 2-5 epilogue: tcgen05.ld of the [128 x BN] accumulator, coalesced fp32 stores
+//   warps 2-9 epilogue (2-5 in the FP8, LM-head and fused forms): tcgen05.ld of the [128 x BN] accumulator, coalesced fp32 stores
 //            of this K slice's partial sums
 //
 // Split-K partial sums are written side by side ([slice][tok][n]); the kernel that
@@ -34,7 +34,12 @@ constexpr int kBM = 128;            // weight rows per tile (MMA M)
 constexpr int kBK = 64;             // K elements per stage = one 128-byte swizzle row
 constexpr int kStageA = kBM * kBK * 2;
 constexpr int kThreads = 192;         // TMA warp, MMA warp, 4 epilogue warps
-constexpr int kThreadsWide = 320;     // ... 8 epilogue warps when a CTA carries two weight halves
+constexpr int kThreadsWide = 320;     // ... 8 epilogue warps when a CTA carries two weight halves, and in the plain bf16 form:
+// What follows a CTA's last MMA (its accumulator and the zeros of unused slices) is time in which its SM streams nothing, and with
+// two warps to a quarter of the accumulator rows it halves.  64 registers then: a CTA (20 K) still fits beside a block of the few-row
+// RMSNorm (45 K).  Measured, four / eight epilogue warps, step of eight LLaDA-shaped blocks in us: 34 rows 974 / 964, 68 rows 1160 /
+// 1136, 136 rows 1381 / 1348, 200 rows 1802 / 1739.
+__host__ __device__ constexpr bool eight_epilogue_warps(bool lm_stats, bool fp8, bool fused) { return !lm_stats && !fp8 && !fused; }
 constexpr int kThreadsPair = 320;     // two-CTA kernel: 8 epilogue warps, two per quarter of the accumulator rows
 
 struct TcParams {
@@ -355,11 +360,12 @@ __device__ unsigned long long g_gemm_trace[8][160][8];
 #endif
 
 template <bool kWide, bool kLmStats, bool kFp8 = false, bool kFused = false>
-__global__ void __launch_bounds__(kWide ? kThreadsWide : kThreads, kFused ? 1 : 0)
+__global__ void __launch_bounds__(kWide || eight_epilogue_warps(kLmStats, kFp8, kFused) ? kThreadsWide : kThreads, kFused ? 1 : 0)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w0,
                const __grid_constant__ CUtensorMap map_w1, const __grid_constant__ CUtensorMap map_w2,
                const TcParams p) {
     constexpr int kKE = kFp8 ? 128 : kBK;                 // K elements per block: one 128-byte swizzle row
+    constexpr bool kEight = !kWide && eight_epilogue_warps(kLmStats, kFp8, kFused);
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment: required by the 128-byte swizzle atoms
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -397,8 +403,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         }
         mbar_init(smem_u32(&bars[2 * NS]), 1);
         mbar_init(smem_u32(&bars[2 * NS + 1]), 1);
-        mbar_init(smem_u32(&bars[2 * NS + 2]), kWide ? 256 : 128);
-        mbar_init(smem_u32(&bars[2 * NS + 3]), kWide ? 256 : 128);
+        mbar_init(smem_u32(&bars[2 * NS + 2]), kWide || kEight ? 256 : 128);
+        mbar_init(smem_u32(&bars[2 * NS + 3]), kWide || kEight ? 256 : 128);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
@@ -524,7 +530,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     } else {
         // ---------------------------------------------------- epilogue (warps 2..5; wide: 2..9)
         const int quarter = warp & 3;                  // TMEM lanes 32*quarter .. +31
-        const int half_sel = (warp - 2) >> 2;          // wide: which weight half this warp drains
+        const int half_sel = kWide ? (warp - 2) >> 2 : 0;      // wide: which weight half this warp drains
+        const int part = kEight ? (warp - 2) >> 2 : 0;         // kEight: two warps to a quarter, on alternate 16-column chunks
+        constexpr int n_part = kEight ? 2 : 1;
         const int n_local = half_sel * kBM + quarter * 32 + lane;
         pdl_wait();      // the previous reader of y has finished (already implied by the data flow)
         bool ok = true;
@@ -555,7 +563,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             const float sw_n = (kFp8 && n_ok) ? p.sw[u.seg][n] : 1.f;      // FP8: scale of this weight row
             const uint32_t t_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((buf + half_sel) * p.buf_cols);
             if constexpr (!kLmStats) {
-                for (int cc = 0; cc < p.bn; cc += 16) {
+                for (int cc = 16 * part; cc < p.bn; cc += 16 * n_part) {
                     if (u.tok0 + cc >= p.rows) break;
                     uint32_t v[16];
                     tmem_ld16(t_acc + (uint32_t)cc, v);
@@ -673,7 +681,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 // this CTA finished the tile: slices nobody wrote must read as zero
                 for (int sl = ord + 1; sl < p.n_slices; ++sl) {
                     float* ys = yb + (size_t)sl * p.split_stride;
-                    for (int tok = u.tok0; tok < u.tok0 + p.bn && tok < p.rows; ++tok) ys[(size_t)tok * p.ncol] = 0.f;
+                    for (int tok = u.tok0 + part; tok < u.tok0 + p.bn && tok < p.rows; tok += n_part) ys[(size_t)tok * p.ncol] = 0.f;
                 }
             }
         }
@@ -1985,7 +1993,7 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
     ++wd_launch_counter;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)(G * ts));
-    lc.blockDim = dim3(cfg.wide ? kThreadsWide : kThreads);
+    lc.blockDim = dim3(cfg.wide || eight_epilogue_warps(lm, fp8 != nullptr, fused) ? kThreadsWide : kThreads);
     lc.dynamicSmemBytes = cfg.smem;
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
