@@ -440,16 +440,6 @@ wd_status encode_bytes(CUtensorMap* m, const void* ptr, int n_rows, int row_byte
 // shares, a unit's sums then being spread over up to n_slices slices.
 struct Split { int grid, n_slices, aligned; };
 
-// Most CTAs that share a unit when the line of n units is cut into G equal shares: with G / n = a + r / q in lowest terms a unit
-// covers at most ceil((q - 1) / q + G / n) of them.
-int sharers(int n, int G) {
-    const int a = G / n;
-    int r = G % n, q = n, x = r;
-    if (r == 0) return a;
-    while (x) { const int t = q % x; q = x; x = t; }       // q = gcd(r, n)
-    return a + (r / q == 1 ? 1 : 2);
-}
-
 // Time of a split: the stages of the longest share, t_stage each, and for every further slice its write and re-read at HBM speed
 // (t_slice) and 0.3 us, for the zero fill where nobody wrote it and for its place in the chain of the kernel that adds the slices
 // (between 0.15 and 1 us the choice is the same).  Beside all SMs the grids tried give G / n_units a denominator of at most eight:
@@ -467,7 +457,7 @@ Split choose_split(int n_units, int kb, int sm_count, int max_slices, double t_s
     double t_best = (double)((n_units + g_unit - 1) / g_unit) * kb * t_stage;
     auto consider = [&](long long G) {
         if (G < 1 || G > sm_count || G > W || W * (G + 1) > INT_MAX) return;
-        const int ns = sharers(n_units, (int)G);
+        const int ns = wd_tc_sharers(n_units, (int)G);
         if (ns > max_slices) return;
         const double t = (double)((W + G - 1) / G) * t_stage + (ns - 1) * (t_slice + 0.3e-6);
         if (t < t_best * 0.999) {

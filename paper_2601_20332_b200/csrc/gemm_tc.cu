@@ -1626,6 +1626,25 @@ int count_slices(int n_units, int kb_total, long long W, long long G) {
     return n;
 }
 
+// Number of equal shares of the K-block line: the blocks of the longest, t_block each, against the slices that the split leaves, a
+// write and a re-read (t_slice) and 0.3 us each (zeros where nobody wrote one, a place in the chain of the kernel that adds them).
+// Tried are all of most CTAs and the grids with which shares start with a tile every few tiles.  Measured against all 148, in us a
+// block (LLaDA shape at 34 rows): q/k/v with 144 shares, two slices instead of three, -0.7; output projection with 128, four instead
+// of six, -0.5; down with 144 -0.3; gate/up stays at 148 (two slices either way; 144 +0.8).  Dream shape, 35 rows: q/k/v 144 -0.7,
+// output projection 140 -0.9.
+long long choose_shares(int n_units, int kb_total, int most, double t_block, double t_slice) {
+    const long long W = (long long)n_units * kb_total;
+    auto cost = [&](long long G) { return (double)((W + G - 1) / G) * t_block + (wd_tc_sharers(n_units, (int)G) - 1) * (t_slice + 0.3e-6); };
+    long long best = most;
+    for (int q = 1; q <= 8; ++q) {
+        const long long j = (long long)most * q / n_units;
+        const long long G = n_units * j / q;
+        if (j < 1 || n_units * j % q || G < 1 || G > W) continue;
+        if (cost(G) < 0.999 * cost(best)) best = G;
+    }
+    return best;
+}
+
 uint32_t make_idesc(int bn, int m = kBM, bool fp8 = false) {
     uint32_t d = 0;
     d |= 1u << 4;                      // D format: f32
@@ -1939,6 +1958,8 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
     // (G = CTAs per token group)
     long long G = (long long)slots / ts;
     if (G > p.W / 2) G = p.W / 2 > 0 ? p.W / 2 : 1;           // at least two K blocks per CTA
+    if (ts == 1 && !cfg.wide && !fused && !force_single_split)
+        G = choose_shares(p.n_units, p.kb_total, (int)G, (kStageA + cfg.bn * kBK * 2) / 63e9, (double)slice * 8.0 / 6.5e12);
     int n_slices = count_slices(p.n_units, p.kb_total, p.W, G);
     p.aligned = 0;
     if (force_single_split || (size_t)n_slices * slice > y_floats || n_slices > WD_TC_MAX_SPLIT || p.W * (G + 1) > INT_MAX) {
