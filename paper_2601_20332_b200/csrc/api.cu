@@ -1292,6 +1292,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         c->chain_dirty = false;
     }
     const bool f32 = d.dtype == WD_F32;
+    // few bf16 rows: 1 / rms multiplies the results of q/k/v and gate/up, where their slices are added
+    const bool split_norm = use_tc(c) && !fused && !c->fp8_on && !c->fp4_on && wd_rmsnorm_split_ok(R_, D);
+    WdRowScale row_scale;
+    if (split_norm) { row_scale.sumsq = c->sumsq; row_scale.inv_d = 1.f / (float)D; row_scale.eps = d.rms_eps; }
     const bool fp8 = c->fp8_on && use_tc(c) && !fused;      // FP8 projections (q/k/v, gate/up, down, LM head)
     const bool fp4 = c->fp4_on && use_tc(c) && !fused;      // NVFP4 projections (the same ones)
     WdFp4Operand x4_d, x4_f, x4_lm;                         // the step's quantised activations, by use
@@ -1432,7 +1436,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                 return s;
         }
         // attention half (FP8 mode: the normalised rows leave the RMSNorm as e4m3 codes + row scales)
-        if (!pq.done)
+        if (split_norm)
+            wd_launch_rmsnorm_split(c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride, c->attn_norm[l], c->xn,
+                                    c->sumsq, R_, D, stream);
+        else if (!pq.done)
             wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
                           c->attn_norm[l], d.rms_eps, c->xn, nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn,
                           fp4 ? &x4_d : nullptr);
@@ -1463,7 +1470,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                           {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
         // (Heads without grouping only, so far.  With 28 query over 4 KV heads a refresh of four blocks would also be 1-2 % faster
         // for it where the rounds are full: 5376 rows 7370 / 7270 us, 6080 rows 8000 / 7830, 6880 rows 9150 / 8990.)
-        if (use_tc(c) && dh == 128 && Hq == Hkv) {
+        if (use_tc(c) && dh == 128 && Hq == Hkv && !split_norm) {
             rope.map_q = c->tc.get(WD_TC_WQ_ROT, l); rope.map_k = c->tc.get(WD_TC_WK_ROT, l);
             rope.row_seq = row_seq; rope.row_pos = row_pos; rope.rope_tab = c->rope_tab;
             rope.q = (__nv_bfloat16*)c->q; rope.kcache = (__nv_bfloat16*)kc; rope.vcache = (__nv_bfloat16*)vc;
@@ -1481,7 +1488,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                                    dh, S, Sp, batch, status, stream);
         else
             wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, row_seq, row_pos, c->rope_tab, c->q, kc,
-                                   vc, R_, Hq, Hkv, dh, S, Sp, batch, status, stream);
+                                   vc, R_, Hq, Hkv, dh, S, Sp, batch, status, stream, row_scale);
         if ((s = attention(l, kc, vc, act)) != WD_OK) return s;
         // from here on the block works on these rows
         const int Rb = act ? NA : R_;
@@ -1519,7 +1526,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             return s;
         }
         // feed-forward half
-        if (!pg.done)
+        if (split_norm)
+            wd_launch_rmsnorm_split(xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], xnb, c->sumsq, Rb, D,
+                                    stream);
+        else if (!pg.done)
             wd_launch_rmsnorm(d.dtype, xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, xnb,
                           nullptr, Rb, D, stream, fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_d : nullptr);
         if (fp4) {
@@ -1542,14 +1552,14 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                 return s;
         } else {
         WdTcSwiglu sg;
-        sg.h = use_tc(c) ? (__nv_bfloat16*)c->h : nullptr;
+        sg.h = use_tc(c) && !split_norm ? (__nv_bfloat16*)c->h : nullptr;
         WdTcEpi epi_sg;
         epi_sg.sg = &sg;
         if (!pg.done) {
             if ((s = run_gemm(c, xnb, xmb, gu, 2, Rb, D, c->part, c->part_floats, status, stream, &go, false,
                               nullptr, nullptr, &epi_sg)) != WD_OK)
                 return s;
-            if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream);
+            if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream, row_scale);
         }
         WdTcSeg wdn[1] = {{c->wd[l], D, c->tc.get(WD_TC_WD, l)}};
         if (f32) {                      // (x is complete: the output projection or the RMSNorm after it has added its sums)
