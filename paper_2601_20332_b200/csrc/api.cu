@@ -76,7 +76,7 @@ struct wd_ctx {
     };
     struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int n_kernels = 0, impl_used = 0; uint64_t last_use = 0; };
     bool graphs_on = true;
-    std::vector<StepGraph> graphs;      // at most kMaxGraphs, least recently used replaced
+    std::vector<StepGraph> graphs;      // at most kMaxGraphs, the least recently used replaced once it is out of use
     std::vector<StepKey> seen;          // configurations met once (capture pays from the second time on)
     uint64_t graph_clock = 0;
     int graphs_captured = 0, graphs_replayed = 0, graph_failures = 0;
@@ -703,10 +703,6 @@ extern "C" wd_status wd_state_reset(wd_state* st, const int32_t* token_ids, cons
         if (token_ids[i] < 0 || token_ids[i] >= st->ctx->d.vocab) return WD_ERR_BAD_PARAM;
     // the pinned staging buffers may still be the source of an earlier reset's copies
     if (st->staged_recorded) WD_CUDA_TRY(cudaEventSynchronize(st->staged));
-    // Launch configurations met once are counted within a generation.  Counted across resets, every refresh step of a second request
-    // of the same lengths was recorded, replayed once and pushed out again: 17 of 230 us each in 64 steps of the small fp32 model.
-    std::vector<wd_ctx::StepKey>& seen = st->ctx->seen;
-    seen.erase(std::remove_if(seen.begin(), seen.end(), [&](const wd_ctx::StepKey& k) { return k.state_uid == st->uid; }), seen.end());
     load_host_mirror(st, token_ids, decoded);
     st->poisoned = false;
     WD_CUDA_TRY(upload_plan_state(st, (cudaStream_t)stream));
@@ -1664,9 +1660,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         key.impl = c->gemm_impl; key.attn_impl = c->attn_impl;
         wd_ctx::StepGraph* hit = nullptr;
         for (wd_ctx::StepGraph& g : c->graphs) if (g.key == key) { hit = &g; break; }
+        ++c->graph_clock;
         if (hit) {
             WD_CUDA_TRY(cudaGraphLaunch(hit->exec, stream));
-            hit->last_use = ++c->graph_clock;
+            hit->last_use = c->graph_clock;
             wd_launch_counter += hit->n_kernels;
             impl_used = hit->impl_used;
             ++c->graphs_replayed;
@@ -1680,9 +1677,17 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             for (int b = 0; b < batch; ++b) live += pend.cp[b].done ? 0 : 1;
             bool seen = !any_refresh && NA == A * live;
             for (const wd_ctx::StepKey& k2 : c->seen) if (k2 == key) { seen = true; break; }
+            // A full cache gives up only a graph that the last 64 steps had no use for.  A job that repeats more configurations than fit
+            // (the refresh steps of a long generation, each of its own row count) would otherwise record each of them, replay it once
+            // and push it out again: 64 steps of the small fp32 model against eight graphs were 17 recordings of 230 us.
+            static const size_t kMaxGraphs = 32;
+            size_t lru = 0;
+            for (size_t i = 1; i < c->graphs.size(); ++i) if (c->graphs[i].last_use < c->graphs[lru].last_use) lru = i;
+            const bool room = c->graphs.size() < kMaxGraphs || c->graphs[lru].last_use + 64 < c->graph_clock;
             if (!seen) {
-                if (c->seen.size() >= 32) c->seen.erase(c->seen.begin());
+                if (c->seen.size() >= 64) c->seen.erase(c->seen.begin());
                 c->seen.push_back(key);
+            } else if (!room) {         // launched directly
             } else if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
                 static const bool gdbg = getenv("WD_GRAPH_DEBUG") != nullptr;
                 const long long k0 = wd_launch_counter;
@@ -1703,11 +1708,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                     cudaGraphDestroy(graph);
                     wd_ctx::StepGraph g;
                     g.key = key; g.exec = exec; g.n_kernels = (int)(wd_launch_counter - k0); g.impl_used = impl_used;
-                    g.last_use = ++c->graph_clock;
-                    static const size_t kMaxGraphs = 8;
+                    g.last_use = c->graph_clock;
                     if (c->graphs.size() >= kMaxGraphs) {
-                        size_t lru = 0;
-                        for (size_t i = 1; i < c->graphs.size(); ++i) if (c->graphs[i].last_use < c->graphs[lru].last_use) lru = i;
                         cudaGraphExecDestroy(c->graphs[lru].exec);
                         c->graphs[lru] = g;
                     } else {
