@@ -18,6 +18,7 @@
 // Split-K partial sums are written side by side ([slice][tok][n]); the kernel that
 // consumes the GEMM output adds them, which keeps the result deterministic.
 // Every wait is bounded: on expiry the CTA records WD_ERR_DEVICE_TIMEOUT and leaves.
+#include <algorithm>
 #include <climits>
 #include <cstdio>
 #include <cstdlib>
@@ -1658,6 +1659,37 @@ uint32_t make_idesc(int bn, int m = kBM, bool fp8 = false) {
     return d;
 }
 
+// whole units pay when every pair gets two or more, or when the one or two rounds are nearly full
+bool full_rounds(long long units, long long pairs) {
+    return units >= 2 * pairs || (units >= pairs && 10 * units >= 9 * pairs * ((units + pairs - 1) / pairs));
+}
+
+// Token tiles of a gate/up launch whose epilogue applies SwiGLU (whole units of a gate and an up tile, dealt to the pairs in rounds),
+// or 0 where equal shares of the K-block line and the SwiGLU kernel are the shorter way.  Fewest tiles are not always best: 1216
+// rows in five tiles of 256 are 240 units for 74 pairs, four rounds, and so are six tiles of 208.  Estimated in us, fitted to both
+// sides measured: a K block of a unit takes its MMAs (0.003 a token) or what a CTA takes in (two weight blocks and half the tokens'
+// at 73 GB/s), a unit's end 4 at 256 tokens; a K block of a share 0.4, its slices' way through the SwiGLU kernel 16 bytes a value at
+// 9.4 TB/s.  Measured, LLaDA shape, us a block against the fewest tiles, or shares where those do not fill their rounds:
+// 352 rows in three tiles -7 (two -4), 440 in three -11, 1100 in six -16 of 177, 1216 in six -31 of 199 (with the power that the fuller rounds draw, -9 and -17 of the whole block); kept at the fewest: 583 rows (four tiles
+// +25), 704 (+24), 900 (five +14), 2100 (ten even); Dream shape 530 (four +25), 1000 (five +8).
+int gate_up_tok_tiles(int tiles, int kb_total, int rows, int pairs, int n) {
+    const int least = (rows + 255) / 256;
+    int best = 0;
+    double t_best = 2.0 * tiles * least * kb_total / pairs * 0.4 + 3.0 + (double)rows * n * 16.0 / 9.4e6;
+    for (int t = least; t < least + 4; ++t) {
+        const int bn = ((rows + t - 1) / t + 15) / 16 * 16;
+        if (!full_rounds((long long)tiles * t, pairs)) continue;
+        const int n_rounds = (tiles * t + pairs - 1) / pairs;
+        const double block = std::max(0.003 * bn, (2 * kStageA + bn * kBK) / 73e3);
+        const double us = n_rounds * (kb_total * block + bn / 64.0);
+        if (us < 0.98 * t_best) {       // (a tile more only for a gain that shows)
+            t_best = us;
+            best = t;
+        }
+    }
+    return best;
+}
+
 // launch of gemm_tc_pair_kernel: same contract as wd_tc_gemm
 wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, int K, float* y, size_t y_floats,
                        int sm_count, int32_t* status, cudaStream_t stream, int* n_split_out, bool force_single_split,
@@ -1680,30 +1712,26 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     // overlaps the next tile.  Measured: pays for the widest weight matrices (gate/up) once every pair
     // gets at least two whole units, costs 10-25 % on the narrow ones.  0 = never, 1 = that rule, 2 = always.
     static const int dual_mode = env_int("WD_GEMM_DUAL", 1);
+    int gu_tok_tiles = 0;
     {
         int tiles_all = 0, ncol_all = 0;
         for (int i = 0; i < nseg; ++i) {
             tiles_all += (segs[i].n + p.tile_rows - 1) / p.tile_rows;
             ncol_all += segs[i].n;
         }
-        // whole units pay when every pair gets two or more, or when the one or two rounds are nearly full
         const long long pairs = sm_count / 2;
-        auto full_rounds = [&](long long units) {
-            return units >= 2 * pairs || (units >= pairs && 10 * units >= 9 * pairs * ((units + pairs - 1) / pairs));
-        };
         const long long dual_units = (long long)tiles_all * ((rows + 511) / 512);
         p.dual = (dual_mode == 2 || (dual_mode == 1 && ncol_all >= 16384 && dual_units >= 2 * pairs)) ? 1 : 0;
         // gate and up against the same tokens, h = silu(gate) * up written by the epilogue: needs whole
         // tiles per pair (no partial sums)
         static const int swiglu_fused = env_int("WD_GEMM_SWIGLU", 1);
-        if (sg && sg->h && swiglu_fused && !fp8 && nseg == 2 && segs[0].n == segs[1].n && dual_mode != 0) {
-            const long long gu_units = (long long)((segs[0].n + p.tile_rows - 1) / p.tile_rows) * ((rows + 255) / 256);
-            if (full_rounds(gu_units)) p.dual = 2;
-        }
+        if (sg && sg->h && swiglu_fused && !fp8 && nseg == 2 && segs[0].n == segs[1].n && dual_mode != 0)
+            gu_tok_tiles = gate_up_tok_tiles((segs[0].n + p.tile_rows - 1) / p.tile_rows, (K + kBK - 1) / kBK, rows, (int)pairs, segs[0].n);
+        if (gu_tok_tiles > 0) p.dual = 2;
         // RoPE or the residual add in the epilogue: the same condition on whole units of one accumulator (with shares of the K-block
         // line a tile's sum is in several pieces)
         static const int epi_on = env_int("WD_GEMM_EPI", 3);
-        if (!fp8 && p.dual != 2 && full_rounds((long long)tiles_all * ((rows + 255) / 256))) {
+        if (!fp8 && p.dual != 2 && full_rounds((long long)tiles_all * ((rows + 255) / 256), pairs)) {
             if (rope && nseg == 3 && (epi_on & 1)) epi = kEpiRope;
             else if (resid && resid->x && nseg == 1 && (epi_on & 2)) epi = kEpiResid;
         }
@@ -1716,7 +1744,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
         p.tok_tiles = (rows + 511) / 512;                                   // super-tiles
         p.bn = ((rows + 2 * p.tok_tiles - 1) / (2 * p.tok_tiles) + 15) / 16 * 16;   // balanced, <= 256
     } else {
-        p.tok_tiles = (rows + 255) / 256;
+        p.tok_tiles = p.dual == 2 ? gu_tok_tiles : (rows + 255) / 256;
         p.bn = ((rows + p.tok_tiles - 1) / p.tok_tiles + 15) / 16 * 16;    // balanced token tiles, <= 256
     }
     int cols = 32;
