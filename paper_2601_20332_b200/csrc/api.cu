@@ -1326,6 +1326,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                           d.n_layers > 1 && NA > 0 && R_ > 256 && 2 * NA <= R_ && !st->taps.layer_out && !st->taps.attn_out;
     // ---- the kernels of the step, from the embedding to the selection (everything after the planner and
     // before the event that a sync waits for); launched directly, or recorded into a CUDA graph and replayed
+    bool copy_logits = false;           // ... unless the kernels are those of a graph: then a copy behind them fills it
     auto run_kernels = [&]() -> wd_status {
     c->tc.x_map_attn.smem_cap = 0;          // set per block below, and only beside the single-key-tile attention
     bool down_pending = false;          // x still lacks the previous block's FFN output (partial sums in part)
@@ -1585,7 +1586,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     bool lm_fused = false;
     int lm_chunks = wd_unmask_chunks(d.vocab);
     if (NA > 0) {
-        float* logits = st->taps.logits ? st->taps.logits : c->logits;      // a tap takes them directly
+        float* logits = st->taps.logits && !copy_logits ? st->taps.logits : c->logits;      // a tap takes them directly
         WdTcSeg lm[1] = {{c->lm_head, d.vocab, c->tc.get(WD_TC_LM, 0)}};
         WdPlainFuse pl;
         if (f32 && !down_pending) {
@@ -1641,7 +1642,9 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) { cudaGetLastError(); cs = cudaStreamCaptureStatusActive; }
         stream_capturing = cs != cudaStreamCaptureStatusNone;
     }
-    const bool taps_on = st->taps.layer_out || st->taps.attn_out || st->taps.logits;
+    // A step of the fp32 path lasts 2-3 us a kernel, and its launches take the host 5 each: with a graph it is also shorter when nothing
+    // is queued and the host waits for every step (9 rows, two blocks of 256 / 688, host to host 105 -> 100 us).
+    const bool taps_on = st->taps.layer_out || st->taps.attn_out || (st->taps.logits && !f32);
     // Only while earlier steps are still queued: the GPU then has work while the host records or submits the
     // graph.  With an empty queue (a caller that syncs after every step) direct launches win, because the GPU
     // starts on the first kernels while the host is still launching the later ones (measured: 230 against 227
@@ -1651,7 +1654,8 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     const bool attn_by_tc = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN;
     const bool attn_by_tiles = d.dtype == WD_F32 && (wd_align_up((size_t)max_vis, 128) + dh) * 4 <= 200 * 1024;
     if (c->graphs_on && dev_mode && !c->prof_on && !taps_on && !fused && !stream_capturing && (attn_by_tc || attn_by_tiles) &&
-        !st->queue.empty()) {
+        (f32 || !st->queue.empty())) {
+        copy_logits = true;
         wd_ctx::StepKey key;
         key.state_uid = st->uid; key.batch = batch; key.rows = R_; key.n_act = NA; key.n_qtiles = (int)n_qtiles;
         key.key_tiles = (max_vis + 127) / 128; key.max_tile_rows = max_tile_rows; key.max_seq_tiles = max_seq_tiles; key.n_aqt = n_aqt;
@@ -1731,7 +1735,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             }
         }
     }
+    if (!graphed) copy_logits = false;
     if (!graphed && (s = run_kernels()) != WD_OK) return s;
+    if (copy_logits && st->taps.logits && NA > 0)
+        WD_CUDA_TRY(cudaMemcpyAsync(st->taps.logits, c->logits, (size_t)NA * d.vocab * 4, cudaMemcpyDeviceToDevice, stream));
     WD_CUDA_TRY(cudaEventRecord(st->done, stream));
     WD_CUDA_TRY(cudaGetLastError());
     if (!dev_mode) pend.plans = st->plans;
