@@ -64,6 +64,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
     return false;
 }
+// One lane of the (converged) warp, the same in every call.
+// The loops that issue TMA and MMA instructions are run by their whole warp, and only the instructions themselves by this lane: their
+// operands (barriers, descriptors, coordinates) then stay in uniform registers, which these instructions take.  In a branch that one
+// lane runs alone each operand is moved there first: four tcgen05.mma and a commit took 400 cycles to issue, 203 like this (and the
+// three instructions of a stage's loads 292), with the waits 620 cycles a K block of the two-CTA GEMM whatever its token tile.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+    return p != 0;
+}
+// Bounded wait of a whole warp, with one answer for all its lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
 // The same wait by a whole warp that goes on either way.  Every lane polls with its own clock, so lanes may give up at different
 // times, and what follows (tcgen05.ld / .st, votes over the full mask) takes the whole warp: a lane that gave up raises the flag,
 // which ends every later wait of the block early, clears ok, and stays with the others.  Nothing that another thread waits for

@@ -418,8 +418,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0 && n_total > 0) {
-            // ------------------------------------------------ TMA producer
+        if (n_total > 0) {
+            // ------------------------------------------------ TMA producer (the whole warp, see elect_one)
+            const bool leader = elect_one();
             uint64_t pol_stream;
             asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
             // walks the K blocks of this CTA's pieces in schedule order without per-block divisions
@@ -447,6 +448,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             const int n_pre = n_total < NS ? n_total : NS;
             Walk w = w0;
             for (int i = 0; i < n_pre; ++i, advance(w)) {
+                if (!leader) continue;
                 mbar_expect_tx(smem_u32(&bars[i]), (uint32_t)stage_bytes);
                 tma_load_2d_hint(smem_u32(smem + (size_t)i * stage_bytes), w.mw, smem_u32(&bars[i]), w.kb * kKE, w.n0,
                                  pol_stream);
@@ -454,34 +456,37 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     tma_load_2d_hint(smem_u32(smem + (size_t)i * stage_bytes) + kStageA, w.mw, smem_u32(&bars[i]),
                                      w.kb * kKE, w.n0 + kBM, pol_stream);
             }
-            G_STAMP(1);
+            if (leader) G_STAMP(1);
             pdl_wait();
-            G_STAMP(2);
+            if (leader) G_STAMP(2);
             Walk wx = w0;
             for (int i = 0; i < n_pre; ++i, advance(wx))
-                tma_load_2d(smem_u32(smem + (size_t)i * stage_bytes) + stage_a, &map_x, smem_u32(&bars[i]), wx.kb * kKE,
+                if (leader) tma_load_2d(smem_u32(smem + (size_t)i * stage_bytes) + stage_a, &map_x, smem_u32(&bars[i]), wx.kb * kKE,
                             wx.tok0);
             int s = n_pre % NS;
             uint32_t ph = (uint32_t)(n_pre / NS) & 1u;
             for (int i = n_pre; i < n_total; ++i, advance(w)) {
-                if (!mbar_wait(smem_u32(&bars[NS + s]), ph ^ 1u, abort_flag)) {
+                if (!mbar_wait_warp(smem_u32(&bars[NS + s]), ph ^ 1u, abort_flag)) {
                     *abort_flag = 1;
                     atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
                     break;
                 }
                 const uint32_t full = smem_u32(&bars[s]);
-                const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
-                mbar_expect_tx(full, (uint32_t)stage_bytes);
-                tma_load_2d_hint(sa, w.mw, full, w.kb * kKE, w.n0, pol_stream);
-                if (kWide) tma_load_2d_hint(sa + kStageA, w.mw, full, w.kb * kKE, w.n0 + kBM, pol_stream);
-                tma_load_2d(sa + stage_a, &map_x, full, w.kb * kKE, w.tok0);
+                const uint32_t sa = smem_u32(smem) + (uint32_t)(s * stage_bytes);
+                if (leader) {
+                    mbar_expect_tx(full, (uint32_t)stage_bytes);
+                    tma_load_2d_hint(sa, w.mw, full, w.kb * kKE, w.n0, pol_stream);
+                    if (kWide) tma_load_2d_hint(sa + kStageA, w.mw, full, w.kb * kKE, w.n0 + kBM, pol_stream);
+                    tma_load_2d(sa + stage_a, &map_x, full, w.kb * kKE, w.tok0);
+                }
                 if (++s == NS) { s = 0; ph ^= 1u; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ------------------------------------------------ MMA issuer
+        {
+            // ------------------------------------------------ MMA issuer (the whole warp)
+            const bool leader = elect_one();
             bool ok = true;
             int s = 0;
             uint32_t ph = 0;
@@ -492,36 +497,38 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 const int buf = kWide ? 0 : (piece & 1);
                 const uint32_t par = kWide ? ((uint32_t)piece & 1u) : ((uint32_t)(piece >> 1) & 1u);
                 // the epilogue has drained this accumulator (free at the start)
-                if (!(ok = mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), par ^ 1u, abort_flag))) break;
+                if (!(ok = mbar_wait_warp(smem_u32(&bars[2 * NS + 2 + buf]), par ^ 1u, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t acc = tmem_base + (uint32_t)(buf * p.buf_cols);
                 for (int j = 0; j < len; ++j) {
-                    if (!(ok = mbar_wait(smem_u32(&bars[s]), ph, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[s]), ph, abort_flag))) break;
                     tc_fence_after();
-                    if (piece == 0 && j == 0) G_STAMP(3);
-                    const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
+                    if (leader && piece == 0 && j == 0) G_STAMP(3);
+                    const uint32_t sa = smem_u32(smem) + (uint32_t)(s * stage_bytes);
                     const uint64_t adesc = make_sdesc(sa);
                     const uint64_t bdesc = make_sdesc(sa + stage_a);
                     const uint64_t adesc1 = make_sdesc(sa + kStageA);   // second weight half (wide)
+                    if (leader) {
 #pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk) {
-                        // 16 bf16 = 32 bytes further along K inside the swizzle row: +2 in 16-byte units
-                        if (kFp8)
-                            umma_f8(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
-                                    (j > 0 || kk > 0) ? 1u : 0u);
-                        else
-                            umma_bf16(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
-                                      (j > 0 || kk > 0) ? 1u : 0u);
-                        if (kWide)
-                            umma_bf16(acc + (uint32_t)p.buf_cols, adesc1 + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk),
-                                      p.idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < kBK / 16; ++kk) {
+                            // 16 bf16 = 32 bytes further along K inside the swizzle row: +2 in 16-byte units
+                            if (kFp8)
+                                umma_f8(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
+                                        (j > 0 || kk > 0) ? 1u : 0u);
+                            else
+                                umma_bf16(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
+                                          (j > 0 || kk > 0) ? 1u : 0u);
+                            if (kWide)
+                                umma_bf16(acc + (uint32_t)p.buf_cols, adesc1 + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk),
+                                          p.idesc, (j > 0 || kk > 0) ? 1u : 0u);
+                        }
+                        umma_commit(smem_u32(&bars[NS + s]));          // stage free once these MMAs have read it
                     }
-                    umma_commit(smem_u32(&bars[NS + s]));          // stage free once these MMAs have read it
                     if (++s == NS) { s = 0; ph ^= 1u; }
                 }
-                if (ok) umma_commit(smem_u32(&bars[2 * NS + buf]));  // this piece's accumulator complete
+                if (ok && leader) umma_commit(smem_u32(&bars[2 * NS + buf]));  // this piece's accumulator complete
             }
-            G_STAMP(4);
+            if (leader) G_STAMP(4);
             if (!ok) {
                 *abort_flag = 1;
                 atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
@@ -1229,8 +1236,10 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0 && n_total > 0) {
-            // ------------------------------------------------ TMA producer (both CTAs, own halves)
+        if (n_total > 0) {
+            // ------------------------------------------------ TMA producer (both CTAs, own halves; the whole warp, see elect_one)
+            const bool leader = elect_one();
+            const uint32_t full0 = cluster_map(smem_u32(&bars[0]), 0);         // the even CTA's barriers
             // weights that one or two units use are streamed past the L2 (evict first); with more token
             // tiles the same weight block is wanted again by the units that follow: keep it (evict last)
             uint64_t pol_stream;
@@ -1266,40 +1275,42 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             const int n_pre = n_total < NS ? n_total : NS;
             Walk w = w0;
             for (int i = 0; i < n_pre; ++i, advance(w)) {
+                const uint32_t full = full0 + 8u * (uint32_t)i, sa = smem_u32(smem) + (uint32_t)(i * stage_bytes);
+                if (!leader) continue;
                 if (rank == 0) mbar_expect_tx(smem_u32(&bars[i]), 2u * (uint32_t)stage_bytes);
-                load_w(w, smem_u32(smem + (size_t)i * stage_bytes), cluster_map(smem_u32(&bars[i]), 0));
-                if (gate_up)
-                    tma2_load_2d_hint(smem_u32(smem + (size_t)i * stage_bytes) + kStageA, &map_w1,
-                                      cluster_map(smem_u32(&bars[i]), 0), w.kb * kKE, w.n0, pol_stream);
+                load_w(w, sa, full);
+                if (gate_up) tma2_load_2d_hint(sa + kStageA, &map_w1, full, w.kb * kKE, w.n0, pol_stream);
             }
-            G_STAMP(1);
+            if (leader) G_STAMP(1);
             pdl_wait();
-            G_STAMP(2);
+            if (leader) G_STAMP(2);
             Walk wx = w0;
             for (int i = 0; i < n_pre; ++i, advance(wx))
-                tma2_load_2d(smem_u32(smem + (size_t)i * stage_bytes) + stage_a, &map_x,
-                             cluster_map(smem_u32(&bars[i]), 0), wx.kb * kKE, wx.tok0);
+                if (leader)
+                    tma2_load_2d(smem_u32(smem) + (uint32_t)(i * stage_bytes) + stage_a, &map_x, full0 + 8u * (uint32_t)i, wx.kb * kKE, wx.tok0);
             int s = n_pre % NS;
             uint32_t ph = (uint32_t)(n_pre / NS) & 1u;
             for (int i = n_pre; i < n_total; ++i, advance(w)) {
-                if (!mbar_wait(smem_u32(&bars[NS + s]), ph ^ 1u, abort_flag)) {
+                if (!mbar_wait_warp(smem_u32(&bars[NS + s]), ph ^ 1u, abort_flag)) {
                     *abort_flag = 1;
                     atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
                     break;
                 }
-                const uint32_t full = cluster_map(smem_u32(&bars[s]), 0);
-                const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
-                if (rank == 0) mbar_expect_tx(smem_u32(&bars[s]), 2u * (uint32_t)stage_bytes);
-                load_w(w, sa, full);
-                if (gate_up) tma2_load_2d_hint(sa + kStageA, &map_w1, full, w.kb * kKE, w.n0, pol_stream);
-                tma2_load_2d(sa + stage_a, &map_x, full, w.kb * kKE, w.tok0);
+                const uint32_t full = full0 + 8u * (uint32_t)s, sa = smem_u32(smem) + (uint32_t)(s * stage_bytes);
+                if (leader) {
+                    if (rank == 0) mbar_expect_tx(smem_u32(&bars[s]), 2u * (uint32_t)stage_bytes);
+                    load_w(w, sa, full);
+                    if (gate_up) tma2_load_2d_hint(sa + kStageA, &map_w1, full, w.kb * kKE, w.n0, pol_stream);
+                    tma2_load_2d(sa + stage_a, &map_x, full, w.kb * kKE, w.tok0);
+                }
                 if (++s == NS) { s = 0; ph ^= 1u; }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
-            // ------------------------------------------------ MMA issuer (even CTA only)
+        if (rank == 0) {
+            // ------------------------------------------------ MMA issuer (even CTA only; the whole warp)
+            const bool leader = elect_one();
             bool ok = true;
             int s = 0;
             uint32_t ph = 0;
@@ -1309,45 +1320,47 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 const int buf = n_sets == 2 ? piece & 1 : 0;
                 const uint32_t par = (uint32_t)(n_sets == 2 ? piece >> 1 : piece) & 1u;
                 // the epilogues of both CTAs have drained this accumulator set (free at the start)
-                if (!(ok = mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), par ^ 1u, abort_flag))) break;
+                if (!(ok = mbar_wait_warp(smem_u32(&bars[2 * NS + 2 + buf]), par ^ 1u, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t acc = tmem_base + (uint32_t)(buf * set_cols);
                 for (int j = 0; j < len; ++j) {
-                    if (!(ok = mbar_wait(smem_u32(&bars[s]), ph, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[s]), ph, abort_flag))) break;
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
+                    const uint32_t sa = smem_u32(smem) + (uint32_t)(s * stage_bytes);
                     const uint64_t adesc = make_sdesc(sa);
                     const uint64_t bdesc = make_sdesc(sa + stage_a);
-#pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk) {
-                        if (kFp8)
-                            umma2_f8(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
-                                     (j > 0 || kk > 0) ? 1u : 0u);
-                        else
-                            umma2_bf16(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
-                                       (j > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    if (p.dual) {
-                        // second accumulator: the same weight rows against the other half of the token rows
-                        // (offset of half_bn rows of 128 bytes, in 16-byte units), or the up weights against
-                        // the same token rows
-                        const uint64_t adesc1 = gate_up ? adesc + (uint64_t)(kStageA >> 4) : adesc;
-                        const uint64_t bdesc1 = gate_up ? bdesc : bdesc + (uint64_t)(half_bn * 8);
-                        const uint32_t acc1 = acc + (uint32_t)p.buf_cols;
+                    if (leader) {
 #pragma unroll
                         for (int kk = 0; kk < kBK / 16; ++kk) {
                             if (kFp8)
-                                umma2_f8(acc1, adesc1 + (uint64_t)(2 * kk), bdesc1 + (uint64_t)(2 * kk), p.idesc,
+                                umma2_f8(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
                                          (j > 0 || kk > 0) ? 1u : 0u);
                             else
-                                umma2_bf16(acc1, adesc1 + (uint64_t)(2 * kk), bdesc1 + (uint64_t)(2 * kk), p.idesc,
+                                umma2_bf16(acc, adesc + (uint64_t)(2 * kk), bdesc + (uint64_t)(2 * kk), p.idesc,
                                            (j > 0 || kk > 0) ? 1u : 0u);
                         }
+                        if (p.dual) {
+                            // second accumulator: the same weight rows against the other half of the token rows
+                            // (offset of half_bn rows of 128 bytes, in 16-byte units), or the up weights against
+                            // the same token rows
+                            const uint64_t adesc1 = gate_up ? adesc + (uint64_t)(kStageA >> 4) : adesc;
+                            const uint64_t bdesc1 = gate_up ? bdesc : bdesc + (uint64_t)(half_bn * 8);
+                            const uint32_t acc1 = acc + (uint32_t)p.buf_cols;
+#pragma unroll
+                            for (int kk = 0; kk < kBK / 16; ++kk) {
+                                if (kFp8)
+                                    umma2_f8(acc1, adesc1 + (uint64_t)(2 * kk), bdesc1 + (uint64_t)(2 * kk), p.idesc,
+                                             (j > 0 || kk > 0) ? 1u : 0u);
+                                else
+                                    umma2_bf16(acc1, adesc1 + (uint64_t)(2 * kk), bdesc1 + (uint64_t)(2 * kk), p.idesc,
+                                               (j > 0 || kk > 0) ? 1u : 0u);
+                            }
+                        }
+                        umma2_commit_mc(smem_u32(&bars[NS + s]), 3);          // stage free in both CTAs
                     }
-                    umma2_commit_mc(smem_u32(&bars[NS + s]), 3);          // stage free in both CTAs
                     if (++s == NS) { s = 0; ph ^= 1u; }
                 }
-                if (ok) umma2_commit_mc(smem_u32(&bars[2 * NS + buf]), 3);  // accumulator complete in both CTAs
+                if (ok && leader) umma2_commit_mc(smem_u32(&bars[2 * NS + buf]), 3);  // accumulator complete in both CTAs
             }
             if (!ok) {
                 *abort_flag = 1;
