@@ -186,14 +186,16 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
     if (!has_work) {
         // nothing to compute
     } else if (warp == 0) {
-        if (lane == 0) {
-            // ---------------------------------------------------- TMA producer
+        {
+            // ---------------------------------------------------- TMA producer (the whole warp, see elect_one)
+            const bool leader = elect_one();
             const uint32_t qf = smem_u32(&bars[kQFull]);
             // slot j: rows [row0, row0 + slot) of head h + j at tile rows [j * slot, ...); slots without a head
             // stay unwritten (their rows of S and O are never read)
-            mbar_expect_tx(qf, (uint32_t)(n_slots * p.slot * 256));
+            if (leader) mbar_expect_tx(qf, (uint32_t)(n_slots * p.slot * 256));
             for (int j = 0; j < n_slots; ++j) {
                 const uint32_t dst = smem_u32(sQ) + (uint32_t)(j * p.slot * 128);
+                if (!leader) continue;
                 tma_load_2d(dst, &map_q, qf, (h + j) * kTile, row0);
                 tma_load_2d(dst + kAtom, &map_q, qf, (h + j) * kTile + 64, row0);
             }
@@ -202,12 +204,14 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
                 const int ks = j % NS;
                 const uint32_t ph = (uint32_t)(j / NS) & 1u;
                 const uint32_t kfull = smem_u32(&bars[kKFull + ks]);
-                if (!mbar_wait(smem_u32(&bars[kKEmpty + ks]), ph ^ 1u, abort_flag)) return false;   // stage free
-                const uint32_t sk = smem_u32(sK + (size_t)ks * kOperand);
+                if (!mbar_wait_warp(smem_u32(&bars[kKEmpty + ks]), ph ^ 1u, abort_flag)) return false;   // stage free
+                const uint32_t sk = smem_u32(sK) + (uint32_t)(ks * kOperand);
                 const int kv0 = (kt_begin + j) * kTile;
-                mbar_expect_tx(kfull, kOperand);
-                tma_load_4d(sk, &map_k, kfull, 0, kv0, bh, p.layer);            // keys kv0.., dims 0..63
-                tma_load_4d(sk + kAtom, &map_k, kfull, 64, kv0, bh, p.layer);   // dims 64..127
+                if (leader) {
+                    mbar_expect_tx(kfull, kOperand);
+                    tma_load_4d(sk, &map_k, kfull, 0, kv0, bh, p.layer);            // keys kv0.., dims 0..63
+                    tma_load_4d(sk + kAtom, &map_k, kfull, 64, kv0, bh, p.layer);   // dims 64..127
+                }
                 return true;
             };
             // order of need: K(0), K(1), V(0), K(2), V(1), ...
@@ -217,12 +221,14 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
                 const int vs = i % NS;
                 const uint32_t ph = (uint32_t)(i / NS) & 1u;
                 const uint32_t vfull = smem_u32(&bars[kVFull + vs]);
-                const uint32_t sv = smem_u32(sV + (size_t)vs * kOperand);
+                const uint32_t sv = smem_u32(sV) + (uint32_t)(vs * kOperand);
                 const int kv0 = (kt_begin + i) * kTile;
-                if (!(ok = mbar_wait(smem_u32(&bars[kVEmpty + vs]), ph ^ 1u, abort_flag))) break;   // stage free
-                mbar_expect_tx(vfull, kOperand);
-                tma_load_4d(sv, &map_vt, vfull, kv0, 0, bh, p.layer);           // all dims, keys kv0..kv0+63
-                tma_load_4d(sv + kAtom, &map_vt, vfull, kv0 + 64, 0, bh, p.layer);
+                if (!(ok = mbar_wait_warp(smem_u32(&bars[kVEmpty + vs]), ph ^ 1u, abort_flag))) break;   // stage free
+                if (leader) {
+                    mbar_expect_tx(vfull, kOperand);
+                    tma_load_4d(sv, &map_vt, vfull, kv0, 0, bh, p.layer);           // all dims, keys kv0..kv0+63
+                    tma_load_4d(sv + kAtom, &map_vt, vfull, kv0 + 64, 0, bh, p.layer);
+                }
             }
             if (!ok) {
                 *abort_flag = 1;
@@ -231,24 +237,27 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------------------------------------------- MMA issuer
+        {
+            // ---------------------------------------------------- MMA issuer (the whole warp)
+            const bool leader = elect_one();
             // tile i uses K/V stage i % 3, S buffer i & 1, O_tile buffer i & 1
-            bool ok = mbar_wait(smem_u32(&bars[kQFull]), 0, abort_flag);
+            bool ok = mbar_wait_warp(smem_u32(&bars[kQFull]), 0, abort_flag);
             const uint64_t qd0 = make_sdesc(smem_u32(sQ)), qd1 = make_sdesc(smem_u32(sQ) + kAtom);
             auto issue_qk = [&](int j) -> bool {           // S[j&1] = Q K(j)^T
                 const int s = j & 1, ks = j % NS;
-                if (!mbar_wait(smem_u32(&bars[kKFull + ks]), (uint32_t)(j / NS) & 1u, abort_flag)) return false;   // K(j) landed
+                if (!mbar_wait_warp(smem_u32(&bars[kKFull + ks]), (uint32_t)(j / NS) & 1u, abort_flag)) return false;   // K(j) landed
                 tc_fence_after();
-                const uint32_t sk = smem_u32(sK + (size_t)ks * kOperand);
+                const uint32_t sk = smem_u32(sK) + (uint32_t)(ks * kOperand);
                 const uint64_t kd0 = make_sdesc(sk), kd1 = make_sdesc(sk + kAtom);
                 const uint32_t acc = tmem_base + (uint32_t)(s * kTile);
+                if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) umma_bf16(acc, qd0 + 2 * kk, kd0 + 2 * kk, p.idesc, kk > 0);
+                    for (int kk = 0; kk < 4; ++kk) umma_bf16(acc, qd0 + 2 * kk, kd0 + 2 * kk, p.idesc, kk > 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) umma_bf16(acc, qd1 + 2 * kk, kd1 + 2 * kk, p.idesc, 1u);
-                umma_commit(smem_u32(&bars[kKEmpty + ks]));    // K stage free once these MMAs have read it
-                umma_commit(smem_u32(&bars[kSFull + s]));
+                    for (int kk = 0; kk < 4; ++kk) umma_bf16(acc, qd1 + 2 * kk, kd1 + 2 * kk, p.idesc, 1u);
+                    umma_commit(smem_u32(&bars[kKEmpty + ks]));    // K stage free once these MMAs have read it
+                    umma_commit(smem_u32(&bars[kSFull + s]));
+                }
                 return true;
             };
             ok = ok && issue_qk(0);
@@ -256,21 +265,23 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_q, cons
                 const int s = i & 1, vs = i % NS;
                 const uint32_t ph = (uint32_t)(i >> 1) & 1u;
                 if (i + 1 < n_kt && !(ok = issue_qk(i + 1))) break;                           // runs ahead of the softmax
-                if (!(ok = mbar_wait(smem_u32(&bars[kVFull + vs]), (uint32_t)(i / NS) & 1u, abort_flag))) break;   // V(i) landed
-                if (!(ok = mbar_wait(smem_u32(&bars[kPFull + s]), ph, abort_flag))) break;              // P(i) written
-                if (!(ok = mbar_wait(smem_u32(&bars[kOEmpty + s]), ph ^ 1u, abort_flag))) break;        // O_tile(i-2) folded
+                if (!(ok = mbar_wait_warp(smem_u32(&bars[kVFull + vs]), (uint32_t)(i / NS) & 1u, abort_flag))) break;   // V(i) landed
+                if (!(ok = mbar_wait_warp(smem_u32(&bars[kPFull + s]), ph, abort_flag))) break;              // P(i) written
+                if (!(ok = mbar_wait_warp(smem_u32(&bars[kOEmpty + s]), ph ^ 1u, abort_flag))) break;        // O_tile(i-2) folded
                 tc_fence_after();
-                const uint32_t sv = smem_u32(sV + (size_t)vs * kOperand);
+                const uint32_t sv = smem_u32(sV) + (uint32_t)(vs * kOperand);
                 const uint64_t vd0 = make_sdesc(sv), vd1 = make_sdesc(sv + kAtom);
                 const uint32_t acc = tmem_base + kOBase + (uint32_t)(s * kTile);
                 const uint32_t pa = tmem_base + (uint32_t)(s * kTile);       // P(i): 64 columns over S(i)
                 // O_tile = P V: reduction over the 128 keys of the tile, 16 keys = 8 columns of P per MMA
+                if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) umma_bf16_ta(acc, pa + 8 * kk, vd0 + 2 * kk, p.idesc, kk > 0);
+                    for (int kk = 0; kk < 4; ++kk) umma_bf16_ta(acc, pa + 8 * kk, vd0 + 2 * kk, p.idesc, kk > 0);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) umma_bf16_ta(acc, pa + 32 + 8 * kk, vd1 + 2 * kk, p.idesc, 1u);
-                umma_commit(smem_u32(&bars[kVEmpty + vs]));    // V stage free
-                umma_commit(smem_u32(&bars[kOFull + s]));      // O_tile(i) ready
+                    for (int kk = 0; kk < 4; ++kk) umma_bf16_ta(acc, pa + 32 + 8 * kk, vd1 + 2 * kk, p.idesc, 1u);
+                    umma_commit(smem_u32(&bars[kVEmpty + vs]));    // V stage free
+                    umma_commit(smem_u32(&bars[kOFull + s]));      // O_tile(i) ready
+                }
             }
             if (!ok) {
                 *abort_flag = 1;
@@ -644,14 +655,16 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (warp == 0) {
-            if (lane == 0) {
-                // ---------------------------------------------------- TMA producer
+            {
+                // ---------------------------------------------------- TMA producer (the whole warp)
+                const bool leader = elect_one();
                 const int bh = b * p.Hkv + kvh;
                 auto load_q = [&](int t) {
                     const Item q = item(t);
                     const uint32_t qf = smem_u32(&bars[kDQ + t]);
-                    mbar_expect_tx(qf, (uint32_t)(q.n_slots * p.slot * 256));
+                    if (leader) mbar_expect_tx(qf, (uint32_t)(q.n_slots * p.slot * 256));
                     for (int j = 0; j < q.n_slots; ++j) {
+                        if (!leader) continue;
                         const uint32_t dst = smem_u32(sQ) + (uint32_t)(t * kOperand + j * p.slot * 128);
                         tma_load_2d(dst, &map_q, qf, (q.h + j) * kTile, q.row0);
                         tma_load_2d(dst + kAtom, &map_q, qf, (q.h + j) * kTile + 64, q.row0);
@@ -663,16 +676,20 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     const int s = i & 1, kv0 = i * kTile;
                     const uint32_t ph = ((uint32_t)(i >> 1) & 1u) ^ 1u;
                     const uint32_t kf = smem_u32(&bars[kDKFull + s]), vf = smem_u32(&bars[kDVFull + s]);
-                    const uint32_t sk = smem_u32(sK + (size_t)s * kOperand), sv = smem_u32(sV + (size_t)s * kOperand);
-                    if (!(ok = mbar_wait(smem_u32(&bars[kDKEmpty + s]), ph, abort_flag))) break;
-                    mbar_expect_tx(kf, kOperand);
-                    tma_load_4d(sk, &map_k, kf, 0, kv0, bh, p.layer);             // keys kv0.., dims 0..63
-                    tma_load_4d(sk + kAtom, &map_k, kf, 64, kv0, bh, p.layer);    // dims 64..127
+                    const uint32_t sk = smem_u32(sK) + (uint32_t)(s * kOperand), sv = smem_u32(sV) + (uint32_t)(s * kOperand);
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[kDKEmpty + s]), ph, abort_flag))) break;
+                    if (leader) {
+                        mbar_expect_tx(kf, kOperand);
+                        tma_load_4d(sk, &map_k, kf, 0, kv0, bh, p.layer);             // keys kv0.., dims 0..63
+                        tma_load_4d(sk + kAtom, &map_k, kf, 64, kv0, bh, p.layer);    // dims 64..127
+                    }
                     if (i == 0 && n_q == 2) load_q(1);
-                    if (!(ok = mbar_wait(smem_u32(&bars[kDVEmpty + s]), ph, abort_flag))) break;
-                    mbar_expect_tx(vf, kOperand);
-                    tma_load_4d(sv, &map_vt, vf, kv0, 0, bh, p.layer);            // all dims, keys kv0..kv0+63
-                    tma_load_4d(sv + kAtom, &map_vt, vf, kv0 + 64, 0, bh, p.layer);
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[kDVEmpty + s]), ph, abort_flag))) break;
+                    if (leader) {
+                        mbar_expect_tx(vf, kOperand);
+                        tma_load_4d(sv, &map_vt, vf, kv0, 0, bh, p.layer);            // all dims, keys kv0..kv0+63
+                        tma_load_4d(sv + kAtom, &map_vt, vf, kv0 + 64, 0, bh, p.layer);
+                    }
                 }
                 if (!ok) {
                     *abort_flag = 1;
@@ -681,13 +698,15 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
             }
             __syncwarp();
         } else if (warp == 1) {
-            if (lane == 0) {
-                // ---------------------------------------------------- MMA issuer
+            {
+                // ---------------------------------------------------- MMA issuer (the whole warp)
+                const bool leader = elect_one();
                 auto issue_qk = [&](int t, int i) {                   // S_t = Q_t K(i)^T
-                    const uint64_t qd = make_sdesc(smem_u32(sQ + (size_t)t * kOperand));
-                    const uint64_t kd = make_sdesc(smem_u32(sK + (size_t)(i & 1) * kOperand));
+                    if (!leader) return;
+                    const uint64_t qd = make_sdesc(smem_u32(sQ) + (uint32_t)(t * kOperand));
+                    const uint64_t kd = make_sdesc(smem_u32(sK) + (uint32_t)((i & 1) * kOperand));
                     const uint32_t acc = tmem_base + (uint32_t)(t * kTile);
-    #pragma unroll
+#pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {
                         const uint64_t o = (uint64_t)((kk >> 2) * (kAtom >> 4) + 2 * (kk & 3));
                         umma_bf16(acc, qd + o, kd + o, p.idesc, kk > 0);
@@ -695,27 +714,29 @@ attention_tc_dual_kernel(const __grid_constant__ CUtensorMap map_q, const __grid
                     umma_commit(smem_u32(&bars[kDSFull + t]));
                     if (t == n_q - 1) umma_commit(smem_u32(&bars[kDKEmpty + (i & 1)]));     // K stage free
                 };
-                bool ok = mbar_wait(smem_u32(&bars[kDKFull]), 0, abort_flag);
+                bool ok = mbar_wait_warp(smem_u32(&bars[kDKFull]), 0, abort_flag);
                 for (int t = 0; t < n_q && ok; ++t) {
-                    if (!(ok = mbar_wait(smem_u32(&bars[kDQ + t]), 0, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[kDQ + t]), 0, abort_flag))) break;
                     tc_fence_after();
                     issue_qk(t, 0);
                 }
                 for (int i = 0; i < n_kt && ok; ++i) {
                     const uint32_t ph = (uint32_t)(i >> 1) & 1u;
-                    if (!(ok = mbar_wait(smem_u32(&bars[kDVFull + (i & 1)]), ph, abort_flag))) break;          // V(i) landed
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[kDVFull + (i & 1)]), ph, abort_flag))) break;          // V(i) landed
                     for (int t = 0; t < n_q; ++t) {
-                        if (!(ok = mbar_wait(smem_u32(&bars[kDPFull + t]), (uint32_t)i & 1u, abort_flag))) break;   // P_t(i) written, O_t rescaled
+                        if (!(ok = mbar_wait_warp(smem_u32(&bars[kDPFull + t]), (uint32_t)i & 1u, abort_flag))) break;   // P_t(i) written, O_t rescaled
                         tc_fence_after();
-                        const uint64_t vd = make_sdesc(smem_u32(sV + (size_t)(i & 1) * kOperand));
+                        const uint64_t vd = make_sdesc(smem_u32(sV) + (uint32_t)((i & 1) * kOperand));
                         const uint32_t acc = tmem_base + (uint32_t)(2 * kTile + t * kTile), pa = tmem_base + (uint32_t)(t * kTile);
-    #pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)                // 16 keys = 8 columns of P per MMA
-                            umma_bf16_ta(acc, pa + 8 * kk, vd + (uint64_t)((kk >> 2) * (kAtom >> 4) + 2 * (kk & 3)), p.idesc, (i > 0 || kk > 0) ? 1u : 0u);
-                        if (t == n_q - 1) umma_commit(smem_u32(&bars[kDVEmpty + (i & 1)]));     // V stage free
-                        if (i == n_kt - 1) umma_commit(smem_u32(&bars[kDODone + t]));
+                        if (leader) {
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk)                // 16 keys = 8 columns of P per MMA
+                                umma_bf16_ta(acc, pa + 8 * kk, vd + (uint64_t)((kk >> 2) * (kAtom >> 4) + 2 * (kk & 3)), p.idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                            if (t == n_q - 1) umma_commit(smem_u32(&bars[kDVEmpty + (i & 1)]));     // V stage free
+                            if (i == n_kt - 1) umma_commit(smem_u32(&bars[kDODone + t]));
+                        }
                         if (i + 1 < n_kt) {
-                            if (t == 0 && !(ok = mbar_wait(smem_u32(&bars[kDKFull + ((i + 1) & 1)]), (uint32_t)((i + 1) >> 1) & 1u, abort_flag))) break;
+                            if (t == 0 && !(ok = mbar_wait_warp(smem_u32(&bars[kDKFull + ((i + 1) & 1)]), (uint32_t)((i + 1) >> 1) & 1u, abort_flag))) break;
                             tc_fence_after();
                             issue_qk(t, i + 1);
                         }

@@ -128,8 +128,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const uint32_t tmem_sf = tmem_base + 2u * (uint32_t)p.buf_cols;      // two slots of 32 columns: 16 for A, 16 for B
 
     if (warp == 0) {
-        if (lane == 0 && n_total > 0) {
-            // ------------------------------------------------ TMA producer
+        if (n_total > 0) {
+            // ------------------------------------------------ TMA producer (the whole warp, see elect_one)
+            const bool leader = elect_one();
             uint64_t pol_stream;
             asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
             struct Walk { int g, left, kb, n0, tok0; };
@@ -143,13 +144,15 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 if (--w.left == 0 && w.g < g_end) enter(w);
             };
             auto load_w = [&](const Walk& w, int s) {
-                const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes), full = smem_u32(&bars[s]);
+                if (!leader) return;
+                const uint32_t sa = smem_u32(smem) + (uint32_t)(s * stage_bytes), full = smem_u32(&bars[s]);
                 mbar_expect_tx(full, (uint32_t)(kStageW + x_bytes + kSfW + sfx_bytes));
                 tma_load_2d_hint(sa, &map_w, full, w.kb * 128, w.n0, pol_stream);
                 tma_load_2d(sa + kStageW + x_bytes, &map_sw, full, w.kb * 16, w.n0);
             };
             auto load_x = [&](const Walk& w, int s) {
-                const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes), full = smem_u32(&bars[s]);
+                if (!leader) return;
+                const uint32_t sa = smem_u32(smem) + (uint32_t)(s * stage_bytes), full = smem_u32(&bars[s]);
                 tma_load_2d(sa + kStageW, &map_x, full, w.kb * 128, w.tok0);
                 tma_load_2d(sa + kStageW + x_bytes + kSfW, &map_sx, full, w.kb * 16, w.tok0);
             };
@@ -169,7 +172,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             int s = n_pre % NS;
             uint32_t ph = (uint32_t)(n_pre / NS) & 1u;
             for (int i = n_pre; i < n_total; ++i, advance(w)) {
-                if (!mbar_wait(smem_u32(&bars[NS + s]), ph ^ 1u, abort_flag)) {
+                if (!mbar_wait_warp(smem_u32(&bars[NS + s]), ph ^ 1u, abort_flag)) {
                     *abort_flag = 1;
                     atomicCAS(p.status, 0, WD_ERR_DEVICE_TIMEOUT);
                     break;
@@ -181,8 +184,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ------------------------------------------------ MMA issuer
+        {
+            // ------------------------------------------------ MMA issuer (the whole warp)
+            const bool leader = elect_one();
             bool ok = true;
             int s = 0, i = 0;
             uint32_t ph = 0;
@@ -192,26 +196,28 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 g += kbn;
                 const int buf = u & 1;
                 const uint32_t par = (uint32_t)(u >> 1) & 1u;
-                if (!(ok = mbar_wait(smem_u32(&acc_empty[buf]), par ^ 1u, abort_flag))) break;
+                if (!(ok = mbar_wait_warp(smem_u32(&acc_empty[buf]), par ^ 1u, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t acc = tmem_base + (uint32_t)(buf * p.buf_cols);
                 for (int j = 0; j < kbn; ++j, ++i) {
                     const int slot = i & 1;
-                    if (!(ok = mbar_wait(smem_u32(&bars[s]), ph, abort_flag))) break;                       // codes landed
-                    if (!(ok = mbar_wait(smem_u32(&sf_full[slot]), (uint32_t)(i >> 1) & 1u, abort_flag))) break;   // scales in tensor memory
+                    if (!(ok = mbar_wait_warp(smem_u32(&bars[s]), ph, abort_flag))) break;                       // codes landed
+                    if (!(ok = mbar_wait_warp(smem_u32(&sf_full[slot]), (uint32_t)(i >> 1) & 1u, abort_flag))) break;   // scales in tensor memory
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
+                    const uint32_t sa = smem_u32(smem) + (uint32_t)(s * stage_bytes);
                     const uint64_t adesc = make_sdesc(sa), bdesc = make_sdesc(sa + kStageW);
                     const uint32_t sf = tmem_sf + (uint32_t)(slot * 32);
+                    if (leader) {
 #pragma unroll
-                    for (int kq = 0; kq < 4; ++kq)       // 64 elements = 32 bytes further along K: +2 in 16-byte units
-                        umma_fp4(acc, adesc + (uint64_t)(2 * kq), bdesc + (uint64_t)(2 * kq), p.idesc, sf + (uint32_t)(4 * kq),
-                                 sf + 16u + (uint32_t)(4 * kq), (j > 0 || kq > 0) ? 1u : 0u);
-                    umma_commit(smem_u32(&bars[NS + s]));      // stage free once these MMAs have read it
-                    umma_commit(smem_u32(&sf_free[slot]));     // ... and the scale slot
+                        for (int kq = 0; kq < 4; ++kq)       // 64 elements = 32 bytes further along K: +2 in 16-byte units
+                            umma_fp4(acc, adesc + (uint64_t)(2 * kq), bdesc + (uint64_t)(2 * kq), p.idesc, sf + (uint32_t)(4 * kq),
+                                     sf + 16u + (uint32_t)(4 * kq), (j > 0 || kq > 0) ? 1u : 0u);
+                        umma_commit(smem_u32(&bars[NS + s]));      // stage free once these MMAs have read it
+                        umma_commit(smem_u32(&sf_free[slot]));     // ... and the scale slot
+                    }
                     if (++s == NS) { s = 0; ph ^= 1u; }
                 }
-                if (ok) umma_commit(smem_u32(&acc_full[buf]));
+                if (ok && leader) umma_commit(smem_u32(&acc_full[buf]));
             }
             if (!ok) {
                 *abort_flag = 1;
