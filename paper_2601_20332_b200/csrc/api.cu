@@ -1465,9 +1465,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         } else {
         WdTcSeg qkv[3] = {{c->wq[l], hq, c->tc.get(WD_TC_WQ, l)}, {c->wk[l], hkv, c->tc.get(WD_TC_WK, l)},
                           {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
-        // (Heads without grouping only, so far.  With 28 query over 4 KV heads a refresh of four blocks would also be 1-2 % faster
-        // for it where the rounds are full: 5376 rows 7370 / 7270 us, 6080 rows 8000 / 7830, 6880 rows 9150 / 8990.)
-        if (use_tc(c) && dh == 128 && Hq == Hkv && !split_norm) {
+        if (use_tc(c) && dh == 128 && !split_norm) {
             rope.map_q = c->tc.get(WD_TC_WQ_ROT, l); rope.map_k = c->tc.get(WD_TC_WK_ROT, l);
             rope.row_seq = row_seq; rope.row_pos = row_pos; rope.rope_tab = c->rope_tab;
             rope.q = (__nv_bfloat16*)c->q; rope.kcache = (__nv_bfloat16*)kc; rope.vcache = (__nv_bfloat16*)vc;

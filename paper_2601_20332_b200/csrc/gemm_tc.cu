@@ -1703,6 +1703,40 @@ int gate_up_tok_tiles(int tiles, int kb_total, int rows, int pairs, int n) {
     return best;
 }
 
+// Token tiles of a launch with one accumulator set in whole units (a round of them walks K in step, so that a weight block and a token
+// block are fetched by all who want them at about the same time), or 0 for equal shares of the K-block line.  Estimated in us at
+// 1.8 GHz: a K block of a whole unit takes 390 cycles to load and issue, or its MMAs, 2 a token; one of a share 700 (the pairs are
+// everywhere in the line, operands come from farther away; 620 with one group of pairs per token tile); a share's slices are written
+// and read again, and the rotation kernel runs that a unit's epilogue replaces.  A unit's end 3 at 256 tokens.  More tiles than the
+// fewest only for a gain of 5 %: full rounds also draw more power.
+// Measured against the fewest tiles, whole where two rounds were full and shares otherwise, us a block: LLaDA shape, output / down
+// projection: 583 rows in four tiles -8 / -10, 900 in four -10 / -18, 1216 in eight -15 / -9, 1551 in nine -24 / -21 (352 in four
+// 0 / +10: shares); q/k/v 352 in two -9, 1216 in six -5 (1551 in nine +5: seven).  Dream shape, down 530 rows in four -21, 1000 in five
+// -38; output projection 530 in five -6, 1000 in eight -11; q/k/v 530 in four -5, 1000 in four -9.
+int whole_unit_tok_tiles(int tiles, int kb_total, int rows, int ncol, int pairs, int epi) {
+    const int least = (rows + 255) / 256, bn_least = ((rows + least - 1) / least + 15) / 16 * 16;
+    const bool groups = least == 2 && pairs % 2 == 0;
+    const double bytes = 4.0 * rows * ncol;
+    const double rotation = epi == kEpiRope ? 2.0 + bytes * 0.5 / 5e6 : 0.0;
+    const int units_shared = groups ? tiles : tiles * least, pairs_shared = groups ? pairs / 2 : pairs;
+    const int slices = wd_tc_sharers(units_shared, pairs_shared);
+    double t_best = (double)tiles * least * kb_total / pairs * std::max(groups ? 620 : 700, 2 * bn_least) / 1800.0 + 3.0 +
+                    bytes * slices * 0.22e-6 + rotation;
+    if (tiles * least >= 2 * pairs) t_best = 1e30;              // (many units: rounds of whole ones are full enough)
+    int best = 0;
+    for (int t = least; t < least + 6; ++t) {
+        const int bn = ((rows + t - 1) / t + 15) / 16 * 16, n_rounds = (tiles * t + pairs - 1) / pairs;
+        if (10 * tiles * t < 7 * pairs) continue;
+        const double us = (double)n_rounds * kb_total * std::max(390, 2 * bn) / 1800.0 + 3.0 + bn * 3.0 / 256 +
+                          (epi == kEpiPlain ? bytes / 5e6 : 0.0);
+        if (us < (best ? 0.95 : 1.0) * t_best) {
+            t_best = us;
+            best = t;
+        }
+    }
+    return best;
+}
+
 // launch of gemm_tc_pair_kernel: same contract as wd_tc_gemm
 wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, int K, float* y, size_t y_floats,
                        int sm_count, int32_t* status, cudaStream_t stream, int* n_split_out, bool force_single_split,
@@ -1725,7 +1759,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     // overlaps the next tile.  Measured: pays for the widest weight matrices (gate/up) once every pair
     // gets at least two whole units, costs 10-25 % on the narrow ones.  0 = never, 1 = that rule, 2 = always.
     static const int dual_mode = env_int("WD_GEMM_DUAL", 1);
-    int gu_tok_tiles = 0;
+    int gu_tok_tiles = 0, unit_tok_tiles = 0;
     {
         int tiles_all = 0, ncol_all = 0;
         for (int i = 0; i < nseg; ++i) {
@@ -1741,23 +1775,25 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
         if (sg && sg->h && swiglu_fused && !fp8 && nseg == 2 && segs[0].n == segs[1].n && dual_mode != 0)
             gu_tok_tiles = gate_up_tok_tiles((segs[0].n + p.tile_rows - 1) / p.tile_rows, (K + kBK - 1) / kBK, rows, (int)pairs, segs[0].n);
         if (gu_tok_tiles > 0) p.dual = 2;
-        // RoPE or the residual add in the epilogue: the same condition on whole units of one accumulator (with shares of the K-block
-        // line a tile's sum is in several pieces)
+        // one accumulator: whole units (with RoPE or the residual add in their epilogue where the launch has one: with shares of the
+        // K-block line a tile's sum is in several pieces), or shares
         static const int epi_on = env_int("WD_GEMM_EPI", 3);
-        if (!fp8 && p.dual != 2 && full_rounds((long long)tiles_all * ((rows + 255) / 256), pairs)) {
-            if (rope && nseg == 3 && (epi_on & 1)) epi = kEpiRope;
-            else if (resid && resid->x && nseg == 1 && (epi_on & 2)) epi = kEpiResid;
-        }
-        if (epi != kEpiPlain) {
-            p.dual = 0;
-            force_single_split = true;
+        if (!fp8 && p.dual == 0 && !force_single_split) {
+            int want = kEpiPlain;
+            if (rope && nseg == 3 && (epi_on & 1)) want = kEpiRope;
+            else if (resid && resid->x && nseg == 1 && (epi_on & 2)) want = kEpiResid;
+            unit_tok_tiles = whole_unit_tok_tiles(tiles_all, (K + kBK - 1) / kBK, rows, ncol_all, (int)pairs, want);
+            if (unit_tok_tiles > 0) {
+                epi = want;
+                force_single_split = true;
+            }
         }
     }
     if (p.dual == 1) {
         p.tok_tiles = (rows + 511) / 512;                                   // super-tiles
         p.bn = ((rows + 2 * p.tok_tiles - 1) / (2 * p.tok_tiles) + 15) / 16 * 16;   // balanced, <= 256
     } else {
-        p.tok_tiles = p.dual == 2 ? gu_tok_tiles : (rows + 255) / 256;
+        p.tok_tiles = p.dual == 2 ? gu_tok_tiles : unit_tok_tiles > 0 ? unit_tok_tiles : (rows + 255) / 256;
         p.bn = ((rows + p.tok_tiles - 1) / p.tok_tiles + 15) / 16 * 16;    // balanced token tiles, <= 256
     }
     int cols = 32;
@@ -1798,7 +1834,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
     p.rows = rows;
     p.kb_total = (K + kke - 1) / kke;
     // two token tiles: one group of pairs per token tile, walking the weight K blocks in step
-    const int ts = (!p.dual && epi == kEpiPlain && p.tok_tiles == 2 && (sm_count / 2) % 2 == 0) ? 2 : 1;
+    const int ts = (!p.dual && unit_tok_tiles == 0 && p.tok_tiles == 2 && (sm_count / 2) % 2 == 0) ? 2 : 1;
     p.tok_split = ts;
     p.n_units = ts > 1 ? tiles : tiles * p.tok_tiles;
     if ((long long)p.n_units * p.kb_total > INT_MAX) return WD_ERR_CAPACITY;
