@@ -1288,10 +1288,6 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         c->chain_dirty = false;
     }
     const bool f32 = d.dtype == WD_F32;
-    // few bf16 rows: 1 / rms multiplies the results of q/k/v and gate/up, where their slices are added
-    const bool split_norm = use_tc(c) && !fused && !c->fp8_on && !c->fp4_on && wd_rmsnorm_split_ok(R_, D);
-    WdRowScale row_scale;
-    if (split_norm) { row_scale.sumsq = c->sumsq; row_scale.inv_d = 1.f / (float)D; row_scale.eps = d.rms_eps; }
     const bool fp8 = c->fp8_on && use_tc(c) && !fused;      // FP8 projections (q/k/v, gate/up, down, LM head)
     const bool fp4 = c->fp4_on && use_tc(c) && !fused;      // NVFP4 projections (the same ones)
     WdFp4Operand x4_d, x4_f, x4_lm;                         // the step's quantised activations, by use
@@ -1433,10 +1429,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                 return s;
         }
         // attention half (FP8 mode: the normalised rows leave the RMSNorm as e4m3 codes + row scales)
-        if (split_norm)
-            wd_launch_rmsnorm_split(c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride, c->attn_norm[l], c->xn,
-                                    c->sumsq, R_, D, stream);
-        else if (!pq.done)
+        if (!pq.done)
             wd_launch_rmsnorm(d.dtype, c->x, down_pending ? c->part : nullptr, down_go.n_split, down_go.split_stride,
                           c->attn_norm[l], d.rms_eps, c->xn, nullptr, R_, D, stream, fp8 ? c->xn8 : nullptr, c->sxn,
                           fp4 ? &x4_d : nullptr);
@@ -1465,7 +1458,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         } else {
         WdTcSeg qkv[3] = {{c->wq[l], hq, c->tc.get(WD_TC_WQ, l)}, {c->wk[l], hkv, c->tc.get(WD_TC_WK, l)},
                           {c->wv[l], hkv, c->tc.get(WD_TC_WV, l)}};
-        if (use_tc(c) && dh == 128 && !split_norm) {
+        if (use_tc(c) && dh == 128) {
             rope.map_q = c->tc.get(WD_TC_WQ_ROT, l); rope.map_k = c->tc.get(WD_TC_WK_ROT, l);
             rope.row_seq = row_seq; rope.row_pos = row_pos; rope.rope_tab = c->rope_tab;
             rope.q = (__nv_bfloat16*)c->q; rope.kcache = (__nv_bfloat16*)kc; rope.vcache = (__nv_bfloat16*)vc;
@@ -1483,7 +1476,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                                    dh, S, Sp, batch, status, stream);
         else
             wd_launch_rope_scatter(d.dtype, c->part, go.n_split, go.split_stride, row_seq, row_pos, c->rope_tab, c->q, kc,
-                                   vc, R_, Hq, Hkv, dh, S, Sp, batch, status, stream, row_scale);
+                                   vc, R_, Hq, Hkv, dh, S, Sp, batch, status, stream);
         if ((s = attention(l, kc, vc, act)) != WD_OK) return s;
         // from here on the block works on these rows
         const int Rb = act ? NA : R_;
@@ -1521,10 +1514,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             return s;
         }
         // feed-forward half
-        if (split_norm)
-            wd_launch_rmsnorm_split(xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], xnb, c->sumsq, Rb, D,
-                                    stream);
-        else if (!pg.done)
+        if (!pg.done)
             wd_launch_rmsnorm(d.dtype, xb, resid_o.done ? nullptr : c->part, go.n_split, go.split_stride, c->ffn_norm[l], d.rms_eps, xnb,
                           nullptr, Rb, D, stream, fp8 ? c->xn8 : nullptr, c->sxn, fp4 ? &x4_d : nullptr);
         if (fp4) {
@@ -1547,14 +1537,14 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                 return s;
         } else {
         WdTcSwiglu sg;
-        sg.h = use_tc(c) && !split_norm ? (__nv_bfloat16*)c->h : nullptr;
+        sg.h = use_tc(c) ? (__nv_bfloat16*)c->h : nullptr;
         WdTcEpi epi_sg;
         epi_sg.sg = &sg;
         if (!pg.done) {
             if ((s = run_gemm(c, xnb, xmb, gu, 2, Rb, D, c->part, c->part_floats, status, stream, &go, false,
                               nullptr, nullptr, &epi_sg)) != WD_OK)
                 return s;
-            if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream, row_scale);
+            if (!sg.done) wd_launch_swiglu(d.dtype, c->part, go.n_split, go.split_stride, c->h, Rb, F, stream);
         }
         WdTcSeg wdn[1] = {{c->wd[l], D, c->tc.get(WD_TC_WD, l)}};
         if (f32) {                      // (x is complete: the output projection or the RMSNorm after it has added its sums)

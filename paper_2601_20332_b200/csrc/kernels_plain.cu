@@ -551,50 +551,6 @@ __global__ void __maxnreg__(88) rmsnorm_rows_kernel(float* __restrict__ x, const
     }
 }
 
-// The residual add and the gains alone, for steps of few rows: with a block to a row the 130 KB of a row and its K slices come in
-// through one SM, about 2 us, and the row's sum has to be complete before anything is written.  Here four blocks share a row, write
-// xg = bf16(x * gain) as soon as x is complete and leave the sum of squares of their quarter; 1 / rms multiplies the projection's
-// result instead, where its slices are added anyway (WdRowScale: RoPE, SwiGLU).  As many rounding steps as before, bf16 being as
-// exact at any scale.  Bound by one round trip to the L2, beside the next GEMM's weights that come into the same SMs.  Measured with
-// one block to a row / four, 34 rows of 4096, step of eight blocks 960 / 946 us (4.1 -> 3.4 us a launch); 68 rows 3.6 -> 3.0 us a launch.
-constexpr int kNormParts = 4;
-__global__ void __launch_bounds__(256) rmsnorm_split_kernel(float* __restrict__ x, const float* __restrict__ part, int n_split,
-                                                            size_t split_stride, const float* __restrict__ gain,
-                                                            __nv_bfloat16* __restrict__ xg, float* __restrict__ sumsq, int d) {
-    __shared__ float red[8];
-    pdl_launch_dependents();
-    const int nv = d >> 4, r = blockIdx.y;                      // float4 of this block
-    const size_t c = 4 * ((size_t)blockIdx.x * nv + threadIdx.x), at = (size_t)r * d + c;
-    const bool on = (int)threadIdx.x < nv;
-    const float4 g = on ? ld_f4_pinned(gain + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-    pdl_wait();
-    S_STAMP(1);
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (on) {
-        a = ld_f4_pinned(x + at);
-        if (part) {
-            const float4 add = sum_slices4_pinned(part + at, n_split, split_stride);
-            a.x += add.x; a.y += add.y; a.z += add.z; a.w += add.w;
-            *reinterpret_cast<float4*>(x + at) = a;
-        }
-        Vec4<__nv_bfloat16>::store(xg + at, a.x * g.x, a.y * g.y, a.z * g.z, a.w * g.w);
-    }
-    const float ss = warp_sum(a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        sumsq[(size_t)r * kNormParts + blockIdx.x] = t;
-    }
-}
-// the factor of row r
-__device__ __forceinline__ float row_scale(const WdRowScale& sc, int r) {
-    if (!sc.sumsq) return 1.f;
-    const float4 s = ld_f4_pinned(sc.sumsq + (size_t)r * kNormParts);
-    return rsqrtf(((s.x + s.y) + (s.z + s.w)) * sc.inv_d + sc.eps);
-}
-
 // The same with NVFP4 output of the bfloat16 rounding of the normalised row (a kernel of its own, so that the
 // bf16 path's kernel carries neither its arguments nor its code): row scale max / (6 * 448), then blocks of 16
 // elements held by four neighbouring lanes.  d % 16 == 0.
@@ -665,8 +621,7 @@ __global__ void __launch_bounds__(256, 4) rope_scatter_kernel(const float* __res
                                     const int32_t* __restrict__ row_seq, const int32_t* __restrict__ row_pos,
                                     const float2* __restrict__ rope_tab, T* __restrict__ q, T* __restrict__ kcache,
                                     T* __restrict__ vcache, int n_rows, int Hq, int Hkv, int dh, int S, int Sp,
-                                    int n_qk, int qk_groups, int n_qk_blocks, int batch, int32_t* __restrict__ status,
-                                    const WdRowScale scale) {
+                                    int n_qk, int qk_groups, int n_qk_blocks, int batch, int32_t* __restrict__ status) {
     __shared__ float tile[32][33];
     pdl_launch_dependents();
     pdl_wait();
@@ -683,7 +638,6 @@ __global__ void __launch_bounds__(256, 4) rope_scatter_kernel(const float* __res
             const bool in_range = (unsigned)pos < (unsigned)S && (unsigned)b < (unsigned)batch;
             if (!in_range && threadIdx.x == 0) atomicCAS(status, 0, WD_ERR_BOUNDS);
             const float* pr = part + (size_t)r * ncol;
-            const float inv = row_scale(scale, r);
             if ((half & 3) == 0) {
                 // four rotation pairs per thread (float4 loads, 8-byte bf16 stores): half/4 threads per head
                 const int tph = half >> 2, hpb = blockDim.x / tph;
@@ -717,8 +671,6 @@ __global__ void __launch_bounds__(256, 4) rope_scatter_kernel(const float* __res
                         c23 = *reinterpret_cast<const float4*>(rope_tab + (size_t)r * half + j + 2);
                     }
                     if (h >= Hq && !in_range) continue;
-                    a.x *= inv; a.y *= inv; a.z *= inv; a.w *= inv;
-                    bb.x *= inv; bb.y *= inv; bb.z *= inv; bb.w *= inv;
                     T* dst = h < Hq ? q + ((size_t)r * Hq + h) * dh : kcache + (((size_t)b * Hkv + (h - Hq)) * S + pos) * dh;
                     Vec4<T>::store(dst + j, a.x * c01.x - bb.x * c01.y, a.y * c01.z - bb.y * c01.w, a.z * c23.x - bb.z * c23.y,
                                    a.w * c23.z - bb.w * c23.w);
@@ -732,8 +684,8 @@ __global__ void __launch_bounds__(256, 4) rope_scatter_kernel(const float* __res
                 const int h = h0 + i / half, j = i % half;
                 if (h >= Hq + Hkv) break;
                 if (h >= Hq && !in_range) continue;
-                const float a = sum_slices1(pr + h * dh + j, n_split, split_stride) * inv;
-                const float bb = sum_slices1(pr + h * dh + j + half, n_split, split_stride) * inv;
+                const float a = sum_slices1(pr + h * dh + j, n_split, split_stride);
+                const float bb = sum_slices1(pr + h * dh + j + half, n_split, split_stride);
                 const float2 cs = rope_tab[(size_t)r * half + j];
                 const float ra = a * cs.x - bb * cs.y, rb = bb * cs.x + a * cs.y;
                 T* dst = h < Hq ? q + ((size_t)r * Hq + h) * dh : kcache + (((size_t)b * Hkv + (h - Hq)) * S + pos) * dh;
@@ -755,17 +707,13 @@ __global__ void __launch_bounds__(256, 4) rope_scatter_kernel(const float* __res
         // one float4 (four head dims of one row) per thread
         const int rr = threadIdx.x >> 3, d4 = (threadIdx.x & 7) * 4, r = r0 + rr;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        float inv = 1.f;
-        if (r < n_rows && d0 + d4 < dh) {
-            inv = row_scale(scale, r);
-            v = sum_slices4(part + (size_t)r * ncol + vcol + d4, n_split, split_stride);
-        }
-        tile[rr][d4] = v.x * inv; tile[rr][d4 + 1] = v.y * inv; tile[rr][d4 + 2] = v.z * inv; tile[rr][d4 + 3] = v.w * inv;
+        if (r < n_rows && d0 + d4 < dh) v = sum_slices4(part + (size_t)r * ncol + vcol + d4, n_split, split_stride);
+        tile[rr][d4] = v.x; tile[rr][d4 + 1] = v.y; tile[rr][d4 + 2] = v.z; tile[rr][d4 + 3] = v.w;
     } else {
         for (int rr = ly; rr < 32; rr += 8) {
             const int r = r0 + rr;
             tile[rr][lx] = (r < n_rows && d0 + lx < dh)
-                ? sum_slices1(part + (size_t)r * ncol + vcol + lx, n_split, split_stride) * row_scale(scale, r) : 0.f;
+                ? sum_slices1(part + (size_t)r * ncol + vcol + lx, n_split, split_stride) : 0.f;
         }
     }
     __syncthreads();
@@ -1012,7 +960,7 @@ __global__ void __launch_bounds__(256, 5) swiglu_kernel(const float* __restrict_
 // slices each) in flight together; registers capped like the kernel above, for the same reason.
 template <typename T>
 __global__ void __launch_bounds__(256, 5) swiglu_rows_kernel(const float* __restrict__ part, int n_split, size_t split_stride,
-                                                             T* __restrict__ h, int n_rows, int F, const WdRowScale scale) {
+                                                             T* __restrict__ h, int n_rows, int F) {
     pdl_launch_dependents();
     pdl_wait();
     S_STAMP(3);
@@ -1022,7 +970,6 @@ __global__ void __launch_bounds__(256, 5) swiglu_rows_kernel(const float* __rest
     const int r = i / f4, c = i - r * f4;
     const float* pg = part + (size_t)r * 2 * F + 4 * c;
     float4 tg[4], tu[4];
-    const float inv = row_scale(scale, r);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         tg[k] = tu[k] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1043,8 +990,6 @@ __global__ void __launch_bounds__(256, 5) swiglu_rows_kernel(const float* __rest
         g.x += a.x; g.y += a.y; g.z += a.z; g.w += a.w;
         u.x += b.x; u.y += b.y; u.z += b.z; u.w += b.w;
     }
-    g.x *= inv; g.y *= inv; g.z *= inv; g.w *= inv;
-    u.x *= inv; u.y *= inv; u.z *= inv; u.w *= inv;
     Vec4<T>::store(h + (size_t)r * F + 4 * c, g.x / (1.f + __expf(-g.x)) * u.x, g.y / (1.f + __expf(-g.y)) * u.y,
                    g.z / (1.f + __expf(-g.z)) * u.z, g.w / (1.f + __expf(-g.w)) * u.w);
 }
@@ -1400,19 +1345,6 @@ void wd_launch_rmsnorm(int dtype, float* x, const float* part, int n_split, size
     }
 }
 
-// Up to 128 rows, where a block to a row leaves SMs idle (beyond, the RMSNorm of one block to a row is bound by its bytes), widths that
-// fill the four blocks' 128 to 256 threads.
-bool wd_rmsnorm_split_ok(int n_rows, int d) {
-    return n_rows <= 128 && d % 64 == 0 && d >= 2048 && d <= 4096;
-}
-
-void wd_launch_rmsnorm_split(float* x, const float* part, int n_split, size_t split_stride, const float* gain, void* xg, float* sumsq,
-                             int n_rows, int d, cudaStream_t st) {
-    if (n_rows <= 0) return;
-    launch_pdl(rmsnorm_split_kernel, dim3(kNormParts, n_rows), dim3((d / 16 + 31) / 32 * 32), 0, st, x, part, n_split, split_stride,
-               gain, (__nv_bfloat16*)xg, sumsq, d);
-}
-
 void wd_launch_gather_active(const float* x, const void* xn, const float2* rope_tab, const int32_t* row_seq, const int32_t* act_row,
                              float* x_act, void* xn_act, float2* rope_act, int32_t* seq_act, int n_act, int d, int half, cudaStream_t st) {
     if (n_act <= 0) return;
@@ -1423,7 +1355,7 @@ void wd_launch_gather_active(const float* x, const void* xn, const float2* rope_
 void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t split_stride,
                             const int32_t* row_seq, const int32_t* row_pos, const float2* rope_tab, void* q,
                             void* kcache, void* vcache, int n_rows, int Hq, int Hkv, int dh, int S, int Sp,
-                            int batch, int32_t* status, cudaStream_t st, const WdRowScale& scale) {
+                            int batch, int32_t* status, cudaStream_t st) {
     if (n_rows <= 0) return;
     const int half = dh >> 1;
     const int qk_groups = (half & 3) == 0 ? wd_ceil_div(Hq + Hkv, std::max(1, 256 / (half >> 2))) : wd_ceil_div(Hq + Hkv, 4);
@@ -1432,7 +1364,7 @@ void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t sp
     const int n_qk_blocks = std::min(n_qk, 148 * 8);
     WD_DISPATCH(dtype, launch_pdl(rope_scatter_kernel<T>, dim3(n_qk_blocks + n_v), dim3(256), 0, st, part, n_split,
                                   split_stride, row_seq, row_pos, rope_tab, (T*)q, (T*)kcache, (T*)vcache, n_rows, Hq,
-                                  Hkv, dh, S, Sp, n_qk, qk_groups, n_qk_blocks, batch, status, scale));
+                                  Hkv, dh, S, Sp, n_qk, qk_groups, n_qk_blocks, batch, status));
 }
 
 template <typename T, bool kVec, bool kFew>
@@ -1478,7 +1410,7 @@ void wd_launch_attention_plain(int dtype, const void* q, const void* kcache, con
 }
 
 void wd_launch_swiglu(int dtype, const float* part, int n_split, size_t split_stride, void* h,
-                      int n_rows, int F, cudaStream_t st, const WdRowScale& scale) {
+                      int n_rows, int F, cudaStream_t st) {
     if (n_rows <= 0) return;
     const size_t total = (size_t)n_rows * (F >> 2);
     static const int sw_rows = getenv("WD_SWIGLU_ROWS") ? atoi(getenv("WD_SWIGLU_ROWS")) : 1;
@@ -1486,9 +1418,9 @@ void wd_launch_swiglu(int dtype, const float* part, int n_split, size_t split_st
     // rows, 10.4 / 7.7 us at 352 rows, where two pay).  Normal step of four blocks, one / two, in us: 12288 wide 170 rows 665 / 687,
     // 204 rows 730 / 753, 238 rows 777 / 798, 272 rows 958 / 958; 18944 wide 140 rows 589 / 585, 210 rows 686 / 678.
     static const int sw_rows_max = getenv("WD_SWIGLU_ROWS_MAX") ? atoi(getenv("WD_SWIGLU_ROWS_MAX")) : 600000;
-    if (scale.sumsq || (sw_rows && total <= (size_t)sw_rows_max)) {
+    if (sw_rows && total <= (size_t)sw_rows_max) {
         WD_DISPATCH(dtype, launch_pdl(swiglu_rows_kernel<T>, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, part, n_split,
-                                      split_stride, (T*)h, n_rows, F, scale));
+                                      split_stride, (T*)h, n_rows, F));
         return;
     }
     const int blocks = (int)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);

@@ -112,17 +112,6 @@ void wd_launch_rmsnorm(int dtype, float* x, const float* part, int n_split, size
 // (xq != null: FP8 output instead of xn: e4m3 codes [n_rows][d] and one scale per row;
 //  x4 != null: NVFP4 output instead of xn, quantised from the bfloat16 rounding of the normalised row; d % 16 == 0)
 
-// The same for steps of few rows without the division by the root mean square: x += sum_s part[s], xg = bf16(x * gain), and the sums
-// of squares of each row's four quarters, sumsq[n_rows][4], from which whoever adds the projection's slices takes 1 / rms
-// (WdRowScale).  wd_rmsnorm_split_ok: the rows and widths that it serves.
-struct WdRowScale {
-    const float* sumsq = nullptr;   // null: 1
-    float inv_d = 0.f, eps = 0.f;
-};
-bool wd_rmsnorm_split_ok(int n_rows, int d);
-void wd_launch_rmsnorm_split(float* x, const float* part, int n_split, size_t split_stride, const float* gain, void* xg, float* sumsq,
-                             int n_rows, int d, cudaStream_t st);
-
 // plain GEMM (gemm_plain.cu): y[rows, n_0 + n_1 + ...] (float, leading dimension ldy) = x[rows,k] * [w_0; w_1; ...]^T for up
 // to three matrices.  w_static: the weights were complete before the previous kernel of the stream started.
 void wd_launch_gemm_plain(int dtype, const void* x, const void* const* w, const int* n, int n_mat, float* y, int rows, int k,
@@ -158,7 +147,7 @@ bool wd_launch_gemm_plain_fused(const WdPlainFuse& f, const void* const* w, cons
 void wd_launch_rope_scatter(int dtype, const float* part, int n_split, size_t split_stride,
                             const int32_t* row_seq, const int32_t* row_pos, const float2* rope_tab, void* q,
                             void* kcache, void* vcache, int n_rows, int Hq, int Hkv, int dh, int S, int Sp,
-                            int batch, int32_t* status, cudaStream_t st, const WdRowScale& scale = WdRowScale());
+                            int batch, int32_t* status, cudaStream_t st);
 // (a row whose position or sequence index is outside the state records WD_ERR_BOUNDS and writes no cache row)
 
 // The active rows of a step, one after the other: x_act[i] = x[act_row[i]], xn_act (bf16), rope_act and seq_act likewise.
@@ -178,7 +167,7 @@ void wd_launch_attention_plain(int dtype, const void* q, const void* kcache, con
 
 // h = silu(gate) * up from partials [n_split][n_rows][2F] (columns = [gate | up]); F % 4 == 0
 void wd_launch_swiglu(int dtype, const float* part, int n_split, size_t split_stride, void* h,
-                      int n_rows, int F, cudaStream_t st, const WdRowScale& scale = WdRowScale());
+                      int n_rows, int F, cudaStream_t st);
 
 // FP8: h as e4m3 codes [n_rows][F] with one scale per row (F <= 32768)
 wd_status wd_launch_swiglu_fp8(const float* part, int n_split, size_t split_stride, uint8_t* hq, float* sh, int n_rows,
