@@ -1929,9 +1929,9 @@ extern "C" wd_status wd_op_gemm_fp4(const void* x, const void* w, float* y, int3
     WD_CUDA_TRY(cudaGetLastError());
     int ns = 1;
     const size_t slice = (size_t)rows * n_out;
-    wd_status s = wd_fp4_gemm(&ox, &ow, (float*)p, wd_tc_scratch_bytes(rows, n_out, k_in) / 4, sm, status, stream, &ns, false, false);
+    wd_status s = wd_fp4_gemm(&ox, &ow, (float*)p, wd_tc_scratch_bytes(rows, n_out, k_in) / 4, sm, status, stream, &ns, false, false, y);
     if (s != WD_OK) return s;
-    wd_launch_reduce_slices((const float*)p, ns, slice, y, slice, stream);
+    if (ns > 1) wd_launch_reduce_slices((const float*)p, ns, slice, y, slice, stream);
     WD_CUDA_TRY(cudaGetLastError());
     return WD_OK;
 }
@@ -1970,9 +1970,9 @@ extern "C" wd_status wd_op_gemm_nvfp4(const void* xq, const void* wq, float* y, 
     wd_fp4_operand_split(const_cast<void*>(wq), n_out, k_in, &ow);
     int ns = 1;
     const size_t slice = (size_t)rows * n_out;
-    wd_status s = wd_fp4_gemm(&ox, &ow, (float*)scratch, scratch_bytes / 4, sm, status, stream, &ns, false, false);
+    wd_status s = wd_fp4_gemm(&ox, &ow, (float*)scratch, scratch_bytes / 4, sm, status, stream, &ns, false, false, y);
     if (s != WD_OK) return s;
-    wd_launch_reduce_slices((const float*)scratch, ns, slice, y, slice, stream);
+    if (ns > 1) wd_launch_reduce_slices((const float*)scratch, ns, slice, y, slice, stream);
     WD_CUDA_TRY(cudaGetLastError());
     return WD_OK;
 }

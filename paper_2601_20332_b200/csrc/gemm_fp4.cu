@@ -21,9 +21,9 @@
 // Persistent, one CTA per SM: the K blocks of all (weight tile, token tile) units form one line that is cut into
 // equal shares (stream-K, see choose_split), or whole units per CTA when that is cheaper.  The partial sums of a unit that several
 // CTAs share are written side by side ([slice][tok][n]) and added by the consumer, as in the bf16 kernel.
-// Measured at 34 rows, quantised input to summed result, 12288 x 4096 / 24576 x 4096 / 4096 x 12288: 15.4 / 22.8 / 16.0 us
+// Measured at 34 rows, quantised input to summed result, 12288 x 4096 / 24576 x 4096 / 4096 x 12288: 11.0 / 16.4 / 12.2 us
 // against 4.7 / 9.3 / 4.6 us for the bytes alone; what remains is start-up (2-3 us to the first complete stage, 2 us from the
-// last MMA to the stores) around 0.44 us a stage.  (Bringing the weights into the L2 ahead of the dependency wait made it
+// last MMA to the stores) around 0.28-0.39 us a stage.  (Bringing the weights into the L2 ahead of the dependency wait made it
 // slower: 24.4 instead of 23.8 us for the middle shape, 107 instead of 90 us at 600 rows.)
 // Every wait is bounded; on expiry the CTA records WD_ERR_DEVICE_TIMEOUT and leaves.
 #include <algorithm>
@@ -446,26 +446,29 @@ wd_status encode_bytes(CUtensorMap* m, const void* ptr, int n_rows, int row_byte
 // shares, a unit's sums then being spread over up to n_slices slices.
 struct Split { int grid, n_slices, aligned; };
 
-// Time of a split: the stages of the longest share, t_stage each, and for every further slice its write and re-read at HBM speed
-// (t_slice) and 0.3 us, for the zero fill where nobody wrote it and for its place in the chain of the kernel that adds the slices
-// (between 0.15 and 1 us the choice is the same).  Beside all SMs the grids tried give G / n_units a denominator of at most eight:
-// shares then start with a unit every few units, which costs hardly a stage and saves slices.  With fewer slices allowed than all
-// SMs would make (a long K with few units, little scratch) it is a smaller grid, not whole units.
-// Measured at 34 rows, step of eight blocks 4096 / 12288 wide: 740 us; with all SMs whenever the line is cut 766, its down
-// projections leaving six slices after 11 stages instead of four after 12, its q/k/v three instead of two after the same 11;
-// fixed K splits dealt round-robin 739, but 850 at 68 rows against 830.  5 rows of 300, K 16384, quantiser and sum with it:
-// 12.3 us (48 CTAs), with whole units 34.8 (3 CTAs).
-Split choose_split(int n_units, int kb, int sm_count, int max_slices, double t_stage, double t_slice) {
+// Time of a split: the stages of the longest share, and for every further slice its write and re-read at HBM speed (t_slice) and 0.3
+// us, for the zero fill where nobody wrote it and for its place in the chain of the kernel that adds the slices; t_sum where there is
+// such a kernel only because of them (a single operation's). A stage of one CTA takes 280 ns to load and issue, what comes in at 85
+// GB/s, or its part of the HBM rate beside the other CTAs: at 34 rows 390 ns with 148 CTAs, 280 with up to 106, so whole units on
+// fewer CTAs lose little.  Beside all SMs the grids tried give G / n_units a denominator of at most eight: shares then start with a
+// unit every few units, which costs hardly a stage and saves slices.  With fewer slices allowed than all SMs would make (a long K
+// with few units, little scratch) it is a smaller grid, not whole units.
+// Measured at 34 rows, quantised input to summed result: 12288 x 4096 13.2 us with 144 shares and two slices, 11.0 with 96 whole units;
+// 24576 x 4096 19.4, 16.4 with 192 whole units on 96 CTAs; 4096 x 12288 keeps 144 shares, five slices.  5 rows of 300, K 16384: 12.3 us
+// (48 CTAs), with whole units 34.8 (3 CTAs).
+Split choose_split(int n_units, int kb, int sm_count, int max_slices, int w_bytes, int x_bytes, double t_slice, double t_sum) {
     const long long W = (long long)n_units * kb;
-    const int g_unit = std::min(sm_count, n_units);
-    Split best = {g_unit, 1, 1};
+    auto stage = [&](int G) { return std::max({280e-9, (w_bytes + x_bytes) / 85e9, (double)w_bytes * G / 7.0e12}); };
+    const int per_cta = (n_units + sm_count - 1) / sm_count, g_unit = (n_units + per_cta - 1) / per_cta;
+    Split best = {std::min(sm_count, n_units), 1, 1};
     if (n_units >= 4 * sm_count) return best;               // rounds of whole units are full enough
-    double t_best = (double)((n_units + g_unit - 1) / g_unit) * kb * t_stage;
+    best.grid = g_unit;
+    double t_best = (double)per_cta * kb * stage(g_unit);
     auto consider = [&](long long G) {
         if (G < 1 || G > sm_count || G > W || W * (G + 1) > INT_MAX) return;
         const int ns = wd_tc_sharers(n_units, (int)G);
         if (ns > max_slices) return;
-        const double t = (double)((W + G - 1) / G) * t_stage + (ns - 1) * (t_slice + 0.3e-6);
+        const double t = (double)((W + G - 1) / G) * stage((int)G) + (ns - 1) * (t_slice + 0.3e-6) + (ns > 1 ? t_sum : 0.0);
         if (t < t_best * 0.999) {
             t_best = t;
             best = {(int)G, ns, 0};
@@ -514,7 +517,7 @@ void wd_launch_quantize_nvfp4(int dtype, const void* x, int n_rows, int K, const
 }
 
 wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, size_t y_floats, int sm_count, int32_t* status,
-                      cudaStream_t stream, int* n_split_out, bool force_single_split, bool w_static) {
+                      cudaStream_t stream, int* n_split_out, bool force_single_split, bool w_static, float* y_sum) {
     if (!x || !w || !y || !status) return WD_ERR_NULL;
     const int rows = x->n_rows, n_out = w->n_rows, K = x->K;
     if (rows < 1 || n_out < 1 || K < kKB || K % kKB || w->K != K) return WD_ERR_BAD_PARAM;
@@ -531,8 +534,9 @@ wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, si
     const size_t slice = (size_t)rows * n_out;
     if (slice > y_floats) return WD_ERR_CAPACITY;
     const int max_slices = (int)std::min<size_t>(WD_TC_MAX_SPLIT, y_floats / slice);
-    const double t_stage = (double)(kStageW + p.bn * 128 + kSfW + p.bn * 16) / 63e9;      // what one SM takes in, whatever the source
-    const Split sp = choose_split(p.n_units, p.kb_total, sm_count, force_single_split ? 1 : max_slices, t_stage, (double)slice * 8.0 / 6.5e12);
+    const Split sp = choose_split(p.n_units, p.kb_total, sm_count, force_single_split ? 1 : max_slices, kStageW + kSfW, p.bn * 144,
+                                  (double)slice * 8.0 / 6.5e12, y_sum ? 4e-6 : 0.0);
+    if (y_sum && sp.n_slices == 1) y = y_sum;
     p.aligned = sp.aligned;
     p.n_slices = sp.n_slices;
     const int grid = sp.grid;

@@ -201,6 +201,7 @@ void wd_launch_quantize_nvfp4(int dtype, const void* x, int n_rows, int K, const
 // w_static: the weights were quantised before the previous kernel on the stream started, so the kernel may
 // fetch them ahead of its dependency wait.
 wd_status wd_fp4_gemm(const WdFp4Operand* x, const WdFp4Operand* w, float* y, size_t y_floats, int sm_count, int32_t* status,
-                      cudaStream_t stream, int* n_split_out, bool force_single_split, bool w_static);
+                      cudaStream_t stream, int* n_split_out, bool force_single_split, bool w_static, float* y_sum = nullptr);
+// (y_sum: where the caller wants the sum of the slices; a result of one slice goes there, and nothing is left to add)
 // adds the K slices of a GEMM result: y[i] = sum_s part[s * stride + i]
 void wd_launch_reduce_slices(const float* part, int n_split, size_t stride, float* y, size_t total, cudaStream_t st);

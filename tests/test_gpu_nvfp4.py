@@ -34,10 +34,10 @@ def test_quantise_edges_are_the_oracles_bytes(rows, k, shift):
 
 
 # a unit shared by many SMs, units that start and end inside a share, a grid cut down to the most slices (three units, one unit),
-# whole units per SM because there are many; two units in three equal shares, every share a fixed part of a unit, more sharers
+# whole units per SM because there are many, and two each on half of the SMs; two units in three equal shares, every share a fixed part of a unit, more sharers
 # than units
 @pytest.mark.parametrize("rows,n,k", [(34, 1000, 4096), (129, 2000, 1024), (5, 300, 16384), (600, 16000, 256), (5, 128, 16384),
-                                      (34, 12288, 4096), (16, 4096, 1024), (64, 600, 8192)])
+                                      (34, 12288, 4096), (16, 4096, 1024), (64, 600, 8192), (16, 19200, 512)])
 def test_gemm_edges(rows, n, k):
     g = torch.Generator(device=DEV).manual_seed(rows + n)
     x = torch.randn(rows, k, device=DEV, generator=g).to(torch.bfloat16)
