@@ -378,7 +378,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     uint32_t* tmem_slot = (uint32_t*)(bars + 2 * NS + 4);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
     int* last_flag = (int*)(tmem_slot + 2);
-    float* lm_scratch = (float*)(tmem_slot + 4);           // 23 KB for the LM-head statistics
+    float* lm_scratch = (float*)(tmem_slot + 4);           // 32 KB for the LM-head statistics
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = gridDim.x / (p.tok_split > 1 ? p.tok_split : 1), c = blockIdx.x % G;
@@ -555,7 +555,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             int ord = 0;
             if (!p.aligned && kb0) ord = c - ((unit * p.kb_total + 1) * G - 1) / p.W;     // (else it is the first)
             // FP8: the row scales of this token tile go to shared memory while the MMAs still run
-            float* sx_s = lm_scratch + (kLmStats ? 5664 : 0);
+            float* sx_s = lm_scratch + (kLmStats ? 8224 : 0);
             if (kFp8) {
                 epi_sync();                                        // the previous piece's readers are done
                 for (int i = (int)threadIdx.x - 64; i < ((p.bn + 31) & ~31); i += 128)
@@ -586,17 +586,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     }
                 }
             } else {
-                // LM head: per token maximum / lowest argmax / sum exp over this tile's 128 logits, folded
-                // into the CTA's running statistics.  A thread holds one vocabulary entry for 32 tokens;
-                // the chunk is transposed through shared memory so that a thread then owns one token and
-                // a quarter of the tile's vocabulary entries, and the four quarters are merged per token.
-                float* run_m = lm_scratch;                          // [256] running statistics of this CTA
-                int* run_i = (int*)(lm_scratch + 256);
-                double* run_s = (double*)(lm_scratch + 512);
-                float* g_m = lm_scratch + 1024;                     // [4 quarters][32 tokens]
-                int* g_i = (int*)(lm_scratch + 1152);
-                double* g_s = (double*)(lm_scratch + 1280);
-                float* tr = lm_scratch + 1536;                      // [32 tokens][129]: padded against bank conflicts
+                // LM head: per token maximum / lowest argmax / sum exp over this tile's 128 logits.  A thread holds one
+                // vocabulary entry for 32 tokens; the chunk is transposed through shared memory so that a thread then owns one
+                // token and a quarter of the tile's vocabulary entries, whose running statistics over the CTA's tiles it keeps;
+                // the four quarters of a token are merged once, at the end.  (Merged per chunk, by 32 threads with five
+                // exponentials in double one after the other, the epilogue of 256 tokens took longer than the tile's MMAs.)
+                float* run_m = lm_scratch;                          // [chunk of 32 tokens][thread]
+                int* run_i = (int*)(lm_scratch + 1024);
+                double* run_s = (double*)(lm_scratch + 2048);
+                float* tr = lm_scratch + 4096;                      // [32 tokens][129]: padded against bank conflicts
                 const int e = (int)threadIdx.x - 64, tt = e & 31, gq = e >> 5;
                 for (int cc = 0; cc < p.bn; cc += 32) {
                     if (u.tok0 + cc >= p.rows) break;
@@ -624,38 +622,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                         x[j] = tr[tt * 129 + 32 * gq + j];
                         if (x[j] > bm) { bm = x[j]; bj = j; }       // strict: the lowest index stays on ties
                     }
+                    epi_sync();                     // everyone has read the transpose tile: the next chunk may be written over it
                     // single-precision exp (1 ulp) of each term, double accumulation: sums good to ~1e-9
                     double sm = 0.0;
                     if (bm > -INFINITY) {
 #pragma unroll
                         for (int j = 0; j < 32; ++j) sm += (double)expf(x[j] - bm);
                     }
-                    g_m[gq * 32 + tt] = bm;
-                    g_i[gq * 32 + tt] = u.n0 + 32 * gq + bj;
-                    g_s[gq * 32 + tt] = sm;
-                    epi_sync();
-                    if (e < 32 && u.tok0 + cc + e < p.rows) {
-                        // quarters ascend in vocabulary index, and so do the tiles of a CTA: on equal
-                        // maxima the earlier index stays
-                        float tm = g_m[e];
-                        int ti = g_i[e];
-                        for (int w = 1; w < 4; ++w)
-                            if (g_m[w * 32 + e] > tm) { tm = g_m[w * 32 + e]; ti = g_i[w * 32 + e]; }
-                        double ts = 0.0;
-                        for (int w = 0; w < 4; ++w)
-                            if (g_m[w * 32 + e] > -INFINITY) ts += g_s[w * 32 + e] * exp((double)g_m[w * 32 + e] - (double)tm);
-                        const int tl = cc + e;
-                        if (piece == 0) {
-                            run_m[tl] = tm; run_i[tl] = ti; run_s[tl] = ts;
-                        } else if (tm > run_m[tl]) {
-                            run_s[tl] = run_s[tl] * exp((double)run_m[tl] - (double)tm) + ts;
-                            run_m[tl] = tm; run_i[tl] = ti;
+                    const int slot = (cc >> 5) * 128 + e;
+                    if (piece == 0) {
+                        run_m[slot] = bm; run_i[slot] = u.n0 + 32 * gq + bj; run_s[slot] = sm;
+                    } else if (bm > -INFINITY) {
+                        // (the tiles of a CTA ascend in vocabulary index: on equal maxima the earlier index stays)
+                        const float m = run_m[slot];
+                        if (bm > m) {
+                            run_s[slot] = run_s[slot] * exp((double)m - (double)bm) + sm;
+                            run_m[slot] = bm; run_i[slot] = u.n0 + 32 * gq + bj;
                         } else {
-                            run_s[tl] += ts * exp((double)tm - (double)run_m[tl]);
+                            run_s[slot] += sm * exp((double)bm - (double)m);
                         }
                     }
-                    // the next chunk's writes to the transpose tile and to the quarter statistics come
-                    // after its own barrier, which every thread reaches only after the reads above
                 }
             }
             tc_fence_before();
@@ -700,16 +686,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         }
         if (kLmStats && sch.n_pieces > 0) {
             // one (max, argmax, sum exp) per token for all the vocabulary tiles this CTA covered
-            float* run_m = lm_scratch;
-            int* run_i = (int*)(lm_scratch + 256);
-            double* run_s = (double*)(lm_scratch + 512);
+            const float* run_m = lm_scratch;
+            const int* run_i = (const int*)(lm_scratch + 1024);
+            const double* run_s = (const double*)(lm_scratch + 2048);
             epi_sync();
             // this CTA's token tile: rows tok_group * bn .. ; entry c of the row's G statistics
             for (int t = (int)threadIdx.x - 64; t < p.bn && tok_group * p.bn + t < p.rows; t += 128) {
                 const size_t si = (size_t)(tok_group * p.bn + t) * G + c;
-                p.f.st_max[si] = run_m[t];
-                p.f.st_idx[si] = run_i[t];
-                p.f.st_sum[si] = run_s[t];
+                const int slot = (t >> 5) * 128 + (t & 31);             // quarter w at slot + 32 w
+                float tm = run_m[slot];
+                int ti = run_i[slot];
+                for (int w = 1; w < 4; ++w) {
+                    const float m = run_m[slot + 32 * w];
+                    const int i = run_i[slot + 32 * w];
+                    if (m > tm || (m == tm && i < ti)) { tm = m; ti = i; }
+                }
+                double ts = 0.0;
+                for (int w = 0; w < 4; ++w)
+                    if (run_m[slot + 32 * w] > -INFINITY) ts += run_s[slot + 32 * w] * exp((double)run_m[slot + 32 * w] - (double)tm);
+                p.f.st_max[si] = tm;
+                p.f.st_idx[si] = ti;
+                p.f.st_sum[si] = ts;
             }
         }
         tc_fence_before();
@@ -1618,7 +1615,7 @@ TcConfig pick_config(int rows, bool allow_wide, bool lm_stats) {
     c.n_stages = ((c.ctas_per_sm == 2 ? 96 : 192) * 1024) / stage;
     if (c.n_stages > 10) c.n_stages = 10;
     if (c.n_stages < 2) c.n_stages = 2;
-    c.smem = (size_t)c.n_stages * stage + (2 * c.n_stages + 4) * 8 + 16 + (lm_stats ? 24576 : 8192) + 1024;
+    c.smem = (size_t)c.n_stages * stage + (2 * c.n_stages + 4) * 8 + 16 + (lm_stats ? 8480 * 4 : 8192) + 1024;
     return c;
 }
 
@@ -2079,10 +2076,10 @@ wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, in
     if (!attr_done[dev]) {
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-        WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        WD_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, false, false, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, false, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-        WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, true, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        WD_CUDA_TRY(cudaFuncSetAttribute((gemm_tc_kernel<false, true, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_done[dev] = true;
     }
     const CUtensorMap& m0 = *segs[0].map;
