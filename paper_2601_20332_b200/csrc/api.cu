@@ -77,7 +77,8 @@ struct wd_ctx {
     struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int n_kernels = 0, impl_used = 0; uint64_t last_use = 0; };
     bool graphs_on = true;
     std::vector<StepGraph> graphs;      // at most kMaxGraphs, the least recently used replaced once it is out of use
-    std::vector<StepKey> seen;          // configurations met once (capture pays from the second time on)
+    struct SeenKey { StepKey key; int times; };
+    std::vector<SeenKey> seen;          // configurations met and not recorded, the last ones
     uint64_t graph_clock = 0;
     int graphs_captured = 0, graphs_replayed = 0, graph_failures = 0;
 
@@ -1633,16 +1634,14 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
     // A step of the fp32 path lasts 2-3 us a kernel, and its launches take the host 5 each: with a graph it is also shorter when nothing
     // is queued and the host waits for every step (9 rows, two blocks of 256 / 688, host to host 105 -> 100 us).
     const bool taps_on = st->taps.layer_out || st->taps.attn_out || (st->taps.logits && !f32);
-    // Only while earlier steps are still queued: the GPU then has work while the host records or submits the
-    // graph.  With an empty queue (a caller that syncs after every step) direct launches win, because the GPU
-    // starts on the first kernels while the host is still launching the later ones (measured: 230 against 227
-    // tokens/s end to end).
+    // Replaying pays with an empty queue too (a caller that syncs after every step: 34 rows, 3.43 ms a step with direct launches, 3.34
+    // with a graph).  Recording then keeps the GPU waiting, 1.3 ms for the 290 kernels of that step, so it is left until the configuration
+    // has come back often enough to pay for it; with earlier steps queued the GPU has work meanwhile.
     // bf16 needs the tensor-core attention.  fp32 steps take the index-list kernel with room for whole key tiles (its
     // scores in shared memory), so a recorded launch holds while the visible count grows within the last tile.
     const bool attn_by_tc = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN;
     const bool attn_by_tiles = d.dtype == WD_F32 && (wd_align_up((size_t)max_vis, 128) + dh) * 4 <= 200 * 1024;
-    if (c->graphs_on && dev_mode && !c->prof_on && !taps_on && !fused && !stream_capturing && (attn_by_tc || attn_by_tiles) &&
-        (f32 || !st->queue.empty())) {
+    if (c->graphs_on && dev_mode && !c->prof_on && !taps_on && !fused && !stream_capturing && (attn_by_tc || attn_by_tiles)) {
         copy_logits = true;
         wd_ctx::StepKey key;
         key.state_uid = st->uid; key.batch = batch; key.rows = R_; key.n_act = NA; key.n_qtiles = (int)n_qtiles;
@@ -1667,8 +1666,10 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             // phases: record it at once
             int live = 0;
             for (int b = 0; b < batch; ++b) live += pend.cp[b].done ? 0 : 1;
-            bool seen = !any_refresh && NA == A * live;
-            for (const wd_ctx::StepKey& k2 : c->seen) if (k2 == key) { seen = true; break; }
+            const int enough = f32 || !st->queue.empty() ? 1 : 8;         // times that it has to have come before
+            wd_ctx::SeenKey* known = nullptr;
+            for (wd_ctx::SeenKey& k2 : c->seen) if (k2.key == key) { known = &k2; break; }
+            const bool seen = (enough == 1 && !any_refresh && NA == A * live) || (known && known->times >= enough);
             // A full cache gives up only a graph that the last 64 steps had no use for.  A job that repeats more configurations than fit
             // (the refresh steps of a long generation, each of its own row count) would otherwise record each of them, replay it once
             // and push it out again: 64 steps of the small fp32 model against eight graphs were 17 recordings of 230 us.
@@ -1676,9 +1677,12 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             size_t lru = 0;
             for (size_t i = 1; i < c->graphs.size(); ++i) if (c->graphs[i].last_use < c->graphs[lru].last_use) lru = i;
             const bool room = c->graphs.size() < kMaxGraphs || c->graphs[lru].last_use + 64 < c->graph_clock;
+            if (known) ++known->times;
             if (!seen) {
-                if (c->seen.size() >= 64) c->seen.erase(c->seen.begin());
-                c->seen.push_back(key);
+                if (!known) {
+                    if (c->seen.size() >= 64) c->seen.erase(c->seen.begin());
+                    c->seen.push_back({key, 1});
+                }
             } else if (!room) {         // launched directly
             } else if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
                 static const bool gdbg = getenv("WD_GRAPH_DEBUG") != nullptr;

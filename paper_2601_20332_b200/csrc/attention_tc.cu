@@ -574,9 +574,10 @@ attention_tc_single_kernel(const __grid_constant__ CUtensorMap map_q, const __gr
 // Tensor memory: S (and P over it) 2 x 128 columns, O 2 x 128.  Shared memory: two Q tiles, two K and two V stages, 192 KB.
 // The tensor core runs Q K^T and P V in issue order, so S(i + 1) complete means P V(i) has read P(i) and has been added to O;
 // one barrier each for S and P of a tile suffices (P(i + 1) needs S(i + 1), which is issued only after P(i) has been seen).
-// What bounds it: 3900 cycles per key tile and pair of query tiles.  The MMAs alone, issued without waiting for any softmax, take
-// 3280 (M = N = 128 runs at 62 % of the peak rate: both operands' slices of a Q K^T use up the shared-memory bandwidth), the
-// softmax without the MMAs 3100, and the K/V loads hide completely.  Beside the loop a CTA spends 3 us until its first scores, 1.1
+// What bounds it: the softmax, 3100 cycles per key tile and pair of query tiles without the MMAs, of which 2048 are the exponentials' (16 a
+// cycle); K/V loads and MMAs hide behind it, now that their issue loops are run by converged warps (one lane alone took 3280 cycles for
+// the MMAs of a key tile, and the launch of 1792 rows, 128 heads 255 us instead of 225; 640 rows, 40 heads, 2048 keys 43.5 / 38.1).
+// Beside the loop a CTA spends 3 us until its first scores, 1.1
 // us after the last exponentials and the write of O, so a few key tiles are dominated by both ends: one row of O per thread took
 // 2.1-4.6 us (a warp's store touched 32 lines), staged through shared memory 0.5-1; loading tile 0 and its keys before tile 1, and
 // zeroing V columns by 16 bytes while the scores are still being computed, the rest of 113 -> 98 us for eight sequences of
