@@ -1775,12 +1775,16 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
         // one accumulator: whole units (with RoPE or the residual add in their epilogue where the launch has one: with shares of the
         // K-block line a tile's sum is in several pieces), or shares
         static const int epi_on = env_int("WD_GEMM_EPI", 3);
-        if (!fp8 && p.dual == 0 && !force_single_split) {
-            int want = kEpiPlain;
-            if (rope && nseg == 3 && (epi_on & 1)) want = kEpiRope;
-            else if (resid && resid->x && nseg == 1 && (epi_on & 2)) want = kEpiResid;
+        int want = kEpiPlain;
+        if (rope && nseg == 3 && (epi_on & 1)) want = kEpiRope;
+        else if (resid && resid->x && nseg == 1 && (epi_on & 2)) want = kEpiResid;
+        if (!fp8 && p.dual != 2 && (p.dual == 0 || want != kEpiPlain) && !force_single_split) {
             unit_tok_tiles = whole_unit_tok_tiles(tiles_all, (K + kBK - 1) / kBK, rows, ncol_all, (int)pairs, want);
             if (unit_tok_tiles > 0) {
+                // An epilogue goes before the second accumulator.  Measured, us a block (wide q/k/v, d_ffn 1024) with two accumulators
+                // and the rotation kernel / with the epilogue: 64 heads, d 8192, 600 rows 390 / 360, 1216 705 / 665, 2100 1229 /
+                // 1108; 128 heads over 8, d 4096, 600 rows 218 / 216, 2100 770 / 706; 50 heads, d 5120, 1100 rows 395 / 349.
+                p.dual = 0;
                 epi = want;
                 force_single_split = true;
             }

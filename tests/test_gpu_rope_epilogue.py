@@ -42,3 +42,18 @@ def test_rope_epilogue_grouped_heads(Hq, Hkv, batch, P):
     assert par.log[0]["info"]["n_rows"] == batch * (P + 56)
     assert launches[0] < launches[1]        # no rotation kernel
     par.close()
+
+
+# q/k/v of 16384 columns or more, enough units of 512 tokens for two rounds: the epilogue before a second accumulator.  24576 columns
+# without grouping, and 18432 of 128 query heads over 8
+@pytest.mark.parametrize("Hq,Hkv", [(64, 64), (128, 8)])
+def test_rope_epilogue_wide(Hq, Hkv):
+    cfg = synth.get_config("llada8b", L=1, d=256, Hq=Hq, Hkv=Hkv, dh=128, F=512, V=1000, P=544 if Hkv == 64 else 1046, G=100)
+    par = Parity(cfg, synth.make_weights(cfg, DEV, gain_jitter=0.1), synth.make_prompts(cfg))
+    launches = []
+    for _ in range(2):
+        assert par.step(16, 40, 4, 2, 1) is not None
+        launches.append(par.log[-1]["info"]["n_launches"])
+    assert par.log[0]["info"]["n_rows"] == cfg["P"] + 56
+    assert launches[0] == launches[1] - 1   # no rotation kernel
+    par.close()
