@@ -1631,12 +1631,11 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
         if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) { cudaGetLastError(); cs = cudaStreamCaptureStatusActive; }
         stream_capturing = cs != cudaStreamCaptureStatusNone;
     }
-    // A step of the fp32 path lasts 2-3 us a kernel, and its launches take the host 5 each: with a graph it is also shorter when nothing
-    // is queued and the host waits for every step (9 rows, two blocks of 256 / 688, host to host 105 -> 100 us).
     const bool taps_on = st->taps.layer_out || st->taps.attn_out || (st->taps.logits && !f32);
     // Replaying pays with an empty queue too (a caller that syncs after every step: 34 rows, 3.43 ms a step with direct launches, 3.34
-    // with a graph).  Recording then keeps the GPU waiting, 1.3 ms for the 290 kernels of that step, so it is left until the configuration
-    // has come back often enough to pay for it; with earlier steps queued the GPU has work meanwhile.
+    // with a graph; fp32, 9 rows, two blocks of 256 / 688: 62 and 59.5 us).  Recording then keeps the GPU waiting, 1.3 ms for the 290
+    // kernels of the former and 110 us for the latter (another 75 where a graph has to go for it), so it is left until the configuration
+    // has come back often enough to expect that it pays; with earlier steps queued the GPU has work meanwhile.
     // bf16 needs the tensor-core attention.  fp32 steps take the index-list kernel with room for whole key tiles (its
     // scores in shared memory), so a recorded launch holds while the visible count grows within the last tile.
     const bool attn_by_tc = use_tc(c) && st->attn_tc && all_contig && c->attn_impl != WD_GEMM_PLAIN;
@@ -1666,7 +1665,7 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             // phases: record it at once
             int live = 0;
             for (int b = 0; b < batch; ++b) live += pend.cp[b].done ? 0 : 1;
-            const int enough = f32 || !st->queue.empty() ? 1 : 8;         // times that it has to have come before
+            const int enough = !st->queue.empty() ? 1 : f32 ? 32 : 8;     // times that it has to have come before
             wd_ctx::SeenKey* known = nullptr;
             for (wd_ctx::SeenKey& k2 : c->seen) if (k2.key == key) { known = &k2; break; }
             const bool seen = (enough == 1 && !any_refresh && NA == A * live) || (known && known->times >= enough);

@@ -1,0 +1,50 @@
+"""Which steps are recorded as graphs and replayed, and what the context keeps of them."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_20332_b200 import binding as wd
+from paper_2601_20332_b200 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _context(name="tiny", **over):
+    cfg = synth.get_config(name, P=20, G=140, **over)
+    ids = synth.make_prompts(cfg)
+    S = ids.shape[1]
+    return cfg, ids, wd.Context(cfg, synth.make_weights(cfg, DEV), 1, S, S, 128)
+
+
+def test_fp32_steps_synced_one_by_one():
+    """With nothing queued an fp32 configuration is recorded after it has come 32 times.  A graph's kernels write the context's logits:
+    the tap of a step is filled behind them, and left alone by the other steps."""
+    runs = []
+    for on in (False, True):
+        cfg, ids, ctx = _context()
+        ctx.set_graphs(on)
+        stream = torch.cuda.Stream(device=DEV)
+        st = wd.State(ctx, ids)
+        taps = [torch.full((128, cfg["V"]), -1.0, device=DEV) for _ in range(2)]
+        torch.cuda.synchronize()
+        got, stats = [], []
+        for i in range(1 + 48):                 # a refresh, then normal steps of one configuration
+            st.set_taps(logits=taps[i % 3] if i % 3 < 2 else None)
+            st.step(8, 120, 1000, 1, 1, stream)
+            out = st.sync()
+            got.append([t.clone() for t in taps] + [out["positions"], out["token_ids"], out["confidence"]])
+            stats.append(ctx.graph_stats())
+            for t in taps:
+                t.fill_(-1.0)
+            torch.cuda.synchronize()
+        runs.append((got, stats))
+        st.close()
+        ctx.close()
+    for i, (a, b) in enumerate(zip(runs[0][0], runs[1][0], strict=True)):
+        for j in range(2):
+            assert torch.equal(a[j], b[j])
+            assert bool((b[j][:8] != -1.0).all()) == (i % 3 == j) and bool((b[j][8:] == -1.0).all())
+        assert all(np.array_equal(x, y) for x, y in zip(a[2:], b[2:], strict=True))
+    assert runs[0][1][-1] == (0, 0)
+    assert runs[1][1][32:34] == [(0, 0), (1, 0)] and runs[1][1][-1] == (1, 15)
