@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
 
 #include "wd_internal.h"
@@ -74,9 +75,15 @@ struct wd_ctx {
                    impl == o.impl && attn_impl == o.attn_impl;
         }
     };
-    struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int n_kernels = 0, impl_used = 0; uint64_t last_use = 0; };
+    struct StepGraph {
+        StepKey key;
+        std::weak_ptr<const char> state;        // expired once the state is destroyed
+        cudaGraphExec_t exec = nullptr;
+        int n_kernels = 0, impl_used = 0;
+        uint64_t last_use = 0;
+    };
     bool graphs_on = true;
-    std::vector<StepGraph> graphs;      // at most kMaxGraphs, the least recently used replaced once it is out of use
+    std::vector<StepGraph> graphs;      // at most kMaxGraphs; replaced: one of a destroyed state, or the least recently used once it is out of use
     struct SeenKey { StepKey key; int times; };
     std::vector<SeenKey> seen;          // configurations met and not recorded, the last ones
     uint64_t graph_clock = 0;
@@ -553,6 +560,8 @@ static std::atomic<uint64_t> g_state_uid{0};
 struct wd_state {
     wd_ctx* ctx = nullptr;
     uint64_t uid = ++g_state_uid;       // never reused, unlike the address (keys the step graphs)
+    std::shared_ptr<const char> life = std::make_shared<const char>('\0');      // what the step graphs watch: a state may outlive its
+                                        // context, or be destroyed while another thread steps another one, so it leaves their list alone
     int batch = 0, S = 0;
     std::vector<WdSeq> seqs;
     std::vector<WdSeqPlan> plans;       // of the pending step
@@ -1672,10 +1681,13 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             // A full cache gives up only a graph that the last 64 steps had no use for.  A job that repeats more configurations than fit
             // (the refresh steps of a long generation, each of its own row count) would otherwise record each of them, replay it once
             // and push it out again: 64 steps of the small fp32 model against eight graphs were 17 recordings of 230 us.
+            // The graphs of a destroyed state, which can match no step any more, go first.
             static const size_t kMaxGraphs = 32;
-            size_t lru = 0;
-            for (size_t i = 1; i < c->graphs.size(); ++i) if (c->graphs[i].last_use < c->graphs[lru].last_use) lru = i;
-            const bool room = c->graphs.size() < kMaxGraphs || c->graphs[lru].last_use + 64 < c->graph_clock;
+            size_t victim = 0;
+            for (size_t i = 1; i < c->graphs.size() && !c->graphs[victim].state.expired(); ++i)
+                if (c->graphs[i].state.expired() || c->graphs[i].last_use < c->graphs[victim].last_use) victim = i;
+            const bool room = c->graphs.size() < kMaxGraphs || c->graphs[victim].state.expired() ||
+                              c->graphs[victim].last_use + 64 < c->graph_clock;
             if (known) ++known->times;
             if (!seen) {
                 if (!known) {
@@ -1702,11 +1714,11 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                 if (ie == cudaSuccess) {
                     cudaGraphDestroy(graph);
                     wd_ctx::StepGraph g;
-                    g.key = key; g.exec = exec; g.n_kernels = (int)(wd_launch_counter - k0); g.impl_used = impl_used;
+                    g.key = key; g.state = st->life; g.exec = exec; g.n_kernels = (int)(wd_launch_counter - k0); g.impl_used = impl_used;
                     g.last_use = c->graph_clock;
                     if (c->graphs.size() >= kMaxGraphs) {
-                        cudaGraphExecDestroy(c->graphs[lru].exec);
-                        c->graphs[lru] = g;
+                        cudaGraphExecDestroy(c->graphs[victim].exec);
+                        c->graphs[victim] = g;
                     } else {
                         c->graphs.push_back(g);
                     }

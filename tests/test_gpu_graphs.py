@@ -17,6 +17,15 @@ def _context(name="tiny", **over):
     return cfg, ids, wd.Context(cfg, synth.make_weights(cfg, DEV), 1, S, S, 128)
 
 
+def _steps(st, windows, stream):
+    """A step for each number of active positions, ten at a time behind one of 64, so that they find steps queued.  They unmask nothing
+    (the same window can be taken again), and only the first step of a state refreshes."""
+    for i in range(0, len(windows), 10):
+        for A in [64] + windows[i:i + 10]:
+            st.step(A, 128 - A, 1000, 1, 0, stream)
+        st.sync_all()
+
+
 def test_fp32_steps_synced_one_by_one():
     """With nothing queued an fp32 configuration is recorded after it has come 32 times.  A graph's kernels write the context's logits:
     the tap of a step is filled behind them, and left alone by the other steps."""
@@ -48,3 +57,19 @@ def test_fp32_steps_synced_one_by_one():
         assert all(np.array_equal(x, y) for x, y in zip(a[2:], b[2:], strict=True))
     assert runs[0][1][-1] == (0, 0)
     assert runs[1][1][32:34] == [(0, 0), (1, 0)] and runs[1][1][-1] == (1, 15)
+
+
+def test_graphs_of_destroyed_states_make_room():
+    """A state that filled the context's graphs and is gone does not keep the next one's steps from being recorded."""
+    cfg, ids, ctx = _context()
+    stream = torch.cuda.Stream(device=DEV)
+    st = wd.State(ctx, ids)
+    _steps(st, list(range(1, 41)), stream)      # more windows than there is room for
+    st.close()
+    captured, replayed = ctx.graph_stats()
+    assert captured == 32 and replayed == 0
+    st = wd.State(ctx, ids)
+    _steps(st, [8] * 10, stream)
+    assert ctx.graph_stats() == (captured + 1, replayed + 9)
+    st.close()
+    ctx.close()
