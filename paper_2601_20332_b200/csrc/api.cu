@@ -85,7 +85,7 @@ struct wd_ctx {
     bool graphs_on = true;
     std::vector<StepGraph> graphs;      // at most kMaxGraphs; replaced: one of a destroyed state, or the least recently used once it is out of use
     struct SeenKey { StepKey key; int times; };
-    std::vector<SeenKey> seen;          // configurations met and not recorded, the last ones
+    std::vector<SeenKey> seen;          // configurations met and not recorded, the last 64, in the order of their last meeting
     uint64_t graph_clock = 0;
     int graphs_captured = 0, graphs_replayed = 0, graph_failures = 0;
 
@@ -1675,9 +1675,14 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
             int live = 0;
             for (int b = 0; b < batch; ++b) live += pend.cp[b].done ? 0 : 1;
             const int enough = !st->queue.empty() ? 1 : f32 ? 32 : 8;     // times that it has to have come before
-            wd_ctx::SeenKey* known = nullptr;
-            for (wd_ctx::SeenKey& k2 : c->seen) if (k2.key == key) { known = &k2; break; }
-            const bool seen = (enough == 1 && !any_refresh && NA == A * live) || (known && known->times >= enough);
+            int times = 0;
+            for (size_t i = 0; i < c->seen.size(); ++i)
+                if (c->seen[i].key == key) {
+                    times = c->seen[i].times;
+                    c->seen.erase(c->seen.begin() + i);
+                    break;
+                }
+            const bool seen = (enough == 1 && !any_refresh && NA == A * live) || times >= enough;
             // A full cache gives up only a graph that the last 64 steps had no use for.  A job that repeats more configurations than fit
             // (the refresh steps of a long generation, each of its own row count) would otherwise record each of them, replay it once
             // and push it out again: 64 steps of the small fp32 model against eight graphs were 17 recordings of 230 us.
@@ -1688,13 +1693,9 @@ extern "C" wd_status wd_step(wd_state* st, int32_t A, int32_t B, int32_t R, int3
                 if (c->graphs[i].state.expired() || c->graphs[i].last_use < c->graphs[victim].last_use) victim = i;
             const bool room = c->graphs.size() < kMaxGraphs || c->graphs[victim].state.expired() ||
                               c->graphs[victim].last_use + 64 < c->graph_clock;
-            if (known) ++known->times;
-            if (!seen) {
-                if (!known) {
-                    if (c->seen.size() >= 64) c->seen.erase(c->seen.begin());
-                    c->seen.push_back({key, 1});
-                }
-            } else if (!room) {         // launched directly
+            if (!seen || !room) {       // launched directly
+                if (c->seen.size() >= 64) c->seen.erase(c->seen.begin());
+                c->seen.push_back({key, times + 1});
             } else if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
                 static const bool gdbg = getenv("WD_GRAPH_DEBUG") != nullptr;
                 const long long k0 = wd_launch_counter;

@@ -8,6 +8,7 @@ from paper_2601_20332_b200 import synth
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
+BF16 = dict(dtype="bf16", dh=128, Hq=2, Hkv=2, F=704)       # the small model with the widths of the tensor-core path
 
 
 def _context(name="tiny", **over):
@@ -71,5 +72,28 @@ def test_graphs_of_destroyed_states_make_room():
     st = wd.State(ctx, ids)
     _steps(st, [8] * 10, stream)
     assert ctx.graph_stats() == (captured + 1, replayed + 9)
+    st.close()
+    ctx.close()
+
+
+def test_a_window_that_keeps_coming_back_is_counted():
+    """With nothing queued a bf16 configuration is recorded after it has come eight times, however many windows that come once lie
+    between."""
+    cfg, ids, ctx = _context(**BF16)
+    stream = torch.cuda.Stream(device=DEV)
+    st = wd.State(ctx, ids)
+
+    def step(A):
+        st.step(A, 128 - A, 1000, 1, 0, stream)
+        st.sync()
+
+    step(64)
+    for i in range(81):
+        step(1 + i)
+        if i % 10 == 0:
+            step(100)
+    assert ctx.graph_stats() == (1, 0)          # recorded at the ninth
+    step(100)
+    assert ctx.graph_stats() == (1, 1)
     st.close()
     ctx.close()
