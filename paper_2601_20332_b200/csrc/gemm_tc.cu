@@ -1669,37 +1669,6 @@ uint32_t make_idesc(int bn, int m = kBM, bool fp8 = false) {
     return d;
 }
 
-// whole units pay when every pair gets two or more, or when the one or two rounds are nearly full
-bool full_rounds(long long units, long long pairs) {
-    return units >= 2 * pairs || (units >= pairs && 10 * units >= 9 * pairs * ((units + pairs - 1) / pairs));
-}
-
-// Token tiles of a gate/up launch whose epilogue applies SwiGLU (whole units of a gate and an up tile, dealt to the pairs in rounds),
-// or 0 where equal shares of the K-block line and the SwiGLU kernel are the shorter way.  Fewest tiles are not always best: 1216
-// rows in five tiles of 256 are 240 units for 74 pairs, four rounds, and so are six tiles of 208.  Estimated in us, fitted to both
-// sides measured: a K block of a unit takes its MMAs (0.003 a token) or what a CTA takes in (two weight blocks and half the tokens'
-// at 73 GB/s), a unit's end 4 at 256 tokens; a K block of a share 0.4, its slices' way through the SwiGLU kernel 16 bytes a value at
-// 9.4 TB/s.  Measured, LLaDA shape, us a block against the fewest tiles, or shares where those do not fill their rounds:
-// 352 rows in three tiles -7 (two -4), 440 in three -11, 1100 in six -16 of 177, 1216 in six -31 of 199 (with the power that the fuller rounds draw, -9 and -17 of the whole block); kept at the fewest: 583 rows (four tiles
-// +25), 704 (+24), 900 (five +14), 2100 (ten even); Dream shape 530 (four +25), 1000 (five +8).
-int gate_up_tok_tiles(int tiles, int kb_total, int rows, int pairs, int n) {
-    const int least = (rows + 255) / 256;
-    int best = 0;
-    double t_best = 2.0 * tiles * least * kb_total / pairs * 0.4 + 3.0 + (double)rows * n * 16.0 / 9.4e6;
-    for (int t = least; t < least + 4; ++t) {
-        const int bn = ((rows + t - 1) / t + 15) / 16 * 16;
-        if (!full_rounds((long long)tiles * t, pairs)) continue;
-        const int n_rounds = (tiles * t + pairs - 1) / pairs;
-        const double block = std::max(0.003 * bn, (2 * kStageA + bn * kBK) / 73e3);
-        const double us = n_rounds * (kb_total * block + bn / 64.0);
-        if (us < 0.98 * t_best) {       // (a tile more only for a gain that shows)
-            t_best = us;
-            best = t;
-        }
-    }
-    return best;
-}
-
 // Token tiles of a launch with one accumulator set in whole units (a round of them walks K in step, so that a weight block and a token
 // block are fetched by all who want them at about the same time), or 0 for equal shares of the K-block line.  Estimated in us at
 // 1.8 GHz: a K block of a whole unit takes 390 cycles to load and issue, or its MMAs, 2 a token; one of a share 700 (the pairs are
@@ -1710,7 +1679,7 @@ int gate_up_tok_tiles(int tiles, int kb_total, int rows, int pairs, int n) {
 // projection: 583 rows in four tiles -8 / -10, 900 in four -10 / -18, 1216 in eight -15 / -9, 1551 in nine -24 / -21 (352 in four
 // 0 / +10: shares); q/k/v 352 in two -9, 1216 in six -5 (1551 in nine +5: seven).  Dream shape, down 530 rows in four -21, 1000 in five
 // -38; output projection 530 in five -6, 1000 in eight -11; q/k/v 530 in four -5, 1000 in four -9.
-int whole_unit_tok_tiles(int tiles, int kb_total, int rows, int ncol, int pairs, int epi) {
+int whole_unit_tok_tiles(int tiles, int kb_total, int rows, int ncol, int pairs, int epi, double* us_out = nullptr) {
     const int least = (rows + 255) / 256, bn_least = ((rows + least - 1) / least + 15) / 16 * 16;
     const bool groups = least == 2 && pairs % 2 == 0;
     const double bytes = 4.0 * rows * ncol;
@@ -1728,6 +1697,44 @@ int whole_unit_tok_tiles(int tiles, int kb_total, int rows, int ncol, int pairs,
                           (epi == kEpiPlain ? bytes / 5e6 : 0.0);
         if (us < (best ? 0.95 : 1.0) * t_best) {
             t_best = us;
+            best = t;
+        }
+    }
+    if (us_out) *us_out = t_best;
+    return best;
+}
+
+// Token tiles of a gate/up launch whose epilogue applies SwiGLU (whole units of a gate and an up tile, dealt to the pairs in rounds),
+// or 0 where the launch without it (of one accumulator or, dual, of token super-tiles) and the SwiGLU kernel are the shorter way.
+// Fewest tiles are not always best: 1216 rows in five tiles of 256 are 240 units for 74 pairs, four rounds, and so are six tiles of
+// 208.  Estimated in us.  Two accumulators: a K block takes its MMAs, 0.0025 a token, and 0.015 more, or 0.25 to load and issue; a unit's
+// end 5.6 at 256 tokens.  One: 0.0012 a token, or 0.19; 3.  The other side's values are written, and read again, at 5.4 TB/s together.  The
+// epilogue has to be 7 % shorter: the fuller its rounds, the more power they draw, and the block's other launches slow down.
+// Fitted to every token tile count against the other side, at 272 to 1551 rows of five shapes (d_model / d_ffn 4096 / 12288, 3584 / 18944,
+// 2048 / 8192, 5120 / 13824, 8192 / 28672).  Measured, us a block of the fewest tiles / this rule's, against the other side: 4096 / 12288,
+// 320 rows +11 / +3 (three tiles), 352 +12 / 0 (the other side; three tiles +1), 384 +18 / -5 (three), 440 +11 / -8 (three), 512 +22 / -12
+// (three), 583 -30 / -30, 1024 -27 / -31 (six), 1216 +14 / -17 (six); 3584 / 18944, 352 rows -10 / -10, 530 -24 / -24; 2048 / 8192, 352 rows
+// -6 / -6; 5120 / 13824, 440 rows +19 / 0 (the other side), 1216 -42 / -60 (eight); 8192 / 28672, 352 rows +8 / -65 (three), 900 -60 /
+// -118 (five).
+int gate_up_tok_tiles(int tiles, int kb_total, int rows, int pairs, int n, bool dual) {
+    const int least = (rows + 255) / 256, super = (rows + 511) / 512;
+    const double values = 8.0 * rows * n / 5.4e6;
+    auto width = [&](int t) { return ((rows + t - 1) / t + 15) / 16 * 16; };
+    auto rounds = [&](int units) { return (double)((units + pairs - 1) / pairs); };
+    auto two = [&](int t) { return rounds(tiles * t) * (kb_total * std::max(0.25, 0.015 + 0.0025 * width(t)) + 0.022 * width(t)); };
+    double other;
+    if (dual) {
+        other = two(2 * super) + 3.0 + values;          // (a unit is a tile of either matrix and twice as many tokens)
+    } else {
+        const int t = whole_unit_tok_tiles(2 * tiles, kb_total, rows, 2 * n, pairs, kEpiPlain, &other);
+        if (t > 0) other = rounds(2 * tiles * t) * kb_total * std::max(0.19, 0.0012 * width(t)) + 3.0 + width(t) * 3.0 / 256 + values;
+    }
+    double t_best = 0.93 * other;
+    int best = 0;
+    for (int t = least; t < least + 4; ++t) {
+        if (10 * tiles * t < 7 * pairs) continue;       // (few units: not measured)
+        if (two(t) < (best ? 0.98 : 1.0) * t_best) {    // (a tile more only for a gain that shows)
+            t_best = two(t);
             best = t;
         }
     }
@@ -1770,7 +1777,7 @@ wd_status tc_gemm_pair(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, 
         // tiles per pair (no partial sums)
         static const int swiglu_fused = env_int("WD_GEMM_SWIGLU", 1);
         if (sg && sg->h && swiglu_fused && !fp8 && nseg == 2 && segs[0].n == segs[1].n && dual_mode != 0)
-            gu_tok_tiles = gate_up_tok_tiles((segs[0].n + p.tile_rows - 1) / p.tile_rows, (K + kBK - 1) / kBK, rows, (int)pairs, segs[0].n);
+            gu_tok_tiles = gate_up_tok_tiles((segs[0].n + p.tile_rows - 1) / p.tile_rows, (K + kBK - 1) / kBK, rows, (int)pairs, segs[0].n, p.dual == 1);
         if (gu_tok_tiles > 0) p.dual = 2;
         // one accumulator: whole units (with RoPE or the residual add in their epilogue where the launch has one: with shares of the
         // K-block line a tile's sum is in several pieces), or shares

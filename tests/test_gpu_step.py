@@ -104,6 +104,24 @@ def test_gate_up_swiglu_epilogue_with_ragged_ffn_width_and_token_tile():
         assert logs[3]["info"]["n_launches"] == logs[0]["info"]["n_launches"] - 1
 
 
+# the rule that takes it has no holes between row counts: 4096 / 12288 from two token tiles to four, whatever part of a round they fill
+@pytest.mark.parametrize("rows", [320, 360, 384, 416, 440, 464, 512, 583, 704, 1024])
+def test_gate_up_takes_its_epilogue(rows):
+    cfg = synth.get_config("llada8b", L=1, d=4096, Hq=2, Hkv=2, dh=128, F=12288, V=1000, P=rows - 56, G=60)
+    ids = synth.make_prompts(cfg)
+    S = ids.shape[1]
+    ctx = wd.Context(cfg, synth.make_weights(cfg, DEV), 1, S, S, 16)
+    st = wd.State(ctx, ids)
+    launches = []
+    for _ in range(2):
+        _, info = st.step(16, 40, 4, 2, 1)
+        st.sync()
+        launches.append((info["n_rows"], info["n_launches"]))
+    assert launches[0] == (rows, launches[1][1] - 1)        # no SwiGLU kernel
+    st.close()
+    ctx.close()
+
+
 @pytest.mark.parametrize("batch,A", [(2, 160), (4, 150), (4, 250)])
 def test_lm_head_statistics_with_several_token_tiles(batch, A):
     """More than 256 active rows: the LM-head epilogue runs one CTA group per token tile (two
