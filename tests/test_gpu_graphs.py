@@ -97,3 +97,52 @@ def test_a_window_that_keeps_coming_back_is_counted():
     assert ctx.graph_stats() == (1, 1)
     st.close()
     ctx.close()
+
+
+def test_more_windows_than_graphs():
+    """32 windows have graphs; another gets one only once 64 steps had no use for theirs.  The logits are those of direct launches."""
+    runs = []
+    for on in (False, True):
+        cfg, ids, ctx = _context()
+        ctx.set_graphs(on)
+        stream = torch.cuda.Stream(device=DEV)
+        st = wd.State(ctx, ids)
+        logits = torch.zeros(128, cfg["V"], device=DEV)
+        st.set_taps(logits=logits)
+        torch.cuda.synchronize()
+        got, stats = [], []
+        for windows in (list(range(1, 41)), list(range(40, 0, -1)), [50] * 90):
+            for i in range(0, len(windows), 10):
+                _steps(st, windows[i:i + 10], stream)
+                got.append(logits.clone())      # of the ten's last step, and what larger ones left behind
+            stats.append(ctx.graph_stats())
+        runs.append((got, stats))
+        st.close()
+        ctx.close()
+    assert all(torch.equal(a, b) for a, b in zip(runs[0][0], runs[1][0], strict=True))
+    assert runs[0][1] == [(0, 0)] * 3
+    # 1 to 32 recorded, then replayed.  Window 32, the first of those to be used for the last time, was step 54 of 88 (each ten has
+    # one of 64 active before it): step 119, the 28th of the window of 50, gets its place
+    assert runs[1][1] == [(32, 0), (32, 32), (33, 32 + 90 - 28)]
+
+
+def test_bf16_steps_synced_one_by_one():
+    """A caller that waits for every step: the steps recorded with nothing queued, and those replayed, are the ones launched directly."""
+    runs = []
+    for on in (False, True):
+        cfg, ids, ctx = _context(**BF16)
+        ctx.set_graphs(on)
+        stream = torch.cuda.Stream(device=DEV)
+        st = wd.State(ctx, ids)
+        outs = []
+        for _ in range(40):
+            st.step(8, 100, 20, 1, 1, stream)
+            outs.append(st.sync())
+        runs.append((st.read(0)["ids"], outs, ctx.graph_stats()))
+        st.close()
+        ctx.close()
+    assert np.array_equal(runs[0][0], runs[1][0])
+    for a, b in zip(runs[0][1], runs[1][1], strict=True):
+        assert all(np.array_equal(a[n], b[n]) for n in ("n_unmasked", "positions", "token_ids", "confidence"))
+    # two phases (of one and two key tiles) of a refresh and nineteen normal steps, the ninth of which is recorded
+    assert runs[0][2] == (0, 0) and runs[1][2] == (2, 20)
