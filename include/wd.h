@@ -163,7 +163,7 @@ typedef struct wd_step_out {
  * half of them active, computes the last block for the active rows only (nothing else reads its output), and its
  * products there are split otherwise, so that the logits of a step with and without these two taps may
  * differ in their last bits.  logits alone changes nothing: the LM head writes there instead of to its own
- * buffer. */
+ * buffer, or behind a step replayed from a graph (wd_set_graphs) a copy fills it. */
 typedef struct wd_debug_taps {
     float* layer_out;
     float* attn_out;
@@ -235,17 +235,24 @@ WD_API wd_status wd_set_fusion(wd_ctx* ctx, int32_t mode);
 
 /* CUDA graphs for the kernels of a step (Section 4.3: the normal steps of a phase repeat the same
  * launch configuration).  On by default.  A step that the device plans (see wd_step) and whose launch
- * configuration — batch, computed rows, active rows, query tiles, key tiles, projection mode — recurs is
- * recorded into a graph (a normal step with full active windows at once, any other step the second time its
- * configuration occurs) and replayed
- * from then on (at most 8 graphs per context, least recently used replaced); the planner kernel and the
- * copy of the result block stay ordinary launches on the caller's stream.  bf16 models need the
- * tensor-core kernels (head_dim 128) for it.  Graphs are used only while earlier steps are still queued: a caller that calls
- * wd_step_sync after every step gets direct launches, which are faster then.  Steps with debug taps, with
- * profiling on, with a fused-consumer mode, planned on the host, or issued on a stream that is itself being
- * captured or that cannot be captured (the legacy default stream) are launched directly.  Results are
- * bit-identical either way.  wd_debug_graph_stats reports how many graphs were recorded and how many steps
- * were replayed since the context was created. */
+ * configuration — state, batch, computed rows, active rows, query tiles, key tiles, projection mode — recurs is
+ * recorded into a graph, from the embedding to the selection, and replayed from then on; the planner kernel
+ * stays an ordinary launch on the caller's stream.
+ * When a configuration is recorded: while earlier steps are queued, that of a normal step with full active
+ * windows at once, any other the second time that it occurs.  With nothing queued (a caller that calls
+ * wd_step_sync after every step) recording keeps the GPU waiting, about 1.3 ms for a step of 32 blocks and
+ * 0.1 ms for one of two, and is left until the configuration has occurred 8 times before, in an fp32 model 32 times.
+ * A context keeps at most 32 graphs.  With that many, one gives way only if its state has been destroyed
+ * or if the last 64 steps that could have been replayed had no use for it; until then other configurations are launched
+ * directly.
+ * bf16 models need the tensor-core kernels (head_dim 128) for it.  Steps with debug taps (of an fp32 model:
+ * taps of the blocks; its logits tap is filled by a copy behind the graph), with profiling on, with a
+ * fused-consumer mode, planned on the host, or issued on a stream that is itself being captured or that cannot
+ * be captured (the legacy default stream) are launched directly.  Results are bit-identical either way.
+ * While a step is being recorded the CUDA runtime refuses work that another thread gives to the legacy default stream,
+ * unless the step's stream was created with cudaStreamNonBlocking.
+ * wd_debug_graph_stats reports how many graphs were recorded and how many steps were replayed since the
+ * context was created. */
 WD_API wd_status wd_set_graphs(wd_ctx* ctx, int32_t on);
 WD_API wd_status wd_debug_graph_stats(const wd_ctx* ctx, int32_t* captured, int32_t* replayed);
 

@@ -67,8 +67,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // One lane of the (converged) warp, the same in every call.
 // The loops that issue TMA and MMA instructions are run by their whole warp, and only the instructions themselves by this lane: their
 // operands (barriers, descriptors, coordinates) then stay in uniform registers, which these instructions take.  In a branch that one
-// lane runs alone each operand is moved there first: four tcgen05.mma and a commit took 400 cycles to issue, 203 like this (and the
-// three instructions of a stage's loads 292), with the waits 620 cycles a K block of the two-CTA GEMM whatever its token tile.
+// lane runs alone each operand is moved there first: in the two-CTA GEMM four tcgen05.mma and a commit took 400 cycles to issue, 250
+// like this, the instructions of a stage's loads 292 and 250, and a K block with the waits 620 whatever its token tile, 353 at 64 tokens.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(p));

@@ -351,7 +351,7 @@ void launch(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaS
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-constexpr int kFusedBlocks = 9 * 148;       // see wd_launch_gemm_plain_fused
+constexpr int kFusedBlocks = 9 * 148;       // nine to an SM of a B200, see wd_launch_gemm_plain_fused
 
 template <typename T, bool kVec, int kEpi = kEpiNone, bool kNorm = false>
 void launch_rows(const void* x, const Segs& segs, float* y, int rows, int n, int k, int ldy, bool w_static, cudaStream_t st,

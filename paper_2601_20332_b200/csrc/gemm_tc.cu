@@ -1639,10 +1639,12 @@ int count_slices(int n_units, int kb_total, long long W, long long G) {
 
 // Number of equal shares of the K-block line: the blocks of the longest, t_block each, against the slices that the split leaves, a
 // write and a re-read (t_slice) and 0.3 us each (zeros where nobody wrote one, a place in the chain of the kernel that adds them).
+// t_block is a CTA's part of the HBM rate beside 147 others, 45 GB/s of weights, 63 with the token block of a few rows beside them.
 // Tried are all of most CTAs and the grids with which shares start with a tile every few tiles.  Measured against all 148, in us a
-// block (LLaDA shape at 34 rows): q/k/v with 144 shares, two slices instead of three, -0.7; output projection with 128, four instead
-// of six, -0.5; down with 144 -0.3; gate/up stays at 148 (two slices either way; 144 +0.8).  Dream shape, 35 rows: q/k/v 144 -0.7,
-// output projection 140 -0.9.
+// block: LLaDA shape, 34 rows: q/k/v with 144 shares, two slices instead of three, -1.1; output projection with 128, four instead
+// of six, -0.4 (96, three: another -0.4); down with 144 -0.2; gate/up stays at 148 (two slices either way; 144 +0.6).  66 rows: q/k/v
+// -1.2, output projection -0.4, down -0.7; 136 rows: q/k/v -2.6, the others within their noise of 1.  Dream shape, 35 rows: q/k/v 144
+// -0.4, output projection 140 -0.9.
 long long choose_shares(int n_units, int kb_total, int most, double t_block, double t_slice) {
     const long long W = (long long)n_units * kb_total;
     auto cost = [&](long long G) { return (double)((W + G - 1) / G) * t_block + (wd_tc_sharers(n_units, (int)G) - 1) * (t_slice + 0.3e-6); };

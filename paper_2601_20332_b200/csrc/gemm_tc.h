@@ -137,8 +137,6 @@ struct WdTcEpi {
     const WdTcResid* resid = nullptr;
 };
 
-// y[split][rows][sum n_i] = x * [w_0; w_1; ...]^T, split-K partial sums side by side
-// (split_stride = rows * sum n_i floats).  The consumer adds the slices.
 // Most CTAs that share a unit when the line of n units is cut into G equal shares: with G / n = a + r / q in lowest terms a unit
 // covers at most ceil((q - 1) / q + G / n) of them.
 inline int wd_tc_sharers(int n, int G) {
@@ -149,6 +147,8 @@ inline int wd_tc_sharers(int n, int G) {
     return a + (r / q == 1 ? 1 : 2);
 }
 
+// y[split][rows][sum n_i] = x * [w_0; w_1; ...]^T, split-K partial sums side by side
+// (split_stride = rows * sum n_i floats).  The consumer adds the slices.
 wd_status wd_tc_gemm(const WdTcX* x, const WdTcSeg* segs, int nseg, int rows, int K, float* y, size_t y_floats,
                      int sm_count, int32_t* status, cudaStream_t stream, int* n_split_out,
                      bool force_single_split = false, const WdTcFuse* fuse = nullptr, const WdTcFp8* fp8 = nullptr,
