@@ -362,7 +362,8 @@ void launch_rows(const void* x, const Segs& segs, float* y, int rows, int n, int
         // Four rows to a warp while the grid stays small (nine rows waste less, and each warp has half the loads and sums in its
         // chain); then also the whole of k up to 768 in one go, one round trip instead of two.  Step of the fp32 model, two blocks of
         // 256 / 688: 9 rows 63 -> 52 us, 40 81 -> 72, 72 98 -> 89; with 13 blocks to an SM instead of nine 96.  (The add after a
-        // short k is the exception: eight rows 2.3 us, four 3.7, always; not understood.)
+        // short k is the exception: eight rows 2.1-2.4 us, four 3.7-3.8, in either block of the step, with a graph and without, and the
+        // step 47.5 -> 50.9 us.  The cause was not found.)
         if (!(kEpi == kEpiAdd && k <= 256) && (long long)wd_ceil_div(n, 16) * wd_ceil_div(rows, 4) <= kFusedBlocks) {
             r = 4;
             kernel = k <= 256 ? gemm_rows_kernel<T, 4, 2, kVec, kEpi, kNorm>
